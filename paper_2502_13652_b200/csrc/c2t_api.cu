@@ -83,9 +83,7 @@ size_t carve(const c2t_config *c, void *base, TreeState *t) {
   const size_t B = c->batch, F = c->frontier_cap, K = c->topk;
   const size_t cap = tree_capacity_unchecked(c), Nw = c2t_final_width(c);
   const int eb = c->dtype == C2T_BF16 ? 2 : 4;
-  // (expand workers outnumber arg-max CTAs, and their spans may be shorter)
-  const size_t ms = max_splits_for(c->vocab, eb, kMaxSms * kExpandCtasPerSm * kExpandWarps, kSegmentPad,
-                                   expand_min_span(c->vocab, eb, c->topk));
+  const size_t ms = max_splits_for(c->vocab, eb, kMaxSms * kPassCtasPerSm);
   TreeState s;
   memset(&s, 0, sizeof s);
   for (int i = 0; i < 2; ++i) {
@@ -124,15 +122,21 @@ size_t carve(const c2t_config *c, void *base, TreeState *t) {
   s.info_target = w.take<PassInfo>(1);
   s.row_off_draft = w.take<int32_t>(B + 1);
   s.topm = w.take<double2>(B * F);
+  // every segment of the expand pass (with M > 0) ends a warp's span or a row
+  const size_t segs = B * F + (size_t)kMaxSms * kExpandWarps;
+  s.n_segs = (int64_t)segs;
+  s.n_chunks = (int64_t)(B * F * row_chunks(c->vocab, eb));
   if (c->entropy_top_m > 0 && c->entropy_top_m < c->vocab) {   // the expand pass sets Eq. 3's candidates aside
     s.topm_pool_vecs = (long long)topm_pool_vectors(B, F, c->vocab, eb);
     s.topm_pool = w.take<uint4>((size_t)s.topm_pool_vecs);
-    s.topm_seg = w.take<TopmSegment>(B * F * ms);
+    s.topm_seg = w.take<TopmSegment>(segs);
     s.topm_done = w.take<int32_t>(B * F);
   }
-  s.part_stats = w.take<float4>(B * F * ms);
-  s.part_keys = w.take<unsigned long long>(B * F * ms * K);
-  s.part_held = w.take<unsigned long long>(B * F * ms * kHeldPerSlot);
+  s.rows = w.take<RowResult>(B * F);
+  s.row_keys = w.take<unsigned long long>(B * F * K);
+  s.row_done = w.take<int32_t>(B * F);
+  s.cells = w.take<uint32_t>((size_t)s.n_chunks * 32);
+  s.sums = w.take<SumRecord>((size_t)s.n_chunks);
   s.part_best = w.take<unsigned long long>(B * Nw * ms);
   s.w1 = w.take<float>(3 * C2T_MAX_HIDDEN);
   s.b1 = w.take<float>(C2T_MAX_HIDDEN);
@@ -140,6 +144,22 @@ size_t carve(const c2t_config *c, void *base, TreeState *t) {
   s.b2 = w.take<float>(4);
   if (t) *t = s;
   return (w.off + 255) & ~(size_t)255;
+}
+
+// the expand pass of a level over rows of `vocab` tokens (the whole vocabulary, or one shard of it)
+PassParams expand_params(const TreeState &t, int level, const void *logits, int64_t seq_stride, int64_t row_stride, int vocab) {
+  PassParams p;
+  memset(&p, 0, sizeof p);
+  p.logits = logits; p.seq_stride = seq_stride; p.row_stride = row_stride;
+  p.V = vocab; p.K = t.K; p.B = t.B; p.rows_per_seq_max = t.F;
+  p.counts = t.frontier_n[level & 1];
+  p.status = t.status;
+  p.info = t.info_draft;
+  p.row_off = t.row_off_draft;
+  p.rows = t.rows; p.row_keys = t.row_keys; p.row_done = t.row_done;
+  p.cells = t.cells; p.sums = t.sums;
+  p.n_chunks = t.n_chunks; p.n_segs = t.n_segs;
+  return p;
 }
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
@@ -199,7 +219,7 @@ int c2t_init(const c2t_config *cfg, void *workspace_dev, size_t workspace_bytes,
   ctx->cfg = *cfg;
   ctx->cfg.w1 = ctx->cfg.b1 = ctx->cfg.w2 = ctx->cfg.b2 = nullptr;
   ctx->grid = grid;
-  ctx->grid_expand = grid / kPassCtasPerSm * kExpandCtasPerSm;
+  ctx->grid_expand = grid / kPassCtasPerSm;
   ctx->elem_bytes = cfg->dtype == C2T_BF16 ? 2 : 4;
   carve(cfg, workspace_dev, &ctx->t);
   TreeState &t = ctx->t;
@@ -209,9 +229,8 @@ int c2t_init(const c2t_config *cfg, void *workspace_dev, size_t workspace_bytes,
   t.hidden = cfg->classifier == C2T_CLS_MLP ? cfg->hidden : 0;
   t.classifier = cfg->classifier; t.tree_add = cfg->tree_add; t.beta = cfg->threshold;
   t.entropy_top_m = cfg->entropy_top_m;
-  t.min_span = expand_min_span(cfg->vocab, (int)ctx->elem_bytes, cfg->topk);
-  t.max_splits = max_splits_for(cfg->vocab, (int)ctx->elem_bytes, ctx->grid_expand * kExpandWarps, kSegmentPad, t.min_span);
-  t.max_splits_tgt = max_splits_for(cfg->vocab, (int)ctx->elem_bytes, ctx->grid, 0);
+  t.topm_place = topm_floor_place(cfg->vocab, (int)ctx->elem_bytes, cfg->entropy_top_m);
+  t.max_splits_tgt = max_splits_for(cfg->vocab, (int)ctx->elem_bytes, ctx->grid);
 
   cudaError_t e = cudaSuccess;
   if (cfg->classifier == C2T_CLS_MLP) {
@@ -223,6 +242,7 @@ int c2t_init(const c2t_config *cfg, void *workspace_dev, size_t workspace_bytes,
   }
   if (e == cudaSuccess) e = cudaMemset(t.status, 0, sizeof(uint32_t) * cfg->batch);
   if (e == cudaSuccess) e = cudaMemset(t.ticket, 0, sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMemset(t.row_done, 0, sizeof(int32_t) * cfg->batch * cfg->frontier_cap);
   if (e != cudaSuccess) { cudaGetLastError(); delete ctx; return C2T_ECUDA; }
   *out = ctx;
   return C2T_OK;
@@ -253,20 +273,9 @@ int c2t_expand_level(c2t_ctx *ctx, int level, const void *logits_dev, int64_t se
   if (!aligned16(logits_dev) || (seq_stride * ctx->elem_bytes) % 16 || (row_stride * ctx->elem_bytes) % 16)
     return C2T_EALIGN;
   const TreeState &t = ctx->t;
-  PassParams p;
-  memset(&p, 0, sizeof p);
-  p.logits = logits_dev; p.seq_stride = seq_stride; p.row_stride = row_stride;
-  p.V = t.V; p.K = t.K; p.B = t.B; p.rows_per_seq_max = t.F;
-  p.counts = t.frontier_n[level & 1];
-  p.max_splits = t.max_splits;
-  p.min_span = t.min_span;
-  p.n_slots = (int64_t)t.B * t.F * t.max_splits;
-  p.status = t.status;
-  p.info = t.info_draft;
-  p.part_stats = t.part_stats; p.part_keys = t.part_keys; p.part_held = t.part_held;
-  p.row_off = t.row_off_draft;
+  PassParams p = expand_params(t, level, logits_dev, seq_stride, row_stride, t.V);
   const bool truncated = t.entropy_top_m > 0 && t.entropy_top_m < t.V;   // Eq. 3: the sums over the M most probable tokens
-  if (truncated) { p.topm_pool = t.topm_pool; p.topm_pool_vecs = t.topm_pool_vecs; p.topm_seg = t.topm_seg; }
+  if (truncated) { p.topm_pool = t.topm_pool; p.topm_pool_vecs = t.topm_pool_vecs; p.topm_seg = t.topm_seg; p.topm_place = t.topm_place; }
   if (launch_expand_pass(p, ctx->cfg.dtype, ctx->grid_expand, (cudaStream_t)stream) != cudaSuccess)
     return C2T_ECUDA;
   ctx->launches += 1;
@@ -315,18 +324,7 @@ int c2t_expand_prune_level(c2t_ctx *ctx, int level, const void *logits_dev, int6
   if (seq_stride < 0 || row_stride < ctx->cfg.vocab) return C2T_EINVAL;
   if (!aligned16(logits_dev) || (seq_stride * ctx->elem_bytes) % 16 || (row_stride * ctx->elem_bytes) % 16)
     return C2T_EALIGN;
-  PassParams p;
-  memset(&p, 0, sizeof p);
-  p.logits = logits_dev; p.seq_stride = seq_stride; p.row_stride = row_stride;
-  p.V = t.V; p.K = t.K; p.B = t.B; p.rows_per_seq_max = t.F;
-  p.counts = t.frontier_n[level & 1];
-  p.max_splits = t.max_splits;
-  p.min_span = t.min_span;
-  p.n_slots = (int64_t)t.B * t.F * t.max_splits;
-  p.status = t.status;
-  p.info = t.info_draft;
-  p.part_stats = t.part_stats; p.part_keys = t.part_keys; p.part_held = t.part_held;
-  p.row_off = t.row_off_draft;
+  PassParams p = expand_params(t, level, logits_dev, seq_stride, row_stride, t.V);
   if (launch_expand_prune(p, t, level, out, ctx->cfg.dtype, ctx->grid_expand, (cudaStream_t)stream) != cudaSuccess)
     return C2T_ECUDA;
   ctx->launches += 1;
@@ -345,18 +343,7 @@ int c2t_expand_level_shard(c2t_ctx *ctx, int level, const void *logits_dev, int6
   if (!aligned16(logits_dev) || (seq_stride * ctx->elem_bytes) % 16 || (row_stride * ctx->elem_bytes) % 16)
     return C2T_EALIGN;
   const TreeState &t = ctx->t;
-  PassParams p;
-  memset(&p, 0, sizeof p);
-  p.logits = logits_dev; p.seq_stride = seq_stride; p.row_stride = row_stride;
-  p.V = vocab_count; p.K = t.K; p.B = t.B; p.rows_per_seq_max = t.F;
-  p.counts = t.frontier_n[level & 1];
-  p.max_splits = t.max_splits;                    // sized for whole rows: enough for any part of one
-  p.min_span = t.min_span;
-  p.n_slots = (int64_t)t.B * t.F * t.max_splits;
-  p.status = t.status;
-  p.info = t.info_draft;
-  p.part_stats = t.part_stats; p.part_keys = t.part_keys; p.part_held = t.part_held;
-  p.row_off = t.row_off_draft;
+  PassParams p = expand_params(t, level, logits_dev, seq_stride, row_stride, vocab_count);
   if (launch_expand_pass(p, ctx->cfg.dtype, ctx->grid_expand, (cudaStream_t)stream) != cudaSuccess)
     return C2T_ECUDA;
   ctx->launches += 1;
@@ -370,7 +357,7 @@ int c2t_export_row_records(c2t_ctx *ctx, int level, int32_t vocab_begin, c2t_row
   if (!ctx || !records_dev) return C2T_EINVAL;
   if (!ctx->shard_expanded || level != ctx->next_level) return C2T_EORDER;
   if (vocab_begin < 0 || (int64_t)vocab_begin + ctx->shard_vocab > ctx->cfg.vocab) return C2T_EINVAL;
-  if (launch_export_rows(ctx->t, level, ctx->shard_vocab, vocab_begin, records_dev, (cudaStream_t)stream) !=
+  if (launch_export_rows(ctx->t, level, vocab_begin, records_dev, (cudaStream_t)stream) !=
       cudaSuccess)
     return C2T_ECUDA;
   ctx->launches += 1;

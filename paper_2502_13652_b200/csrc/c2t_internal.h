@@ -87,30 +87,32 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
 constexpr int kPassThreads = 512;     // threads per CTA of the vocabulary pass
 constexpr int kPassCtasPerSm = 2;
 constexpr int kMinSpanVectors = 1024; // a CTA never gets fewer 16-byte vectors than this
-// the expand pass: every warp is a worker of its own (a span of the rows, its own partial records).
-// 20 warps per SM: 96 registers per thread (no spills) and fewer segments to open than with 24; measured
-// 3 % faster than 24 warps and 4 % faster than 16.
-constexpr int kExpandThreads = 640;
-// 16-byte vectors a lane holds of one group (a group is 32 times this).  Measured on 640 rows of 128256 bf16 logits:
-// 4 with 20 warps 44 us; 2 with 24 warps 45 us; 8 with 10 or 14 warps 67 us.
-constexpr int kExpandVecPerLane = 4;
-constexpr int kExpandCtasPerSm = 1;
-constexpr int kExpandWarps = kExpandThreads / 32;
-// Opening a segment (filter warm-up, extra drains while the filter is still loose, the record)
-// costs a warp about as much as streaming this many vectors (measured: the 640-row level is
-// fastest with 1024 to 2048).  The expand pass cuts the rows into spans of equal COST: every row
-// is preceded by this many virtual vectors, the padded rows are laid end to end and cut evenly,
-// and a worker streams the real vectors of its piece.
-constexpr int kSegmentPad = 1024;
-constexpr int kHeldPerSlot = 1;       // exact keys held out of the fp32 sums per partial record
+// the expand pass: one CTA per SM, 12 warps that stream and 4 that complete rows
+constexpr int kExpandWarps = 12;
+constexpr int kExpandThreads = (kExpandWarps + 4) * 32;
+constexpr int kChunkVecs = 512;       // 16-byte vectors of a chunk: 16 per lane
 
 // What one launch of the vocabulary pass derived from the device-side row counts.
 struct PassInfo {
   int32_t n_rows;       // active rows
   int32_t vec_per_row;  // 16-byte vectors per row (last one may be ragged)
-  int64_t span;         // vectors per worker (a CTA of the arg-max pass, a warp of the expand pass)
-  int32_t pad;          // expand pass: virtual vectors in front of every row (see kSegmentPad), else 0
-  int32_t reserved;
+  int64_t span;         // vectors per CTA (the expand pass counts both in chunks)
+};
+
+// What the expand pass leaves per active row, at (b, j) of [B, F]; its K largest keys are in row_keys.
+struct RowResult {
+  double M, S, T, L;            // row maximum; sums over every other element of e^(x - M) and e^(x - M)(x - M); ln(1 + S)
+  unsigned long long top;       // the row's best key (0: none)
+  int32_t n_valid;              // keys that exist (at most K)
+  uint32_t fault;               // C2T_ST_* bits of the row's data
+};
+
+// The sums over the chunks of a row that one warp streamed, base 2, relative to an integer offset; the lane and chunk with
+// the largest value are kept apart, so that a row can be completed without its largest element by summing one lane's
+// vectors of one chunk again.
+struct alignas(16) SumRecord {
+  float4 rest;                  // S and U of everything else, the offset, the largest value
+  float4 held;                  // S and U of that lane and chunk, their numbers (as int bits)
 };
 
 struct TopmSegment;
@@ -122,34 +124,38 @@ struct PassParams {
   int32_t rows_per_seq_max;         // F (draft) or Nw (target)
   const int32_t *counts;            // [B] active rows per sequence, device
   const int32_t *row_sel;           // arg-max pass only, may be null: [B] the row of sequence b to read (then counts is 0 or 1)
-  int32_t max_splits;               // partial slots per row
-  int32_t min_span;                 // expand: the fewest vectors a worker gets (expand_min_span)
-  int64_t n_slots;                  // partial slots in the workspace (rows the workspace was carved for x max_splits)
+  int32_t max_splits;               // arg-max: partial slots per row
+  int64_t n_slots;                  // arg-max: partial slots in the workspace (rows the workspace was carved for x max_splits)
   uint32_t *status;                 // may be null: a status word for C2T_ST_INTERNAL (the first sequence's)
-  PassInfo *info;                   // written by CTA 0
-  int32_t *row_off;                 // may be null: [B+1] first active row of every sequence, written by CTA 0
-  // expand: per (row, split) partial
-  float4 *part_stats;               // {offset c, S, U, n_keys as int bits}: base-2 sums, see expand_pass.cu
-  unsigned long long *part_keys;    // [.. * K] the segment's K largest keys, sorted descending, 0-padded
-  unsigned long long *part_held;    // [.. * kHeldPerSlot] keys excluded from S and U (0 = none)
-  // expand with M > 0 (else null): the pool of candidate vectors, cut evenly among the workers, and a record per (row, split)
+  PassInfo *info;                   // written by CTA 0 (expand: only with M > 0)
+  int32_t *row_off;                 // expand with M > 0: [B+1] first active row of every sequence, written by CTA 0
+  // expand: results per row, and what the warps that stream a row leave for the pair that completes it
+  RowResult *rows;                  // [B, F]
+  unsigned long long *row_keys;     // [B, F, K] the row's K largest keys, sorted descending, 0-padded
+  int32_t *row_done;                // [B * F] finished chunks of a row shared by several CTAs; 0 between launches
+  uint32_t *cells;                  // [chunk, 32] lane maxima (expand_pass.cu)
+  SumRecord *sums;                  // [chunk] at a warp's last chunk of a row
+  int64_t n_chunks, n_segs;
+  int32_t cta_tasks;                // barriers in a CTA's shared memory (set at launch)
+  // expand with M > 0 (else null): the pool of candidate vectors, cut evenly among the warps, and a record per segment
   uint4 *topm_pool;
   long long topm_pool_vecs;
-  TopmSegment *topm_seg;
+  int32_t topm_place;               // the floor's place among the lane maxima (topm_floor_place)
+  TopmSegment *topm_seg;            // [warp + row]
   // argmax: per (row, split) best key
   unsigned long long *part_best;
 };
 
 // ---------------------------------------------------------------- candidates of the truncated entropy (Eq. 3)
 // With entropy_top_m = M > 0 the expand pass also sets aside every 16-byte vector that holds an element at or above
-// a floor of its segment: the kTopmRank-th largest of the 32 lane maxima over the segment's first two groups, about
-// the top 2 % of the elements seen there (M = 1000 of 128256 is the top 0.8 %).  The vectors go, in stream order, to
+// a floor of its segment (the part of a row that one warp streams): one of the 32 lane maxima over the segment's first two
+// groups, the place among them chosen so that about 3 M of the row's elements reach it (if the segment's head looks like
+// the row).  The vectors go, in stream order, to
 // a region of the warp's own in a pool in global memory; the segment's record says where they are and what the floor
 // was.  A small kernel per row then takes the elements at or above the row's highest floor F from those vectors: if
 // there are at least M of them the M-th largest is among them and so is everything above it, and Eq. 3's sums follow
 // without reading the row again.  Rows for which that fails (a region ran full, fewer than M elements at or above F,
 // more than fit in shared memory) are left to the pass that reads the row again.
-constexpr int kTopmRank = 24;
 constexpr int kTopmPoolDivisor = 3;      // the pool holds a third of the largest level's vectors (twice what is expected)
 constexpr float kTopmLowestFloor = -1.7e38f;   // above -2^127, the value that pads a ragged vector
 struct TopmSegment {
@@ -158,27 +164,23 @@ struct TopmSegment {
   float floor;
   int pad;
 };
+int topm_floor_place(int vocab, int elem_bytes, int M);
 size_t topm_pool_vectors(size_t batch, size_t rows_per_seq, int vocab, int elem_bytes);
 
-// partial slots a row can need; workers: CTAs (arg-max, pad 0) or warps (expand, pad kSegmentPad)
-int max_splits_for(int vocab, int elem_bytes, int workers, int pad, int min_span = kMinSpanVectors);
-// Keys of a row's partial lists that one warp of the row merge stages in shared memory; a row with more takes a slow path.
-constexpr int kStageKeys = 320;
-// The fewest vectors a worker of the expand pass gets: as few as the row merge allows (at most 31 partial lists per
-// row, and K keys apiece must fit the staging area), so that launches with few rows still spread over the chip.
-int expand_min_span(int vocab, int elem_bytes, int K);
+int max_splits_for(int vocab, int elem_bytes, int workers);   // partial slots a row of the arg-max pass can need
+int row_chunks(int vocab, int elem_bytes);                     // chunks of a row of the expand pass
 
 cudaError_t prepare_expand_pass();   // once per device: opt in to the kernel's shared-memory size
-cudaError_t launch_expand_pass(const PassParams &p, int dtype, int grid, cudaStream_t s);
+cudaError_t launch_expand_pass(PassParams p, int dtype, int grid, cudaStream_t s);
 cudaError_t launch_argmax_pass(const PassParams &p, int dtype, int grid, cudaStream_t s);
 struct TreeState;
 // expand and prune of a level in one launch (batches of at most C2T_FUSED_MAX_BATCH sequences)
-cudaError_t launch_expand_prune(const PassParams &p, const TreeState &t, int level, const c2t_frontier *out, int dtype,
+cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, const c2t_frontier *out, int dtype,
                                 int grid, cudaStream_t s);
 // ---------------------------------------------------------------- tree state -
 
 struct TreeState {
-  int32_t B, V, K, F, D, N, Nw, W, cap, hidden, classifier, tree_add, max_splits, max_splits_tgt, min_span;
+  int32_t B, V, K, F, D, N, Nw, W, cap, hidden, classifier, tree_add, max_splits_tgt;
   float beta;
   // frontier, double buffered by level parity
   int32_t *frontier_n[2];      // [B]
@@ -198,19 +200,22 @@ struct TreeState {
   int32_t *node_argmax;        // [B, Nw]
   int32_t *root_tok, *prefix_len;                   // [B]
   int32_t *walk_active, *walk_cur, *walk_len;       // [B] state of the lazy acceptance walk
-  int32_t entropy_top_m;       // M of Eq. 3 (0: exact entropy)
+  int32_t entropy_top_m, topm_place;   // M of Eq. 3 (0: exact entropy); the place of the collection floor
   double2 *topm;               // [B, F] {S_M, T_M} of the last expand call when M > 0
   uint4 *topm_pool;            // M > 0: candidate vectors set aside by the expand pass
   long long topm_pool_vecs;
-  TopmSegment *topm_seg;       // M > 0: [B * F * max_splits] where each segment's candidates are
+  TopmSegment *topm_seg;       // M > 0: [n_segs] where each segment's candidates are
   int32_t *topm_done;          // M > 0: [B, F] 1 where the row's sums came from the candidate vectors
   uint32_t *status;            // [B]
   uint32_t *ticket;            // one counter: CTAs of a fused expand + prune launch that have finished (0 between launches)
   PassInfo *info_draft, *info_target;
   int32_t *row_off_draft;          // [B+1] first row of every sequence in the last expand pass
-  float4 *part_stats;
-  unsigned long long *part_keys;
-  unsigned long long *part_held;
+  RowResult *rows;                 // the expand pass: see PassParams
+  unsigned long long *row_keys;
+  int32_t *row_done;
+  uint32_t *cells;
+  SumRecord *sums;
+  int64_t n_chunks, n_segs;
   unsigned long long *part_best;
   float *w1, *b1, *w2, *b2;
 };
@@ -231,8 +236,7 @@ cudaError_t launch_begin_step(const TreeState &t, const int32_t *root_tok, const
 // records == nullptr: rows merged from this context's own expand pass; else from n_shards gathered records per row
 cudaError_t launch_prune_level(const TreeState &t, int level, const c2t_frontier *out, const c2t_row_record *records,
                                int n_shards, cudaStream_t s);
-cudaError_t launch_export_rows(const TreeState &t, int level, int vocab_count, int vocab_begin, c2t_row_record *out,
-                               cudaStream_t s);
+cudaError_t launch_export_rows(const TreeState &t, int level, int vocab_begin, c2t_row_record *out, cudaStream_t s);
 cudaError_t launch_final_prune(const TreeState &t, cudaStream_t s);
 cudaError_t launch_build_verify(const TreeState &t, const c2t_verify *out, cudaStream_t s);
 cudaError_t launch_dense_mask(const TreeState &t, void *out, int out_dtype, int64_t kv_len, cudaStream_t s);

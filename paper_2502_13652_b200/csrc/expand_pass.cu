@@ -2,462 +2,689 @@
 // softmax normaliser and entropy sums and the K largest logits (ties to the lower token id)
 //                                                        (Sec. 4.2.1, Eq. 2, Sec. 4.2.2).
 //
-// Work partition.  The active rows (a device-side count per sequence) are laid end to end as
-// n_rows * vec_per_row 16-byte vectors and cut into contiguous spans of equal cost, one per WARP
-// of a persistent grid (one CTA of 20 warps per SM).  A span may cover the tail of one row and
-// the head of the next; each (row, warp) piece is a "segment" and produces one partial record.
-// Opening a segment costs about as much as streaming kSegmentPad vectors, so the cut is even
-// in vectors + kSegmentPad per row opened.
-// The pruning kernel merges the partials of a row in double precision.  After one barrier at
-// the start (the row list) the warps never wait for each other: while one warp is between
-// segments the other 19 on the SM keep the memory pipe full.  (One CTA per SM rather than
-// three smaller ones: the warps of an older CTA are served first, and its work would end early.)
+// Work partition.  A row is cut into chunks of 512 consecutive 16-byte vectors (8 KB).  The chunks
+// of the active rows (a device-side count per sequence), laid end to end, are dealt out in
+// contiguous equal ranges, one per CTA of a persistent grid (one CTA per SM).  Most warps of a CTA
+// stream, taking its chunks in turn; the others complete rows, in pairs, as soon as all chunks of
+// a row are done: while the stream goes on, but for the last row.
 //
-// Data movement.  A warp works on groups of 128 consecutive vectors (2 KB), four per lane, 32
-// apart, and owns kRingSlots shared-memory slots of 2 KB: while group n is in registers, groups
-// n+1 .. n+kRingSlots are in flight, across segment boundaries too.  bf16 rows: each lane owns 4 x 16
-// bytes of a slot, fills them with cp.async and reads back only what it copied itself, so the only
-// wait is on its own copies (cp.async.wait_group).  fp32 rows: lane 0 fills a slot with ONE bulk copy
-// (cp.async.bulk: the TMA unit moves the bytes and reports them to the slot's transaction barrier),
-// the warp waits on the barrier (a bounded poll: a wait that runs out sets C2T_ST_INTERNAL instead of
-// hanging), every lane takes its four vectors, and after a warp barrier the slot is requested again.
+// Stream.  A warp keeps one chunk in registers, 16 vectors per lane, in four groups; as soon as a
+// group has been consumed the same registers are requested for the same group of the warp's next chunk,
+// so three to four groups (6 to 8 KB per warp) are in flight all the time.  Per element the
+// stream does nothing but the sums and a running maximum: no comparison with a filter, no vote, no
+// branch that depends on the data.  Selection of the K largest is left to the row's end, where the
+// maxima say where to look.
 //
-// Sums.  In base-2 units relative to a warp-uniform offset c = -m log2(e):  t = x log2(e) + c,
-// S = sum 2^t, U = sum 2^t t  (one unpack, FMA, ex2, add, FMA per element).  m is the largest
-// value the warp has met when c was last set, and only vectors whose elements are all below the
-// filter (hence below m) are summed in the stream, so t <= 0.  (x log2(e) uses the fp32
-// constant: a relative error of 1.3e-8 |x| in an element's weight, far inside tolerance.)
+// Sums.  Per lane, in base-2 units relative to an integer offset c = -rint(m log2(e)), m the largest value of the first
+// group of the row that the warp meets:  t = x log2(e) + c,  S = sum 2^t,  U = sum 2^t t,  two elements at a time (packed
+// fp32 FMA and add).  A chunk with a value more than 100 octaves above m (the first group was all -inf, or a hostile row)
+// is summed again with a better offset.  Offsets are integers so that rescaling is by exact powers of two.  (x log2(e)
+// uses the fp32 constant: a relative error of 1.3e-8 |x| in an element's weight.)
 //
-// Top-K.  A vector with an element at or above the filter is not summed but set aside in the
-// warp's queue in shared memory (ballot-ranked places, so the order is fixed).  When the queue
-// is nearly full, and at the end of the segment, the warp drains it, one element per lane and
-// step: elements below the filter join the sums; the others join a small pool of keys next to
-// the K largest keys found so far, the pool is ranked by counting, the K largest stay and the
-// rest join the sums.  At the end of the segment all of the K largest but the first join the
-// sums too: the segment's largest key stays out and is handed on exactly, so the sums keep fp32
-// relative accuracy with respect to "everything but the maximum" however peaked the row is.
-// The filter starts as the K-th largest lane maximum of the segment's first two groups (K
-// distinct elements are at or above it) and after every drain is just above the K-th largest
-// value so far: later elements of that value have higher token ids and lose the tie.
-// Everything depends only on the warp's own data in a fixed order, so the results are
-// reproducible bit for bit.
+// Top-K.  Every lane records the maxima of its vectors in each half of a chunk, its "cells".  When all chunks of a
+// row are done the row is completed: the K-th largest of the 32 lanes' column maxima
+// is a lower bound on the row's K-th largest element, the few cells that reach it are read again (128 bytes each,
+// usually from L2), their elements at or above the bound are ranked by key, and the warps' sums are merged in double
+// precision.  The row's largest element stays out of the sums, so that they keep fp32 relative accuracy with respect to
+// "everything but the maximum" however peaked the row is: the one lane and chunk that holds it is summed again without it.
+// Everything is computed in an order that does not depend on timing, so the results are reproducible bit for bit.
+#include <math.h>
+
 #include "vocab_common.cuh"
 #include "level_prune.cuh"
 
 namespace c2t {
 namespace {
 
-constexpr int kEWarps = kExpandThreads / 32;
-constexpr int kVPL = kExpandVecPerLane;               // vectors of a group per lane, 32 apart
-constexpr int kGroupVecs = 32 * kVPL;                 // vectors of one group of a warp
-constexpr int kRingSlots = 2;                         // groups in flight per warp behind the one in registers (3 measured 3 % slower)
-constexpr int kDrainAt = 12;                          // queued vectors that trigger a drain: early drains keep the filter tight
-constexpr int kQueueCap = kDrainAt + kGroupVecs;      // a whole group always fits behind kDrainAt vectors
+constexpr int kStreamWarps = kExpandWarps;            // the first warps of a CTA stream ...
+constexpr int kEWarps = kExpandThreads / 32;          // ... the others only complete rows
+constexpr int kPairs = kEWarps / 2;
+constexpr int kGroups = kChunkVecs / 128;             // groups of a chunk; a lane holds 4 vectors of each, 32 apart
+constexpr int kListCap = 128;                         // cells of a row that are read again
+constexpr int kPoolCap = 128;                         // keys ranked at a time
+static_assert(kStreamWarps % 2 == 0 && kPairs <= 15, "pairs of warps, one named barrier each");
 
-// What one warp owns in shared memory.
-constexpr int kPool = 64;                             // keys ranked at a time (the K kept ones and up to 32 + 32 - K new)
-struct WarpShared {
-  uint4 ring[kRingSlots][kGroupVecs];
-  unsigned long long mbar[kRingSlots];  // one transaction barrier per ring slot
-  uint4 qdata[kQueueCap];
-  int qindex[kQueueCap];
-  unsigned long long pool[kPool];      // [0, K): the K largest keys so far, sorted (0 = none); behind them the new ones
-  unsigned long long ranked[C2T_MAX_TOPK];
+// What a pair of warps needs in shared memory to complete a row.
+struct PairShared {
+  unsigned long long pool[kPoolCap];
+  __align__(16) float colmax[64];
+  int list[kListCap], vecs[kListCap];
 };
 
-// ---------------------------------------------------------------- sums
-
-struct Acc {
-  float S0, S1, U0, U1;
+// A CTA's shared memory; behind it a transaction barrier per task (a row, or the CTA's part of one) and the row list.
+struct CtaShared {
+  PairShared scratch[kPairs];
+  int task, flag[kPairs], task_of[kPairs];            // the next task; what the first warp of a pair tells the other
+  int pad;
+  __device__ unsigned long long *bars() { return reinterpret_cast<unsigned long long *>(this + 1); }
 };
 
-// move the offset from c to new_c (the reference only rises, so new_c <= c)
-__device__ __forceinline__ void acc_rescale(Acc &a, float c, float new_c) {
-  const float S = a.S0 + a.S1, U = a.U0 + a.U1;
-  const float d = fmaxf(new_c - c, -1e30f);          // every t shifts by d
-  const float f = ex2f(d);
-  a.S0 = S * f;
-  a.U0 = f * (U + d * S);
-  a.S1 = a.U1 = 0.f;
+// ---------------------------------------------------------------- packed sums
+
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
 }
-
-__device__ __forceinline__ void acc_scalar(Acc &a, float c, float x) {
-  const float t = fmaf(x, kLog2e, c);
-  const float e = ex2f(t);
-  a.S0 += e;
-  a.U0 = fmaf(e, t, a.U0);
+__device__ __forceinline__ void unpack2(f32x2 a, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a)); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
 }
-
-// the sums of one vector; t = x scale + c (scale is log2(e), or 0 to leave the vector out)
-template <bool BF16>
-__device__ __forceinline__ void acc_vector(Acc &a, const uint4 &q, float scale, float c) {
-  float x[Vec<BF16>::N];
-  Vec<BF16>::unpack(q, x);
-#pragma unroll
-  for (int i = 0; i < Vec<BF16>::N; i += 2) {
-    const float t0 = fmaf(x[i], scale, c), t1 = fmaf(x[i + 1], scale, c);
-    const float e0 = ex2f(t0), e1 = ex2f(t1);
-    a.S0 += e0;
-    a.S1 += e1;
-    a.U0 = fmaf(e0, t0, a.U0);
-    a.U1 = fmaf(e1, t1, a.U1);
-  }
-}
-
-// ---------------------------------------------------------------- per-warp state of a segment
-
-struct SegState {
-  Acc acc;                    // per lane
-  float c;                    // warp-uniform offset of the sums, -m log2(e)
-  float m;                    // warp-uniform reference value
-  float thr;                  // warp-uniform filter
-  int qn;                     // warp-uniform: vectors in the queue
-};
-
-struct Group {
-  uint4 q[kVPL];
-};
-
-// ---------------------------------------------------------------- segments of a span
-
-// a / b for non-negative operands; the 32-bit division is much shorter when both fit
-__device__ __forceinline__ long long div_floor(long long a, long long b) {
-  if (((unsigned long long)(a | b) >> 32) == 0) return (long long)((unsigned)a / (unsigned)b);
-  return a / b;
-}
-
-// Position x of the padded rows laid end to end -> position in the real rows laid end to end
-// (a position inside a row's pad is the row's start).
-__device__ __forceinline__ long long real_position(long long x, long long vrow, long long vtotal, int vpr) {
-  if (x >= vtotal) x = vtotal;
-  const long long row = div_floor(x, vrow);
-  const long long off = x - row * vrow - kSegmentPad;
-  return row * vpr + (off > 0 ? off : 0);
-}
-
-
-struct Segment {
-  const char *row;
-  int a, v0, v1;     // vectors [v0, v1) of active row a
-};
-
-struct SegWalk {
-  int a, v0, left, vec_per_row;
-  __device__ SegWalk(long long start, long long end, int vpr) : vec_per_row(vpr) {
-    a = (int)div_floor(start, vpr);
-    v0 = (int)(start - (long long)a * vpr);
-    left = (int)(end - start);
-  }
-  __device__ bool done() const { return left <= 0; }
-  __device__ Segment take(const PassParams &p, const int *s_off, size_t esz) {
-    Segment g;
-    const int room = vec_per_row - v0;
-    const int n = left < room ? left : room;
-    g.a = a; g.v0 = v0; g.v1 = v0 + n;
-    const int b = find_sequence(s_off, p.B, a);
-    const int j = a - s_off[b];
-    g.row = reinterpret_cast<const char *>(p.logits) + ((size_t)b * p.seq_stride + (size_t)j * p.row_stride) * esz;
-    left -= n;
-    ++a;
-    v0 = 0;
-    return g;
-  }
-};
-
-// The groups of a warp's span in order; all lanes hold the same cursor.
-struct GroupCursor {
-  SegWalk walk;
-  Segment seg;     // the segment the current group belongs to
-  int tv0;         // first vector of the current group; the lane's are tv0 + lane + 32 u
-  bool valid;
-  __device__ GroupCursor(long long start, long long end, int vpr, const PassParams &p, const int *s_off, size_t esz)
-      : walk(start, end, vpr) {
-    seg = walk.take(p, s_off, esz);
-    tv0 = seg.v0;
-    valid = true;
-  }
-  __device__ bool last_of_segment() const { return tv0 + kGroupVecs >= seg.v1; }
-  __device__ void advance(const PassParams &p, const int *s_off, size_t esz) {
-    tv0 += kGroupVecs;
-    if (tv0 >= seg.v1) {
-      if (walk.done()) { valid = false; return; }
-      seg = walk.take(p, s_off, esz);
-      tv0 = seg.v0;
-    }
-  }
-};
-
-// ---------------------------------------------------------------- asynchronous prefetch ring
-
-__device__ __forceinline__ unsigned next_slot(unsigned slot) { return slot + 1 == kRingSlots ? 0u : slot + 1; }
-
-// Two ways to fill a ring slot.  bf16 rows: every lane copies its own four vectors with cp.async and waits for its
-// own copies (cp.async.wait_group); the kernel is bound by instruction issue there, and this form needs the fewest
-// issue slots.  fp32 rows (half the elements per byte, so the memory side weighs more): one bulk copy per slot, below;
-// measured on a 640-row level, bulk copies against cp.async: fp32 63.6 against 67.6 us, bf16 50 against 47.2 us.
-template <int OFF>   // both addresses + OFF bytes
-__device__ __forceinline__ void cp_async_16(uint32_t smem_dst, const void *gmem_src) {
-  asm volatile("cp.async.cg.shared.global [%0 + %2], [%1 + %2], 16;" ::"r"(smem_dst), "l"(gmem_src), "n"(OFF) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-// the lane's kVPL copies of a whole group / of a group cut off at vector lim
-template <int U>
-struct LaneCopies {
-  static __device__ __forceinline__ void all(uint32_t dst, const uint4 *src) {
-    LaneCopies<U - 1>::all(dst, src);
-    cp_async_16<(U - 1) * 512>(dst, src);
-  }
-  static __device__ __forceinline__ void below(uint32_t dst, const uint4 *src, int vt, int lim) {
-    LaneCopies<U - 1>::below(dst, src, vt, lim);
-    if (vt + (U - 1) * 32 < lim) cp_async_16<(U - 1) * 512>(dst, src);
-  }
-};
-template <>
-struct LaneCopies<0> {
-  static __device__ __forceinline__ void all(uint32_t, const uint4 *) {}
-  static __device__ __forceinline__ void below(uint32_t, const uint4 *, int, int) {}
-};
-
-// A warp's ring of bulk copies: every slot is filled by ONE bulk copy (the TMA unit moves up to 2 KB from global to shared memory
-// and reports the bytes to the slot's transaction barrier), issued by lane 0.  All lanes hold the same state.
-constexpr int kRingWaitLimit = 1 << 22;               // polls of a barrier before the warp gives up (and says so)
-struct Ring {
-  uint32_t bar0;             // shared-memory address of the first slot's barrier; the others follow at 8 bytes
-  uint32_t phase;            // bit s: parity of the phase slot s's next wait completes
-  uint32_t pending;          // bit s: a copy into slot s was issued and has not been waited for
-  __device__ __forceinline__ void init(WarpShared *ws, int lane) {
-    bar0 = (uint32_t)__cvta_generic_to_shared(&ws->mbar[0]);
-    phase = 0u;
-    pending = 0u;
-    if (lane == 0) {
-#pragma unroll
-      for (int i = 0; i < kRingSlots; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8u * i) : "memory");
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncwarp();
-  }
-  // n_vec whole vectors from src into the slot (lane 0 issues; the slot's last readers are behind a __syncwarp)
-  __device__ __forceinline__ void issue(unsigned s, uint4 *slot, const uint4 *src, int n_vec, int lane) {
-    if (n_vec <= 0) return;
-    if (lane == 0) {
-      const uint32_t bar = bar0 + 8u * s, bytes = (uint32_t)n_vec * 16u;
-      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(slot);
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                   ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-    }
-    pending |= 1u << s;
-  }
-  // until the slot's copy (if one is outstanding) has landed; false if the wait ran out
-  __device__ __forceinline__ bool wait(unsigned s) {
-    if (!((pending >> s) & 1u)) return true;
-    const uint32_t bar = bar0 + 8u * s, par = (phase >> s) & 1u;
-    uint32_t done = 0u;
-    for (int i = 0; i < kRingWaitLimit && !done; ++i)
-      asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                   : "=r"(done) : "r"(bar), "r"(par) : "memory");
-    phase ^= 1u << s;
-    pending &= ~(1u << s);
-    return done != 0u;
-  }
-};
-
-// Requests the whole vectors of the cursor's group into a ring slot.
-template <bool BULK>
-__device__ __forceinline__ void prefetch_group(Ring &ring, unsigned s, const GroupCursor &c, uint4 *slot, int v_full, int lane) {
-  if (c.valid) {
-    const int lim = c.seg.v1 < v_full ? c.seg.v1 : v_full;
-    if (BULK) {
-      const int n = lim - c.tv0;
-      ring.issue(s, slot, reinterpret_cast<const uint4 *>(c.seg.row) + c.tv0, n < kGroupVecs ? n : kGroupVecs, lane);
-    } else {
-      const uint4 *src = reinterpret_cast<const uint4 *>(c.seg.row) + c.tv0 + lane;
-      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(slot + lane);
-      if (c.tv0 + kGroupVecs <= lim) LaneCopies<kVPL>::all(dst, src);
-      else LaneCopies<kVPL>::below(dst, src, c.tv0 + lane, lim);
-    }
-  }
-  if (!BULK) cp_async_commit();
-}
-
-// Until the copies into slot s have landed (cp.async: s is the oldest request, the only one ever waited for).
-template <bool BULK>
-__device__ __forceinline__ bool ring_wait(Ring &ring, unsigned s) {
-  if (BULK) return ring.wait(s);
-  cp_async_wait<kRingSlots - 1>();
-  return true;
-}
-
-// Takes the cursor's group out of a ring slot (its copies have completed) into registers and
-// clamps it.  Vectors past the segment end become -2^127, which adds exactly 0 to the sums; a
-// ragged last vector of a row is assembled from scalar loads.
-template <bool BF16>
-__device__ __forceinline__ void take_group(Group &g, const GroupCursor &c, const uint4 *slot, int v_full, int V,
-                                           int lane) {
-  using VT = Vec<BF16>;
-  const uint32_t lo = BF16 ? kLowestBf16x2 : __float_as_uint(kLowestF32);
-  const int vt = c.tv0 + lane;
-  if (c.tv0 + kGroupVecs <= (c.seg.v1 < v_full ? c.seg.v1 : v_full)) {
-#pragma unroll
-    for (int u = 0; u < kVPL; ++u) g.q[u] = slot[lane + u * 32];
-  } else {
-#pragma unroll
-    for (int u = 0; u < kVPL; ++u) {
-      const int v = vt + u * 32;
-      g.q[u] = make_uint4(lo, lo, lo, lo);
-      if (v < c.seg.v1) g.q[u] = v < v_full ? slot[lane + u * 32] : VT::load(c.seg.row, v, v_full, V);
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < kVPL; ++u) VT::clamp(g.q[u]);
-}
-
-// ---------------------------------------------------------------- start of a segment
-
-// the float just above the value of an orderable word
-__device__ __forceinline__ float value_just_above(uint32_t orderable) {
-  return __uint_as_float(f32_from_orderable(orderable + 1u));
-}
-
-// The filter and the reference of a new segment, from the lane maxima over its first two
-// groups (the first is in registers, the second has landed in the ring: the caller has waited for it); TOPM: also the
-// floor of the candidate collection (.z).
-template <bool BF16, bool TOPM>
-__device__ __noinline__ float4 segment_warmup(int K, Group g, int vt, int v1, int v_full, const uint4 *next_slot) {
-  using VT = Vec<BF16>;
-  const int lane = threadIdx.x & 31;
-  float lmax = -INFINITY;
-#pragma unroll
-  for (int u = 0; u < kVPL; ++u) {
-    if (vt + u * 32 < v1) {
-      const float vm = VT::vmax(g.q[u]);
-      if (vm == vm) lmax = fmaxf(lmax, vm);
-    }
-  }
-  const int lim = v1 < v_full ? v1 : v_full;
-#pragma unroll
-  for (int u = 0; u < kVPL; ++u) {
-    if (vt + kGroupVecs + u * 32 < lim) {  // same segment, whole vector: it is in the ring
-      uint4 q = next_slot[lane + u * 32];
-      VT::clamp(q);
-      const float vm = VT::vmax(q);
-      if (vm == vm) lmax = fmaxf(lmax, vm);
-    }
-  }
-  uint32_t live = f32_orderable(__float_as_uint(lmax)), kth = 0, first = 0, low = 0;
-  const int rounds = TOPM && K < kTopmRank ? kTopmRank : K;
-  for (int r = 0; r < rounds; ++r) {       // K-th largest lane maximum
-    const uint32_t cur = __reduce_max_sync(kFull, live);
-    if (r == 0) first = cur;
-    if (r == K - 1) kth = cur;
-    if (TOPM && r == kTopmRank - 1) low = cur;
-    const unsigned bal = __ballot_sync(kFull, live == cur);
-    if (lane == __ffs(bal) - 1) live = 0;
-  }
-  const uint32_t none = f32_orderable(0xFF800000u);   // -inf: a lane without data
-  float4 out;
-  out.x = kth <= none ? -INFINITY : __uint_as_float(f32_from_orderable(kth));      // filter
-  out.y = first <= none ? 0.f : __uint_as_float(f32_from_orderable(first));        // reference (any finite value if no data)
-  out.z = low <= none ? kTopmLowestFloor : fmaxf(__uint_as_float(f32_from_orderable(low)), kTopmLowestFloor);
-  out.w = 0.f;
-  return out;
-}
-
-// ---------------------------------------------------------------- draining the queue
-
-struct Drained {
-  Acc acc;
-  float c, m, thr;
-};
-
-// Empties the warp's queue, one element per lane and step.  Elements below the filter are
-// summed.  The others are appended to the pool behind the K largest keys so far; whenever
-// another step might not fit, and at the end, the pool is ranked by counting: the K largest
-// keys stay (sorted, not summed yet), the rest is summed.
-template <bool BF16>
-__device__ __forceinline__ Drained drain_queue(WarpShared *ws, int qn, int K, Acc acc, float c, float m, float thr,
-                                               uint32_t *status) {
-  constexpr int EPV = Vec<BF16>::N;        // elements per vector
-  constexpr int VPS = 32 / EPV;            // vectors per step
-  const int lane = threadIdx.x & 31;
-  const unsigned lt_mask = (1u << lane) - 1u;
-  const int sub = lane / EPV, e = lane % EPV;
-  int pn = K;
-  for (int base = 0;; base += VPS) {
-    const bool more = base < qn;
-    if (!more || pn > kPool - 32) {
-      // ---- rank the pool: lane l owns keys l and l + 32
-      __syncwarp();
-      const unsigned long long a = lane < pn ? ws->pool[lane] : 0ull;
-      const unsigned long long b = lane + 32 < pn ? ws->pool[lane + 32] : 0ull;
-      if (lane < K) ws->ranked[lane] = 0ull;
-      int ra = 0, rb = 0;
-      if (pn <= 32) {
-#pragma unroll 4
-        for (int r = 0; r < pn; ++r) ra += ws->pool[r] > a;
-      } else {
-#pragma unroll 4
-        for (int r = 0; r < pn; ++r) {
-          const unsigned long long kr = ws->pool[r];
-          ra += kr > a;
-          rb += kr > b;
-        }
-      }
-      __syncwarp();
-      // the reference follows the largest key before anything of the pool is summed
-      const uint32_t top_hi = (a != 0ull && ra == 0) ? (uint32_t)(a >> 32) : ((b != 0ull && rb == 0) ? (uint32_t)(b >> 32) : 0u);
-      const unsigned owner = __ballot_sync(kFull, top_hi != 0u);
-      if (owner) {
-        const float hm = __uint_as_float(f32_from_orderable(__shfl_sync(kFull, top_hi, __ffs(owner) - 1)));
-        if (hm > m) {
-          const float new_c = -hm * kLog2e;
-          acc_rescale(acc, c, new_c);
-          c = new_c;
-          m = hm;
-        }
-      }
-      if (a != 0ull) {
-        if (ra < K) ws->ranked[ra] = a;
-        else acc_scalar(acc, c, key_value(a));
-      }
-      if (b != 0ull) {
-        if (rb < K) ws->ranked[rb] = b;
-        else acc_scalar(acc, c, key_value(b));
-      }
-      __syncwarp();
-      if (lane < K) ws->pool[lane] = ws->ranked[lane];
-      pn = K;
-      if (!more) break;
-    }
-    const int j = base + sub;
-    bool cand = false;
-    unsigned long long key = 0ull;
-    if (j < qn) {
-      float x;
-      if (BF16) x = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t *>(ws->qdata + j)[e] << 16);
-      else x = reinterpret_cast<const float *>(ws->qdata + j)[e];
-      cand = x >= thr;
-      if (cand) key = make_key(x, (uint32_t)ws->qindex[j] * EPV + e);
-      else acc_scalar(acc, c, x);                    // (a NaN element poisons the sums, as it must)
-    }
-    const unsigned mask = __ballot_sync(kFull, cand);
-    if (cand && C2T_IN_BOUNDS(pn + __popc(mask & lt_mask), kPool, status)) ws->pool[pn + __popc(mask & lt_mask)] = key;
-    pn += __popc(mask);
-  }
-  __syncwarp();
-  // the list is exact for everything read so far: from now on only values above its K-th matter
-  const unsigned long long kth = ws->pool[K - 1];
-  if (kth != 0ull) thr = fmaxf(thr, value_just_above((uint32_t)(kth >> 32)));
-  Drained d;
-  d.acc = acc; d.c = c; d.m = m; d.thr = thr;
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
 
-// Candidates of the truncated entropy (Eq. 3): where a warp puts the vectors whose largest element reaches its
-// segment's floor (ballot-ranked places in stream order, so the result does not depend on timing).
+// S and U of a lane: two packed accumulators each, so that consecutive additions do not wait for each other.
+struct Acc {
+  f32x2 S[2], U[2];
+  __device__ __forceinline__ void clear() { S[0] = S[1] = U[0] = U[1] = 0ull; }
+  __device__ __forceinline__ void totals(float &s, float &u) const {
+    float a, b, c, d;
+    unpack2(add2(S[0], S[1]), a, b);
+    unpack2(add2(U[0], U[1]), c, d);
+    s = a + b;
+    u = c + d;
+  }
+};
+
+__device__ __forceinline__ void acc_pair(Acc &a, int i, float x0, float x1, f32x2 scale, f32x2 c) {
+  const f32x2 t = fma2(pack2(x0, x1), scale, c);
+  float t0, t1;
+  unpack2(t, t0, t1);
+  const f32x2 e = pack2(ex2f(t0), ex2f(t1));
+  a.S[i] = add2(a.S[i], e);
+  a.U[i] = fma2(e, t, a.U[i]);
+}
+
+template <bool BF16>
+__device__ __forceinline__ void acc_vector(Acc &a, const uint4 &q, f32x2 scale, f32x2 c) {
+  float x[Vec<BF16>::N];
+  Vec<BF16>::unpack(q, x);
+#pragma unroll
+  for (int i = 0; i < Vec<BF16>::N; i += 2) acc_pair(a, (i >> 1) & 1, x[i], x[i + 1], scale, c);
+}
+
+// ---------------------------------------------------------------- maxima
+
+// A running maximum of whole vectors (NaN ignored): packed for bf16, plain for fp32.
+template <bool BF16>
+struct RunMax {
+  uint32_t v;
+  __device__ __forceinline__ void clear() { v = BF16 ? kLowestBf16x2 : __float_as_uint(kLowestF32); }
+  __device__ __forceinline__ void take(const uint4 &q) {
+    if (BF16) v = max_bf16x2(v, max_bf16x2(max_bf16x2(q.x, q.y), max_bf16x2(q.z, q.w)));
+    else v = __float_as_uint(fmaxf(__uint_as_float(v), fmaxf(fmaxf(__uint_as_float(q.x), __uint_as_float(q.y)),
+                                                             fmaxf(__uint_as_float(q.z), __uint_as_float(q.w)))));
+  }
+  __device__ __forceinline__ float value() const {
+    return BF16 ? fmaxf(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u)) : __uint_as_float(v);
+  }
+};
+
+__device__ __forceinline__ float warp_max(float x) {      // not for NaN
+  return __uint_as_float(f32_from_orderable(__reduce_max_sync(kFull, f32_orderable(__float_as_uint(x)))));
+}
+
+// the float just above a value
+__device__ __forceinline__ float just_above(float x) {
+  return __uint_as_float(f32_from_orderable(f32_orderable(__float_as_uint(x)) + 1u));
+}
+
+// ---------------------------------------------------------------- a warp's sums of a row
+
+constexpr float kNoOffset = 3e38f;                    // no data yet: behind every real offset
+constexpr float kSlack = 100.f;                       // octaves a value may lie above the reference
+
+// A lane's sums of the chunks of a row that its warp streams; the chunk with the lane's largest value is kept apart.
+struct LaneSums {
+  Acc acc;                   // the current chunk
+  float S, U;                // finished chunks but the held one
+  float Sh, Uh, hmax;        // the held chunk: its sums and its largest value
+  int hch;
+  f32x2 c2;                  // the offset, twice (warp-uniform)
+  float c, limit;            // the offset; the value from which on it has to move (the lowest while there was no data)
+  __device__ __forceinline__ void start(float m) {
+    acc.clear();
+    S = U = Sh = Uh = 0.f;
+    hmax = kLowestF32;
+    hch = 0;
+    set_offset(m);
+  }
+  __device__ __forceinline__ void set_offset(float m) {
+    const bool none = m <= kNegInfAsFinite;
+    c = none ? 0.f : -rintf(fminf(m, 2e38f) * kLog2e);
+    c2 = pack2(c, c);
+    limit = none ? kNegInfAsFinite : (kSlack - c) * (1.f / kLog2e);
+  }
+  // a new reference: what has been summed follows
+  __device__ __forceinline__ void move_offset(float m) {
+    const float old = c;
+    const bool none = limit == kNegInfAsFinite;
+    set_offset(m);
+    const float d = none ? 0.f : fmaxf(c - old, -1e30f), f = ex2f(d);                // every t shifts by d (no sums yet: by nothing)
+    U = f * fmaf(d, S, U);
+    S *= f;
+    Uh = f * fmaf(d, Sh, Uh);
+    Sh *= f;
+  }
+  __device__ __forceinline__ void end_chunk(float cmax, int ch) {
+    float s, u;
+    acc.totals(s, u);
+    acc.clear();
+    const bool best = cmax > hmax;
+    S += best ? Sh : s;
+    U += best ? Uh : u;
+    Sh = best ? s : Sh;
+    Uh = best ? u : Uh;
+    hch = best ? ch : hch;
+    hmax = fmaxf(hmax, cmax);
+  }
+};
+
+// 2^d for an integer d <= 0
+__device__ __forceinline__ double pow2_f64(float d) { return d < -1000.f ? 0.0 : __hiloint2double((1023 + (int)d) << 20, 0); }
+
+// The lanes' sums over the warp into a record.
+__device__ __forceinline__ void write_record(SumRecord *rec, const LaneSums &ls) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t ord = f32_orderable(__float_as_uint(ls.hmax)), top = __reduce_max_sync(kFull, ord);
+  const int t = __ffs(__ballot_sync(kFull, ord == top)) - 1;
+  float s = ls.S, u = ls.U;
+  if (lane == t) {
+    rec->held = make_float4(ls.Sh, ls.Uh, __int_as_float(t), __int_as_float(ls.hch));
+  } else {
+    s += ls.Sh;
+    u += ls.Uh;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(kFull, s, o);
+    u += __shfl_xor_sync(kFull, u, o);
+  }
+  if (lane == 0) rec->rest = make_float4(s, u, ls.limit == kNegInfAsFinite ? kNoOffset : ls.c, __uint_as_float(f32_from_orderable(top)));
+}
+
+// ---------------------------------------------------------------- rows and chunks
+
+template <bool BF16>
+struct RowShape {
+  int vpr, v_full, nc;         // vectors of a row (the last may be ragged), whole ones, chunks
+  __device__ __forceinline__ explicit RowShape(int V) {
+    vpr = (V + Vec<BF16>::N - 1) / Vec<BF16>::N;
+    v_full = V / Vec<BF16>::N;
+    nc = (vpr + kChunkVecs - 1) / kChunkVecs;
+  }
+};
+
+__device__ __forceinline__ const char *row_pointer(const PassParams &p, int b, int j, size_t esz) {
+  return reinterpret_cast<const char *>(p.logits) + ((size_t)b * p.seq_stride + (size_t)j * p.row_stride) * esz;
+}
+
+// the ragged last vector of a row, assembled from scalar loads
+template <bool BF16>
+__device__ __noinline__ uint4 load_ragged(const void *row, int v, int v_full, int V) { return Vec<BF16>::load(row, v, v_full, V); }
+
+// Requests group g of a chunk: src points at the lane's first vector of the chunk, nv counts the whole vectors from the
+// chunk's start on.  Vectors past them become the lowest value, which adds exactly 0 to the sums.
+template <bool BF16>
+__device__ __forceinline__ void load_group(uint4 (&q)[4], const uint4 *src, int g, int nv, int lane) {
+  const uint32_t lo = BF16 ? kLowestBf16x2 : __float_as_uint(kLowestF32);
+  if (nv >= (g + 1) * 128) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) q[k] = ldg_stream(src + g * 128 + k * 32);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      q[k] = make_uint4(lo, lo, lo, lo);
+      if (g * 128 + k * 32 + lane < nv) q[k] = ldg_stream(src + g * 128 + k * 32);
+    }
+  }
+}
+
+// A chunk's sums of one lane, with plain loads.
+template <bool BF16>
+__device__ __noinline__ float2 sum_again(const char *row, int ch, float c, int V) {
+  const RowShape<BF16> rs(V);
+  const int lane = threadIdx.x & 31, v1 = (ch + 1) * kChunkVecs < rs.vpr ? (ch + 1) * kChunkVecs : rs.vpr;
+  Acc acc;
+  acc.clear();
+  for (int v = ch * kChunkVecs + lane; v < v1; v += 32) {
+    uint4 q = Vec<BF16>::load(row, v, rs.v_full, V);
+    Vec<BF16>::clamp(q);
+    acc_vector<BF16>(acc, q, pack2(kLog2e, kLog2e), pack2(c, c));
+  }
+  float2 su;
+  acc.totals(su.x, su.y);
+  return su;
+}
+
+// Cells are bf16, fp32 maxima rounded towards -inf: the floor taken from them is still reached by K elements, and a cell
+// with an element that reaches the floor still reaches it.
+__device__ __forceinline__ uint32_t cell_bits(float x, bool exact) {
+  uint32_t b = __float_as_uint(x);
+  if (!exact && (b & 0x80000000u)) b += 0xFFFFu;      // (a negative value: towards the larger magnitude)
+  return b >> 16;
+}
+
+// How the launch cut the rows, as one CTA sees it.  CTA i has chunks [i per_cta, (i + 1) per_cta) of the rows laid end to end.
+// Its tasks are its part of its last row, if it shares that row with the next CTA, its part of its first row, if it shares
+// that one, and the rows inside.  It streams them in this order, so that shared rows are complete early.
+//   TOPM: the CTA's range in natural order, an equal contiguous part per warp (a part's floor serves all its chunks).
+template <bool TOPM>
+struct CtaRange {
+  int nc, per_cta, u0, u1;     // chunks per row and per CTA; this CTA's chunks
+  int in0, in1;                // the rows inside
+  int tail, head;              // chunks of the shared last row (if it is not the first as well) and of the shared first row
+  int part, busy;              // TOPM: chunks of a warp; warps of the grid with chunks, as if every CTA had per_cta
+  __device__ __forceinline__ CtaRange(int nc_, int total) : nc(nc_) {
+    per_cta = (total + (int)gridDim.x - 1) / (int)gridDim.x;
+    part = (per_cta + kStreamWarps - 1) / kStreamWarps;
+    u0 = (int)blockIdx.x * per_cta;
+    u1 = u0 + per_cta < total ? u0 + per_cta : total;
+    const int a0 = u0 / nc, a1 = u1 > u0 ? (u1 - 1) / nc : a0;
+    in0 = a0 * nc < u0 ? a0 + 1 : a0;
+    in1 = (a1 + 1) * nc > u1 ? a1 : a1 + 1;
+    head = in0 > a0 ? (in0 * nc < u1 ? in0 * nc : u1) - u0 : 0;
+    if (in0 == a0 && in1 == a0) { head = u1 - u0; in0 = in1 = a0 + 1; }     // a row begins here and ends beyond
+    tail = in1 <= a1 && in1 >= in0 && a1 > a0 ? u1 - a1 * nc : 0;
+    if (in1 < in0) in1 = in0;
+    busy = 0;
+    if (TOPM && per_cta > 0) busy = (total + per_cta - 1) / per_cta * ((per_cta + part - 1) / part);
+  }
+  __device__ __forceinline__ int chunk_at(int i) const {              // the i-th chunk of the work order
+    if (TOPM) return u0 + i;
+    return i < tail ? u1 - tail + i : u0 + i - tail;                  // (the first row's part lies before the rows inside)
+  }
+  __device__ __forceinline__ int n_tasks() const { return (tail > 0) + (head > 0) + in1 - in0; }
+  __device__ __forceinline__ int task_row(int k) const {
+    if (tail > 0 && k-- == 0) return in1;
+    if (head > 0 && k-- == 0) return in0 - 1;
+    return in0 + k;
+  }
+  __device__ __forceinline__ int row_task(int a) const {
+    if (a < in0) return tail > 0;
+    if (a >= in1) return 0;
+    return (tail > 0) + (head > 0) + a - in0;
+  }
+  __device__ __forceinline__ int task_chunks(int a) const { return a < in0 ? head : (a >= in1 ? tail : nc); }
+  // records that the CTA's warps write for row a
+  __device__ __forceinline__ int task_records(int a) const {
+    const int n = task_chunks(a);
+    if (!TOPM) return n < kStreamWarps ? n : kStreamWarps;
+    const int from = (a * nc > u0 ? a * nc : u0) - u0;
+    return (from + n - 1) / part - from / part + 1;
+  }
+  // does the warp that streams chunk u of row a write its record after it?
+  __device__ __forceinline__ bool ends_record(int u, int a) const {
+    const int cta = u / per_cta, row_end = (a + 1) * nc, cta_end = (cta + 1) * per_cta, end = row_end < cta_end ? row_end : cta_end;
+    if (!TOPM) return end - u <= kStreamWarps;
+    return u + 1 == end || (u - cta * per_cta + 1) % part == 0;
+  }
+};
+
+// ---------------------------------------------------------------- completing a row
+
+// vector k of the lane's 8 in a cell (16 in a chunk, a cell being half a chunk)
+__device__ __forceinline__ int cell_vector(int cell, int lane, int k) { return cell * (kChunkVecs / 2) + lane + 32 * k; }
+
+template <bool BF16>
+__device__ __forceinline__ float element(const char *row, int tok) {    // -inf as the lowest finite value
+  const float x = BF16 ? __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short *>(row) + tok) << 16)
+                       : __ldg(reinterpret_cast<const float *>(row) + tok);
+  return x < kLowestF32 ? kLowestF32 : x;
+}
+
+// N vectors of a row, clamped; the lowest value past the row's end
+template <bool BF16, int N>
+__device__ __forceinline__ void load_vectors(uint4 (&q)[N], const char *row, const int (&v)[N], const RowShape<BF16> &rs, int V) {
+  const uint32_t lo = BF16 ? kLowestBf16x2 : __float_as_uint(kLowestF32);
+#pragma unroll
+  for (int u = 0; u < N; ++u) {
+    q[u] = make_uint4(lo, lo, lo, lo);
+    if (v[u] < rs.v_full) q[u] = __ldg(reinterpret_cast<const uint4 *>(row) + v[u]);
+  }
+  if (rs.vpr != rs.v_full) {
+#pragma unroll
+    for (int u = 0; u < N; ++u)
+      if (v[u] == rs.v_full) q[u] = load_ragged<BF16>(row, rs.v_full, rs.v_full, V);
+  }
+#pragma unroll
+  for (int u = 0; u < N; ++u) Vec<BF16>::clamp(q[u]);
+}
+
+// Ranks the first n keys of the pool: the K largest move to pool[0 .. K), sorted, 0-padded.  Returns how many there are.
+__device__ __noinline__ int rank_pool(PairShared *ws, int n, int K) {
+  const int lane = threadIdx.x & 31;
+  if (n <= 32) {                                     // the usual case: a key per lane
+    const unsigned long long key = lane < n ? ws->pool[lane] : 0ull;
+    int place = 0;
+#pragma unroll 8
+    for (int r = 0; r < n; ++r) place += ws->pool[r] > key;
+    if (lane >= n) place = lane;                     // (the zeros behind the keys)
+    __syncwarp();
+    ws->pool[place] = key;
+    __syncwarp();
+    return n < K ? n : K;
+  }
+  unsigned long long mine[kPoolCap / 32];
+  int rank[kPoolCap / 32];
+#pragma unroll
+  for (int i = 0; i < kPoolCap / 32; ++i) {
+    mine[i] = i * 32 + lane < n ? ws->pool[i * 32 + lane] : 0ull;
+    rank[i] = 0;
+  }
+  for (int r = 0; r < n; ++r) {
+    const unsigned long long k = ws->pool[r];
+#pragma unroll
+    for (int i = 0; i < kPoolCap / 32; ++i) rank[i] += k > mine[i];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < kPoolCap / 32; ++i)
+    if (mine[i] != 0ull && rank[i] < K) ws->pool[rank[i]] = mine[i];     // (K <= 32 < n: all K places are taken)
+  __syncwarp();
+  return K;
+}
+
+// Rows whose K largest do not come out of a short list (many equal values, few values): the chunks in order, elements
+// in token order 32 at a time, against a filter that rises.
+template <bool BF16>
+__device__ __noinline__ int select_in_order(const PassParams &p, PairShared *ws, const char *row, int a, float floor) {
+  const RowShape<BF16> rs(p.V);
+  const int lane = threadIdx.x & 31, K = p.K;
+  int have = 0;                                     // keys kept in pool[0 .. K)
+  float thr = floor;
+  constexpr int kBatch = 8;                         // elements of a lane in flight
+  for (int ch = 0; ch < rs.nc; ++ch) {
+    const uint32_t two = p.cells[(size_t)(a * rs.nc + ch) * 32 + lane];
+    // a cell is below the largest value it stands for by less than a bf16 step
+    const float cell = fmaxf(__uint_as_float(two << 16), __uint_as_float(two & 0xFFFF0000u));
+    const float most = BF16 ? cell : __uint_as_float(f32_from_orderable(f32_orderable(__float_as_uint(cell)) + 0xFFFFu));
+    if (!__any_sync(kFull, most >= thr)) continue;
+    const int t1 = (ch + 1) * kChunkVecs * Vec<BF16>::N;
+    const int end = t1 < p.V ? t1 : p.V;
+    for (int t0 = ch * kChunkVecs * Vec<BF16>::N; t0 < end; t0 += 32 * kBatch) {
+      float x[kBatch];
+      bool any = false;
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        const int tok = t0 + i * 32 + lane;
+        x[i] = tok < end ? element<BF16>(row, tok) : -INFINITY;
+        any = any || x[i] >= thr;
+      }
+      if (!__any_sync(kFull, any)) continue;
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        const unsigned long long key = x[i] >= thr ? make_key(x[i], (uint32_t)(t0 + i * 32 + lane)) : 0ull;
+        const bool in = key != 0ull && (have < K || key > ws->pool[K - 1]);
+        const unsigned mask = __ballot_sync(kFull, in);
+        if (mask) {
+          __syncwarp();
+          if (in) ws->pool[have + __popc(mask & ((1u << lane) - 1u))] = key;
+          __syncwarp();
+          have = rank_pool(ws, have + __popc(mask), K);
+          if (have == K) thr = just_above(key_value(ws->pool[K - 1]));   // later tokens of the K-th value lose the tie
+        }
+      }
+    }
+  }
+  if (lane == 0)
+    for (int r = have; r < K; ++r) ws->pool[r] = 0ull;
+  __syncwarp();
+  return have;
+}
+
+// The elements at or above the floor, out of the listed cells, as keys in the pool.  Returns how many there are, or -1 if
+// something overflowed.
+template <bool BF16>
+__device__ __forceinline__ int gather_keys(PairShared *ws, const char *row, const RowShape<BF16> &rs, int V, float floor, int n_list) {
+  constexpr int EPV = Vec<BF16>::N;
+  constexpr int kBatch = 4;                         // 16-byte loads of a lane in flight: 16 cells
+  const int lane = threadIdx.x & 31;
+  const unsigned lt_mask = (1u << lane) - 1u;
+  int n_vec = 0;                                    // vectors with such an element
+  for (int i0 = 0; i0 < n_list * 8; i0 += 32 * kBatch) {
+    uint4 q[kBatch];
+    int v[kBatch];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      const int i = i0 + u * 32 + lane, cell = i < n_list * 8 ? ws->list[i >> 3] : -1;
+      v[u] = cell < 0 ? rs.vpr : cell_vector(cell >> 5, cell & 31, i & 7);
+    }
+    load_vectors<BF16, kBatch>(q, row, v, rs, V);
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      const bool hit = v[u] < rs.vpr && Vec<BF16>::vmax(q[u]) >= floor;
+      const unsigned hm = __ballot_sync(kFull, hit);
+      const int pos = n_vec + __popc(hm & lt_mask);
+      if (hit && pos < kListCap) ws->vecs[pos] = v[u];
+      n_vec += __popc(hm);
+    }
+  }
+  if (n_vec > kListCap) return -1;
+  __syncwarp();
+  int n = 0;
+#pragma unroll 4
+  for (int i0 = 0; i0 < n_vec * EPV; i0 += 32) {
+    const int i = i0 + lane;
+    const int tok = i < n_vec * EPV ? ws->vecs[i / EPV] * EPV + i % EPV : V;
+    const float x = tok < V ? element<BF16>(row, tok) : -INFINITY;
+    const unsigned hm = __ballot_sync(kFull, x >= floor);
+    const int pos = n + __popc(hm & lt_mask);
+    if (x >= floor && pos < kPoolCap) ws->pool[pos] = make_key(x, (uint32_t)tok);
+    n += __popc(hm);
+  }
+  __syncwarp();
+  return n <= kPoolCap ? n : -1;
+}
+
+// A row is completed, all its partial results being in place, in two independent halves, by the two warps of a pair.  Each
+// is a chain of dependent steps, so loads are issued in batches, as early as their addresses are known.
+
+// The K largest.
+template <bool BF16>
+__device__ __forceinline__ void complete_keys(const PassParams &p, PairShared *ws, int a, int b, int j) {
+  constexpr int kBatch = 32;                        // chunks of its column that a lane holds at a time
+  const RowShape<BF16> rs(p.V);
+  const int lane = threadIdx.x & 31, K = p.K;
+  const char *row = row_pointer(p, b, j, BF16 ? 2 : 4);
+  const uint32_t *cells = p.cells + (size_t)a * rs.nc * 32 + lane;
+  uint32_t v[kBatch], cm2 = kLowestBf16x2;
+#pragma unroll
+  for (int i = 0; i < kBatch; ++i) v[i] = i < rs.nc ? cells[i * 32] : kLowestBf16x2;
+#pragma unroll
+  for (int i = 0; i < kBatch; ++i) cm2 = max_bf16x2(cm2, v[i]);
+  for (int c0 = kBatch; c0 < rs.nc; c0 += kBatch) {
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i) v[i] = c0 + i < rs.nc ? cells[(c0 + i) * 32] : kLowestBf16x2;
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i) cm2 = max_bf16x2(cm2, v[i]);
+  }
+  // 32 columns, or for a large K 64 half columns, and their places under (maximum desc, index asc): at least K elements
+  // reach the K-th largest column maximum (if that many columns have data)
+  const float lo = __uint_as_float(cm2 << 16), hi = __uint_as_float(cm2 & 0xFFFF0000u);
+  float floor;
+  if (K <= 16) {
+    const float cm = fmaxf(lo, hi);
+    ws->colmax[lane] = cm;
+    __syncwarp();
+    int place = 0;
+#pragma unroll
+    for (int i = 0; i < 32; i += 4) {
+      const float4 o = *reinterpret_cast<const float4 *>(&ws->colmax[i]);
+      place += o.x > cm || (o.x == cm && i < lane);
+      place += o.y > cm || (o.y == cm && i + 1 < lane);
+      place += o.z > cm || (o.z == cm && i + 2 < lane);
+      place += o.w > cm || (o.w == cm && i + 3 < lane);
+    }
+    floor = __shfl_sync(kFull, cm, __ffs(__ballot_sync(kFull, place == K - 1)) - 1);
+  } else {
+    ws->colmax[lane] = lo;
+    ws->colmax[32 + lane] = hi;
+    __syncwarp();
+    int p0 = 0, p1 = 0;
+#pragma unroll 8
+    for (int i = 0; i < 64; ++i) {
+      const float o = ws->colmax[i];
+      p0 += o > lo || (o == lo && i < lane);
+      p1 += o > hi || (o == hi && i < 32 + lane);
+    }
+    const unsigned b0 = __ballot_sync(kFull, p0 == K - 1), b1 = __ballot_sync(kFull, p1 == K - 1);
+    floor = b0 ? __shfl_sync(kFull, lo, __ffs(b0) - 1) : __shfl_sync(kFull, hi, __ffs(b1) - 1);
+  }
+  const uint32_t fb = __float_as_uint(floor), floor2 = fb | (fb >> 16);
+
+  // ---- the cells that reach it
+  int n_list = 0;
+  for (int c0 = 0; c0 < rs.nc && n_list <= kListCap; c0 += kBatch) {
+    if (rs.nc > kBatch) {
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) v[i] = c0 + i < rs.nc ? cells[(c0 + i) * 32] : kLowestBf16x2;
+    }
+    unsigned long long mask = 0ull;                 // 16 chunks: bits of their first halves, then of their second ones; twice
+#pragma unroll
+    for (int h = 0; h < kBatch / 16; ++h) {
+      uint32_t m = 0u;
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        uint32_t ge;
+        asm("set.ge.u32.bf16x2 %0, %1, %2;" : "=r"(ge) : "r"(v[h * 16 + i]), "r"(floor2));
+        m |= (ge & 0x00010001u) << i;
+      }
+      mask |= (unsigned long long)m << (32 * h);
+    }
+    for (;;) {
+      const unsigned bal = __ballot_sync(kFull, mask != 0ull);
+      if (!bal || n_list > kListCap) break;
+      const int pos = n_list + __popc(bal & ((1u << lane) - 1u));
+      if (mask) {
+        const int bit = __ffsll((long long)mask) - 1, chunk = c0 + ((bit & 32) >> 1) + (bit & 15);
+        if (pos < kListCap) ws->list[pos] = chunk < rs.nc ? (2 * chunk + ((bit >> 4) & 1)) * 32 + lane : -1;
+      }
+      mask &= mask - 1ull;
+      n_list += __popc(bal);
+    }
+  }
+  __syncwarp();
+  const int n_keys = n_list <= kListCap ? gather_keys<BF16>(ws, row, rs, p.V, floor, n_list) : -1;
+  const int n_valid = n_keys >= 0 ? rank_pool(ws, n_keys, K) : select_in_order<BF16>(p, ws, row, a, floor);
+  const size_t slot = (size_t)b * p.rows_per_seq_max + j;
+  for (int i = lane; i < K; i += 32) p.row_keys[slot * K + i] = ws->pool[i];
+  if (lane == 0) {
+    p.rows[slot].top = ws->pool[0];
+    p.rows[slot].n_valid = n_valid;
+  }
+  __syncwarp();
+}
+
+// The maximum and the merged sums.
+template <bool BF16, bool TOPM>
+__device__ __forceinline__ void complete_sums(const PassParams &p, const CtaRange<TOPM> &cr, int a, int b, int j) {
+  constexpr int kBatch = 2;                         // chunks of a lane at a time: 64 of the row
+  const RowShape<BF16> rs(p.V);
+  const int lane = threadIdx.x & 31, first = a * rs.nc;
+  const char *row = row_pointer(p, b, j, BF16 ? 2 : 4);
+  float4 rest[kBatch], held[kBatch];
+  // ---- the row maximum and where it is
+  float m = kLowestF32;
+  int at = 0, tl = 0, tc = 0;                        // the record, its lane and chunk
+  for (int c0 = 0; c0 < rs.nc; c0 += 32 * kBatch) {
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i) {
+      const int ch = c0 + i * 32 + lane;
+      rest[i] = make_float4(0.f, 0.f, kNoOffset, kLowestF32);
+      held[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (ch < rs.nc && cr.ends_record(first + ch, a)) {
+        const SumRecord *r = p.sums + first + ch;
+        rest[i] = r->rest;
+        held[i] = r->held;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i)
+      if (rest[i].w > m) { m = rest[i].w; at = c0 + i * 32 + lane; tl = __float_as_int(held[i].z); tc = __float_as_int(held[i].w); }
+  }
+  const uint32_t ord = f32_orderable(__float_as_uint(m)), top = __reduce_max_sync(kFull, ord);
+  const int owner = __ffs(__ballot_sync(kFull, ord == top)) - 1;
+  const float Mf = __shfl_sync(kFull, m, owner);
+  const int trec = __shfl_sync(kFull, at, owner), tlane = __shfl_sync(kFull, tl, owner), tch = __shfl_sync(kFull, tc, owner);
+
+  // ---- that lane's 16 vectors of the chunk summed again without the maximum (and without its equals, which are counted)
+  const float cM = -rintf(fminf(Mf, 2e38f) * kLog2e);                 // the offset of the maximum: the reference of the merge
+  float s_own, u_own;
+  int equals = 0;
+  {
+    uint4 q[1];
+    const int vec[1] = {lane < 16 ? cell_vector(2 * tch, tlane, lane) : rs.vpr};
+    load_vectors<BF16, 1>(q, row, vec, rs, p.V);
+    float x[Vec<BF16>::N];
+    Vec<BF16>::unpack(q[0], x);
+    Acc acc;
+    acc.clear();
+#pragma unroll
+    for (int e = 0; e < Vec<BF16>::N; ++e)
+      if (x[e] == Mf && lane < 16) { x[e] = kLowestF32; ++equals; }
+#pragma unroll
+    for (int e = 0; e < Vec<BF16>::N; e += 2) acc_pair(acc, (e >> 1) & 1, x[e], x[e + 1], pack2(kLog2e, kLog2e), pack2(cM, cM));
+    acc.totals(s_own, u_own);
+  }
+  const double kLn2 = 0.69314718055994530942;
+  const double M = (double)Mf, g = -(double)cM * kLn2 - M, scale = exp(g);   // x - M = t ln2 + g
+
+  // ---- merge: all records brought to the reference of the maximum
+  double S = (double)s_own, U = (double)u_own;
+  for (int c0 = 0; c0 < rs.nc; c0 += 32 * kBatch) {
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i) {
+      const int ch = c0 + i * 32 + lane;
+      const bool have = ch < rs.nc && cr.ends_record(first + ch, a);
+      if (rs.nc > 32 * kBatch && have) {
+        const SumRecord *r = p.sums + first + ch;
+        rest[i] = r->rest;
+        held[i] = r->held;
+      }
+      if (have) {
+        const double s = (double)rest[i].x + (ch == trec ? 0.0 : (double)held[i].x);
+        const double u = (double)rest[i].y + (ch == trec ? 0.0 : (double)held[i].y);
+        const float d = fmaxf(cM - rest[i].z, -2000.f);               // (never positive)
+        const double f = pow2_f64(d);
+        S += f * s;
+        U += f * (u + (double)d * s);
+      }
+    }
+  }
+  S = warp_sum(S);
+  U = warp_sum(U);
+  equals = __reduce_add_sync(kFull, equals);
+  if (lane == 0) {
+    const double Sn = S * scale + (double)(equals - 1), Tn = scale * (kLn2 * U + g * S);
+    RowResult *r = p.rows + (size_t)b * p.rows_per_seq_max + j;
+    r->M = M; r->S = Sn; r->T = Tn;
+    r->L = log1p(Sn);                               // ln sum_v e^(x_v - M); the maximum contributes the 1
+    r->fault = row_fault_bits(Mf, Sn, Tn);
+  }
+  __syncwarp();
+}
+
+// The CTA's part of a row shared with others is done: is the row complete?  (By one lane; the others' records are visible to it afterwards.)
+__device__ __forceinline__ bool count_shared(const PassParams &p, int a, int chunks, int nc) {
+  __threadfence();                                   // the CTA's records, before its count
+  if (atomicAdd(&p.row_done[a], chunks) + chunks != nc) return false;
+  p.row_done[a] = 0;                                 // for the next launch
+  __threadfence();                                   // the other CTAs' records, after their counts
+  return true;
+}
+
+// ---------------------------------------------------------------- truncated entropy (Eq. 3): setting candidates aside
+
+// Where a warp puts the vectors whose largest element reaches its segment's floor (ballot-ranked places in stream
+// order, so the result does not depend on timing).
 struct TopmState {
   uint4 *region;              // the warp's part of the pool
   int cap, n, first;          // its size in vectors; vectors set aside by the warp so far (may pass cap: then nothing more is stored); n when the segment began
@@ -470,275 +697,269 @@ __device__ __forceinline__ void store_keep_in_l2(uint4 *dst, const uint4 &q, uns
                ::"l"(dst), "r"(q.x), "r"(q.y), "r"(q.z), "r"(q.w), "l"(policy) : "memory");
 }
 
-// One group: vectors that meet the filter go to the queue, the others into the sums.  WHOLE:
-// no lane is past the segment's end (a vector past it holds the lowest value, below every floor).
-template <bool BF16, bool WHOLE, bool TOPM>
-__device__ __forceinline__ void process_group(WarpShared *ws, const Group &g, SegState &st, TopmState &ts, int vt, int v1,
-                                              unsigned lt_mask, uint32_t *status) {
-  using VT = Vec<BF16>;
-  float vm[kVPL];
-#pragma unroll
-  for (int u = 0; u < kVPL; ++u) vm[u] = VT::vmax(g.q[u]);
-  if (TOPM) {
-#pragma unroll
-    for (int u = 0; u < kVPL; ++u) {
-      const bool c = vm[u] >= ts.floor;              // (false for a vector with a NaN; such a row is reported anyway)
-      const unsigned cm = __ballot_sync(kFull, c);
-      const int pos = ts.n + __popc(cm & lt_mask);
-      if (c && pos < ts.cap) store_keep_in_l2(ts.region + pos, g.q[u], ts.keep);
-      ts.n += __popc(cm);
-    }
+// the collection floor of a segment from the lane maxima over its first two groups
+__device__ __forceinline__ float collection_floor(float lmax, int place) {
+  const int lane = threadIdx.x & 31;
+  uint32_t live = f32_orderable(__float_as_uint(lmax)), low = 0;
+  for (int r = 0; r < place; ++r) {
+    low = __reduce_max_sync(kFull, live);
+    if (lane == __ffs(__ballot_sync(kFull, live == low)) - 1) live = 0;
   }
-  float gm = vm[0];
-#pragma unroll
-  for (int u = 1; u < kVPL; ++u) gm = fmaxf(gm, vm[u]);
-  const bool any_hit = gm >= st.thr;
-  if (!__any_sync(kFull, any_hit)) {
-#pragma unroll
-    for (int u = 0; u < kVPL; ++u) acc_vector<BF16>(st.acc, g.q[u], kLog2e, st.c);
-  } else {
-    // The sums still run over all four vectors in one straight line; a vector that goes to the
-    // queue is left out by t = 0 x - 200 (2^-200 flushes to zero and 0 * -200 adds nothing to U).
-    bool hit[kVPL];
-    unsigned mask[kVPL];
-#pragma unroll
-    for (int u = 0; u < kVPL; ++u) {
-      hit[u] = vm[u] >= st.thr && (WHOLE || vt + u * 32 < v1);
-      mask[u] = __ballot_sync(kFull, hit[u]);
-    }
-#pragma unroll
-    for (int u = 0; u < kVPL; ++u) {
-      if (hit[u]) {
-        const int pos = st.qn + __popc(mask[u] & lt_mask);
-        if (C2T_IN_BOUNDS(pos, kQueueCap, status)) {
-          ws->qdata[pos] = g.q[u];
-          ws->qindex[pos] = vt + u * 32;
-        }
-      }
-      st.qn += __popc(mask[u]);
-    }
-#pragma unroll
-    for (int u = 0; u < kVPL; ++u)
-      acc_vector<BF16>(st.acc, g.q[u], hit[u] ? 0.f : kLog2e, hit[u] ? -200.f : st.c);
-  }
-}
-
-template <bool BF16>
-__device__ __forceinline__ void drain_into(WarpShared *ws, SegState &st, int K, uint32_t *status) {
-  __syncwarp();                                      // the queue was written by other lanes
-  const Drained d = drain_queue<BF16>(ws, st.qn, K, st.acc, st.c, st.m, st.thr, status);
-  st.acc = d.acc; st.c = d.c; st.m = d.m; st.thr = d.thr;
-  st.qn = 0;
-  __syncwarp();
+  return fmaxf(__uint_as_float(f32_from_orderable(low)), kTopmLowestFloor);
 }
 
 // ---------------------------------------------------------------- the kernel
 
-// The pass itself: what every warp of the grid does (a warp returns when its span is done).
+// Sums and maxima of the chunk in q, each group of which is requested for the next chunk as soon as it is consumed.
 template <bool BF16, bool TOPM>
-__device__ __forceinline__ void expand_pass_body(const PassParams &p, unsigned char *s_dyn) {
-  using VT = Vec<BF16>;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  WarpShared *ws = reinterpret_cast<WarpShared *>(s_dyn) + warp;
-  int *s_off = reinterpret_cast<int *>(s_dyn + kEWarps * sizeof(WarpShared));
-
-  const int K = p.K;
-  const int n_rows = build_row_offsets(p.counts, p.B, p.rows_per_seq_max, s_off);   // the only barriers
-  if (blockIdx.x == 0 && p.row_off)                  // the pruning kernel finds a sequence's rows with this
-    for (int i = threadIdx.x; i <= p.B; i += kExpandThreads) p.row_off[i] = s_off[i];
-  const int vpr = (p.V + VT::N - 1) / VT::N, v_full = p.V / VT::N;
-  // spans of equal cost: rows behind kSegmentPad virtual vectors each, laid end to end, cut evenly
-  const long long vrow = (long long)vpr + kSegmentPad;
-  const long long vtotal = (long long)n_rows * vrow;
-  const long long workers = (long long)gridDim.x * kEWarps;
-  long long span = div_floor(vtotal + workers - 1, workers);
-  if (span < p.min_span) span = p.min_span;
-  // consecutive workers sit on different SMs: a launch with few rows (level 0) still uses every SM
-  const long long worker = (long long)warp * gridDim.x + blockIdx.x;
-  if (worker == 0 && lane == 0) {
-    p.info->n_rows = n_rows;
-    p.info->vec_per_row = vpr;
-    p.info->span = span;
-    p.info->pad = kSegmentPad;
-  }
-  const long long start = real_position(worker * span, vrow, vtotal, vpr);
-  const long long end = real_position((worker + 1) * span, vrow, vtotal, vpr);
-  if (start >= end) return;
-
-  const size_t esz = BF16 ? 2 : 4;
-  GroupCursor cur(start, end, vpr, p, s_off, esz);   // the group being worked on
-  GroupCursor pre = cur;                             // the group being requested, two ahead
-  constexpr bool BULK = !BF16;                       // how the ring is filled (see above)
-  Ring ring;
-  ring.bar0 = ring.phase = ring.pending = 0u;
-  if (BULK) ring.init(ws, lane);
-  bool landed = true;                                // no wait for a copy has run out
+__device__ __forceinline__ void stream_chunk(uint4 (&q)[kGroups][4], const uint4 *src, int nnv, LaneSums &ls, f32x2 scale, float (&cv)[2],
+                                             TopmState &ts, int lane) {
 #pragma unroll
-  for (int i = 0; i < kRingSlots; ++i) {
-    prefetch_group<BULK>(ring, i, pre, ws->ring[i], v_full, lane);
-    pre.advance(p, s_off, esz);
+  for (int h = 0; h < 2; ++h) {
+    RunMax<BF16> m;
+    m.clear();
+#pragma unroll
+    for (int g = 2 * h; g < 2 * h + 2; ++g) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (TOPM) {
+          RunMax<BF16> one;
+          one.clear();
+          one.take(q[g][k]);
+          const bool hit = one.value() >= ts.floor;            // (false for a vector of NaNs; such a row is reported anyway)
+          const unsigned hm = __ballot_sync(kFull, hit);
+          const int pos = ts.n + __popc(hm & ((1u << lane) - 1u));
+          if (hit && pos < ts.cap) store_keep_in_l2(ts.region + pos, q[g][k], ts.keep);
+          ts.n += __popc(hm);
+        }
+        m.take(q[g][k]);
+        Vec<BF16>::clamp(q[g][k]);
+        acc_vector<BF16>(ls.acc, q[g][k], scale, ls.c2);
+      }
+      load_group<BF16>(q[g], src, g, nnv, lane);
+    }
+    cv[h] = m.value();
   }
-  unsigned n = 0;                                    // ring slot of the current group
+}
 
-  Group g;
-  landed &= ring_wait<BULK>(ring, 0);
-  take_group<BF16>(g, cur, ws->ring[0], v_full, p.V, lane);
-  if (BULK) __syncwarp();                            // every lane has its vectors: the slot may be filled again
-  prefetch_group<BULK>(ring, 0, pre, ws->ring[0], v_full, lane);
-  pre.advance(p, s_off, esz);
-
-  const unsigned lt_mask = (1u << lane) - 1u;
-  SegState st;
+// One warp's stream: every kStreamWarps-th chunk of the CTA's work order (TOPM: a contiguous part of it).
+template <bool BF16, bool TOPM>
+__device__ __forceinline__ void stream(const PassParams &p, CtaShared *cs, const int *s_off, const RowShape<BF16> &rs, const CtaRange<TOPM> &cr) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = cr.u1 - cr.u0, step = TOPM ? 1 : kStreamWarps;
+  int i = TOPM ? warp * cr.part : warp;
+  const int end = TOPM ? (i + cr.part < n ? i + cr.part : n) : n;
+  if (i >= end) {
+    __syncthreads();
+    return;
+  }
+  const size_t esz = BF16 ? 2 : 4;
+  const f32x2 scale = pack2(kLog2e, kLog2e);
+  const int u_first = cr.chunk_at(i);
+  int a = u_first / rs.nc, ch = u_first - a * rs.nc, b = find_sequence(s_off, p.B, a);
+  const char *row = row_pointer(p, b, a - s_off[b], esz);
+  uint4 q[kGroups][4];
+  {
+    const uint4 *src = reinterpret_cast<const uint4 *>(row) + ch * kChunkVecs + lane;
+#pragma unroll
+    for (int g = 0; g < kGroups; ++g) load_group<BF16>(q[g], src, g, rs.v_full - ch * kChunkVecs, lane);
+  }
+  __syncthreads();                                   // the tasks' barriers are set up
   TopmState ts;
   ts.region = nullptr; ts.cap = 0; ts.n = 0; ts.first = 0; ts.floor = INFINITY; ts.keep = 0ull;
+  int region = 0;
   if (TOPM) {
     asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(ts.keep));
-    const long long busy = div_floor(vtotal + span - 1, span);       // workers with a span of this launch
-    const long long cap = div_floor(p.topm_pool_vecs, busy > 0 ? busy : 1);
+    const long long cap = p.topm_pool_vecs / cr.busy;          // an equal part of the pool for every warp with chunks
     ts.cap = (int)(cap < 0x3FFFFFFF ? cap : 0x3FFFFFFF);
-    ts.region = p.topm_pool + worker * ts.cap;
+    region = (int)((long long)((int)blockIdx.x * ((cr.per_cta + cr.part - 1) / cr.part) + warp) * ts.cap);
+    ts.region = p.topm_pool + region;
   }
-  bool fresh = true;                                 // the current group opens a segment
+  LaneSums ls;
+  bool fresh = true;                                 // the chunk is the warp's first of its row
   for (;;) {
-    const Segment seg = cur.seg;
+    // ---- the warp's next chunk
+    const bool more = i + step < end;
+    int na = a, nch = 0, nb = b;
+    const char *nrow = row;
+    if (more) {
+      const int nu = cr.chunk_at(i + step);
+      na = nu / rs.nc;
+      nch = nu - na * rs.nc;
+      if (na != a) {
+        if (na < a) nb = find_sequence(s_off, p.B, na);
+        else while (s_off[nb + 1] <= na) ++nb;
+        nrow = row_pointer(p, nb, na - s_off[nb], esz);
+      }
+    }
+    const uint4 *src = reinterpret_cast<const uint4 *>(nrow) + nch * kChunkVecs + lane;
+    const int nnv = more ? rs.v_full - nch * kChunkVecs : 0;
+    const int nvec = rs.vpr - ch * kChunkVecs;       // vectors from the chunk's start to the row's end
+    if (nvec <= kChunkVecs && rs.vpr != rs.v_full) { // the row's ragged last vector is in this chunk
+      const uint4 t = load_ragged<BF16>(row, rs.v_full, rs.v_full, p.V);
+#pragma unroll
+      for (int g = 0; g < kGroups; ++g)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (g * 128 + k * 32 + lane == nvec - 1) q[g][k] = t;
+    }
     if (fresh) {
-      landed &= ring_wait<BULK>(ring, next_slot(n));   // the group after this one
-      const float4 w = segment_warmup<BF16, TOPM>(K, g, cur.tv0 + lane, seg.v1, v_full, ws->ring[next_slot(n)]);
-      if (TOPM) { ts.floor = w.z; ts.first = ts.n; }
-      st.acc.S0 = st.acc.S1 = st.acc.U0 = st.acc.U1 = 0.f;
-      st.thr = w.x;
-      st.m = w.y;
-      st.c = -w.y * kLog2e;
-      st.qn = 0;
-      if (lane < K) ws->pool[lane] = 0ull;
-      fresh = false;
-    }
-    // ---- the inside of a segment: this group, the next one (in the ring) and the one to be
-    // requested (kRingSlots + 1 ahead) are whole groups of this segment, so nothing needs checking
-    if (pre.valid && pre.seg.a == seg.a) {
-      const int lim = seg.v1 < v_full ? seg.v1 : v_full;
-      const int k = (lim - cur.tv0) / kGroupVecs - (kRingSlots + 1);
-      if (k > 0) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(seg.row) + pre.tv0 + (BULK ? 0 : lane);
-        int vt = cur.tv0 + lane;
-        for (int i = 0; i < k; ++i) {
-          process_group<BF16, true, TOPM>(ws, g, st, ts, vt, 0, lt_mask, p.status);
-          n = next_slot(n);
-          vt += kGroupVecs;
-          landed &= ring_wait<BULK>(ring, n);
-          uint4 *slot = ws->ring[n];
+      RunMax<BF16> head;
+      head.clear();
 #pragma unroll
-          for (int u = 0; u < kVPL; ++u) g.q[u] = slot[lane + u * 32];
+      for (int k = 0; k < 4; ++k) head.take(q[0][k]);
+      ls.start(warp_max(head.value()));
+      if (TOPM) {
 #pragma unroll
-          for (int u = 0; u < kVPL; ++u) VT::clamp(g.q[u]);
-          if (BULK) {
-            __syncwarp();
-            ring.issue(n, slot, src, kGroupVecs, lane);
-          } else {
-            LaneCopies<kVPL>::all((uint32_t)__cvta_generic_to_shared(slot + lane), src);
-            cp_async_commit();
-          }
-          src += kGroupVecs;
-          if (st.qn > kDrainAt) drain_into<BF16>(ws, st, K, p.status);
-        }
-        cur.tv0 += k * kGroupVecs;
-        pre.tv0 += (k - 1) * kGroupVecs;             // the last step may leave the segment
-        pre.advance(p, s_off, esz);
+        for (int k = 0; k < 4; ++k) head.take(q[1][k]);
+        ts.floor = collection_floor(head.value(), p.topm_place);
+        ts.first = ts.n;
       }
     }
-    // ---- one group near the end of a segment, everything checked
-    const int vt = cur.tv0 + lane;
-    process_group<BF16, false, TOPM>(ws, g, st, ts, vt, seg.v1, lt_mask, p.status);
-    const bool last = cur.last_of_segment();
-    cur.advance(p, s_off, esz);
-    n = next_slot(n);
-    if (cur.valid) {                                 // next group (of this or of the next segment) into registers
-      landed &= ring_wait<BULK>(ring, n);
-      uint4 *slot = ws->ring[n];
-      take_group<BF16>(g, cur, slot, v_full, p.V, lane);
-      if (BULK) __syncwarp();
-      prefetch_group<BULK>(ring, n, pre, slot, v_full, lane);
-      pre.advance(p, s_off, esz);
+    float cv[2];                                     // the chunk's two cells
+    stream_chunk<BF16, TOPM>(q, src, nnv, ls, scale, cv, ts, lane);
+    if (__any_sync(kFull, fmaxf(cv[0], cv[1]) > ls.limit)) {
+      const float m = warp_max(fmaxf(cv[0], cv[1]));
+      ls.move_offset(m < INFINITY ? m : 2e38f);
+      const float2 su = sum_again<BF16>(row, ch, ls.c, p.V);
+      ls.acc.clear();
+      ls.acc.S[0] = pack2(su.x, 0.f);
+      ls.acc.U[0] = pack2(su.y, 0.f);
     }
-    if (last || st.qn > kDrainAt) drain_into<BF16>(ws, st, K, p.status);
-    if (last) {
-      // ---- the segment's record: the K largest keys but the first join the sums; sums in a
-      // fixed order, the sorted keys, the held-out head
-      const unsigned long long mine = lane < K ? ws->pool[lane] : 0ull;
-      if (lane > 0 && mine != 0ull) acc_scalar(st.acc, st.c, key_value(mine));
-      float S = st.acc.S0 + st.acc.S1, U = st.acc.U0 + st.acc.U1;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        S += __shfl_down_sync(kFull, S, o);
-        U += __shfl_down_sync(kFull, U, o);
-      }
-      const long long split = worker - div_floor((long long)seg.a * vrow + kSegmentPad, span);   // workers before the row's first
-      const size_t slot_id = (size_t)seg.a * p.max_splits + (size_t)split;
-      const unsigned have = __ballot_sync(kFull, mine != 0ull);
-      const bool slot_ok = C2T_IN_BOUNDS(slot_id, p.n_slots, p.status);
-      if (lane < K && slot_ok) p.part_keys[slot_id * K + lane] = mine;
-      if (lane == 0 && slot_ok) {
-        p.part_held[slot_id] = mine;
-        p.part_stats[slot_id] = make_float4(st.c, S, U, __int_as_float(__popc(have)));
-        if (TOPM) {
-          TopmSegment rec;
-          rec.first = (int)(worker * ts.cap) + ts.first;
-          rec.n = ts.n > ts.cap ? -1 : ts.n - ts.first;
-          rec.floor = ts.floor;
-          rec.pad = 0;
-          p.topm_seg[slot_id] = rec;
+    // ---- the chunk's cells; at the end of the warp's part of the row the record
+    ls.end_chunk(fmaxf(cv[0], cv[1]), ch);
+    const int u = a * rs.nc + ch;
+    fresh = !more || na != a;
+    if (C2T_IN_BOUNDS(u, p.n_chunks, p.status)) {
+      p.cells[(size_t)u * 32 + lane] = cell_bits(cv[0], BF16) | (cell_bits(cv[1], BF16) << 16);
+      if (fresh) write_record(p.sums + u, ls);
+    }
+    if (fresh) {
+      if (TOPM) {
+        const int seg = (int)blockIdx.x * kStreamWarps + warp + a;    // (both only grow along the parts: unique)
+        if (lane == 0 && C2T_IN_BOUNDS(seg, p.n_segs, p.status)) {
+          TopmSegment set;
+          set.first = region + ts.first;
+          set.n = ts.n > ts.cap ? -1 : ts.n - ts.first;
+          set.floor = ts.floor;
+          set.pad = 0;
+          p.topm_seg[seg] = set;
         }
       }
       __syncwarp();
-      if (!cur.valid) break;
-      fresh = true;
+      if (lane == 0) {
+        const uint32_t bar = (uint32_t)__cvta_generic_to_shared(cs->bars() + cr.row_task(a));
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+      }
+    }
+    if (!more) break;
+    i += step; a = na; ch = nch; b = nb; row = nrow;
+  }
+}
+
+// the two warps of a pair wait for each other
+__device__ __forceinline__ void pair_barrier(int pair) { asm volatile("bar.sync %0, 64;" ::"r"(1 + pair) : "memory"); }
+
+// Until all records of a task are written; false if the wait ran out.
+constexpr int kTaskWaitLimit = 1 << 22;               // tries of a task's barrier before a pair gives up (and says so)
+__device__ __forceinline__ bool wait_task(unsigned long long *bar_ptr) {
+  const uint32_t bar = (uint32_t)__cvta_generic_to_shared(bar_ptr);
+  uint32_t done = 0u;
+  for (int i = 0; i < kTaskWaitLimit && !done; ++i)
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done) : "r"(bar) : "memory");
+  return done != 0u;
+}
+
+// A pair's work: the CTA's tasks, one after the other.  A row inside the range is complete when its records are; a
+// shared one if this CTA's part of it was the last.
+template <bool BF16, bool TOPM>
+__device__ __forceinline__ void complete(const PassParams &p, CtaShared *cs, const int *s_off, const RowShape<BF16> &rs, const CtaRange<TOPM> &cr) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pair = warp >> 1, role = warp & 1;
+  const int n_tasks = cr.n_tasks();
+  pair_barrier(pair);                                // (both have done with streaming)
+  for (;;) {
+    if (role == 0 && lane == 0) {
+      const int k = atomicAdd(&cs->task, 1);
+      int go = 0;
+      if (k < n_tasks) {
+        const int a = cr.task_row(k);
+        if (!wait_task(cs->bars() + k)) { if (p.status) atomicOr(p.status, C2T_ST_INTERNAL); }
+        else go = (a >= cr.in0 && a < cr.in1) || count_shared(p, a, cr.task_chunks(a), rs.nc);
+      }
+      cs->task_of[pair] = k;
+      cs->flag[pair] = go;
+    }
+    pair_barrier(pair);
+    const int k = cs->task_of[pair], go = cs->flag[pair];
+    pair_barrier(pair);
+    if (k >= n_tasks) break;
+    if (!go) continue;
+    const int a = cr.task_row(k), b = find_sequence(s_off, p.B, a);
+    if (role == 0) complete_keys<BF16>(p, &cs->scratch[pair], a, b, a - s_off[b]);
+    else complete_sums<BF16, TOPM>(p, cr, a, b, a - s_off[b]);
+  }
+}
+
+// The pass itself: what every warp of the grid does.
+template <bool BF16, bool TOPM>
+__device__ __forceinline__ void expand_pass_body(const PassParams &p, unsigned char *s_dyn) {
+  CtaShared *cs = reinterpret_cast<CtaShared *>(s_dyn);
+  int *s_off = reinterpret_cast<int *>(cs->bars() + p.cta_tasks);
+  const int n_rows = build_row_offsets(p.counts, p.B, p.rows_per_seq_max, s_off);
+  const RowShape<BF16> rs(p.V);
+  const CtaRange<TOPM> cr(rs.nc, n_rows * rs.nc);
+  if (TOPM) {                                        // the selection kernels find a row's segments with these
+    if (blockIdx.x == 0)
+      for (int i = threadIdx.x; i <= p.B; i += kExpandThreads) p.row_off[i] = s_off[i];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      p.info->n_rows = n_rows;
+      p.info->vec_per_row = rs.nc;                   // (in chunks)
+      p.info->span = cr.per_cta;                     // (chunks per CTA)
     }
   }
-  // (every bulk copy that was issued has been waited for: the requests never run past the span)
-  if (!BULK) cp_async_wait<0>();
-  if (!landed && lane == 0 && p.status) atomicOr(p.status, C2T_ST_INTERNAL);
+  if (cr.u0 >= cr.u1) return;
+  for (int k = kExpandThreads - 1 - (int)threadIdx.x; k < cr.n_tasks(); k += kExpandThreads) {   // (the last warps first: they do not stream)
+    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(cs->bars() + k);
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(cr.task_records(cr.task_row(k))) : "memory");
+  }
+  if (threadIdx.x == kExpandThreads - 1) cs->task = 0;
+  if (threadIdx.x < kStreamWarps * 32) stream<BF16, TOPM>(p, cs, s_off, rs, cr);
+  else __syncthreads();
+  complete<BF16, TOPM>(p, cs, s_off, rs, cr);
 }
 
 template <bool BF16, bool TOPM>
-__global__ void __launch_bounds__(kExpandThreads, kExpandCtasPerSm) expand_pass_kernel(PassParams p) {
+__global__ void __launch_bounds__(kExpandThreads, 1) expand_pass_kernel(const __grid_constant__ PassParams p) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
   chain_enter();
   expand_pass_body<BF16, TOPM>(p, s_dyn);
 }
 
 // Expand and prune of a level in one launch, for small batches: the CTA that finishes last (an atomic ticket, nobody
-// waits) has every row's partial records in front of it and does the per-sequence work of c2t_prune for all
-// sequences, one after the other.
+// waits) has every row's result in front of it and does the per-sequence work of c2t_prune for all sequences, one
+// after the other.
 template <bool BF16>
-__global__ void __launch_bounds__(kExpandThreads, kExpandCtasPerSm) expand_prune_kernel(PassParams p, TreeState t, int level,
-                                                                                        c2t_frontier out) {
+__global__ void __launch_bounds__(kExpandThreads, 1) expand_prune_kernel(const __grid_constant__ PassParams p,
+                                                                         const __grid_constant__ TreeState t, int level,
+                                                                         c2t_frontier out) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
   __shared__ unsigned s_ticket;
   chain_enter();
   expand_pass_body<BF16, false>(p, s_dyn);
-  __threadfence();                                   // this CTA's records, before its ticket
+  __threadfence();                                   // this CTA's row results, before its ticket
   __syncthreads();
   if (threadIdx.x == 0) s_ticket = atomicAdd(t.ticket, 1u);
   __syncthreads();
   if (s_ticket != gridDim.x - 1) return;
-  __threadfence();                                   // the other CTAs' records, after their tickets
+  __threadfence();                                   // the other CTAs' results, after their tickets
   if (threadIdx.x == 0) *t.ticket = 0u;              // for the next launch
   // the pass's shared memory is free now
-  static_assert(sizeof(PruneShared<kEWarps>) <= kEWarps * sizeof(WarpShared), "the prune's scratch must fit the warps' areas");
-  PruneShared<kEWarps> &sh = *reinterpret_cast<PruneShared<kEWarps> *>(s_dyn);
+  PruneShared &sh = *reinterpret_cast<PruneShared *>(s_dyn);
   for (int b = 0; b < t.B; ++b) prune_level_body<kExpandThreads, false>(t, level, out, nullptr, 0, b, sh);
 }
 
 }  // namespace
-
-int expand_min_span(int vocab, int elem_bytes, int K) {
-  const int vec = 16 / elem_bytes;
-  const int vec_per_row = (vocab + vec - 1) / vec;
-  int lists = kStageKeys / (K < 1 ? 1 : K) - 1;      // one list in reserve: a row's pieces may start mid-worker
-  lists = lists > 31 ? 31 : (lists < 4 ? 4 : lists);
-  const int span = (vec_per_row + kSegmentPad + lists - 1) / lists;
-  return span < 256 ? 256 : span;
-}
 
 size_t topm_pool_vectors(size_t batch, size_t rows_per_seq, int vocab, int elem_bytes) {
   const size_t vec = 16 / elem_bytes;
@@ -746,42 +967,56 @@ size_t topm_pool_vectors(size_t batch, size_t rows_per_seq, int vocab, int elem_
   return n < 0x7FFFFFFFu ? n : 0x7FFFFFFFu;          // records hold 32-bit positions
 }
 
-int max_splits_for(int vocab, int elem_bytes, int workers, int pad, int min_span) {
+int topm_floor_place(int vocab, int elem_bytes, int M) {
+  const int vec = 16 / elem_bytes;
+  const int vec_per_row = (vocab + vec - 1) / vec, head = vec_per_row < 256 ? vec_per_row : 256;
+  const double per_lane = (double)head * vec / 32.0, share = 3.0 * M / vocab;
+  const int place = share >= 1.0 ? 31 : (int)ceil(32.0 * (1.0 - pow(1.0 - share, per_lane)));
+  return place < 1 ? 1 : (place > 31 ? 31 : place);
+}
+
+int row_chunks(int vocab, int elem_bytes) {
+  const int vec = 16 / elem_bytes;
+  return ((vocab + vec - 1) / vec + kChunkVecs - 1) / kChunkVecs;
+}
+
+int max_splits_for(int vocab, int elem_bytes, int workers) {
   const int vec = 16 / elem_bytes;
   const int vec_per_row = (vocab + vec - 1) / vec;
-  int by_span = (vec_per_row + pad + min_span - 1) / min_span;
+  int by_span = (vec_per_row + kMinSpanVectors - 1) / kMinSpanVectors;
   if (by_span > workers) by_span = workers;
   return by_span + 1;
 }
 
-static size_t expand_dynamic_smem(int B) {
-  return (size_t)kEWarps * sizeof(WarpShared) + ((size_t)B + 1) * sizeof(int);
+// the launch's shared memory
+static size_t plan_shared(PassParams &p, int grid) {
+  p.cta_tasks = (int)((long long)p.B * p.rows_per_seq_max / grid) + 4;       // rows inside a CTA's range, and the two it shares
+  return sizeof(CtaShared) + (size_t)p.cta_tasks * sizeof(unsigned long long) + ((size_t)p.B + 1) * sizeof(int);
 }
 
 cudaError_t prepare_expand_pass() {
-  const int bytes = (int)expand_dynamic_smem(C2T_MAX_BATCH);
-  const int fused = (int)expand_dynamic_smem(C2T_FUSED_MAX_BATCH);
+  const int bytes = 100 * 1024;                      // more than plan_shared asks for at the limits of a configuration
   cudaError_t e = cudaFuncSetAttribute(expand_pass_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_pass_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_pass_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_pass_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_prune_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, fused);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_prune_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, fused);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_prune_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_prune_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   return e;
 }
 
-cudaError_t launch_expand_prune(const PassParams &p, const TreeState &t, int level, const c2t_frontier *out, int dtype,
-                                int grid, cudaStream_t s) {
+cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, const c2t_frontier *out, int dtype, int grid, cudaStream_t s) {
   c2t_frontier o = {nullptr, nullptr, nullptr, nullptr};
   if (out) o = *out;
-  const size_t smem = expand_dynamic_smem(p.B);
+  size_t smem = plan_shared(p, grid);
+  if (smem < sizeof(PruneShared)) smem = sizeof(PruneShared);
   if (dtype == C2T_BF16)
     return launch_chained(expand_prune_kernel<true>, dim3(grid), dim3(kExpandThreads), smem, s, p, t, level, o);
   return launch_chained(expand_prune_kernel<false>, dim3(grid), dim3(kExpandThreads), smem, s, p, t, level, o);
 }
 
-cudaError_t launch_expand_pass(const PassParams &p, int dtype, int grid, cudaStream_t s) {
-  const size_t smem = expand_dynamic_smem(p.B);
+cudaError_t launch_expand_pass(PassParams p, int dtype, int grid, cudaStream_t s) {
+  const size_t smem = plan_shared(p, grid);
   const bool bf16 = dtype == C2T_BF16;
   if (p.topm_pool) {                                 // also sets the candidates of Eq. 3 aside
     if (bf16) return launch_chained(expand_pass_kernel<true, true>, dim3(grid), dim3(kExpandThreads), smem, s, p);

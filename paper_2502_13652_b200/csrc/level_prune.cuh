@@ -1,5 +1,5 @@
-// The per-sequence work of a level (Eq. 1, Eq. 4, Alg. 1, Sec. 4.2.2): merge of the rows' partial records,
-// features, classifier, the two prunings, compaction, tree append.  A device function, so that the pruning kernel
+// The per-sequence work of a level (Eq. 1, Eq. 4, Alg. 1, Sec. 4.2.2): features, classifier, the two prunings,
+// compaction, tree append, from the results that the expand pass (or the merge of gathered records) has per row.  A device function, so that the pruning kernel
 // (one CTA per sequence) and the expand kernel's last CTA (small batches: expand and prune in one launch) share it.
 #pragma once
 
@@ -55,139 +55,16 @@ __device__ double classify(const TreeState &t, const float *s_w, double P, doubl
   return 1.0 / (1.0 + exp(-z));
 }
 
-// What one warp makes of the partial records of one active row of the last expand pass.
+// A row's merged sums, as one warp holds them.
 struct RowMerge {
   double M, S, T;              // row maximum; sums over every other element of e^(x - M) and e^(x - M)(x - M)
   unsigned long long top;      // the row's best key (0: none)
   int n_valid;                 // candidates written (at most K)
 };
 
-// One warp merges the partial records of active row `a` (all lanes return the same values).  The K
-// best (logit, token) pairs go to out_x / out_tok (shared or global memory, best first, padded with
-// -inf / -1), token ids offset by tok_base; vloc is the length of the rows the pass read (tokens at
-// or past it pad a ragged last vector).  sk: the warp's staging area of kStageKeys keys.
-__device__ RowMerge merge_row_partials(const TreeState &t, const PassInfo &info, int seq, int a, int K, int vloc,
-                                       unsigned long long *sk, float *out_x, int *out_tok, int tok_base) {
-  const int lane = threadIdx.x & 31;
-  // the workers that hold a piece of this row: the rows, each behind info.pad virtual vectors, were cut every info.span
-  const long long first_vec = (long long)a * (info.vec_per_row + info.pad) + info.pad;
-  const int c_first = (int)(first_vec / info.span);
-  const int c_last = (int)((first_vec + info.vec_per_row - 1) / info.span);
-  int n_splits = c_last - c_first + 1;
-  if (n_splits > t.max_splits) {                    // the host's sizing and the pass disagree: say so, stay in bounds
-    n_splits = t.max_splits;
-    if (lane == 0) atomicOr(&t.status[seq], C2T_ST_INTERNAL);
-  }
-  const size_t slot0 = (size_t)a * t.max_splits;
-  const int n_keys = n_splits * K;
-
-  // rows with few partials (the usual case): every load is issued before the first use
-  const bool staged = n_splits <= 32 && n_keys <= kStageKeys && kHeldPerSlot == 1;
-  unsigned long long my_held = 0ull;
-  float4 my_stats = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (staged) {
-    if (lane < n_splits) {
-      my_held = t.part_held[slot0 + lane];
-      my_stats = t.part_stats[slot0 + lane];
-    }
-    for (int i = lane; i < n_keys; i += 32) sk[i] = t.part_keys[slot0 * K + i];
-  }
-
-  // the row maximum is the largest key held out of any partial's sums
-  const int n_held = n_splits * kHeldPerSlot;
-  unsigned long long top = my_held;
-  if (!staged) {
-    for (int i = lane; i < n_held; i += 32) {
-      unsigned long long k0 = t.part_held[slot0 * kHeldPerSlot + i];
-      top = k0 > top ? k0 : top;
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    unsigned long long other = __shfl_xor_sync(kFullMask, top, o);
-    top = other > top ? other : top;
-  }
-  const double M = (double)key_value(top);
-
-  // fp32 sums of every split: S = sum 2^t, U = sum 2^t t with t = x log2(e) + c, brought to
-  // natural units relative to M:  x - M = t ln2 + g,  g = -c ln2 - M
-  double S = 0.0, T = 0.0;
-  for (int i = lane; i < n_splits; i += 32) {
-    const float4 st = staged ? my_stats : t.part_stats[slot0 + i];
-    const double Ss = (double)st.y, Us = (double)st.z;
-    if (Ss != 0.0 || Us != 0.0) {               // (NaN passes this test and poisons the sums)
-      const double kLn2 = 0.69314718055994530942;
-      const double g = -(double)st.x * kLn2 - M;
-      const double f = exp(g);
-      S += Ss * f;
-      T += f * (kLn2 * Us + g * Ss);
-    }
-  }
-  // held-out elements are not in those sums: add them exactly, all but the row maximum itself
-  for (int i = lane; i < n_held; i += 32) {
-    const unsigned long long key = staged ? my_held : t.part_held[slot0 * kHeldPerSlot + i];
-    if (key == 0ull || key == top) continue;
-    const float x = key_value(key);
-    if (x > kNegInfAsFinite) {
-      double d = (double)x - M;
-      double e = exp(d);
-      S += e;
-      T += e * d;
-    }
-  }
-  // the K best keys over all splits become the candidates
-  S = warp_sum(S);
-  T = warp_sum(T);
-  int n_valid = 0;
-  if (staged) {
-    // every split's list is sorted and now in shared memory, one list per lane: take the
-    // largest head K times (a key of a token past the vocabulary ends its list: it pads a
-    // ragged last vector and sorts behind every real element)
-    __syncwarp();
-    int pos = 0;
-    for (; n_valid < K; ++n_valid) {
-      unsigned long long h = (lane < n_splits && pos < K) ? sk[lane * K + pos] : 0ull;
-      if (h != 0ull && key_token(h) >= vloc) h = 0ull;
-      const uint32_t hi = (uint32_t)(h >> 32), mx_hi = __reduce_max_sync(kFullMask, hi);
-      const uint32_t mx_lo = __reduce_max_sync(kFullMask, hi == mx_hi ? (uint32_t)h : 0u);
-      const unsigned long long mx = ((unsigned long long)mx_hi << 32) | mx_lo;
-      if (mx == 0ull) break;
-      if (lane == 0) { out_x[n_valid] = key_value(mx); out_tok[n_valid] = key_token(mx) + tok_base; }
-      if (h == mx) ++pos;
-    }
-    __syncwarp();
-  } else {
-    for (int i = lane; i < n_keys; i += 32) {
-      const unsigned long long key = t.part_keys[slot0 * K + i];
-      if (key == 0ull) continue;
-      const int tok = key_token(key);
-      if (tok >= vloc) continue;                    // padding of a ragged last vector
-      int rank = 0;
-      for (int r = 0; r < n_keys; ++r) {
-        unsigned long long other = t.part_keys[slot0 * K + r];
-        rank += (other > key) && (key_token(other) < vloc);
-      }
-      if (rank < K) { out_x[rank] = key_value(key); out_tok[rank] = tok + tok_base; }
-    }
-    for (int i = lane; i < n_keys; i += 32) {
-      unsigned long long key = t.part_keys[slot0 * K + i];
-      n_valid += (key != 0ull && key_token(key) < vloc);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) n_valid += __shfl_xor_sync(kFullMask, n_valid, o);
-    if (n_valid > K) n_valid = K;
-  }
-  // candidates that do not exist (fewer than K tokens in the vocabulary)
-  for (int r = n_valid + lane; r < K; r += 32) { out_x[r] = -INFINITY; out_tok[r] = -1; }
-  RowMerge m;
-  m.M = M; m.S = S; m.T = T; m.top = top; m.n_valid = n_valid;
-  return m;
-}
-
-// status bits of a row from its best key and its sums
-__device__ __forceinline__ uint32_t row_fault_bits(unsigned long long top, double S, double T) {
-  const float top_x = key_value(top);
-  if (top == 0ull || top_x <= kNegInfAsFinite) return C2T_ST_ALL_NEGINF;
+// status bits of a row from its maximum and its sums
+__device__ __forceinline__ uint32_t row_fault_bits(float top_x, double S, double T) {
+  if (!(top_x > kNegInfAsFinite)) return C2T_ST_ALL_NEGINF;
   if (top_x == INFINITY) return C2T_ST_POSINF_LOGIT;
   if (S != S || T != T || isinf(S)) return C2T_ST_NAN_LOGIT;
   return 0u;
@@ -246,14 +123,12 @@ __device__ RowMerge merge_row_records(const TreeState &t, const c2t_row_record *
   return m;
 }
 
-// records == nullptr: the rows come from this context's own expand pass; else from gathered records of n_shards shards
-// The shared memory of prune_level_body for a CTA of NW warps.
-template <int NW>
+// The shared memory of prune_level_body.
 struct PruneShared {
   double rowM[C2T_MAX_FRONTIER], rowL[C2T_MAX_FRONTIER], rowH[C2T_MAX_FRONTIER];
   double C[kMaxCand];
   double logP[kMaxCand];                       // joint log-probability of every candidate
-  unsigned long long keys[NW][kStageKeys];
+  unsigned long long ckey[kMaxCand];           // confidence of every candidate as an orderable integer
   float w[5 * C2T_MAX_HIDDEN + 4];
   float x[kMaxCand];
   int tok[kMaxCand];
@@ -261,16 +136,31 @@ struct PruneShared {
   double fchat[C2T_MAX_FRONTIER];              // its smallest confidence on the path from the root
   int fnode[C2T_MAX_FRONTIER];                 // tree id of every frontier node
   int rowfault[C2T_MAX_FRONTIER];
-  int scan[NW + 1];
+  int scan[33];
   int misc[2];
   unsigned char keep[kMaxCand], sel[kMaxCand];
 };
 
+// One row's maximum, normaliser and entropy into shared memory; its fault into the status word.
+__device__ __forceinline__ void row_stats(const TreeState &t, const RowResult &r, int b, int j, PruneShared &sh) {
+  sh.rowM[j] = r.M;
+  sh.rowL[j] = r.L;
+  if (t.entropy_top_m > 0 && t.entropy_top_m < t.V) {
+    const double2 sm = t.topm[(size_t)b * t.F + j];             // Eq. 3: only the M most probable tokens,
+    sh.rowH[j] = (r.L * sm.x - sm.y) / (1.0 + r.S);             // probabilities of the full softmax
+  } else {
+    sh.rowH[j] = r.L - r.T / (1.0 + r.S);                       // Eq. 2 with natural log
+  }
+  sh.rowfault[j] = (int)r.fault;
+  if (r.fault) atomicOr(&t.status[b], r.fault);
+}
+
 // NT: threads of the CTA; b: the sequence; chained: the caller is a kernel of the launch chain of its own (the
-// classifier's weights are then staged before the wait for the predecessor).
+// classifier's weights are then staged before the wait for the predecessor).  records == nullptr: the rows come from
+// this context's own expand pass; else from gathered records of n_shards shards.
 template <int NT, bool CHAINED>
 __device__ void prune_level_body(const TreeState &t, int level, const c2t_frontier &out, const c2t_row_record *records,
-                                 int n_shards, int b, PruneShared<NT / 32> &sh) {
+                                 int n_shards, int b, PruneShared &sh) {
   constexpr int kTreeThreads = NT, kTreeWarps = NT / 32;
   float *s_w = sh.w;
   double *s_rowM = sh.rowM, *s_rowL = sh.rowL, *s_rowH = sh.rowH;
@@ -281,9 +171,7 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
   unsigned char *s_keep = sh.keep, *s_sel = sh.sel;
   int *s_scan = sh.scan;
   int *s_misc = sh.misc;
-  unsigned long long (*s_keys)[kStageKeys] = sh.keys;
-  unsigned long long *s_ckey = &s_keys[0][0];     // phases 2-3 reuse the staging area: a key per candidate
-  static_assert(kTreeWarps * kStageKeys >= kMaxCand, "candidate keys must fit the staging area");
+  unsigned long long *s_ckey = sh.ckey;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int K = t.K, F = t.F;
@@ -303,8 +191,6 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
   if (CHAINED) chain_wait();
   __syncthreads();                                // (a CTA that serves several sequences: the last one's reads are done)
   int n = t.frontier_n[cur][b];
-  const int row_off = t.row_off_draft[b];         // rows of earlier sequences in the expand pass
-  const PassInfo info = *t.info_draft;            // (loads issued together with the one above)
   const int tree_base = t.tree_n[b];              // (needed last; its latency hides behind everything else)
   // the frontier's nodes, their joint log-probabilities (Eq. 1's left factor) and path confidences: two dependent
   // loads, issued by the last warp (the one least likely to have a row) so that they run beside the rows' merges;
@@ -329,25 +215,28 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
   }
   // (no barrier here: phase 1 reads nothing that was written above)
 
-  // ---- phase 1: one warp per row merges that row's partial records
-  for (int j = warp; j < n; j += kTreeWarps) {
-    uint32_t shard_faults = 0u;
-    const RowMerge m = records
-        ? merge_row_records(t, records, n_shards, b, j, K, &s_x[j * K], &s_tok[j * K], &shard_faults)
-        : merge_row_partials(t, info, b, row_off + j, K, t.V, s_keys[warp], &s_x[j * K], &s_tok[j * K], 0);
-    if (lane == 0) {
-      const uint32_t fault = shard_faults ? shard_faults : row_fault_bits(m.top, m.S, m.T);
-      const double L = log1p(m.S);                // ln sum_v e^(x_v - M); the maximum contributes the 1
-      s_rowM[j] = m.M;
-      s_rowL[j] = L;
-      if (t.entropy_top_m > 0 && t.entropy_top_m < t.V) {
-        const double2 sm = t.topm[(size_t)b * F + j];               // Eq. 3: only the M most probable tokens,
-        s_rowH[j] = (L * sm.x - sm.y) / (1.0 + m.S);               // probabilities of the full softmax
-      } else {
-        s_rowH[j] = L - m.T / (1.0 + m.S);        // Eq. 2 with natural log
+  // ---- phase 1: the rows' sums and candidates.  From the expand pass they are ready (a lane per row, a thread per
+  // candidate); gathered records are merged first, a warp per row.
+  if (!records) {
+    const RowResult *rows = t.rows + (size_t)b * F;
+    const unsigned long long *keys = t.row_keys + cbase;
+    for (int c = tid; c < n * K; c += kTreeThreads) {
+      const unsigned long long key = __ldcg(&keys[c]);
+      s_x[c] = key ? key_value(key) : -INFINITY;
+      s_tok[c] = key ? key_token(key) : -1;
+    }
+    for (int j = tid; j < n; j += kTreeThreads) row_stats(t, rows[j], b, j, sh);
+  } else {
+    for (int j = warp; j < n; j += kTreeWarps) {
+      uint32_t shard_faults = 0u;
+      const RowMerge m = merge_row_records(t, records, n_shards, b, j, K, &s_x[j * K], &s_tok[j * K], &shard_faults);
+      if (lane == 0) {
+        RowResult r;
+        r.M = m.M; r.S = m.S; r.T = m.T;
+        r.L = log1p(m.S);
+        r.fault = shard_faults ? shard_faults : row_fault_bits(m.top ? key_value(m.top) : -INFINITY, m.S, m.T);
+        row_stats(t, r, b, j, sh);
       }
-      s_rowfault[j] = (int)fault;
-      if (fault) atomicOr(&t.status[b], fault);
     }
   }
   __syncthreads();

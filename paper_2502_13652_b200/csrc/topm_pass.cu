@@ -30,13 +30,11 @@ constexpr int kTopmThreads = C2T_TOPM_THREADS;
 constexpr int kTopmBatch = 8;          // independent 16-byte loads a thread keeps in flight
 constexpr int kTopmCand = C2T_TOPM_CAND;   // candidate keys the fast path can hold in shared memory
 
-// Where the expand pass, which runs just before, left what this pass can reuse: the row's maximum
-// is the largest of the keys held out of its partial sums.
+// What the expand pass, which runs just before, left: the rows' results (their maxima), and how it cut the rows.
 struct TopmAux {
-  const unsigned long long *part_held;
+  const RowResult *rows;
   const PassInfo *info;
   const int32_t *row_off;
-  int max_splits;
 };
 
 // The bin, from 255 downwards, in which the need-th largest counted element lies, and how many
@@ -231,17 +229,7 @@ __device__ __forceinline__ void topm_entropy_row(const void *logits, long long s
   // the elements from there upwards are copied to shared memory and the selection runs on them alone;
   // rows where that guess fails (fewer than M such elements, or more than fit) take the general path.
   if (M < V) {
-    const PassInfo info = *aux.info;
-    const int a = aux.row_off[b] + j;
-    const long long first_vec = (long long)a * (info.vec_per_row + info.pad) + info.pad;
-    const int c_first = (int)(first_vec / info.span);
-    int n_splits = (int)((first_vec + info.vec_per_row - 1) / info.span) - c_first + 1;
-    if (n_splits > aux.max_splits) n_splits = aux.max_splits;
-    unsigned long long top = 0ull;
-    for (int sp = 0; sp < n_splits; ++sp) {
-      const unsigned long long k = aux.part_held[(size_t)a * aux.max_splits + sp];
-      top = k > top ? k : top;
-    }
+    const unsigned long long top = aux.rows[(size_t)b * F + j].top;
     const uint32_t top_key = (uint32_t)(top >> 32);
     const int d0 = (int)(top_key >> 24);
     const float mf = key_value(top);
@@ -548,7 +536,7 @@ struct TopmCollected {
 
 constexpr int kFinishThreads = 512;
 constexpr int kFinishCand = 8192;      // keys of a row that fit in shared memory (several CTAs per SM)
-constexpr int kFinishSegs = 64;        // segments of a row the kernel handles
+constexpr int kFinishSegs = 128;       // chunks of a row the kernel handles
 constexpr int kFinishBatch = 4;        // independent 16-byte loads a thread keeps in flight
 constexpr int kFinishMulti = 512;      // vectors of a row with more than one candidate that the list holds
 
@@ -592,53 +580,52 @@ __global__ void __launch_bounds__(kFinishThreads) topm_finish_kernel(int M, int 
   if (j >= n) return;
   const PassInfo info = *aux.info;
   const int a = aux.row_off[b] + j;
-  const long long first_vec = (long long)a * (info.vec_per_row + info.pad) + info.pad;
-  const int c_first = (int)(first_vec / info.span);
-  int n_splits = (int)((first_vec + info.vec_per_row - 1) / info.span) - c_first + 1;
-  if (n_splits > aux.max_splits) n_splits = aux.max_splits;
-  // ---- the row's segments: warp 0, two per lane
+  // ---- the row's segments: warp 0, several chunks of the row per lane.  In the pass a CTA has `span` chunks, its warps equal
+  // parts of those in order; a segment begins with the row, with a CTA's range or with a warp's part.
+  const int nc = info.vec_per_row, n_seg = nc < kFinishSegs ? nc : kFinishSegs;
   if (tid < 32) {
-    unsigned long long top = 0ull;
+    constexpr int PER = kFinishSegs / 32;
+    const unsigned long long top = aux.rows[(size_t)b * F + j].top;
+    const int per_cta = (int)info.span, part = (per_cta + kExpandWarps - 1) / kExpandWarps;
     float floor = kTopmLowestFloor;
-    bool ok = n_splits <= kFinishSegs;
-    int cnt[2] = {0, 0};
+    bool ok = nc <= kFinishSegs;
+    int cnt[PER], sum = 0;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int sp = lane * 2 + h;
-      if (sp < n_splits && sp < kFinishSegs) {
-        const size_t slot = (size_t)a * aux.max_splits + sp;
-        const unsigned long long k = aux.part_held[slot];
-        top = k > top ? k : top;
-        const TopmSegment rec = col.seg[slot];
-        ok = ok && rec.n >= 0;
-        floor = fmaxf(floor, rec.floor);
-        cnt[h] = rec.n > 0 ? rec.n : 0;
-        s_first[sp] = rec.first;
+    for (int h = 0; h < PER; ++h) {
+      const int ch = lane * PER + h;
+      cnt[h] = 0;
+      if (ch < n_seg) {
+        const int u = a * nc + ch, cta = u / per_cta, at = u - cta * per_cta;
+        if (ch == 0 || at % part == 0) {
+          const TopmSegment rec = col.seg[cta * kExpandWarps + at / part + a];
+          ok = ok && rec.n >= 0;
+          floor = fmaxf(floor, rec.floor);
+          cnt[h] = rec.n > 0 ? rec.n : 0;
+          s_first[ch] = rec.first;
+        }
       }
+      sum += cnt[h];
     }
-    int inc = cnt[0] + cnt[1];
+    int inc = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int v = __shfl_up_sync(kFull, inc, o);
       if (lane >= o) inc += v;
     }
-    if (lane * 2 < kFinishSegs) {
-      s_start[lane * 2 + 1] = inc - cnt[1];
-      s_start[lane * 2 + 2] = inc;
+    int run = inc - sum;
+#pragma unroll
+    for (int h = 0; h < PER; ++h) {
+      run += cnt[h];
+      s_start[lane * PER + h + 1] = run;
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long t2 = __shfl_xor_sync(kFull, top, o);
-      top = t2 > top ? t2 : top;
-      floor = fmaxf(floor, __shfl_xor_sync(kFull, floor, o));
-    }
+    for (int o = 16; o > 0; o >>= 1) floor = fmaxf(floor, __shfl_xor_sync(kFull, floor, o));
     ok = __all_sync(kFull, ok);
     if (lane == 0) { s_start[0] = 0; s_top = top; s_floor = floor; s_ok = ok; s_count = 0u; s_multi_n = 0u; }
   }
   __syncthreads();
   const float mf = key_value(s_top);
   const float floor = s_floor;
-  const int n_seg = n_splits < kFinishSegs ? n_splits : kFinishSegs;
   const int total = s_start[n_seg];
   if (s_ok && s_top != 0ull && mf < INFINITY) {      // (uniform)
     // A thread takes a vector at a time.  Nearly every vector holds exactly one element at or above the floor, and
@@ -741,7 +728,7 @@ cudaError_t launch_topm_entropy(const void *logits, int64_t seq_stride, int64_t 
   const long long rows = (long long)B * F;
   const dim3 grid((unsigned)(rows < n_ctas ? rows : n_ctas));     // a CTA fills an SM
   TopmAux aux;
-  aux.part_held = t.part_held; aux.info = t.info_draft; aux.row_off = t.row_off_draft; aux.max_splits = t.max_splits;
+  aux.rows = t.rows; aux.info = t.info_draft; aux.row_off = t.row_off_draft;
   const size_t smem = topm_dynamic_smem();
   if (dtype == C2T_BF16)
     return launch_chained(topm_entropy_kernel<true>, grid, dim3(kTopmThreads), smem, s, logits, seq_stride, row_stride, V, M, F,
@@ -754,7 +741,7 @@ cudaError_t launch_topm_finish(int M, int F, int B, const int32_t *counts, const
                                cudaStream_t s) {
   const dim3 grid(F, B);
   TopmAux aux;
-  aux.part_held = t.part_held; aux.info = t.info_draft; aux.row_off = t.row_off_draft; aux.max_splits = t.max_splits;
+  aux.rows = t.rows; aux.info = t.info_draft; aux.row_off = t.row_off_draft;
   TopmCollected col;
   col.pool = t.topm_pool; col.seg = t.topm_seg; col.done = t.topm_done;
   const size_t smem = (size_t)kFinishCand * sizeof(uint32_t);

@@ -35,24 +35,26 @@ __global__ void begin_step_kernel(TreeState t, const int32_t *root_tok, const in
   t.status[b] = 0u;
 }
 
-// The record of every active row of the last (sharded) expand pass, for c2t_export_row_records.
-__global__ void __launch_bounds__(kTreeThreads) export_rows_kernel(TreeState t, int level, int vloc, int tok_base,
-                                                                   c2t_row_record *out) {
-  __shared__ unsigned long long s_keys[kTreeWarps][kStageKeys];
+// The record of every active row of the last (sharded) expand pass, for c2t_export_row_records: a warp per row.
+constexpr int kExportWarps = 4;
+__global__ void __launch_bounds__(kExportWarps * 32) export_rows_kernel(TreeState t, int level, int tok_base, c2t_row_record *out) {
   chain_enter();
-  const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int n = t.frontier_n[level & 1][b];
-  const int row_off = t.row_off_draft[b];
-  const PassInfo info = *t.info_draft;
-  n = n < 0 ? 0 : (n > t.F ? t.F : n);
-  for (int j = warp; j < n; j += kTreeWarps) {
-    c2t_row_record *r = out + (size_t)b * t.F + j;
-    const RowMerge m = merge_row_partials(t, info, b, row_off + j, t.K, vloc, s_keys[warp], r->x, r->tok, tok_base);
-    if (lane == 0) {
-      r->M = m.M; r->S = m.S; r->T = m.T;
-      r->n = m.n_valid;
-      r->fault = row_fault_bits(m.top, m.S, m.T);
-    }
+  const int lane = threadIdx.x & 31;
+  const long long i = (long long)blockIdx.x * kExportWarps + (threadIdx.x >> 5);
+  if (i >= (long long)t.B * t.F) return;
+  const int b = (int)(i / t.F), j = (int)(i % t.F);
+  if (j >= t.frontier_n[level & 1][b]) return;
+  const RowResult r = t.rows[i];
+  c2t_row_record *o = out + i;
+  if (lane < t.K) {
+    const unsigned long long key = t.row_keys[i * t.K + lane];
+    o->x[lane] = key ? key_value(key) : -INFINITY;
+    o->tok[lane] = key ? key_token(key) + tok_base : -1;
+  }
+  if (lane == 0) {
+    o->M = r.M; o->S = r.S; o->T = r.T;
+    o->n = r.n_valid;
+    o->fault = r.fault;
   }
 }
 
@@ -60,7 +62,7 @@ __global__ void __launch_bounds__(kTreeThreads) export_rows_kernel(TreeState t, 
 __global__ void __launch_bounds__(kTreeThreads) prune_level_kernel(TreeState t, int level, c2t_frontier out,
                                                                    const c2t_row_record *records, int n_shards) {
   extern __shared__ __align__(16) unsigned char s_prune[];
-  PruneShared<kTreeWarps> &sh = *reinterpret_cast<PruneShared<kTreeWarps> *>(s_prune);
+  PruneShared &sh = *reinterpret_cast<PruneShared *>(s_prune);
   prune_level_body<kTreeThreads, true>(t, level, out, records, n_shards, blockIdx.x, sh);
 }
 
@@ -498,22 +500,23 @@ cudaError_t launch_begin_step(const TreeState &t, const int32_t *root_tok, const
   return launch_chained(begin_step_kernel, dim3((t.B + 127) / 128), dim3(128), 0, s, t, root_tok, prefix_len);
 }
 
-cudaError_t launch_export_rows(const TreeState &t, int level, int vocab_count, int vocab_begin, c2t_row_record *out,
-                               cudaStream_t s) {
-  return launch_chained(export_rows_kernel, dim3(t.B), dim3(kTreeThreads), 0, s, t, level, vocab_count, vocab_begin, out);
+cudaError_t launch_export_rows(const TreeState &t, int level, int vocab_begin, c2t_row_record *out, cudaStream_t s) {
+  const long long rows = (long long)t.B * t.F;
+  return launch_chained(export_rows_kernel, dim3((unsigned)((rows + kExportWarps - 1) / kExportWarps)), dim3(kExportWarps * 32), 0, s,
+                        t, level, vocab_begin, out);
 }
 
 cudaError_t launch_prune_level(const TreeState &t, int level, const c2t_frontier *out, const c2t_row_record *records,
                                int n_shards, cudaStream_t s) {
   c2t_frontier o = {nullptr, nullptr, nullptr, nullptr};
   if (out) o = *out;
-  return launch_chained(prune_level_kernel, dim3(t.B), dim3(kTreeThreads), sizeof(PruneShared<kTreeWarps>), s, t, level, o,
+  return launch_chained(prune_level_kernel, dim3(t.B), dim3(kTreeThreads), sizeof(PruneShared), s, t, level, o,
                         records, n_shards);
 }
 
 cudaError_t prepare_tree_kernels() {
   return cudaFuncSetAttribute(prune_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(PruneShared<kTreeWarps>));
+                              (int)sizeof(PruneShared));
 }
 
 cudaError_t launch_final_prune(const TreeState &t, cudaStream_t s) {
