@@ -135,7 +135,7 @@ size_t carve(const c2t_config *c, void *base, TreeState *t) {
   s.rows = w.take<RowResult>(B * F);
   s.row_keys = w.take<unsigned long long>(B * F * K);
   s.row_done = w.take<int32_t>(B * F);
-  s.cells = w.take<uint32_t>((size_t)s.n_chunks * 32);
+  s.cells = w.take<uint32_t>(B * F * ((row_chunks(c->vocab, eb) + 1) / 2) * 32);
   s.sums = w.take<SumRecord>((size_t)s.n_chunks);
   s.part_best = w.take<unsigned long long>(B * Nw * ms);
   s.w1 = w.take<float>(3 * C2T_MAX_HIDDEN);

@@ -2,15 +2,15 @@
 // softmax normaliser and entropy sums and the K largest logits (ties to the lower token id)
 //                                                        (Sec. 4.2.1, Eq. 2, Sec. 4.2.2).
 //
-// Work partition.  A row is cut into chunks of 512 consecutive 16-byte vectors (8 KB).  The chunks
+// Work partition.  A row is cut into chunks of 256 consecutive 16-byte vectors (4 KB).  The chunks
 // of the active rows (a device-side count per sequence), laid end to end, are dealt out in
 // contiguous equal ranges, one per CTA of a persistent grid (one CTA per SM).  Most warps of a CTA
 // stream, taking its chunks in turn; the others complete rows, in pairs, as soon as all chunks of
 // a row are done: while the stream goes on, but for the last row.
 //
-// Stream.  A warp keeps one chunk in registers, 16 vectors per lane, in four groups; as soon as a
+// Stream.  A warp keeps one chunk in registers, 8 vectors per lane, in two groups; as soon as a
 // group has been consumed the same registers are requested for the same group of the warp's next chunk,
-// so three to four groups (6 to 8 KB per warp) are in flight all the time.  Per element the
+// so one to two groups (2 to 4 KB per warp) are in flight all the time.  Per element the
 // stream does nothing but the sums and a running maximum: no comparison with a filter, no vote, no
 // branch that depends on the data.  Selection of the K largest is left to the row's end, where the
 // maxima say where to look.
@@ -21,7 +21,7 @@
 // is summed again with a better offset.  Offsets are integers so that rescaling is by exact powers of two.  (x log2(e)
 // uses the fp32 constant: a relative error of 1.3e-8 |x| in an element's weight.)
 //
-// Top-K.  Every lane records the maxima of its vectors in each half of a chunk, its "cells".  When all chunks of a
+// Top-K.  Every lane records the maximum of its vectors of a chunk, its "cell".  When all chunks of a
 // row are done the row is completed: the K-th largest of the 32 lanes' column maxima
 // is a lower bound on the row's K-th largest element, the few cells that reach it are read again (128 bytes each,
 // usually from L2), their elements at or above the bound are ranked by key, and the warps' sums are merged in double
@@ -214,11 +214,12 @@ __device__ __forceinline__ void write_record(SumRecord *rec, const LaneSums &ls)
 
 template <bool BF16>
 struct RowShape {
-  int vpr, v_full, nc;         // vectors of a row (the last may be ragged), whole ones, chunks
+  int vpr, v_full, nc, words;  // vectors of a row (the last may be ragged), whole ones, chunks, words of two cells per lane
   __device__ __forceinline__ explicit RowShape(int V) {
     vpr = (V + Vec<BF16>::N - 1) / Vec<BF16>::N;
     v_full = V / Vec<BF16>::N;
     nc = (vpr + kChunkVecs - 1) / kChunkVecs;
+    words = (nc + 1) / 2;
   }
 };
 
@@ -330,8 +331,8 @@ struct CtaRange {
 
 // ---------------------------------------------------------------- completing a row
 
-// vector k of the lane's 8 in a cell (16 in a chunk, a cell being half a chunk)
-__device__ __forceinline__ int cell_vector(int cell, int lane, int k) { return cell * (kChunkVecs / 2) + lane + 32 * k; }
+// vector k of the lane's 8 in a chunk
+__device__ __forceinline__ int cell_vector(int chunk, int lane, int k) { return chunk * kChunkVecs + lane + 32 * k; }
 
 template <bool BF16>
 __device__ __forceinline__ float element(const char *row, int tok) {    // -inf as the lowest finite value
@@ -401,15 +402,15 @@ __device__ __noinline__ int select_in_order(const PassParams &p, PairShared *ws,
   int have = 0;                                     // keys kept in pool[0 .. K)
   float thr = floor;
   constexpr int kBatch = 8;                         // elements of a lane in flight
-  for (int ch = 0; ch < rs.nc; ++ch) {
-    const uint32_t two = p.cells[(size_t)(a * rs.nc + ch) * 32 + lane];
+  for (int w = 0; w < rs.words; ++w) {
+    const uint32_t two = p.cells[((size_t)a * rs.words + w) * 32 + lane];
     // a cell is below the largest value it stands for by less than a bf16 step
     const float cell = fmaxf(__uint_as_float(two << 16), __uint_as_float(two & 0xFFFF0000u));
     const float most = BF16 ? cell : __uint_as_float(f32_from_orderable(f32_orderable(__float_as_uint(cell)) + 0xFFFFu));
     if (!__any_sync(kFull, most >= thr)) continue;
-    const int t1 = (ch + 1) * kChunkVecs * Vec<BF16>::N;
+    const int t1 = (w + 1) * 2 * kChunkVecs * Vec<BF16>::N;
     const int end = t1 < p.V ? t1 : p.V;
-    for (int t0 = ch * kChunkVecs * Vec<BF16>::N; t0 < end; t0 += 32 * kBatch) {
+    for (int t0 = w * 2 * kChunkVecs * Vec<BF16>::N; t0 < end; t0 += 32 * kBatch) {
       float x[kBatch];
       bool any = false;
 #pragma unroll
@@ -490,19 +491,19 @@ __device__ __forceinline__ int gather_keys(PairShared *ws, const char *row, cons
 // The K largest.
 template <bool BF16>
 __device__ __forceinline__ void complete_keys(const PassParams &p, PairShared *ws, int a, int b, int j) {
-  constexpr int kBatch = 32;                        // chunks of its column that a lane holds at a time
+  constexpr int kBatch = 32;                        // words of its column that a lane holds at a time: 64 chunks
   const RowShape<BF16> rs(p.V);
   const int lane = threadIdx.x & 31, K = p.K;
   const char *row = row_pointer(p, b, j, BF16 ? 2 : 4);
-  const uint32_t *cells = p.cells + (size_t)a * rs.nc * 32 + lane;
+  const uint32_t *cells = p.cells + (size_t)a * rs.words * 32 + lane;
   uint32_t v[kBatch], cm2 = kLowestBf16x2;
 #pragma unroll
-  for (int i = 0; i < kBatch; ++i) v[i] = i < rs.nc ? cells[i * 32] : kLowestBf16x2;
+  for (int i = 0; i < kBatch; ++i) v[i] = i < rs.words ? cells[i * 32] : kLowestBf16x2;
 #pragma unroll
   for (int i = 0; i < kBatch; ++i) cm2 = max_bf16x2(cm2, v[i]);
-  for (int c0 = kBatch; c0 < rs.nc; c0 += kBatch) {
+  for (int c0 = kBatch; c0 < rs.words; c0 += kBatch) {
 #pragma unroll
-    for (int i = 0; i < kBatch; ++i) v[i] = c0 + i < rs.nc ? cells[(c0 + i) * 32] : kLowestBf16x2;
+    for (int i = 0; i < kBatch; ++i) v[i] = c0 + i < rs.words ? cells[(c0 + i) * 32] : kLowestBf16x2;
 #pragma unroll
     for (int i = 0; i < kBatch; ++i) cm2 = max_bf16x2(cm2, v[i]);
   }
@@ -542,12 +543,12 @@ __device__ __forceinline__ void complete_keys(const PassParams &p, PairShared *w
 
   // ---- the cells that reach it
   int n_list = 0;
-  for (int c0 = 0; c0 < rs.nc && n_list <= kListCap; c0 += kBatch) {
-    if (rs.nc > kBatch) {
+  for (int c0 = 0; c0 < rs.words && n_list <= kListCap; c0 += kBatch) {
+    if (rs.words > kBatch) {
 #pragma unroll
-      for (int i = 0; i < kBatch; ++i) v[i] = c0 + i < rs.nc ? cells[(c0 + i) * 32] : kLowestBf16x2;
+      for (int i = 0; i < kBatch; ++i) v[i] = c0 + i < rs.words ? cells[(c0 + i) * 32] : kLowestBf16x2;
     }
-    unsigned long long mask = 0ull;                 // 16 chunks: bits of their first halves, then of their second ones; twice
+    unsigned long long mask = 0ull;                 // 16 words: bits of their first cells, then of their second ones; twice
 #pragma unroll
     for (int h = 0; h < kBatch / 16; ++h) {
       uint32_t m = 0u;
@@ -564,8 +565,8 @@ __device__ __forceinline__ void complete_keys(const PassParams &p, PairShared *w
       if (!bal || n_list > kListCap) break;
       const int pos = n_list + __popc(bal & ((1u << lane) - 1u));
       if (mask) {
-        const int bit = __ffsll((long long)mask) - 1, chunk = c0 + ((bit & 32) >> 1) + (bit & 15);
-        if (pos < kListCap) ws->list[pos] = chunk < rs.nc ? (2 * chunk + ((bit >> 4) & 1)) * 32 + lane : -1;
+        const int bit = __ffsll((long long)mask) - 1, chunk = 2 * (c0 + ((bit & 32) >> 1) + (bit & 15)) + ((bit >> 4) & 1);
+        if (pos < kListCap) ws->list[pos] = chunk < rs.nc ? chunk * 32 + lane : -1;
       }
       mask &= mask - 1ull;
       n_list += __popc(bal);
@@ -615,13 +616,13 @@ __device__ __forceinline__ void complete_sums(const PassParams &p, const CtaRang
   const float Mf = __shfl_sync(kFull, m, owner);
   const int trec = __shfl_sync(kFull, at, owner), tlane = __shfl_sync(kFull, tl, owner), tch = __shfl_sync(kFull, tc, owner);
 
-  // ---- that lane's 16 vectors of the chunk summed again without the maximum (and without its equals, which are counted)
+  // ---- that lane's vectors of the chunk summed again without the maximum (and without its equals, which are counted)
   const float cM = -rintf(fminf(Mf, 2e38f) * kLog2e);                 // the offset of the maximum: the reference of the merge
   float s_own, u_own;
   int equals = 0;
   {
     uint4 q[1];
-    const int vec[1] = {lane < 16 ? cell_vector(2 * tch, tlane, lane) : rs.vpr};
+    const int vec[1] = {lane < kChunkVecs / 32 ? cell_vector(tch, tlane, lane) : rs.vpr};
     load_vectors<BF16, 1>(q, row, vec, rs, p.V);
     float x[Vec<BF16>::N];
     Vec<BF16>::unpack(q[0], x);
@@ -629,7 +630,7 @@ __device__ __forceinline__ void complete_sums(const PassParams &p, const CtaRang
     acc.clear();
 #pragma unroll
     for (int e = 0; e < Vec<BF16>::N; ++e)
-      if (x[e] == Mf && lane < 16) { x[e] = kLowestF32; ++equals; }
+      if (x[e] == Mf && lane < kChunkVecs / 32) { x[e] = kLowestF32; ++equals; }
 #pragma unroll
     for (int e = 0; e < Vec<BF16>::N; e += 2) acc_pair(acc, (e >> 1) & 1, x[e], x[e + 1], pack2(kLog2e, kLog2e), pack2(cM, cM));
     acc.totals(s_own, u_own);
@@ -710,36 +711,33 @@ __device__ __forceinline__ float collection_floor(float lmax, int place) {
 
 // ---------------------------------------------------------------- the kernel
 
-// Sums and maxima of the chunk in q, each group of which is requested for the next chunk as soon as it is consumed.
+// Sums and maximum of the chunk in q, each group of which is requested for the next chunk as soon as it is consumed.
 template <bool BF16, bool TOPM>
-__device__ __forceinline__ void stream_chunk(uint4 (&q)[kGroups][4], const uint4 *src, int nnv, LaneSums &ls, f32x2 scale, float (&cv)[2],
-                                             TopmState &ts, int lane) {
+__device__ __forceinline__ float stream_chunk(uint4 (&q)[kGroups][4], const uint4 *src, int nnv, LaneSums &ls, f32x2 scale, TopmState &ts,
+                                              int lane) {
+  RunMax<BF16> m;
+  m.clear();
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    RunMax<BF16> m;
-    m.clear();
+  for (int g = 0; g < kGroups; ++g) {
 #pragma unroll
-    for (int g = 2 * h; g < 2 * h + 2; ++g) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (TOPM) {
-          RunMax<BF16> one;
-          one.clear();
-          one.take(q[g][k]);
-          const bool hit = one.value() >= ts.floor;            // (false for a vector of NaNs; such a row is reported anyway)
-          const unsigned hm = __ballot_sync(kFull, hit);
-          const int pos = ts.n + __popc(hm & ((1u << lane) - 1u));
-          if (hit && pos < ts.cap) store_keep_in_l2(ts.region + pos, q[g][k], ts.keep);
-          ts.n += __popc(hm);
-        }
-        m.take(q[g][k]);
-        Vec<BF16>::clamp(q[g][k]);
-        acc_vector<BF16>(ls.acc, q[g][k], scale, ls.c2);
+    for (int k = 0; k < 4; ++k) {
+      if (TOPM) {
+        RunMax<BF16> one;
+        one.clear();
+        one.take(q[g][k]);
+        const bool hit = one.value() >= ts.floor;              // (false for a vector of NaNs; such a row is reported anyway)
+        const unsigned hm = __ballot_sync(kFull, hit);
+        const int pos = ts.n + __popc(hm & ((1u << lane) - 1u));
+        if (hit && pos < ts.cap) store_keep_in_l2(ts.region + pos, q[g][k], ts.keep);
+        ts.n += __popc(hm);
       }
-      load_group<BF16>(q[g], src, g, nnv, lane);
+      m.take(q[g][k]);
+      Vec<BF16>::clamp(q[g][k]);
+      acc_vector<BF16>(ls.acc, q[g][k], scale, ls.c2);
     }
-    cv[h] = m.value();
+    load_group<BF16>(q[g], src, g, nnv, lane);
   }
+  return m.value();
 }
 
 // One warp's stream: every kStreamWarps-th chunk of the CTA's work order (TOPM: a contiguous part of it).
@@ -816,10 +814,9 @@ __device__ __forceinline__ void stream(const PassParams &p, CtaShared *cs, const
         ts.first = ts.n;
       }
     }
-    float cv[2];                                     // the chunk's two cells
-    stream_chunk<BF16, TOPM>(q, src, nnv, ls, scale, cv, ts, lane);
-    if (__any_sync(kFull, fmaxf(cv[0], cv[1]) > ls.limit)) {
-      const float m = warp_max(fmaxf(cv[0], cv[1]));
+    const float cv = stream_chunk<BF16, TOPM>(q, src, nnv, ls, scale, ts, lane);
+    if (__any_sync(kFull, cv > ls.limit)) {
+      const float m = warp_max(cv);
       ls.move_offset(m < INFINITY ? m : 2e38f);
       const float2 su = sum_again<BF16>(row, ch, ls.c, p.V);
       ls.acc.clear();
@@ -827,11 +824,13 @@ __device__ __forceinline__ void stream(const PassParams &p, CtaShared *cs, const
       ls.acc.U[0] = pack2(su.y, 0.f);
     }
     // ---- the chunk's cells; at the end of the warp's part of the row the record
-    ls.end_chunk(fmaxf(cv[0], cv[1]), ch);
+    ls.end_chunk(cv, ch);
     const int u = a * rs.nc + ch;
     fresh = !more || na != a;
     if (C2T_IN_BOUNDS(u, p.n_chunks, p.status)) {
-      p.cells[(size_t)u * 32 + lane] = cell_bits(cv[0], BF16) | (cell_bits(cv[1], BF16) << 16);
+      uint32_t *word = p.cells + ((size_t)a * rs.words + (ch >> 1)) * 32 + lane;
+      if (ch + 1 == rs.nc && !(ch & 1)) *word = cell_bits(cv, BF16) | (kLowestBf16x2 & 0xFFFF0000u);     // (no second cell)
+      else reinterpret_cast<unsigned short *>(word)[ch & 1] = (unsigned short)cell_bits(cv, BF16);
       if (fresh) write_record(p.sums + u, ls);
     }
     if (fresh) {

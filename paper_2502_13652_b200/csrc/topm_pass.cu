@@ -536,7 +536,7 @@ struct TopmCollected {
 
 constexpr int kFinishThreads = 512;
 constexpr int kFinishCand = 8192;      // keys of a row that fit in shared memory (several CTAs per SM)
-constexpr int kFinishSegs = 128;       // chunks of a row the kernel handles
+constexpr int kFinishSegs = 256;       // chunks of a row the kernel handles
 constexpr int kFinishBatch = 4;        // independent 16-byte loads a thread keeps in flight
 constexpr int kFinishMulti = 512;      // vectors of a row with more than one candidate that the list holds
 
