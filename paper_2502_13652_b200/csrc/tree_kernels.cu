@@ -303,30 +303,57 @@ __global__ void __launch_bounds__(kTreeThreads) accept_walk_kernel(TreeState t, 
 
 // ---------------------------------------------------------------- dense mask -
 
-// One CTA per (sequence, final-tree row): the row's ancestor-or-self set as bits in shared
-// memory (a walk up the parent pointers, at most D+1 steps), then the row of kv_len additive
-// mask values, 0 or -inf (Sec. 2.2).
+// Eight rows of a sequence's final tree per CTA, a warp per row: the row's ancestor-or-self set as bits in shared memory (a
+// walk up the parent pointers, at most D+1 steps), then the row of kv_len additive mask values, 0 or -inf (Sec. 2.2).  Bound
+// by the stores, so they are 16 bytes wide; the walk runs on a copy of the parents in shared memory, because one that
+// loads every parent from global memory costs several microseconds before the first store.  64 x 60 rows of 4160
+// bf16 values: 26.6 -> 11.1 us per call (32 MB, 2.9 TB/s).
+constexpr int kMaskRows = 8;
 template <typename T>
-__global__ void __launch_bounds__(256) dense_mask_kernel(TreeState t, T *out, long long kv_len, T zero, T ninf) {
-  __shared__ unsigned long long s_bits[(C2T_MAX_TREE + 63) / 64];   // Nw never exceeds the tree capacity
-  const int b = blockIdx.y, i = blockIdx.x, tid = threadIdx.x;
-  const int Nw = t.Nw, n = t.final_n[b];
-  const int words = (Nw + 63) / 64;
-  for (int w = tid; w < words; w += blockDim.x) s_bits[w] = 0ull;
-  __syncthreads();
-  if (tid == 0 && i < n) {
-    const int32_t *parent = t.final_parent + (size_t)b * Nw;
-    for (int j = i, guard = 0; j >= 0 && guard <= Nw; j = parent[j], ++guard) s_bits[j >> 6] |= 1ull << (j & 63);
-  }
-  __syncthreads();
+__global__ void __launch_bounds__(kMaskRows * 32) dense_mask_kernel(TreeState t, T *out, long long kv_len, T ninf) {
+  extern __shared__ int s_parent[];                  // [Nw], behind it the rows' bits
+  constexpr int E = 16 / sizeof(T);
+  const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = (int)blockIdx.x * kMaskRows + warp;
+  const int Nw = t.Nw, words = (Nw + 31) / 32;
+  unsigned *bits = reinterpret_cast<unsigned *>(s_parent + Nw) + warp * words;
+  chain_enter();
+  const int n = t.final_n[b];
   const long long prefix = t.prefix_len[b];
-  T *row = out + ((size_t)b * Nw + i) * kv_len;
-  for (long long c = tid; c < kv_len; c += blockDim.x) {
-    bool on = c < prefix;
+  for (int j = threadIdx.x; j < Nw; j += kMaskRows * 32) s_parent[j] = t.final_parent[(size_t)b * Nw + j];
+  for (int w = lane; w < words; w += 32) bits[w] = 0u;
+  __syncthreads();
+  if (i >= Nw) return;
+  if (lane == 0 && i < n)
+    for (int j = i, guard = 0; j >= 0 && j < Nw && guard <= Nw; j = s_parent[j], ++guard) bits[j >> 5] |= 1u << (j & 31);
+  __syncwarp();
+  auto value = [&](long long c) -> T {
     const long long j = c - prefix;
-    if (j >= 0 && j < Nw) on = (s_bits[j >> 6] >> (j & 63)) & 1ull;
-    row[c] = on ? zero : ninf;
+    return c < prefix || (j < Nw && ((bits[j >> 5] >> (j & 31)) & 1u)) ? (T)0 : ninf;
+  };
+  T *row = out + ((size_t)b * Nw + i) * kv_len;
+  long long head = (long long)((16 - (reinterpret_cast<uintptr_t>(row) & 15)) & 15) / (int)sizeof(T);     // up to the first 16-byte boundary
+  head = head < kv_len ? head : kv_len;
+  const long long body = (kv_len - head) / E;
+  if (lane < head) row[lane] = value(lane);
+  union { uint4 v; T e[E]; } zeros, ninfs, mixed;
+#pragma unroll
+  for (int k = 0; k < E; ++k) { zeros.e[k] = (T)0; ninfs.e[k] = ninf; }
+  uint4 *dst = reinterpret_cast<uint4 *>(row + head);
+#pragma unroll 4
+  for (long long k = lane; k < body; k += 32) {
+    const long long c = head + k * E;
+    if (c + E <= prefix) {
+      dst[k] = zeros.v;
+    } else if (c >= prefix + Nw) {
+      dst[k] = ninfs.v;
+    } else {
+#pragma unroll
+      for (int q = 0; q < E; ++q) mixed.e[q] = value(c + q);
+      dst[k] = mixed.v;
+    }
   }
+  const long long done = head + body * E;
+  if (lane < kv_len - done) row[done + lane] = value(done + lane);
 }
 
 // ---------------------------------------------------------------- lazy walk --
@@ -472,15 +499,13 @@ __global__ void __launch_bounds__(kWalkThreads) export_lazy_best_kernel(TreeStat
 }  // namespace
 
 cudaError_t launch_dense_mask(const TreeState &t, void *out, int out_dtype, int64_t kv_len, cudaStream_t s) {
-  const dim3 grid(t.Nw, t.B);
-  if (out_dtype == C2T_F32) {
-    dense_mask_kernel<float><<<grid, 256, 0, s>>>(t, reinterpret_cast<float *>(out), kv_len, 0.f, -INFINITY);
-  } else {
-    // bf16 as raw 16-bit words: +0 and -inf
-    dense_mask_kernel<unsigned short><<<grid, 256, 0, s>>>(t, reinterpret_cast<unsigned short *>(out), kv_len,
-                                                          (unsigned short)0x0000, (unsigned short)0xFF80);
-  }
-  return cudaGetLastError();
+  const dim3 grid((t.Nw + kMaskRows - 1) / kMaskRows, t.B);
+  const size_t smem = (size_t)t.Nw * sizeof(int) + (size_t)kMaskRows * ((t.Nw + 31) / 32) * sizeof(unsigned);    // (at most 40 KB)
+  if (out_dtype == C2T_F32)                          // the values as raw words: +0 and -inf
+    return launch_chained(dense_mask_kernel<unsigned>, grid, dim3(kMaskRows * 32), smem, s, t, reinterpret_cast<unsigned *>(out),
+                          (long long)kv_len, 0xFF800000u);
+  return launch_chained(dense_mask_kernel<unsigned short>, grid, dim3(kMaskRows * 32), smem, s, t, reinterpret_cast<unsigned short *>(out),
+                        (long long)kv_len, (unsigned short)0xFF80);
 }
 
 cudaError_t launch_lazy_walk_round(const TreeState &t, int round, const c2t_accept_out *out,
