@@ -9,19 +9,15 @@ namespace {
 
 constexpr int kStaticMaxRows = C2T_STATIC_MAX_ROWS;
 constexpr int kStaticMaxVocab = C2T_STATIC_MAX_VOCAB;
-// slots per row the arg-max pass can need at the largest vocabulary (fp32: 4 elements per vector)
-constexpr int kStaticMaxSplits = (kStaticMaxVocab / 4 + kMinSpanVectors - 1) / kMinSpanVectors + 1;
 constexpr int kMaxDevices = 64;
-// the arg-max kernel keeps one row offset per "sequence" in shared memory, sized by the batch limit
-static_assert(C2T_STATIC_MAX_ROWS <= C2T_MAX_BATCH, "the static entry point passes its rows as the batch of the pass");
 
+// What the CTAs that read pieces of one row meet in; all zeros between calls (and when the library is loaded).
 struct StaticScratch {
-  PassInfo info;                                              // what the pass derived from the row counts
-  int32_t counts[kStaticMaxRows];                             // one active row per "sequence"
-  unsigned long long best[(size_t)kStaticMaxRows * kStaticMaxSplits];   // best key per (row, split)
+  unsigned long long best[kStaticMaxRows];                    // best key so far
+  int32_t done[kStaticMaxRows];                               // vectors seen
 };
 
-// The scratch itself.  Every GPU that loads the library holds these ~2.1 MB until the process exits.
+// The scratch itself.  Every GPU that loads the library holds these 48 KB until the process exits.
 static __device__ __align__(256) unsigned char g_static_scratch[sizeof(StaticScratch)];
 
 // Host side: the array's name is only a handle here; the device address comes from
@@ -32,30 +28,6 @@ struct PerDevice {
 };
 PerDevice g_dev[kMaxDevices];
 std::mutex g_dev_mutex;
-
-__global__ void static_prepare_kernel(StaticScratch *s, int rows, int max_splits) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < rows) s->counts[i] = 1;
-  // stale keys of an earlier call must never be taken for this call's
-  for (size_t k = i; k < (size_t)rows * max_splits; k += (size_t)gridDim.x * blockDim.x) s->best[k] = 0ull;
-}
-
-__global__ void static_finish_kernel(const StaticScratch *s, int rows, int max_splits, int32_t *out) {
-  const int a = blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= rows) return;
-  const PassInfo info = s->info;
-  const long long first_vec = (long long)a * info.vec_per_row;
-  const int c_first = (int)(first_vec / info.span);
-  const int c_last = (int)((first_vec + info.vec_per_row - 1) / info.span);
-  int n_splits = c_last - c_first + 1;
-  if (n_splits > max_splits) n_splits = max_splits;
-  unsigned long long best = 0ull;
-  for (int k = 0; k < n_splits; ++k) {
-    const unsigned long long key = s->best[(size_t)a * max_splits + k];
-    best = key > best ? key : best;
-  }
-  out[a] = best ? key_token(best) : -1;
-}
 
 }  // namespace
 }  // namespace c2t
@@ -90,25 +62,8 @@ extern "C" int c2t_row_argmax_static(const void *logits_dev, int32_t rows, int32
     pd = g_dev[dev];
   }
 
-  cudaStream_t s = (cudaStream_t)stream;
-  const int max_splits = max_splits_for(vocab, eb, pd.grid);   // <= kStaticMaxSplits by the limits above
-  static_prepare_kernel<<<(rows + 255) / 256, 256, 0, s>>>(pd.scratch, rows, max_splits);
-  if (cudaGetLastError() != cudaSuccess) return C2T_ECUDA;
-
-  PassParams p;
-  memset(&p, 0, sizeof p);
-  p.logits = logits_dev;
-  p.seq_stride = row_stride;      // every row is a "sequence" with one active row
-  p.row_stride = row_stride;
-  p.V = vocab; p.K = 1; p.B = rows; p.rows_per_seq_max = 1;
-  p.counts = pd.scratch->counts;  // address arithmetic on a device pointer, never dereferenced here
-  p.max_splits = max_splits;
-  p.n_slots = (int64_t)rows * max_splits;
-  p.info = &pd.scratch->info;
-  p.part_best = pd.scratch->best;
-  if (launch_argmax_pass(p, dtype, pd.grid, s) != cudaSuccess) return C2T_ECUDA;
-
-  static_finish_kernel<<<(rows + 255) / 256, 256, 0, s>>>(pd.scratch, rows, max_splits, argmax_dev);
-  if (cudaGetLastError() != cudaSuccess) return C2T_ECUDA;
+  if (launch_row_argmax(logits_dev, row_stride, rows, vocab, dtype, pd.scratch->best, pd.scratch->done, argmax_dev, pd.grid,
+                        (cudaStream_t)stream) != cudaSuccess)
+    return C2T_ECUDA;                                         // (address arithmetic on device pointers, never dereferenced here)
   return C2T_OK;
 }

@@ -175,7 +175,14 @@ int row_chunks(int vocab, int elem_bytes);                     // chunks of a ro
 cudaError_t prepare_expand_pass();   // once per device: opt in to the kernel's shared-memory size
 cudaError_t launch_expand_pass(PassParams p, int dtype, int grid, cudaStream_t s);
 cudaError_t launch_argmax_pass(const PassParams &p, int dtype, int grid, cudaStream_t s);
+// arg-max of every row of a matrix; best, done: [rows] device scratch, zeros between calls
+cudaError_t launch_row_argmax(const void *logits, int64_t row_stride, int rows, int V, int dtype, unsigned long long *best, int *done,
+                              int32_t *out, int grid, cudaStream_t s);
 struct TreeState;
+cudaError_t prepare_accept_lazy();   // once per device
+// the acceptance walk reading only the rows it visits; grid: CTAs of kPassThreads threads that the chip holds
+cudaError_t launch_accept_lazy(const TreeState &t, const void *logits, int64_t seq_stride, int64_t row_stride, const c2t_accept_out *out,
+                               int dtype, int grid, cudaStream_t s);
 // expand and prune of a level in one launch (batches of at most C2T_FUSED_MAX_BATCH sequences)
 cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, const c2t_frontier *out, int dtype,
                                 int grid, cudaStream_t s);
