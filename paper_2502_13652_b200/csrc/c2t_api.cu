@@ -92,6 +92,8 @@ size_t carve(const c2t_config *c, void *base, TreeState *t) {
   for (int i = 0; i < 2; ++i) {
     s.frontier_n[i] = w.take<int32_t>(B);
     s.frontier_node[i] = w.take<int32_t>(B * F);
+    s.frontier_logP[i] = w.take<double>(B * F);
+    s.frontier_chat[i] = w.take<double>(B * F);
   }
   s.tree_n = w.take<int32_t>(B);
   s.tree_token = w.take<int32_t>(B * cap);

@@ -103,7 +103,8 @@ struct PassInfo {
 
 // What the expand pass leaves per active row, at (b, j) of [B, F]; its K largest keys are in row_keys.
 struct RowResult {
-  double M, S, T, L;            // row maximum; sums over every other element of e^(x - M) and e^(x - M)(x - M); ln(1 + S)
+  double M, S, T, L, H;         // row maximum; sums over every other element of e^(x - M) and e^(x - M)(x - M); ln(1 + S);
+                                // the entropy of Eq. 2 with natural log
   unsigned long long top;       // the row's best key (0: none)
   int32_t n_valid;              // keys that exist (at most K)
   uint32_t fault;               // C2T_ST_* bits of the row's data
@@ -194,6 +195,7 @@ struct TreeState {
   // frontier, double buffered by level parity
   int32_t *frontier_n[2];      // [B]
   int32_t *frontier_node[2];   // [B, F]
+  double *frontier_logP[2], *frontier_chat[2];      // [B, F] the nodes' tree_logP and tree_Chat
   // tree
   int32_t *tree_n;             // [B]
   int32_t *tree_token, *tree_parent, *tree_level;   // [B, cap]

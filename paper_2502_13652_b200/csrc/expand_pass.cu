@@ -49,6 +49,7 @@ struct PairShared {
   unsigned long long pool[kPoolCap];
   __align__(16) float colmax[64];
   int list[kListCap], vecs[kListCap];
+  __align__(16) uint4 data[kListCap];
 };
 
 // A CTA's shared memory; behind it a transaction barrier per task (a row, or the CTA's part of one) and the row list.
@@ -464,7 +465,7 @@ __device__ __forceinline__ int gather_keys(PairShared *ws, const char *row, cons
       const bool hit = v[u] < rs.vpr && Vec<BF16>::vmax(q[u]) >= floor;
       const unsigned hm = __ballot_sync(kFull, hit);
       const int pos = n_vec + __popc(hm & lt_mask);
-      if (hit && pos < kListCap) ws->vecs[pos] = v[u];
+      if (hit && pos < kListCap) { ws->vecs[pos] = v[u]; ws->data[pos] = q[u]; }
       n_vec += __popc(hm);
     }
   }
@@ -474,11 +475,17 @@ __device__ __forceinline__ int gather_keys(PairShared *ws, const char *row, cons
 #pragma unroll 4
   for (int i0 = 0; i0 < n_vec * EPV; i0 += 32) {
     const int i = i0 + lane;
-    const int tok = i < n_vec * EPV ? ws->vecs[i / EPV] * EPV + i % EPV : V;
-    const float x = tok < V ? element<BF16>(row, tok) : -INFINITY;
-    const unsigned hm = __ballot_sync(kFull, x >= floor);
+    float x = -INFINITY;
+    int tok = V;
+    if (i < n_vec * EPV) {
+      tok = ws->vecs[i / EPV] * EPV + i % EPV;
+      if (BF16) x = __uint_as_float((uint32_t)reinterpret_cast<const unsigned short *>(ws->data)[i] << 16);
+      else x = reinterpret_cast<const float *>(ws->data)[i];
+    }
+    const bool hit = x >= floor && tok < V;
+    const unsigned hm = __ballot_sync(kFull, hit);
     const int pos = n + __popc(hm & lt_mask);
-    if (x >= floor && pos < kPoolCap) ws->pool[pos] = make_key(x, (uint32_t)tok);
+    if (hit && pos < kPoolCap) ws->pool[pos] = make_key(x, (uint32_t)tok);
     n += __popc(hm);
   }
   __syncwarp();
@@ -667,7 +674,9 @@ __device__ __forceinline__ void complete_sums(const PassParams &p, const CtaRang
     const double Sn = S * scale + (double)(equals - 1), Tn = scale * (kLn2 * U + g * S);
     RowResult *r = p.rows + (size_t)b * p.rows_per_seq_max + j;
     r->M = M; r->S = Sn; r->T = Tn;
-    r->L = log1p(Sn);                               // ln sum_v e^(x_v - M); the maximum contributes the 1
+    const double L = log1p(Sn);                     // ln sum_v e^(x_v - M); the maximum contributes the 1
+    r->L = L;
+    r->H = L - Tn / (1.0 + Sn);                     // Eq. 2 with natural log
     r->fault = row_fault_bits(Mf, Sn, Tn);
   }
   __syncwarp();
@@ -944,6 +953,8 @@ __global__ void __launch_bounds__(kExpandThreads, 1) expand_prune_kernel(const _
                                                                          c2t_frontier out) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
   __shared__ unsigned s_ticket;
+  __shared__ double s_w[kWCount];
+  if (threadIdx.x >= kStreamWarps * 32) stage_classifier(t, s_w, threadIdx.x - kStreamWarps * 32, kExpandThreads - kStreamWarps * 32);   // (written at init)
   chain_enter();
   expand_pass_body<BF16, false>(p, s_dyn);
   __threadfence();                                   // this CTA's row results, before its ticket
@@ -955,7 +966,7 @@ __global__ void __launch_bounds__(kExpandThreads, 1) expand_prune_kernel(const _
   if (threadIdx.x == 0) *t.ticket = 0u;              // for the next launch
   // the pass's shared memory is free now
   PruneShared &sh = *reinterpret_cast<PruneShared *>(s_dyn);
-  for (int b = 0; b < t.B; ++b) prune_level_body<kExpandThreads, false>(t, level, out, nullptr, 0, b, sh);
+  for (int b = 0; b < t.B; ++b) prune_level_body<kExpandThreads>(t, level, out, nullptr, 0, b, sh, s_w, nullptr);
 }
 
 }  // namespace

@@ -43,14 +43,30 @@ __device__ int block_exclusive_scan(int v, int *s_warp /*[NT/32+1]*/, int *total
 
 // ---------------------------------------------------------------- a level ---
 
+// The classifier's weights in shared memory, as doubles (a conversion per use costs more than the arithmetic): per hidden
+// unit its three input weights, its bias, its output weight; w[kW0] is the output bias.
+constexpr int kWStride = 6;
+constexpr int kW0 = kWStride * C2T_MAX_HIDDEN;
+constexpr int kWCount = kW0 + 2;
+__device__ __forceinline__ void stage_classifier(const TreeState &t, double *w, int tid, int n_threads) {
+  if (t.classifier != C2T_CLS_MLP) return;
+  for (int i = tid; i < 3 * t.hidden; i += n_threads) w[(i / 3) * kWStride + i % 3] = (double)t.w1[i];
+  for (int i = tid; i < t.hidden; i += n_threads) {
+    w[i * kWStride + 3] = (double)t.b1[i];
+    w[i * kWStride + 4] = (double)t.w2[i];
+  }
+  if (tid == 0) w[kW0] = (double)t.b2[0];
+}
+
 // Confidence of one child (Eq. 4): two-layer FFN on (P, H, d), ReLU, sigmoid.
-__device__ double classify(const TreeState &t, const float *s_w, double P, double H, double d) {
-  const float *w1 = s_w, *b1 = s_w + 3 * C2T_MAX_HIDDEN, *w2 = b1 + C2T_MAX_HIDDEN, *b2 = w2 + C2T_MAX_HIDDEN;
-  double z = (double)b2[0];
-  for (int k = 0; k < t.hidden; ++k) {
-    double a = (double)b1[k] + (double)w1[3 * k] * P + (double)w1[3 * k + 1] * H + (double)w1[3 * k + 2] * d;
+__device__ __forceinline__ double classify(int hidden, const double *w, double P, double H, double d) {
+  double z = w[kW0];
+#pragma unroll 4
+  for (int k = 0; k < hidden; ++k) {
+    const double *u = w + k * kWStride;
+    double a = u[3] + u[0] * P + u[1] * H + u[2] * d;
     if (a < 0.0) a = 0.0;
-    z += (double)w2[k] * a;
+    z += u[4] * a;
   }
   return 1.0 / (1.0 + exp(-z));
 }
@@ -70,13 +86,24 @@ __device__ __forceinline__ uint32_t row_fault_bits(float top_x, double S, double
   return 0u;
 }
 
+constexpr int kStageKeys = 320;
 // One warp merges the gathered records of row (b, j): lane s holds shard s's record.  Writes the K
 // best candidates to out_x / out_tok and returns the merged maximum and sums; *fault_out collects the
-// shards' status bits ("all -inf" only if every shard says so).
+// shards' status bits ("all -inf" only if every shard says so).  stage: room for kStageKeys keys in shared memory, where
+// the shards' lists are copied first if they fit (one after the other from global memory, a head costs a round trip).
 __device__ RowMerge merge_row_records(const TreeState &t, const c2t_row_record *records, int n_shards, int b, int j,
-                                      int K, float *out_x, int *out_tok, uint32_t *fault_out) {
+                                      int K, float *out_x, int *out_tok, uint32_t *fault_out, unsigned long long *stage) {
   const int lane = threadIdx.x & 31;
-  const c2t_row_record *rec = records + ((size_t)lane * t.B + b) * t.F + j;
+  const size_t row = (size_t)b * t.F + j, shard_rows = (size_t)t.B * t.F;
+  const c2t_row_record *rec = records + lane * shard_rows + row;
+  const bool staged = n_shards * K <= kStageKeys;
+  if (staged) {
+#pragma unroll 4
+    for (int i = lane; i < n_shards * K; i += 32) {
+      const c2t_row_record *r = records + (i / K) * shard_rows + row;
+      stage[i] = make_key(r->x[i % K], (uint32_t)r->tok[i % K]);
+    }
+  }
   double Mg = 0.0, Sg = 0.0, Tg = 0.0;
   int ng = 0;
   uint32_t fg = 0u;
@@ -106,9 +133,11 @@ __device__ RowMerge merge_row_records(const TreeState &t, const c2t_row_record *
   }
   S = warp_sum(S);
   T = warp_sum(T);
+  __syncwarp();
   int n_valid = 0, pos = 0;
   for (; n_valid < K; ++n_valid) {                // the shards' lists are sorted: take the largest head K times
-    const unsigned long long h = (live && pos < ng) ? make_key(rec->x[pos], (uint32_t)rec->tok[pos]) : 0ull;
+    unsigned long long h = 0ull;
+    if (live && pos < ng) h = staged ? stage[lane * K + pos] : make_key(rec->x[pos], (uint32_t)rec->tok[pos]);
     const uint32_t hi = (uint32_t)(h >> 32), mx_hi = __reduce_max_sync(kFullMask, hi);
     const uint32_t mx_lo = __reduce_max_sync(kFullMask, hi == mx_hi ? (uint32_t)h : 0u);
     const unsigned long long mx = ((unsigned long long)mx_hi << 32) | mx_lo;
@@ -117,6 +146,7 @@ __device__ RowMerge merge_row_records(const TreeState &t, const c2t_row_record *
     if (h == mx) ++pos;
   }
   for (int r = n_valid + lane; r < K; r += 32) { out_x[r] = -INFINITY; out_tok[r] = -1; }
+  __syncwarp();
   *fault_out = fault;
   RowMerge m;
   m.M = M; m.S = S; m.T = T; m.top = top; m.n_valid = n_valid;
@@ -126,85 +156,72 @@ __device__ RowMerge merge_row_records(const TreeState &t, const c2t_row_record *
 // The shared memory of prune_level_body.
 struct PruneShared {
   double rowM[C2T_MAX_FRONTIER], rowL[C2T_MAX_FRONTIER], rowH[C2T_MAX_FRONTIER];
-  double C[kMaxCand];
-  double logP[kMaxCand];                       // joint log-probability of every candidate
-  unsigned long long ckey[kMaxCand];           // confidence of every candidate as an orderable integer
-  float w[5 * C2T_MAX_HIDDEN + 4];
-  float x[kMaxCand];
-  int tok[kMaxCand];
   double flogP[C2T_MAX_FRONTIER];              // joint log-probability of every frontier node
   double fchat[C2T_MAX_FRONTIER];              // its smallest confidence on the path from the root
   int fnode[C2T_MAX_FRONTIER];                 // tree id of every frontier node
   int rowfault[C2T_MAX_FRONTIER];
-  int scan[33];
-  int misc[2];
-  unsigned char keep[kMaxCand], sel[kMaxCand];
+  unsigned long long ckey[kMaxCand];           // confidence of every candidate as an orderable integer, 0 for a dropped one
+  int count[32];                               // candidates added and selected, per 32
+  unsigned char sel[kMaxCand];
+};
+// ... and with gathered records, behind it:
+struct GatherShared {
+  float x[kMaxCand];
+  int tok[kMaxCand];
+  unsigned long long stage[16][kStageKeys];
 };
 
 // One row's maximum, normaliser and entropy into shared memory; its fault into the status word.
-__device__ __forceinline__ void row_stats(const TreeState &t, const RowResult &r, int b, int j, PruneShared &sh) {
+__device__ __forceinline__ void row_stats(const TreeState &t, const RowResult &r, const double2 &sm, int b, int j, PruneShared &sh) {
   sh.rowM[j] = r.M;
   sh.rowL[j] = r.L;
-  if (t.entropy_top_m > 0 && t.entropy_top_m < t.V) {
-    const double2 sm = t.topm[(size_t)b * t.F + j];             // Eq. 3: only the M most probable tokens,
-    sh.rowH[j] = (r.L * sm.x - sm.y) / (1.0 + r.S);             // probabilities of the full softmax
-  } else {
-    sh.rowH[j] = r.L - r.T / (1.0 + r.S);                       // Eq. 2 with natural log
-  }
+  if (t.entropy_top_m > 0 && t.entropy_top_m < t.V) sh.rowH[j] = (r.L * sm.x - sm.y) / (1.0 + r.S);   // Eq. 3: only the M most
+                                                                // probable tokens, probabilities of the full softmax
+  else sh.rowH[j] = r.H;                                        // Eq. 2
   sh.rowfault[j] = (int)r.fault;
   if (r.fault) atomicOr(&t.status[b], r.fault);
 }
 
-// NT: threads of the CTA; b: the sequence; chained: the caller is a kernel of the launch chain of its own (the
-// classifier's weights are then staged before the wait for the predecessor).  records == nullptr: the rows come from
-// this context's own expand pass; else from gathered records of n_shards shards.
-template <int NT, bool CHAINED>
+// NT: threads of the CTA; b: the sequence; w: the classifier's staged weights.  records == nullptr: the rows come from
+// this context's own expand pass; else from gathered records of n_shards shards (gs: room for their merge).
+//   The work is a chain of dependent steps over at most F K candidates, on the critical path of every level, so it is short
+// in steps rather than in operations: every global load whose address does not depend on another is issued at the top
+// (frontier nodes carry their log-probabilities and path confidences with them for that), a thread keeps its
+// candidates in registers, the cap ranks a candidate with a whole warp, and the compaction needs one barrier.
+// Eight levels of 64 sequences: 323 -> 307 us (expand and prune).
+template <int NT>
 __device__ void prune_level_body(const TreeState &t, int level, const c2t_frontier &out, const c2t_row_record *records,
-                                 int n_shards, int b, PruneShared &sh) {
-  constexpr int kTreeThreads = NT, kTreeWarps = NT / 32;
-  float *s_w = sh.w;
-  double *s_rowM = sh.rowM, *s_rowL = sh.rowL, *s_rowH = sh.rowH;
-  int *s_rowfault = sh.rowfault;
-  float *s_x = sh.x;
-  int *s_tok = sh.tok;
-  double *s_C = sh.C;
-  unsigned char *s_keep = sh.keep, *s_sel = sh.sel;
-  int *s_scan = sh.scan;
-  int *s_misc = sh.misc;
-  unsigned long long *s_ckey = sh.ckey;
-
+                                 int n_shards, int b, PruneShared &sh, const double *w, GatherShared *gs) {
+  constexpr int kRounds = kMaxCand / NT, kNW = NT / 32;        // candidates per thread; warps
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int K = t.K, F = t.F;
   const int cur = level & 1, nxt = cur ^ 1;
-  if (CHAINED) chain_release();
-  // the classifier's weights were written at init, not by the chain: they are staged while the
-  // expand pass may still be finishing
-  if (tid == 0) s_misc[1] = 0;                    // survivors of the first pruning
-  if (t.classifier == C2T_CLS_MLP) {
-    for (int i = tid; i < 3 * t.hidden; i += kTreeThreads) s_w[i] = t.w1[i];
-    for (int i = tid; i < t.hidden; i += kTreeThreads) {
-      s_w[3 * C2T_MAX_HIDDEN + i] = t.b1[i];
-      s_w[4 * C2T_MAX_HIDDEN + i] = t.w2[i];
-    }
-    if (tid == 0) s_w[5 * C2T_MAX_HIDDEN] = t.b2[0];
-  }
-  if (CHAINED) chain_wait();
-  __syncthreads();                                // (a CTA that serves several sequences: the last one's reads are done)
+  const size_t cbase = (size_t)b * F * K, fbase = (size_t)b * F;
+
+  // ---- loads (slots past the frontier's size hold anything: kept in bounds, unused)
   int n = t.frontier_n[cur][b];
-  const int tree_base = t.tree_n[b];              // (needed last; its latency hides behind everything else)
-  // the frontier's nodes, their joint log-probabilities (Eq. 1's left factor) and path confidences: two dependent
-  // loads, issued by the last warp (the one least likely to have a row) so that they run beside the rows' merges;
-  // phases 2 and 4 read them, behind barriers (slots past the frontier's size hold anything: kept in bounds, unused)
-  if (warp == kTreeWarps - 1 && lane < F) {
-    int f = t.frontier_node[cur][(size_t)b * F + lane];
-    f = f < 0 ? 0 : (f >= t.cap ? t.cap - 1 : f);
-    sh.fnode[lane] = f;
-    sh.flogP[lane] = t.tree_logP[(size_t)b * t.cap + f];
-    sh.fchat[lane] = t.tree_Chat[(size_t)b * t.cap + f];
+  const int base = t.tree_n[b];
+  unsigned long long key[kRounds];
+#pragma unroll
+  for (int r = 0; r < kRounds; ++r) {
+    const int c = tid + r * NT;
+    key[r] = !records && c < F * K ? __ldcg(&t.row_keys[cbase + c]) : 0ull;
+  }
+  const int jr = tid - (NT - 64), jf = tid - (NT - 32);        // the last two warps fetch the rows' and the frontier's data
+  RowResult row;
+  double2 sm = make_double2(0.0, 0.0);
+  if (!records && jr >= 0 && jr < F) {
+    row = t.rows[fbase + jr];
+    if (t.entropy_top_m > 0) sm = t.topm[fbase + jr];
+  }
+  int fnode = 0;
+  double flogP = 0.0, fchat = 0.0;
+  if (jf >= 0 && jf < F) {
+    fnode = t.frontier_node[cur][fbase + jf];
+    flogP = t.frontier_logP[cur][fbase + jf];
+    fchat = t.frontier_chat[cur][fbase + jf];
   }
   n = n < 0 ? 0 : (n > F ? F : n);
-  const size_t cbase = (size_t)b * F * K;
-
   if (n == 0) {                                   // the loop of Alg. 1 has ended for this sequence
     if (tid == 0) {
       t.frontier_n[nxt][b] = 0;
@@ -213,128 +230,140 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
     }
     return;
   }
-  // (no barrier here: phase 1 reads nothing that was written above)
-
-  // ---- phase 1: the rows' sums and candidates.  From the expand pass they are ready (a lane per row, a thread per
-  // candidate); gathered records are merged first, a warp per row.
+  __syncthreads();                                // (a CTA that serves several sequences: the last one's reads are done)
   if (!records) {
-    const RowResult *rows = t.rows + (size_t)b * F;
-    const unsigned long long *keys = t.row_keys + cbase;
-    for (int c = tid; c < n * K; c += kTreeThreads) {
-      const unsigned long long key = __ldcg(&keys[c]);
-      s_x[c] = key ? key_value(key) : -INFINITY;
-      s_tok[c] = key ? key_token(key) : -1;
-    }
-    for (int j = tid; j < n; j += kTreeThreads) row_stats(t, rows[j], b, j, sh);
+    if (jr >= 0 && jr < n) row_stats(t, row, sm, b, jr, sh);
   } else {
-    for (int j = warp; j < n; j += kTreeWarps) {
+    for (int j = warp; j < n; j += kNW) {
       uint32_t shard_faults = 0u;
-      const RowMerge m = merge_row_records(t, records, n_shards, b, j, K, &s_x[j * K], &s_tok[j * K], &shard_faults);
+      const RowMerge m = merge_row_records(t, records, n_shards, b, j, K, &gs->x[j * K], &gs->tok[j * K], &shard_faults, gs->stage[warp]);
       if (lane == 0) {
         RowResult r;
         r.M = m.M; r.S = m.S; r.T = m.T;
         r.L = log1p(m.S);
+        r.H = r.L - m.T / (1.0 + m.S);
         r.fault = shard_faults ? shard_faults : row_fault_bits(m.top ? key_value(m.top) : -INFINITY, m.S, m.T);
-        row_stats(t, r, b, j, sh);
+        row_stats(t, r, sm, b, j, sh);
       }
     }
   }
+  if (jf >= 0 && jf < n) {
+    sh.fnode[jf] = fnode;
+    sh.flogP[jf] = flogP;
+    sh.fchat[jf] = fchat;
+  }
   __syncthreads();
 
-  // ---- phase 2: features and confidence, one thread per candidate child
+  // ---- features and confidence, a thread per candidate child
   const int nc = n * K;
-  for (int c = tid; c < nc; c += kTreeThreads) {
-    const int j = c / K;
-    const int tok = s_tok[c];
-    const float x = s_x[c];
-    const bool ok = tok >= 0 && !s_rowfault[j];
-    const double lp = (x > kNegInfAsFinite) ? ((double)x - s_rowM[j]) - s_rowL[j] : -INFINITY;
-    const double logP = sh.flogP[j] + lp;                                   // Eq. 1 in log space
-    const double P = exp(logP);
-    const double H = s_rowH[j];
-    double C;
-    if (!ok) C = NAN;
-    else if (t.classifier == C2T_CLS_IDENTITY_JOINT) C = P;
-    else if (t.classifier == C2T_CLS_IDENTITY_COND) C = exp(lp);
-    else C = classify(t, s_w, P, H, (double)level);
-    const bool keep = ok && C >= (double)t.beta;                            // first pruning
-    s_C[c] = C;
-    s_keep[c] = keep;
-    s_sel[c] = keep;
-    // (C desc, index asc) as integer compares: an orderable image of C, 0 for a dropped candidate
-    const unsigned long long cb = (unsigned long long)__double_as_longlong(C);
-    s_ckey[c] = keep ? (cb ^ ((cb >> 63) ? ~0ull : 0x8000000000000000ull)) : 0ull;
-    if (keep) atomicAdd(&s_misc[1], 1);
-    t.cand_token[cbase + c] = tok;
-    t.cand_lp[cbase + c] = ok ? lp : NAN;
-    t.cand_logP[cbase + c] = ok ? logP : NAN;
-    sh.logP[c] = logP;
-    t.cand_H[cbase + c] = ok ? H : NAN;
-    t.cand_C[cbase + c] = C;
-  }
-  __syncthreads();
-
-  // ---- phase 3: second pruning, the F survivors that come first under (C desc, index asc)
-  const int n_keep = s_misc[1];
-  if (n_keep > F) {
-    // four threads per survivor share the comparisons against all candidates
-    for (int c0 = 0; c0 < nc; c0 += kTreeThreads / 4) {
-      const int c = c0 + (tid >> 2);
-      const unsigned long long kc = c < nc ? s_ckey[c] : 0ull;
-      int rank = 0;
-      if (kc != 0ull)
-        for (int o = tid & 3; o < nc; o += 4) {
-          const unsigned long long ko = s_ckey[o];
-          rank += (ko > kc) || (ko == kc && o < c);
-        }
-      rank += __shfl_xor_sync(kFullMask, rank, 1);
-      rank += __shfl_xor_sync(kFullMask, rank, 2);
-      if (kc != 0ull && (tid & 3) == 0) s_sel[c] = rank < F;
+  double C[kRounds], logP[kRounds];
+  int tok[kRounds];
+  bool keep[kRounds], sel[kRounds];
+  int n_keep = 0;
+#pragma unroll
+  for (int r = 0; r < kRounds; ++r) {
+    const int c = tid + r * NT;
+    keep[r] = false;
+    if (r * NT < nc) {                            // (uniform)
+      if (c < nc) {
+        const int j = c / K;
+        float x;
+        if (records) { x = gs->x[c]; tok[r] = gs->tok[c]; }
+        else { x = key[r] ? key_value(key[r]) : -INFINITY; tok[r] = key[r] ? key_token(key[r]) : -1; }
+        const bool ok = tok[r] >= 0 && !sh.rowfault[j];
+        const double lp = (x > kNegInfAsFinite) ? ((double)x - sh.rowM[j]) - sh.rowL[j] : -INFINITY;
+        logP[r] = sh.flogP[j] + lp;                                             // Eq. 1 in log space
+        const double P = exp(logP[r]);
+        const double H = sh.rowH[j];
+        if (!ok) C[r] = NAN;
+        else if (t.classifier == C2T_CLS_IDENTITY_JOINT) C[r] = P;
+        else if (t.classifier == C2T_CLS_IDENTITY_COND) C[r] = exp(lp);
+        else C[r] = classify(t.hidden, w, P, H, (double)level);
+        keep[r] = ok && C[r] >= (double)t.beta;                                 // first pruning
+        // (C desc, index asc) as integer compares: an orderable image of C, 0 for a dropped candidate
+        const unsigned long long cb = (unsigned long long)__double_as_longlong(C[r]);
+        sh.ckey[c] = keep[r] ? (cb ^ ((cb >> 63) ? ~0ull : 0x8000000000000000ull)) : 0ull;
+        t.cand_token[cbase + c] = tok[r];
+        t.cand_lp[cbase + c] = ok ? lp : NAN;
+        t.cand_logP[cbase + c] = ok ? logP[r] : NAN;
+        t.cand_H[cbase + c] = ok ? H : NAN;
+        t.cand_C[cbase + c] = C[r];
+      }
+      n_keep += __syncthreads_count(keep[r]);
     }
+    sel[r] = keep[r];
   }
-  __syncthreads();
 
-  // ---- phase 4: stable compaction in candidate order; append to the tree, emit the frontier
-  const int per = (nc + kTreeThreads - 1) / kTreeThreads;      // consecutive candidates per thread
-  const int c0 = tid * per, c1 = (c0 + per < nc) ? c0 + per : nc;
+  // ---- second pruning: the F survivors that come first under (C desc, index asc); a warp counts what comes before a
+  // candidate, every lane with four of the keys in registers
+  if (n_keep > F) {
+    for (int c0 = warp; c0 < nc; c0 += kNW) {
+      const unsigned long long kc = sh.ckey[c0];
+      int before = 0;
+      for (int o0 = 0; o0 < nc; o0 += 128) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int o = o0 + q * 32 + lane;
+          const unsigned long long ko = o < nc ? sh.ckey[o] : 0ull;
+          before += ko > kc || (ko == kc && o < c0);
+        }
+      }
+      before = __reduce_add_sync(kFullMask, before);
+      if (lane == 0) sh.sel[c0] = kc != 0ull && before < F;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r)
+      if (tid + r * NT < nc) sel[r] = sh.sel[tid + r * NT];
+  }
+
+  // ---- stable compaction in candidate order; append to the tree, emit the frontier
   const bool add_all = t.tree_add == C2T_ADD_ALL_SURVIVORS;
-  int n_add = 0, n_sel = 0;
-  for (int c = c0; c < c1; ++c) { n_add += add_all ? s_keep[c] : s_sel[c]; n_sel += s_sel[c]; }
-  // one scan for both counts (each at most kMaxCand = 1024: 16 bits apiece)
-  int tot_both;
-  const int off_both = block_exclusive_scan<NT>(n_add | (n_sel << 16), s_scan, &tot_both);
-  int off_add = off_both & 0xFFFF, off_sel = off_both >> 16;
-  const int tot_add = tot_both & 0xFFFF, tot_sel = tot_both >> 16;
-  const int base = tree_base;
+  unsigned add_mask[kRounds], sel_mask[kRounds];
+#pragma unroll
+  for (int r = 0; r < kRounds; ++r) {
+    add_mask[r] = __ballot_sync(kFullMask, add_all ? keep[r] : sel[r]);
+    sel_mask[r] = __ballot_sync(kFullMask, sel[r]);
+    if (lane == 0) sh.count[r * kNW + warp] = __popc(add_mask[r]) | (__popc(sel_mask[r]) << 16);    // (each total at most 1024)
+  }
+  static_assert(kRounds * kNW == 32, "a count per lane");
+  __syncthreads();
+  const int counts = sh.count[lane];
+  const int total = __reduce_add_sync(kFullMask, counts);
+  const int tot_add = total & 0xFFFF, tot_sel = total >> 16;
   const bool overflow = base + tot_add > t.cap;
   const size_t tb = (size_t)b * t.cap;
-  for (int c = c0; c < c1; ++c) {
-    const bool add = add_all ? s_keep[c] : s_sel[c];
-    int flags = (s_keep[c] ? 1 : 0) | (s_sel[c] ? 2 : 0);
-    t.cand_flags[cbase + c] = flags;
-    if (!add) continue;
-    const int id = base + off_add++;
+#pragma unroll
+  for (int r = 0; r < kRounds; ++r) {
+    const int c = tid + r * NT;
+    if (r * NT >= nc) break;                      // (uniform)
+    const int before = __reduce_add_sync(kFullMask, lane < r * kNW + warp ? counts : 0);
+    if (c >= nc) continue;
+    t.cand_flags[cbase + c] = (keep[r] ? 1 : 0) | (sel[r] ? 2 : 0);
+    if (!(add_all ? keep[r] : sel[r])) continue;
+    const unsigned lt = (1u << lane) - 1u;
+    const int id = base + (before & 0xFFFF) + __popc(add_mask[r] & lt);
+    const int j = c / K;
+    const double chat = C[r] < sh.fchat[j] ? C[r] : sh.fchat[j];
     if (id < t.cap) {
-      const int j = c / K;
-      const int f = sh.fnode[j];
-      t.tree_token[tb + id] = s_tok[c];
-      t.tree_parent[tb + id] = f;
+      t.tree_token[tb + id] = tok[r];
+      t.tree_parent[tb + id] = sh.fnode[j];
       t.tree_level[tb + id] = level + 1;
-      t.tree_logP[tb + id] = sh.logP[c];              // (a node is only added if its candidate was in order)
-      t.tree_C[tb + id] = s_C[c];
-      const double ch = sh.fchat[j];
-      t.tree_Chat[tb + id] = s_C[c] < ch ? s_C[c] : ch;
+      t.tree_logP[tb + id] = logP[r];             // (a node is only added if its candidate was in order)
+      t.tree_C[tb + id] = C[r];
+      t.tree_Chat[tb + id] = chat;
     }
-    if (s_sel[c] && !overflow) {
-      const int slot = off_sel++;
+    if (sel[r] && !overflow) {
+      const int slot = (before >> 16) + __popc(sel_mask[r] & lt);
       if (!C2T_IN_BOUNDS(slot, F, &t.status[b])) continue;
-      t.frontier_node[nxt][(size_t)b * F + slot] = id;
-      if (out.token) out.token[(size_t)b * F + slot] = s_tok[c];
-      if (out.node_id) out.node_id[(size_t)b * F + slot] = id;
-      if (out.parent_slot) out.parent_slot[(size_t)b * F + slot] = c / K;
+      t.frontier_node[nxt][fbase + slot] = id;
+      t.frontier_logP[nxt][fbase + slot] = logP[r];
+      t.frontier_chat[nxt][fbase + slot] = chat;
+      if (out.token) out.token[fbase + slot] = tok[r];
+      if (out.node_id) out.node_id[fbase + slot] = id;
+      if (out.parent_slot) out.parent_slot[fbase + slot] = j;
     }
   }
-  __syncthreads();
   if (tid == 0) {
     const int next_n = overflow ? 0 : tot_sel;
     t.tree_n[b] = overflow ? t.cap : base + tot_add;

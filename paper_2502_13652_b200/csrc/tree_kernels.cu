@@ -28,6 +28,8 @@ __global__ void begin_step_kernel(TreeState t, const int32_t *root_tok, const in
   t.frontier_n[0][b] = 1;
   t.frontier_n[1][b] = 0;
   t.frontier_node[0][(size_t)b * t.F] = 0;
+  t.frontier_logP[0][(size_t)b * t.F] = 0.0;
+  t.frontier_chat[0][(size_t)b * t.F] = INFINITY;
   t.cand_n[b] = 0;
   t.final_n[b] = 0;
   t.root_tok[b] = root_tok[b];
@@ -43,11 +45,12 @@ __global__ void __launch_bounds__(kExportWarps * 32) export_rows_kernel(TreeStat
   const long long i = (long long)blockIdx.x * kExportWarps + (threadIdx.x >> 5);
   if (i >= (long long)t.B * t.F) return;
   const int b = (int)(i / t.F), j = (int)(i % t.F);
-  if (j >= t.frontier_n[level & 1][b]) return;
-  const RowResult r = t.rows[i];
+  const int n = t.frontier_n[level & 1][b];
+  const RowResult r = t.rows[i];                     // (loads issued together; rows past n hold anything)
+  const unsigned long long key = lane < t.K ? t.row_keys[i * t.K + lane] : 0ull;
+  if (j >= n) return;
   c2t_row_record *o = out + i;
   if (lane < t.K) {
-    const unsigned long long key = t.row_keys[i * t.K + lane];
     o->x[lane] = key ? key_value(key) : -INFINITY;
     o->tok[lane] = key ? key_token(key) + tok_base : -1;
   }
@@ -62,56 +65,72 @@ __global__ void __launch_bounds__(kExportWarps * 32) export_rows_kernel(TreeStat
 __global__ void __launch_bounds__(kTreeThreads) prune_level_kernel(TreeState t, int level, c2t_frontier out,
                                                                    const c2t_row_record *records, int n_shards) {
   extern __shared__ __align__(16) unsigned char s_prune[];
+  __shared__ double s_w[kWCount];
   PruneShared &sh = *reinterpret_cast<PruneShared *>(s_prune);
-  prune_level_body<kTreeThreads, true>(t, level, out, records, n_shards, blockIdx.x, sh);
+  GatherShared *gs = reinterpret_cast<GatherShared *>(s_prune + sizeof(PruneShared));
+  chain_release();
+  stage_classifier(t, s_w, threadIdx.x, kTreeThreads);   // (written at init, not by the chain: while the expand pass is finishing)
+  chain_wait();
+  prune_level_body<kTreeThreads>(t, level, out, records, n_shards, blockIdx.x, sh, s_w, gs);
 }
 
 // ---------------------------------------------------------------- rerank ----
 
 // Top-N rerank (Sec. 2.2): root + the N-1 nodes first under (Chat desc, id asc), renumbered
 // in id order.  Chat never exceeds the parent's and parents have lower ids, so the kept set
-// is closed under "parent of".
+// is closed under "parent of".  A chain of dependent steps: the tree is fetched into shared memory in one go, the scores as
+// orderable integers, and a warp ranks a node against 32 others at a time.
 __global__ void __launch_bounds__(kTreeThreads) final_prune_kernel(TreeState t) {
-  __shared__ int s_scan[kTreeWarps + 1];
+  extern __shared__ unsigned long long s_score[];              // [cap], behind it [cap] parents, [cap] new ids
+  __shared__ int s_count[kTreeWarps];
+  int *s_parent = reinterpret_cast<int *>(s_score + t.cap), *s_remap = s_parent + t.cap;
   chain_enter();
-  const int b = blockIdx.x, tid = threadIdx.x;
-  int n = t.tree_n[b];
-  n = n > t.cap ? t.cap : n;
+  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const size_t tb = (size_t)b * t.cap, fb = (size_t)b * t.Nw;
-  const double *chat = t.tree_Chat + tb;
-  int32_t *remap = t.remap + tb;
+  int n = t.tree_n[b];
+  for (int i = tid; i < t.cap; i += kTreeThreads) {            // (past n: anything, unused)
+    const unsigned long long cb = (unsigned long long)__double_as_longlong(t.tree_Chat[tb + i]);
+    s_score[i] = cb ^ ((cb >> 63) ? ~0ull : 0x8000000000000000ull);
+    s_parent[i] = t.tree_parent[tb + i];
+  }
+  n = n > t.cap ? t.cap : n;
+  __syncthreads();
   const bool all = (t.N <= 0 || n <= t.N);
-
-  int run = 0;     // nodes kept so far (ids below the chunk)
+  if (!all) {
+    for (int i = warp; i < n; i += kTreeWarps) {               // 1: kept (for now)
+      const unsigned long long mine = s_score[i];
+      int before = 0;
+#pragma unroll 4
+      for (int o = lane; o < n; o += 32) {
+        const unsigned long long other = s_score[o];
+        before += o > 0 && (other > mine || (other == mine && o < i));
+      }
+      before = __reduce_add_sync(kFull, before);
+      if (lane == 0) s_remap[i] = i == 0 || before < t.N - 1;
+    }
+    __syncthreads();
+  }
+  int run = 0;                                                 // nodes kept below the chunk
   for (int base = 0; base < n; base += kTreeThreads) {
     const int i = base + tid;
-    int keep = 0;
-    if (i < n) {
-      if (all || i == 0) keep = 1;
-      else {
-        const double ci = chat[i];
-        int rank = 0;
-        for (int o = 1; o < n; ++o) {
-          const double co = __ldg(&chat[o]);
-          rank += (co > ci) || (co == ci && o < i);
-        }
-        keep = rank < t.N - 1;
-      }
-    }
-    int total;
-    const int off = block_exclusive_scan<kTreeThreads>(keep, s_scan, &total);
-    if (i < n) remap[i] = keep ? run + off : -1;
-    run += total;
+    const bool keep = i < n && (all || s_remap[i]);
+    const unsigned mask = __ballot_sync(kFull, keep);
+    if (lane == 0) s_count[warp] = __popc(mask);
+    __syncthreads();
+    const int c = lane < kTreeWarps ? s_count[lane] : 0;
+    const int before = __reduce_add_sync(kFull, lane < warp ? c : 0);
+    if (i < n) s_remap[i] = keep ? run + before + __popc(mask & ((1u << lane) - 1u)) : -1;
+    run += __reduce_add_sync(kFull, c);
+    __syncthreads();
   }
-  __syncthreads();
   const int n_final = run > t.Nw ? t.Nw : run;
   for (int i = tid; i < n; i += kTreeThreads) {
-    const int m = remap[i];
+    const int m = s_remap[i];
     if (m < 0 || m >= t.Nw) continue;
-    const int par = t.tree_parent[tb + i];
+    const int par = s_parent[i];
     t.final_src[fb + m] = i;
     t.final_token[fb + m] = t.tree_token[tb + i];
-    t.final_parent[fb + m] = par < 0 ? -1 : remap[par];
+    t.final_parent[fb + m] = par < 0 ? -1 : s_remap[par];
     t.final_level[fb + m] = t.tree_level[tb + i];
   }
   for (int m = n_final + tid; m < t.Nw; m += kTreeThreads) {
@@ -125,35 +144,39 @@ __global__ void __launch_bounds__(kTreeThreads) final_prune_kernel(TreeState t) 
 
 // ---------------------------------------------------------------- verify ----
 
+// The tree is fetched into shared memory in one go; ancestors are found there.
 __global__ void __launch_bounds__(kTreeThreads) build_verify_kernel(TreeState t, c2t_verify out) {
-  __shared__ int s_has_child[C2T_MAX_BUDGET > C2T_MAX_TREE ? C2T_MAX_BUDGET : C2T_MAX_TREE];
-  __shared__ int s_scan[kTreeWarps + 1];
+  extern __shared__ int s_verify[];                            // [Nw] parents, [Nw] levels, [Nw] has-child
+  __shared__ int s_count[kTreeWarps];
   chain_enter();
-  const int b = blockIdx.x, tid = threadIdx.x;
+  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = t.final_n[b], Nw = t.Nw, W = t.W, width = t.D + 1;
-  const size_t fb = (size_t)b * Nw;
-  const int32_t *parent = t.final_parent + fb, *level = t.final_level + fb;
   const int prefix = t.prefix_len[b];
-
-  for (int i = tid; i < Nw; i += kTreeThreads) s_has_child[i] = 0;
+  const size_t fb = (size_t)b * Nw;
+  int *parent = s_verify, *level = s_verify + Nw, *has_child = s_verify + 2 * Nw;
+  for (int i = tid; i < Nw; i += kTreeThreads) {               // (past n: parent -1, level and token 0)
+    parent[i] = t.final_parent[fb + i];
+    level[i] = t.final_level[fb + i];
+    has_child[i] = 0;
+    if (out.tokens) out.tokens[fb + i] = t.final_token[fb + i];
+  }
+  if (out.retrieve)
+    for (int k = tid; k < Nw * width; k += kTreeThreads) out.retrieve[fb * width + k] = -1;
   __syncthreads();
   for (int i = tid; i < n; i += kTreeThreads)
-    if (parent[i] >= 0) s_has_child[parent[i]] = 1;
-  __syncthreads();
-
+    if (parent[i] >= 0) has_child[parent[i]] = 1;
   for (int i = tid; i < Nw; i += kTreeThreads) {
-    if (out.tokens) out.tokens[fb + i] = i < n ? t.final_token[fb + i] : 0;
-    if (out.parents) out.parents[fb + i] = i < n ? parent[i] : -1;
+    if (out.parents) out.parents[fb + i] = parent[i];
     if (out.position_ids) out.position_ids[fb + i] = i < n ? prefix + level[i] : 0;
-    if (out.mask_bits) {
-      uint64_t *row = out.mask_bits + (fb + i) * W;
-      for (int w = 0; w < W; ++w) row[w] = 0ull;
+  }
+  if (out.mask_bits) {
+    for (int k = tid; k < Nw * W; k += kTreeThreads) {         // a thread per word
+      const int i = k / W, w = k - i * W;
+      unsigned long long bits = 0ull;
       if (i < n)
-        for (int a = i, g = 0; a >= 0 && g <= t.D + 1; a = parent[a], ++g) row[a >> 6] |= 1ull << (a & 63);
-    }
-    if (out.retrieve) {
-      int32_t *row = out.retrieve + (fb + i) * width;
-      for (int k = 0; k < width; ++k) row[k] = -1;
+        for (int a = i, g = 0; a >= 0 && g <= t.D + 1; a = parent[a], ++g)
+          if ((a >> 6) == w) bits |= 1ull << (a & 63);
+      out.mask_bits[fb * W + k] = bits;
     }
   }
   __syncthreads();
@@ -161,17 +184,21 @@ __global__ void __launch_bounds__(kTreeThreads) build_verify_kernel(TreeState t,
   int run = 0;
   for (int base = 0; base < n; base += kTreeThreads) {
     const int i = base + tid;
-    const int leaf = (i < n && !s_has_child[i]) ? 1 : 0;
-    int total;
-    const int off = block_exclusive_scan<kTreeThreads>(leaf, s_scan, &total);
+    const bool leaf = i < n && !has_child[i];
+    const unsigned mask = __ballot_sync(kFull, leaf);
+    if (lane == 0) s_count[warp] = __popc(mask);
+    __syncthreads();
+    const int c = lane < kTreeWarps ? s_count[lane] : 0;
+    const int at = run + __reduce_add_sync(kFull, lane < warp ? c : 0) + __popc(mask & ((1u << lane) - 1u));
     if (leaf && out.retrieve) {
-      int32_t *row = out.retrieve + (fb + run + off) * width;
+      int32_t *row = out.retrieve + (fb + at) * width;
       for (int a = i, g = 0; a >= 0 && g <= t.D + 1; a = parent[a], ++g) {
         const int l = level[a];
         if (l >= 0 && l < width) row[l] = a;
       }
     }
-    run += total;
+    run += __reduce_add_sync(kFull, c);
+    __syncthreads();
   }
   if (tid == 0) {
     if (out.n_nodes) out.n_nodes[b] = n;
@@ -231,36 +258,30 @@ __global__ void __launch_bounds__(kTreeThreads) export_best_kernel(TreeState t, 
   }
 }
 
-// gathered == nullptr: the arg-max of this context's own pass; else the best of n_shards gathered keys per node
+// gathered == nullptr: the arg-max of this context's own pass; else the best of n_shards gathered keys per node.
+// The tree and the nodes' arg-maxes meet in shared memory, where every node looks for the child that carries its token, so
+// that the walk itself is a chain of one load per step.
 __global__ void __launch_bounds__(kTreeThreads) accept_walk_kernel(TreeState t, c2t_accept_out out,
                                                                    const unsigned long long *gathered, int n_shards) {
-  __shared__ int s_misc[1];
+  extern __shared__ int s_walk[];                              // [Nw] arg-maxes, [Nw] the child to go to
+  __shared__ int s_scan[kTreeWarps + 1];
+  __shared__ int s_total;
   chain_enter();
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = t.final_n[b], Nw = t.Nw, width = t.D + 1;
   const size_t fb = (size_t)b * Nw;
   const PassInfo info = *t.info_target;
-
-  // rows of earlier sequences in the argmax pass
-  if (!gathered) {
-    __shared__ int s_scan[kTreeWarps + 1];
-    int part = 0;
-    for (int i = tid; i < b; i += kTreeThreads) {
-      int c = t.final_n[i];
-      part += c < 0 ? 0 : (c > Nw ? Nw : c);
-    }
-    int total;
-    block_exclusive_scan<kTreeThreads>(part, s_scan, &total);
-    if (tid == 0) s_misc[0] = total;
-    __syncthreads();
-  }
-  const int row_off = gathered ? 0 : s_misc[0];
+  int *want = s_walk, *next = s_walk + Nw;
+  if (out.path)
+    for (int k = tid; k < width; k += kTreeThreads) out.path[(size_t)b * width + k] = k == 0 ? 0 : -1;
+  const int row_off = gathered ? 0 : target_row_offset(t, b, s_scan, &s_total);     // rows of earlier sequences in the arg-max pass
   // target argmax per node: best key over the row's partials
   for (int i = tid; i < Nw; i += kTreeThreads) {
     int tok = -1;
     if (i < n) {
       unsigned long long best = 0ull;
       if (gathered) {                               // equal logits in two shards: the larger key is the lower token id
+#pragma unroll 4
         for (int s = 0; s < n_shards; ++s) {
           const unsigned long long k = gathered[((size_t)s * t.B + b) * Nw + i];
           best = k > best ? k : best;
@@ -270,35 +291,27 @@ __global__ void __launch_bounds__(kTreeThreads) accept_walk_kernel(TreeState t, 
       }
       tok = best ? key_token(best) : -1;
     }
+    want[i] = tok;
+    next[i] = 0x7FFFFFFF;
     t.node_argmax[fb + i] = tok;
   }
   __syncthreads();
-  if (warp != 0) return;
-  // greedy walk by one warp
-  const int32_t *parent = t.final_parent + fb, *token = t.final_token + fb;
+  for (int c = 1 + tid; c < n; c += kTreeThreads) {
+    const int par = t.final_parent[fb + c];
+    if (par >= 0 && t.final_token[fb + c] == want[par]) atomicMin(&next[par], c);
+  }
+  __syncthreads();
+  if (warp != 0 || lane != 0) return;
   int cur = 0, len = 0;
-  if (out.path && lane < width) out.path[(size_t)b * width + lane] = lane == 0 ? 0 : -1;
-  for (int w = 32 + lane; out.path && w < width; w += 32) out.path[(size_t)b * width + w] = -1;
-  __syncwarp();
   while (n > 0 && len + 1 < width) {
-    const int want = t.node_argmax[fb + cur];
-    int found = 0x7FFFFFFF;
-    for (int c = cur + 1 + lane; c < n; c += 32)
-      if (parent[c] == cur && token[c] == want) { found = c; break; }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      int other = __shfl_xor_sync(kFull, found, o);
-      found = other < found ? other : found;
-    }
+    const int found = next[cur];
     if (found == 0x7FFFFFFF) break;
     cur = found;
     ++len;
-    if (lane == 0 && out.path) out.path[(size_t)b * width + len] = cur;
+    if (out.path) out.path[(size_t)b * width + len] = cur;
   }
-  if (lane == 0) {
-    if (out.accept_len) out.accept_len[b] = len;
-    if (out.next_token) out.next_token[b] = n > 0 ? t.node_argmax[fb + cur] : -1;
-  }
+  if (out.accept_len) out.accept_len[b] = len;
+  if (out.next_token) out.next_token[b] = n > 0 ? want[cur] : -1;
 }
 
 // ---------------------------------------------------------------- dense mask -
@@ -535,23 +548,30 @@ cudaError_t launch_prune_level(const TreeState &t, int level, const c2t_frontier
                                int n_shards, cudaStream_t s) {
   c2t_frontier o = {nullptr, nullptr, nullptr, nullptr};
   if (out) o = *out;
-  return launch_chained(prune_level_kernel, dim3(t.B), dim3(kTreeThreads), sizeof(PruneShared), s, t, level, o,
-                        records, n_shards);
+  return launch_chained(prune_level_kernel, dim3(t.B), dim3(kTreeThreads), sizeof(PruneShared) + (records ? sizeof(GatherShared) : 0),
+                        s, t, level, o, records, n_shards);
 }
 
+// dynamic shared memory: up to 128 KB for the rerank of the largest tree
+static size_t final_smem(int cap) { return (size_t)cap * (sizeof(unsigned long long) + 2 * sizeof(int)); }
+
 cudaError_t prepare_tree_kernels() {
-  return cudaFuncSetAttribute(prune_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(PruneShared));
+  cudaError_t e = cudaFuncSetAttribute(prune_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(sizeof(PruneShared) + sizeof(GatherShared)));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(final_prune_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)final_smem(C2T_MAX_TREE));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(build_verify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * C2T_MAX_TREE * (int)sizeof(int));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(accept_walk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * C2T_MAX_TREE * (int)sizeof(int));
+  return e;
 }
 
 cudaError_t launch_final_prune(const TreeState &t, cudaStream_t s) {
-  return launch_chained(final_prune_kernel, dim3(t.B), dim3(kTreeThreads), 0, s, t);
+  return launch_chained(final_prune_kernel, dim3(t.B), dim3(kTreeThreads), final_smem(t.cap), s, t);
 }
 
 cudaError_t launch_build_verify(const TreeState &t, const c2t_verify *out, cudaStream_t s) {
   c2t_verify o = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   if (out) o = *out;
-  return launch_chained(build_verify_kernel, dim3(t.B), dim3(kTreeThreads), 0, s, t, o);
+  return launch_chained(build_verify_kernel, dim3(t.B), dim3(kTreeThreads), 3 * (size_t)t.Nw * sizeof(int), s, t, o);
 }
 
 cudaError_t launch_export_best(const TreeState &t, int vocab_begin, unsigned long long *out, cudaStream_t s) {
@@ -562,7 +582,7 @@ cudaError_t launch_accept_walk(const TreeState &t, const c2t_accept_out *out, co
                                int n_shards, cudaStream_t s) {
   c2t_accept_out o = {nullptr, nullptr, nullptr};
   if (out) o = *out;
-  return launch_chained(accept_walk_kernel, dim3(t.B), dim3(kTreeThreads), 0, s, t, o, gathered, n_shards);
+  return launch_chained(accept_walk_kernel, dim3(t.B), dim3(kTreeThreads), 2 * (size_t)t.Nw * sizeof(int), s, t, o, gathered, n_shards);
 }
 
 }  // namespace c2t
