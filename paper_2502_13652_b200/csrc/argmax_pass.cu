@@ -1,8 +1,12 @@
 // Arg-max over rows of logits, per row the largest logit, ties to the lower token id.
-//   argmax_pass_kernel: the rows of all final nodes, for the greedy acceptance walk (Sec. 5 Metrics).  Same even
-// partition of the active rows as everywhere; plain 128-bit loads, four in flight per thread.
+//   argmax_pass_kernel: the rows of all final nodes, for the greedy acceptance walk (Sec. 5 Metrics).
 //   row_argmax_kernel: the rows of a matrix, from the logits to the token ids in one launch.
 //   accept_lazy_kernel: the acceptance walk that reads only the rows it visits, in one launch.
+// argmax_pass_kernel lays the rows end to end and cuts them into equal spans, one per CTA.  The warps of a CTA take groups of
+// 128 or 256 vectors (four or eight 16-byte loads per lane, all in flight) in turn, through rows and across them, and a warp brings its
+// best key of a row to the row's place by an atomic maximum: nothing waits at a row's end.  (With one key per CTA and row, two
+// barriers at every row's end cost more than a short row's loads: 3840 rows of 16032 bf16 values took 54.8 us.  With
+// a span per warp a CTA reads 16 places at once: 1 % slower on long rows.)
 #include "vocab_common.cuh"
 
 namespace c2t {
@@ -15,9 +19,10 @@ struct BestVector {
   int v;
   uint4 q;
   __device__ __forceinline__ void clear() { m = -INFINITY; v = -1; q = make_uint4(0u, 0u, 0u, 0u); }   // (clamped values are finite)
-  __device__ __forceinline__ void take(uint4 x, int at) {
-    Vec<BF16>::clamp(x);
-    const float vm = Vec<BF16>::vmax(x);
+  // (-inf counts as -2^127 here as everywhere: applied to the maximum, it costs one select per vector)
+  __device__ __forceinline__ void take(const uint4 &x, int at) {
+    float vm = Vec<BF16>::vmax(x);
+    vm = vm < kLowestF32 ? kLowestF32 : vm;
     if (vm > m) { m = vm; v = at; q = x; }
   }
   // the key of its largest element, the lowest token among equals (0: only NaN so far); V: length of the row
@@ -28,7 +33,7 @@ struct BestVector {
       Vec<BF16>::unpack(q, x);
 #pragma unroll
       for (int i = Vec<BF16>::N - 1; i >= 0; --i)
-        if (x[i] == m && v * Vec<BF16>::N + i < V) best = make_key(m, (uint32_t)(v * Vec<BF16>::N + i));
+        if ((x[i] < kLowestF32 ? kLowestF32 : x[i]) == m && v * Vec<BF16>::N + i < V) best = make_key(m, (uint32_t)(v * Vec<BF16>::N + i));
     }
     return best;
   }
@@ -43,69 +48,80 @@ __device__ __forceinline__ unsigned long long warp_best(unsigned long long best)
   return best;
 }
 
-// The CTA's largest key over vectors [v0, v1) of a row, in thread 0.
-template <bool BF16>
-__device__ __forceinline__ unsigned long long piece_best(const char *row, int v0, int v1, int v_full, int V, unsigned long long *s_best) {
-  using VT = Vec<BF16>;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  BestVector<BF16> bv;
-  bv.clear();
-  int v = v0 + tid;
-  for (; v + 3 * kPassThreads < v1; v += 4 * kPassThreads) {
-    uint4 q[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) q[i] = VT::load(row, v + i * kPassThreads, v_full, V);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) bv.take(q[i], v + i * kPassThreads);
-  }
-  for (; v < v1; v += kPassThreads) bv.take(VT::load(row, v, v_full, V), v);
-  unsigned long long best = warp_best(bv.key(V));
-  if (lane == 0) s_best[warp] = best;
-  __syncthreads();
-  if (warp == 0) best = warp_best(lane < kWarps ? s_best[lane] : 0ull);
-  __syncthreads();
-  return best;
-}
+constexpr int kMinPassSpan = 1024;     // a CTA of the pass never gets fewer vectors than this
+// Loads of a lane per group.  Small groups keep a CTA's reads closer together (rows of 16032 vectors: 156.7 -> 145.7 us for
+// 985 MB of bf16; 32064: 105.6 -> 98.5 us for 657 MB of fp32), large ones leave fewer row ends to a warp (rows of 2004 vectors:
+// 33.8 -> 27.1 us for 123 MB; 835 vectors: 13.4 -> 11.6 us); rows of 4000 to 8000 vectors do not care.
+constexpr int kLongRow = 4096;
 
-template <bool BF16>
+template <bool BF16, int kGroupLoads>
 __global__ void __launch_bounds__(kPassThreads, kPassCtasPerSm) argmax_pass_kernel(PassParams p) {
   using VT = Vec<BF16>;
+  constexpr int kGroup = 32 * kGroupLoads;
   __shared__ int s_off[C2T_MAX_BATCH + 1];
-  __shared__ unsigned long long s_best[kWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   chain_enter();
   const int n_rows = build_row_offsets(p.counts, p.B, p.rows_per_seq_max, s_off);
-  const Partition pt = make_partition<VT::N>(p, n_rows);
-  if (pt.start >= pt.end) return;
+  const int vpr = (p.V + VT::N - 1) / VT::N, v_full = p.V / VT::N;
+  const long long total = (long long)n_rows * vpr;
+  long long span = (total + gridDim.x - 1) / gridDim.x;
+  if (span < kMinPassSpan) span = kMinPassSpan;
+  long long pos = (long long)blockIdx.x * span;
+  const long long end = pos + span < total ? pos + span : total;
+  if (pos >= end) return;
   const size_t esz = BF16 ? 2 : 4;
-  long long pos = pt.start;
-  int a = (int)(pt.start / pt.vec_per_row);
-  int v0 = (int)(pt.start - (long long)a * pt.vec_per_row);
-  while (pos < pt.end) {
-    const long long left = pt.end - pos;
-    const int seg = left < (long long)(pt.vec_per_row - v0) ? (int)left : pt.vec_per_row - v0;
-    const int b = find_sequence(s_off, p.B, a);
-    const int j = p.row_sel ? p.row_sel[b] : a - s_off[b];
-    const char *row = reinterpret_cast<const char *>(p.logits) +
-                      ((size_t)b * p.seq_stride + (size_t)j * p.row_stride) * esz;
-    const int split = blockIdx.x - (int)(((long long)a * pt.vec_per_row) / pt.span);
-    const size_t slot = (size_t)a * p.max_splits + split;
-    const unsigned long long best = piece_best<BF16>(row, v0, v0 + seg, pt.v_full, p.V, s_best);
-    if (threadIdx.x == 0 && C2T_IN_BOUNDS(slot, p.n_slots, p.status)) p.part_best[slot] = best;
+  int a = (int)(pos / vpr), v0 = (int)(pos - (long long)a * vpr);
+  int turn = warp;                                   // groups until this warp's next
+  for (; pos < end; ++a, v0 = 0) {
+    const long long left = end - pos;
+    const int seg = left < (long long)(vpr - v0) ? (int)left : vpr - v0;
+    const int v1 = v0 + seg, groups = (seg + kGroup - 1) / kGroup;
     pos += seg;
-    ++a;
-    v0 = 0;
+    if (turn < groups) {
+      const int b = find_sequence(s_off, p.B, a), i = a - s_off[b], j = p.row_sel ? p.row_sel[b] : i;
+      const char *row = reinterpret_cast<const char *>(p.logits) + ((size_t)b * p.seq_stride + (size_t)j * p.row_stride) * esz;
+      const int whole = v1 < v_full ? v1 : v_full;   // (only the last vector of a ragged row is not whole)
+      BestVector<BF16> bv;
+      bv.clear();
+      do {
+        const int v = v0 + turn * kGroup + lane;
+        uint4 q[kGroupLoads];
+        if (v0 + (turn + 1) * kGroup <= whole) {
+#pragma unroll
+          for (int k = 0; k < kGroupLoads; ++k) q[k] = ldg_stream(reinterpret_cast<const uint4 *>(row) + v + k * 32);
+#pragma unroll
+          for (int k = 0; k < kGroupLoads; ++k) bv.take(q[k], v + k * 32);
+        } else {
+#pragma unroll
+          for (int k = 0; k < kGroupLoads; ++k)
+            if (v + k * 32 < whole) q[k] = ldg_stream(reinterpret_cast<const uint4 *>(row) + v + k * 32);
+#pragma unroll
+          for (int k = 0; k < kGroupLoads; ++k)
+            if (v + k * 32 < whole) bv.take(q[k], v + k * 32);
+          if (v1 > v_full && (v_full - v0) / kGroup == turn && lane == ((v_full - v0) & 31)) bv.take(VT::load(row, v_full, v_full, p.V), v_full);
+        }
+        turn += kWarps;
+      } while (turn < groups);
+      const unsigned long long best = warp_best(bv.key(p.V));
+      const size_t slot = (size_t)b * p.rows_per_seq_max + i;
+      if (lane == 0 && best && C2T_IN_BOUNDS(slot, p.n_slots, p.status)) atomicMax(&p.best[slot], best);
+    }
+    turn -= groups;
   }
 }
 
-// Rows a * row_stride of a matrix.  A row that lies in one CTA's piece is answered by that CTA; the pieces of a row cut
-// between CTAs meet in best[row] (atomic maximum) and done[row] (vectors seen; both 0 between calls), and the CTA that
-// completes the count answers and puts the zeros back: no launch before this one to clear anything, none after it to
-// gather.  256 rows of 128256 bf16 values: 23.9 -> 14.9 us per call (66 MB, 4.4 TB/s).
+// Rows a * row_stride of a matrix, in equal spans, one per CTA.  A row that lies in one span is answered by that CTA; the pieces
+// of a row cut between CTAs meet in best[row] (atomic maximum) and done[row] (vectors seen; both 0 between calls), and the CTA
+// that completes the count answers and puts the zeros back: no launch before this one to clear anything, none after it to
+// gather.  256 rows of 128256 bf16 values: 23.9 -> 14.9 us per call (66 MB); a span per warp makes it 18 pieces to a row, with
+// two fences each, and 19.4 us.
+constexpr int kMinSpanVectors = 1024;  // a CTA never gets fewer 16-byte vectors than this
 template <bool BF16>
 __global__ void __launch_bounds__(kPassThreads, kPassCtasPerSm) row_argmax_kernel(const char *logits, long long row_bytes, int rows, int V,
                                                                                  unsigned long long *best, int *done, int32_t *out) {
   using VT = Vec<BF16>;
   __shared__ unsigned long long s_best[kWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   chain_enter();
   const int vpr = (V + VT::N - 1) / VT::N, v_full = V / VT::N;
   const long long total = (long long)rows * vpr;
@@ -116,9 +132,25 @@ __global__ void __launch_bounds__(kPassThreads, kPassCtasPerSm) row_argmax_kerne
   int a = (int)(pos / vpr), v0 = (int)(pos - (long long)a * vpr);
   for (; pos < end; ++a, v0 = 0) {
     const long long left = end - pos;
-    const int seg = left < (long long)(vpr - v0) ? (int)left : vpr - v0;
-    unsigned long long key = piece_best<BF16>(logits + (size_t)a * row_bytes, v0, v0 + seg, v_full, V, s_best);
-    if (threadIdx.x == 0) {
+    const int seg = left < (long long)(vpr - v0) ? (int)left : vpr - v0, v1 = v0 + seg;
+    const char *row = logits + (size_t)a * row_bytes;
+    BestVector<BF16> bv;
+    bv.clear();
+    int v = v0 + tid;
+    for (; v + 3 * kPassThreads < v1; v += 4 * kPassThreads) {
+      uint4 q[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) q[i] = VT::load(row, v + i * kPassThreads, v_full, V);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) bv.take(q[i], v + i * kPassThreads);
+    }
+    for (; v < v1; v += kPassThreads) bv.take(VT::load(row, v, v_full, V), v);
+    unsigned long long key = warp_best(bv.key(V));
+    if (lane == 0) s_best[warp] = key;
+    __syncthreads();
+    if (warp == 0) key = warp_best(lane < kWarps ? s_best[lane] : 0ull);
+    __syncthreads();
+    if (tid == 0) {
       bool whole = seg == vpr;
       if (!whole) {
         if (key) atomicMax(&best[a], key);
@@ -233,8 +265,11 @@ __global__ void __launch_bounds__(kPassThreads, kPassCtasPerSm) accept_lazy_kern
 }  // namespace
 
 cudaError_t launch_argmax_pass(const PassParams &p, int dtype, int grid, cudaStream_t s) {
-  if (dtype == C2T_BF16) return launch_chained(argmax_pass_kernel<true>, dim3(grid), dim3(kPassThreads), 0, s, p);
-  return launch_chained(argmax_pass_kernel<false>, dim3(grid), dim3(kPassThreads), 0, s, p);
+  const int vec = dtype == C2T_BF16 ? 8 : 4;
+  const bool long_rows = (p.V + vec - 1) / vec >= kLongRow;
+  if (dtype == C2T_BF16)
+    return launch_chained(long_rows ? argmax_pass_kernel<true, 4> : argmax_pass_kernel<true, 8>, dim3(grid), dim3(kPassThreads), 0, s, p);
+  return launch_chained(long_rows ? argmax_pass_kernel<false, 4> : argmax_pass_kernel<false, 8>, dim3(grid), dim3(kPassThreads), 0, s, p);
 }
 
 cudaError_t launch_row_argmax(const void *logits, int64_t row_stride, int rows, int V, int dtype, unsigned long long *best, int *done,

@@ -86,7 +86,6 @@ size_t carve(const c2t_config *c, void *base, TreeState *t) {
   const size_t B = c->batch, F = c->frontier_cap, K = c->topk;
   const size_t cap = tree_capacity_unchecked(c), Nw = c2t_final_width(c);
   const int eb = c->dtype == C2T_BF16 ? 2 : 4;
-  const size_t ms = max_splits_for(c->vocab, eb, kMaxSms * kPassCtasPerSm);
   TreeState s;
   memset(&s, 0, sizeof s);
   for (int i = 0; i < 2; ++i) {
@@ -124,7 +123,6 @@ size_t carve(const c2t_config *c, void *base, TreeState *t) {
   s.status = w.take<uint32_t>(B);
   s.ticket = w.take<uint32_t>(1);
   s.info_draft = w.take<PassInfo>(1);
-  s.info_target = w.take<PassInfo>(1);
   s.row_off_draft = w.take<int32_t>(B + 1);
   s.topm = w.take<double2>(B * F);
   // every segment of the expand pass (with M > 0) ends a warp's span or a row
@@ -142,7 +140,7 @@ size_t carve(const c2t_config *c, void *base, TreeState *t) {
   s.row_done = w.take<int32_t>(B * F);
   s.cells = w.take<uint32_t>(B * F * ((row_chunks(c->vocab, eb) + 1) / 2) * 32);
   s.sums = w.take<SumRecord>((size_t)s.n_chunks);
-  s.part_best = w.take<unsigned long long>(B * Nw * ms);
+  s.best = w.take<unsigned long long>(B * Nw);
   s.w1 = w.take<float>(3 * C2T_MAX_HIDDEN);
   s.b1 = w.take<float>(C2T_MAX_HIDDEN);
   s.w2 = w.take<float>(C2T_MAX_HIDDEN);
@@ -164,6 +162,20 @@ PassParams expand_params(const TreeState &t, int level, const void *logits, int6
   p.rows = t.rows; p.row_keys = t.row_keys; p.row_done = t.row_done;
   p.cells = t.cells; p.sums = t.sums;
   p.n_chunks = t.n_chunks; p.n_segs = t.n_segs;
+  return p;
+}
+
+// the arg-max pass over the rows of all final nodes, or (walk) over the current node's row of every walking sequence
+PassParams argmax_params(const TreeState &t, const void *logits, int64_t seq_stride, int64_t row_stride, int vocab, bool walk) {
+  PassParams p;
+  memset(&p, 0, sizeof p);
+  p.logits = logits; p.seq_stride = seq_stride; p.row_stride = row_stride;
+  p.V = vocab; p.K = 1; p.B = t.B; p.rows_per_seq_max = walk ? 1 : t.Nw;
+  p.counts = walk ? t.walk_active : t.final_n;
+  p.row_sel = walk ? t.walk_cur : nullptr;
+  p.status = t.status;
+  p.best = t.best;
+  p.n_slots = (int64_t)t.B * t.Nw;
   return p;
 }
 
@@ -235,8 +247,6 @@ int c2t_init(const c2t_config *cfg, void *workspace_dev, size_t workspace_bytes,
   t.classifier = cfg->classifier; t.tree_add = cfg->tree_add; t.beta = cfg->threshold;
   t.entropy_top_m = cfg->entropy_top_m;
   t.topm_place = topm_floor_place(cfg->vocab, (int)ctx->elem_bytes, cfg->entropy_top_m);
-  t.max_splits_tgt = max_splits_for(cfg->vocab, (int)ctx->elem_bytes, ctx->grid);
-
   cudaError_t e = cudaSuccess;
   if (cfg->classifier == C2T_CLS_MLP) {
     const size_t h = cfg->hidden;
@@ -247,6 +257,7 @@ int c2t_init(const c2t_config *cfg, void *workspace_dev, size_t workspace_bytes,
   }
   if (e == cudaSuccess) e = cudaMemset(t.status, 0, sizeof(uint32_t) * cfg->batch);
   if (e == cudaSuccess) e = cudaMemset(t.ticket, 0, sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMemset(t.best, 0, sizeof(unsigned long long) * cfg->batch * t.Nw);
   if (e == cudaSuccess) e = cudaMemset(t.row_done, 0, sizeof(int32_t) * cfg->batch * cfg->frontier_cap);
   if (e != cudaSuccess) { cudaGetLastError(); delete ctx; return C2T_ECUDA; }
   *out = ctx;
@@ -418,16 +429,7 @@ int c2t_accept(c2t_ctx *ctx, const void *target_logits_dev, int64_t seq_stride, 
       (row_stride * ctx->elem_bytes) % 16)
     return C2T_EALIGN;
   const TreeState &t = ctx->t;
-  PassParams p;
-  memset(&p, 0, sizeof p);
-  p.logits = target_logits_dev; p.seq_stride = seq_stride; p.row_stride = row_stride;
-  p.V = t.V; p.K = 1; p.B = t.B; p.rows_per_seq_max = t.Nw;
-  p.counts = t.final_n;
-  p.max_splits = t.max_splits_tgt;
-  p.n_slots = (int64_t)t.B * t.Nw * t.max_splits_tgt;
-  p.status = t.status;
-  p.info = t.info_target;
-  p.part_best = t.part_best;
+  const PassParams p = argmax_params(t, target_logits_dev, seq_stride, row_stride, t.V, false);
   if (launch_argmax_pass(p, ctx->cfg.dtype, ctx->grid, (cudaStream_t)stream) != cudaSuccess)
     return C2T_ECUDA;
   if (launch_accept_walk(t, out, nullptr, 0, (cudaStream_t)stream) != cudaSuccess) return C2T_ECUDA;
@@ -446,16 +448,7 @@ int c2t_argmax_shard(c2t_ctx *ctx, const void *target_logits_dev, int64_t seq_st
       (row_stride * ctx->elem_bytes) % 16)
     return C2T_EALIGN;
   const TreeState &t = ctx->t;
-  PassParams p;
-  memset(&p, 0, sizeof p);
-  p.logits = target_logits_dev; p.seq_stride = seq_stride; p.row_stride = row_stride;
-  p.V = vocab_count; p.K = 1; p.B = t.B; p.rows_per_seq_max = t.Nw;
-  p.counts = t.final_n;
-  p.max_splits = t.max_splits_tgt;
-  p.n_slots = (int64_t)t.B * t.Nw * t.max_splits_tgt;
-  p.status = t.status;
-  p.info = t.info_target;
-  p.part_best = t.part_best;
+  const PassParams p = argmax_params(t, target_logits_dev, seq_stride, row_stride, vocab_count, false);
   if (launch_argmax_pass(p, ctx->cfg.dtype, ctx->grid, (cudaStream_t)stream) != cudaSuccess)
     return C2T_ECUDA;
   if (launch_export_best(t, vocab_begin, reinterpret_cast<unsigned long long *>(keys_dev), (cudaStream_t)stream) !=
@@ -510,17 +503,7 @@ int c2t_lazy_argmax_shard(c2t_ctx *ctx, const void *target_logits_dev, int64_t s
   if (!aligned16(target_logits_dev) || (seq_stride * ctx->elem_bytes) % 16 || (row_stride * ctx->elem_bytes) % 16)
     return C2T_EALIGN;
   const TreeState &t = ctx->t;
-  PassParams p;
-  memset(&p, 0, sizeof p);
-  p.logits = target_logits_dev; p.seq_stride = seq_stride; p.row_stride = row_stride;
-  p.V = vocab_count; p.K = 1; p.B = t.B; p.rows_per_seq_max = 1;
-  p.counts = t.walk_active;          // one row per sequence that is still walking ...
-  p.row_sel = t.walk_cur;            // ... the row of its current node
-  p.max_splits = t.max_splits_tgt;
-  p.n_slots = (int64_t)t.B * t.Nw * t.max_splits_tgt;
-  p.status = t.status;
-  p.info = t.info_target;
-  p.part_best = t.part_best;
+  const PassParams p = argmax_params(t, target_logits_dev, seq_stride, row_stride, vocab_count, true);
   cudaStream_t s = (cudaStream_t)stream;
   if (launch_argmax_pass(p, ctx->cfg.dtype, ctx->grid, s) != cudaSuccess) return C2T_ECUDA;
   if (launch_export_lazy_best(t, vocab_begin, reinterpret_cast<unsigned long long *>(keys_dev), s) != cudaSuccess)

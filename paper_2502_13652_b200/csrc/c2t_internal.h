@@ -86,7 +86,6 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
 
 constexpr int kPassThreads = 512;     // threads per CTA of the vocabulary pass
 constexpr int kPassCtasPerSm = 2;
-constexpr int kMinSpanVectors = 1024; // a CTA never gets fewer 16-byte vectors than this
 // the expand pass: one CTA per SM, 12 warps that stream and 4 that complete rows.  Measured on eight levels of 640 rows of
 // 128256 tokens (bf16 / fp32): 12 streaming warps 323 / 472 us, 16 325 / 462, 20 342 / 477, 24 372 / 550 (fewer registers per
 // thread: spills); chunks of 8 KB in 12 warps 335 / 468 (the unrolled chunk no longer fits the instruction caches).
@@ -94,11 +93,12 @@ constexpr int kExpandWarps = 12;
 constexpr int kExpandThreads = (kExpandWarps + 4) * 32;
 constexpr int kChunkVecs = 256;       // 16-byte vectors of a chunk: 8 per lane
 
-// What one launch of the vocabulary pass derived from the device-side row counts.
+// How the expand pass cut the rows (with M > 0: for the selection kernels).
 struct PassInfo {
   int32_t n_rows;       // active rows
-  int32_t vec_per_row;  // 16-byte vectors per row (last one may be ragged)
-  int64_t span;         // vectors per CTA (the expand pass counts both in chunks)
+  int32_t row_chunks;   // chunks per row
+  int32_t cta_chunks;   // chunks per CTA
+  int32_t reserved;
 };
 
 // What the expand pass leaves per active row, at (b, j) of [B, F]; its K largest keys are in row_keys.
@@ -127,10 +127,8 @@ struct PassParams {
   int32_t rows_per_seq_max;         // F (draft) or Nw (target)
   const int32_t *counts;            // [B] active rows per sequence, device
   const int32_t *row_sel;           // arg-max pass only, may be null: [B] the row of sequence b to read (then counts is 0 or 1)
-  int32_t max_splits;               // arg-max: partial slots per row
-  int64_t n_slots;                  // arg-max: partial slots in the workspace (rows the workspace was carved for x max_splits)
   uint32_t *status;                 // may be null: a status word for C2T_ST_INTERNAL (the first sequence's)
-  PassInfo *info;                   // written by CTA 0 (expand: only with M > 0)
+  PassInfo *info;                   // expand with M > 0: written by CTA 0
   int32_t *row_off;                 // expand with M > 0: [B+1] first active row of every sequence, written by CTA 0
   // expand: results per row, and what the warps that stream a row leave for the pair that completes it
   RowResult *rows;                  // [B, F]
@@ -145,8 +143,10 @@ struct PassParams {
   long long topm_pool_vecs;
   int32_t topm_place;               // the floor's place among the lane maxima (topm_floor_place)
   TopmSegment *topm_seg;            // [warp + row]
-  // argmax: per (row, split) best key
-  unsigned long long *part_best;
+  // argmax: [B, rows_per_seq_max] best key per row, the largest of what is there and of the row's keys (0 before the pass;
+  // the kernel that reads a key puts the 0 back)
+  unsigned long long *best;
+  int64_t n_slots;
 };
 
 // ---------------------------------------------------------------- candidates of the truncated entropy (Eq. 3)
@@ -170,8 +170,7 @@ struct TopmSegment {
 int topm_floor_place(int vocab, int elem_bytes, int M);
 size_t topm_pool_vectors(size_t batch, size_t rows_per_seq, int vocab, int elem_bytes);
 
-int max_splits_for(int vocab, int elem_bytes, int workers);   // partial slots a row of the arg-max pass can need
-int row_chunks(int vocab, int elem_bytes);                     // chunks of a row of the expand pass
+int row_chunks(int vocab, int elem_bytes);   // chunks of a row of the expand pass
 
 cudaError_t prepare_expand_pass();   // once per device: opt in to the kernel's shared-memory size
 cudaError_t launch_expand_pass(PassParams p, int dtype, int grid, cudaStream_t s);
@@ -190,7 +189,7 @@ cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, con
 // ---------------------------------------------------------------- tree state -
 
 struct TreeState {
-  int32_t B, V, K, F, D, N, Nw, W, cap, hidden, classifier, tree_add, max_splits_tgt;
+  int32_t B, V, K, F, D, N, Nw, W, cap, hidden, classifier, tree_add;
   float beta;
   // frontier, double buffered by level parity
   int32_t *frontier_n[2];      // [B]
@@ -219,7 +218,7 @@ struct TreeState {
   int32_t *topm_done;          // M > 0: [B, F] 1 where the row's sums came from the candidate vectors
   uint32_t *status;            // [B]
   uint32_t *ticket;            // one counter: CTAs of a fused expand + prune launch that have finished (0 between launches)
-  PassInfo *info_draft, *info_target;
+  PassInfo *info_draft;
   int32_t *row_off_draft;          // [B+1] first row of every sequence in the last expand pass
   RowResult *rows;                 // the expand pass: see PassParams
   unsigned long long *row_keys;
@@ -227,7 +226,7 @@ struct TreeState {
   uint32_t *cells;
   SumRecord *sums;
   int64_t n_chunks, n_segs;
-  unsigned long long *part_best;
+  unsigned long long *best;        // [B, Nw] best key per row of the last arg-max pass; zeros between passes
   float *w1, *b1, *w2, *b2;
 };
 
@@ -255,8 +254,7 @@ cudaError_t launch_dense_mask(const TreeState &t, void *out, int out_dtype, int6
 cudaError_t launch_accept_walk(const TreeState &t, const c2t_accept_out *out, const unsigned long long *gathered,
                                int n_shards, cudaStream_t s);
 cudaError_t launch_export_best(const TreeState &t, int vocab_begin, unsigned long long *out, cudaStream_t s);
-// one round of the lazy walk: round 0 starts it, round r > 0 consumes the arg-max of round r-1
-// gathered == nullptr: the round consumes this context's own arg-max pass; else n_shards gathered keys per sequence
+// one round of the lazy walk over sharded rows: round 0 starts it, round r > 0 takes n_shards gathered keys per sequence
 cudaError_t launch_lazy_walk_round(const TreeState &t, int round, const c2t_accept_out *out,
                                    const unsigned long long *gathered, int n_shards, cudaStream_t s);
 cudaError_t launch_export_lazy_best(const TreeState &t, int vocab_begin, unsigned long long *out, cudaStream_t s);

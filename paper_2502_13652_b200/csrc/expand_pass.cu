@@ -922,8 +922,8 @@ __device__ __forceinline__ void expand_pass_body(const PassParams &p, unsigned c
       for (int i = threadIdx.x; i <= p.B; i += kExpandThreads) p.row_off[i] = s_off[i];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       p.info->n_rows = n_rows;
-      p.info->vec_per_row = rs.nc;                   // (in chunks)
-      p.info->span = cr.per_cta;                     // (chunks per CTA)
+      p.info->row_chunks = rs.nc;
+      p.info->cta_chunks = cr.per_cta;
     }
   }
   if (cr.u0 >= cr.u1) return;
@@ -988,14 +988,6 @@ int topm_floor_place(int vocab, int elem_bytes, int M) {
 int row_chunks(int vocab, int elem_bytes) {
   const int vec = 16 / elem_bytes;
   return ((vocab + vec - 1) / vec + kChunkVecs - 1) / kChunkVecs;
-}
-
-int max_splits_for(int vocab, int elem_bytes, int workers) {
-  const int vec = 16 / elem_bytes;
-  const int vec_per_row = (vocab + vec - 1) / vec;
-  int by_span = (vec_per_row + kMinSpanVectors - 1) / kMinSpanVectors;
-  if (by_span > workers) by_span = workers;
-  return by_span + 1;
 }
 
 // the launch's shared memory

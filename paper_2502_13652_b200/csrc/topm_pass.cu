@@ -580,13 +580,13 @@ __global__ void __launch_bounds__(kFinishThreads) topm_finish_kernel(int M, int 
   if (j >= n) return;
   const PassInfo info = *aux.info;
   const int a = aux.row_off[b] + j;
-  // ---- the row's segments: warp 0, several chunks of the row per lane.  In the pass a CTA has `span` chunks, its warps equal
+  // ---- the row's segments: warp 0, several chunks of the row per lane.  In the pass a CTA has cta_chunks chunks, its warps equal
   // parts of those in order; a segment begins with the row, with a CTA's range or with a warp's part.
-  const int nc = info.vec_per_row, n_seg = nc < kFinishSegs ? nc : kFinishSegs;
+  const int nc = info.row_chunks, n_seg = nc < kFinishSegs ? nc : kFinishSegs;
   if (tid < 32) {
     constexpr int PER = kFinishSegs / 32;
     const unsigned long long top = aux.rows[(size_t)b * F + j].top;
-    const int per_cta = (int)info.span, part = (per_cta + kExpandWarps - 1) / kExpandWarps;
+    const int per_cta = info.cta_chunks, part = (per_cta + kExpandWarps - 1) / kExpandWarps;
     float floor = kTopmLowestFloor;
     bool ok = nc <= kFinishSegs;
     int cnt[PER], sum = 0;

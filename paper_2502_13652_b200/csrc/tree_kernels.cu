@@ -79,10 +79,13 @@ __global__ void __launch_bounds__(kTreeThreads) prune_level_kernel(TreeState t, 
 // Top-N rerank (Sec. 2.2): root + the N-1 nodes first under (Chat desc, id asc), renumbered
 // in id order.  Chat never exceeds the parent's and parents have lower ids, so the kept set
 // is closed under "parent of".  A chain of dependent steps: the tree is fetched into shared memory in one go, the scores as
-// orderable integers, and a warp ranks a node against 32 others at a time.
+// orderable integers.  Up to kRankNodes nodes a warp ranks a node against 32 others at a time; beyond that the work of
+// all pairs is the longer way (511 nodes: 30.9 us) and the cut is searched by its bits, one count of the whole tree per bit.
+constexpr int kRankNodes = 192;
 __global__ void __launch_bounds__(kTreeThreads) final_prune_kernel(TreeState t) {
   extern __shared__ unsigned long long s_score[];              // [cap], behind it [cap] parents, [cap] new ids
   __shared__ int s_count[kTreeWarps];
+  __shared__ unsigned long long s_and, s_or;
   int *s_parent = reinterpret_cast<int *>(s_score + t.cap), *s_remap = s_parent + t.cap;
   chain_enter();
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -96,7 +99,54 @@ __global__ void __launch_bounds__(kTreeThreads) final_prune_kernel(TreeState t) 
   n = n > t.cap ? t.cap : n;
   __syncthreads();
   const bool all = (t.N <= 0 || n <= t.N);
-  if (!all) {
+  if (!all && n > kRankNodes) {
+    // the (N-1)-th largest score by its bits, from the highest in which the scores differ down, until a count fits exactly
+    // (equal scores at the cut: the lower ids)
+    const int quota = t.N - 1;
+    if (tid == 0) { s_and = ~0ull; s_or = 0ull; }
+    __syncthreads();
+    unsigned long long al = ~0ull, ol = 0ull;
+    for (int i = 1 + tid; i < n; i += kTreeThreads) { al &= s_score[i]; ol |= s_score[i]; }
+    atomicAnd(&s_and, al);
+    atomicOr(&s_or, ol);
+    __syncthreads();
+    const unsigned long long common = s_and, differ = common ^ s_or;
+    int bit = differ ? 63 - __clzll((long long)differ) : -1;
+    unsigned long long cutoff = bit >= 63 ? 0ull : common & ~((1ull << (bit + 1)) - 1ull);
+    if (bit < 0) cutoff = common;
+    bool exact = false;
+    for (; bit >= 0 && !exact; --bit) {
+      const unsigned long long trial = cutoff | (1ull << bit);
+      int reach = 0;
+      for (int base = 0; base < n; base += kTreeThreads) {
+        const int i = base + tid;
+        reach += __syncthreads_count(i > 0 && i < n && s_score[i] >= trial);
+      }
+      if (reach >= quota) cutoff = trial;
+      exact = reach == quota;
+    }
+    int ties = n;                                              // nodes with the cutoff's score that may stay
+    if (!exact) {
+      ties = quota;
+      for (int base = 0; base < n; base += kTreeThreads) {
+        const int i = base + tid;
+        ties -= __syncthreads_count(i > 0 && i < n && s_score[i] > cutoff);
+      }
+    }
+    int seen = 0;
+    for (int base = 0; base < n; base += kTreeThreads) {
+      const int i = base + tid;
+      const bool tie = i > 0 && i < n && s_score[i] == cutoff;
+      const unsigned mask = __ballot_sync(kFull, tie);
+      if (lane == 0) s_count[warp] = __popc(mask);
+      __syncthreads();
+      const int c = lane < kTreeWarps ? s_count[lane] : 0;
+      const int before = seen + __reduce_add_sync(kFull, lane < warp ? c : 0) + __popc(mask & ((1u << lane) - 1u));
+      if (i < n) s_remap[i] = i == 0 || s_score[i] > cutoff || (tie && before < ties);
+      seen += __reduce_add_sync(kFull, c);
+      __syncthreads();
+    }
+  } else if (!all) {
     for (int i = warp; i < n; i += kTreeWarps) {               // 1: kept (for now)
       const unsigned long long mine = s_score[i];
       int before = 0;
@@ -208,54 +258,20 @@ __global__ void __launch_bounds__(kTreeThreads) build_verify_kernel(TreeState t,
 
 // ---------------------------------------------------------------- accept ----
 
-// best key of active row `a` of the last arg-max pass (0: none)
-__device__ __forceinline__ unsigned long long row_best_key(const TreeState &t, const PassInfo &info, int seq, int a) {
-  const long long first_vec = (long long)a * info.vec_per_row;
-  const int c_first = (int)(first_vec / info.span);
-  const int c_last = (int)((first_vec + info.vec_per_row - 1) / info.span);
-  int n_splits = c_last - c_first + 1;
-  if (n_splits > t.max_splits_tgt) {
-    n_splits = t.max_splits_tgt;
-    atomicOr(&t.status[seq], C2T_ST_INTERNAL);
-  }
-  unsigned long long best = 0ull;
-  for (int s = 0; s < n_splits; ++s) {
-    unsigned long long k = t.part_best[(size_t)a * t.max_splits_tgt + s];
-    best = k > best ? k : best;
-  }
+// takes a key of the last arg-max pass (0: none) and leaves the zero that the next pass starts from
+__device__ __forceinline__ unsigned long long take_best(const TreeState &t, size_t slot) {
+  const unsigned long long best = t.best[slot];
+  if (best) t.best[slot] = 0ull;
   return best;
-}
-
-// rows of earlier sequences in the arg-max pass over the final trees (all threads of the CTA call this)
-__device__ int target_row_offset(const TreeState &t, int b, int *s_scan, int *s_total) {
-  int part = 0;
-  for (int i = threadIdx.x; i < b; i += kTreeThreads) {
-    int c = t.final_n[i];
-    part += c < 0 ? 0 : (c > t.Nw ? t.Nw : c);
-  }
-  int total;
-  block_exclusive_scan<kTreeThreads>(part, s_scan, &total);
-  if (threadIdx.x == 0) *s_total = total;
-  __syncthreads();
-  return *s_total;
 }
 
 // The best key of every final node's row over one token range, token ids made global, for c2t_argmax_shard.
 __global__ void __launch_bounds__(kTreeThreads) export_best_kernel(TreeState t, int tok_base, unsigned long long *out) {
-  __shared__ int s_scan[kTreeWarps + 1];
-  __shared__ int s_total;
   chain_enter();
-  const int b = blockIdx.x, n = t.final_n[b], Nw = t.Nw;
-  const PassInfo info = *t.info_target;
-  const int row_off = target_row_offset(t, b, s_scan, &s_total);
-  for (int i = threadIdx.x; i < Nw; i += kTreeThreads) {
-    unsigned long long key = 0ull;
-    if (i < n) {
-      const unsigned long long best = row_best_key(t, info, b, row_off + i);
-      if (best) key = (best & 0xFFFFFFFF00000000ull) | (0xFFFFFFFFu - (uint32_t)(key_token(best) + tok_base));
-    }
-    out[(size_t)b * Nw + i] = key;
-  }
+  const size_t i = (size_t)blockIdx.x * kTreeThreads + threadIdx.x;
+  if (i >= (size_t)t.B * t.Nw) return;
+  const unsigned long long best = take_best(t, i);             // (nodes that do not exist have none)
+  out[i] = best ? (best & 0xFFFFFFFF00000000ull) | (0xFFFFFFFFu - (uint32_t)(key_token(best) + tok_base)) : 0ull;
 }
 
 // gathered == nullptr: the arg-max of this context's own pass; else the best of n_shards gathered keys per node.
@@ -264,33 +280,25 @@ __global__ void __launch_bounds__(kTreeThreads) export_best_kernel(TreeState t, 
 __global__ void __launch_bounds__(kTreeThreads) accept_walk_kernel(TreeState t, c2t_accept_out out,
                                                                    const unsigned long long *gathered, int n_shards) {
   extern __shared__ int s_walk[];                              // [Nw] arg-maxes, [Nw] the child to go to
-  __shared__ int s_scan[kTreeWarps + 1];
-  __shared__ int s_total;
   chain_enter();
-  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = blockIdx.x, tid = threadIdx.x;
   const int n = t.final_n[b], Nw = t.Nw, width = t.D + 1;
   const size_t fb = (size_t)b * Nw;
-  const PassInfo info = *t.info_target;
   int *want = s_walk, *next = s_walk + Nw;
   if (out.path)
     for (int k = tid; k < width; k += kTreeThreads) out.path[(size_t)b * width + k] = k == 0 ? 0 : -1;
-  const int row_off = gathered ? 0 : target_row_offset(t, b, s_scan, &s_total);     // rows of earlier sequences in the arg-max pass
-  // target argmax per node: best key over the row's partials
   for (int i = tid; i < Nw; i += kTreeThreads) {
-    int tok = -1;
-    if (i < n) {
-      unsigned long long best = 0ull;
-      if (gathered) {                               // equal logits in two shards: the larger key is the lower token id
+    unsigned long long best = 0ull;
+    if (gathered) {                                 // equal logits in two shards: the larger key is the lower token id
 #pragma unroll 4
-        for (int s = 0; s < n_shards; ++s) {
-          const unsigned long long k = gathered[((size_t)s * t.B + b) * Nw + i];
-          best = k > best ? k : best;
-        }
-      } else {
-        best = row_best_key(t, info, b, row_off + i);
+      for (int s = 0; s < n_shards; ++s) {
+        const unsigned long long k = gathered[((size_t)s * t.B + b) * Nw + i];
+        best = k > best ? k : best;
       }
-      tok = best ? key_token(best) : -1;
+    } else {
+      best = take_best(t, fb + i);
     }
+    const int tok = best && i < n ? key_token(best) : -1;
     want[i] = tok;
     next[i] = 0x7FFFFFFF;
     t.node_argmax[fb + i] = tok;
@@ -301,7 +309,7 @@ __global__ void __launch_bounds__(kTreeThreads) accept_walk_kernel(TreeState t, 
     if (par >= 0 && t.final_token[fb + c] == want[par]) atomicMin(&next[par], c);
   }
   __syncthreads();
-  if (warp != 0 || lane != 0) return;
+  if (tid != 0) return;
   int cur = 0, len = 0;
   while (n > 0 && len + 1 < width) {
     const int found = next[cur];
@@ -316,197 +324,123 @@ __global__ void __launch_bounds__(kTreeThreads) accept_walk_kernel(TreeState t, 
 
 // ---------------------------------------------------------------- dense mask -
 
-// Eight rows of a sequence's final tree per CTA, a warp per row: the row's ancestor-or-self set as bits in shared memory (a
-// walk up the parent pointers, at most D+1 steps), then the row of kv_len additive mask values, 0 or -inf (Sec. 2.2).  Bound
-// by the stores, so they are 16 bytes wide; the walk runs on a copy of the parents in shared memory, because one that
-// loads every parent from global memory costs several microseconds before the first store.  64 x 60 rows of 4160
-// bf16 values: 26.6 -> 11.1 us per call (32 MB, 2.9 TB/s).
-constexpr int kMaskRows = 8;
+// Four rows of a sequence's final tree per CTA, two warps per row.  Most of a row does not depend on the tree (its
+// prefix, and what lies behind the tree), and is stored first, 16 bytes at a time; then the row's ancestor-or-self set (Sec. 2.2)
+// is found by a walk up the parent pointers in shared memory (at most D+1 steps; through global memory it costs
+// microseconds), and the few vectors that hold tree nodes follow.  Bound by the stores: 64 x 60 rows of 4160 bf16
+// values 26.6 -> 9.8 us per call (32 MB).
+constexpr int kMaskRows = 4, kMaskThreads = kMaskRows * 64;
 template <typename T>
-__global__ void __launch_bounds__(kMaskRows * 32) dense_mask_kernel(TreeState t, T *out, long long kv_len, T ninf) {
+__global__ void __launch_bounds__(kMaskThreads) dense_mask_kernel(TreeState t, T *out, long long kv_len, T ninf) {
   extern __shared__ int s_parent[];                  // [Nw], behind it the rows' bits
   constexpr int E = 16 / sizeof(T);
-  const int b = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = (int)blockIdx.x * kMaskRows + warp;
+  const int b = blockIdx.y, tid = threadIdx.x, r = tid >> 6, k0 = tid & 63, i = (int)blockIdx.x * kMaskRows + r;
   const int Nw = t.Nw, words = (Nw + 31) / 32;
-  unsigned *bits = reinterpret_cast<unsigned *>(s_parent + Nw) + warp * words;
+  unsigned *bits = reinterpret_cast<unsigned *>(s_parent + Nw) + r * words;
   chain_enter();
-  const int n = t.final_n[b];
   const long long prefix = t.prefix_len[b];
-  for (int j = threadIdx.x; j < Nw; j += kMaskRows * 32) s_parent[j] = t.final_parent[(size_t)b * Nw + j];
-  for (int w = lane; w < words; w += 32) bits[w] = 0u;
-  __syncthreads();
-  if (i >= Nw) return;
-  if (lane == 0 && i < n)
-    for (int j = i, guard = 0; j >= 0 && j < Nw && guard <= Nw; j = s_parent[j], ++guard) bits[j >> 5] |= 1u << (j & 31);
-  __syncwarp();
-  auto value = [&](long long c) -> T {
-    const long long j = c - prefix;
-    return c < prefix || (j < Nw && ((bits[j >> 5] >> (j & 31)) & 1u)) ? (T)0 : ninf;
-  };
+  const int n = t.final_n[b];
+  for (int j = tid; j < Nw; j += kMaskThreads) s_parent[j] = t.final_parent[(size_t)b * Nw + j];
+  for (int w = k0; w < words; w += 64) bits[w] = 0u;
   T *row = out + ((size_t)b * Nw + i) * kv_len;
   long long head = (long long)((16 - (reinterpret_cast<uintptr_t>(row) & 15)) & 15) / (int)sizeof(T);     // up to the first 16-byte boundary
   head = head < kv_len ? head : kv_len;
   const long long body = (kv_len - head) / E;
-  if (lane < head) row[lane] = value(lane);
-  union { uint4 v; T e[E]; } zeros, ninfs, mixed;
-#pragma unroll
-  for (int k = 0; k < E; ++k) { zeros.e[k] = (T)0; ninfs.e[k] = ninf; }
   uint4 *dst = reinterpret_cast<uint4 *>(row + head);
+  // vectors [0, k1) lie in the prefix, [k2, body) behind the tree
+  long long k1 = prefix > head ? (prefix - head) / E : 0, k2 = prefix + Nw > head ? (prefix + Nw - head + E - 1) / E : 0;
+  k1 = k1 < body ? k1 : body;
+  k2 = k2 < body ? k2 : body;
+  union { uint4 v; T e[E]; } fill, mixed;
+  if (i < Nw) {
 #pragma unroll 4
-  for (long long k = lane; k < body; k += 32) {
-    const long long c = head + k * E;
-    if (c + E <= prefix) {
-      dst[k] = zeros.v;
-    } else if (c >= prefix + Nw) {
-      dst[k] = ninfs.v;
-    } else {
+    for (long long k = k0; k < k1; k += 64) dst[k] = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-      for (int q = 0; q < E; ++q) mixed.e[q] = value(c + q);
-      dst[k] = mixed.v;
-    }
+    for (int q = 0; q < E; ++q) fill.e[q] = ninf;
+#pragma unroll 4
+    for (long long k = k2 + k0; k < body; k += 64) dst[k] = fill.v;
   }
+  __syncthreads();
+  if (k0 == 0 && i < n)
+    for (int j = i, guard = 0; j >= 0 && j < Nw && guard <= Nw; j = s_parent[j], ++guard) bits[j >> 5] |= 1u << (j & 31);
+  __syncthreads();
+  if (i >= Nw) return;
+  auto value = [&](long long c) -> T {
+    const long long j = c - prefix;
+    return c < prefix || (j < Nw && ((bits[j >> 5] >> (j & 31)) & 1u)) ? (T)0 : ninf;
+  };
+  for (long long k = k1 + k0; k < k2; k += 64) {
+#pragma unroll
+    for (int q = 0; q < E; ++q) mixed.e[q] = value(head + k * E + q);
+    dst[k] = mixed.v;
+  }
+  if (k0 < head) row[k0] = value(k0);
   const long long done = head + body * E;
-  if (lane < kv_len - done) row[done + lane] = value(done + lane);
+  if (k0 < kv_len - done) row[done + k0] = value(done + k0);
 }
 
 // ---------------------------------------------------------------- lazy walk --
 
-// One round of the acceptance walk that reads only the rows it visits (Sec. 5 Metrics).
-// Round 0 puts every sequence with a tree on its root.  Round r > 0 follows the arg-max pass
-// over the current nodes' rows (one row per walking sequence, in sequence order): the
-// sequence moves to the child that carries the arg-max token, or stops.  A single CTA serves
-// all sequences, 1024 at a time; the scan numbers the walking sequences the way the pass did.
-constexpr int kWalkThreads = 1024;
-
-// gathered == nullptr: the arg-max of this context's own pass over whole rows; else the best of n_shards gathered keys
-// per sequence ([n_shards, B], one key for the sequence's current node, 0 for a sequence that has stopped).
+// One round of the acceptance walk over target rows sharded over the vocabulary, reading only the rows it visits (Sec. 5
+// Metrics).  Round 0 puts every sequence with a tree on its root.  Round r > 0 takes the best of the n_shards gathered keys
+// per sequence ([n_shards, B], one key for the sequence's current node, 0 for a sequence that has stopped): the
+// sequence moves to the child that carries that token, or stops.  A thread per sequence.
+constexpr int kWalkThreads = 128;
 __global__ void __launch_bounds__(kWalkThreads) lazy_walk_round_kernel(TreeState t, int round, c2t_accept_out out,
                                                                        const unsigned long long *gathered, int n_shards) {
-  __shared__ int s_warp[kWalkThreads / 32 + 1];
   chain_enter();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = blockIdx.x * kWalkThreads + threadIdx.x;
   const int Nw = t.Nw, width = t.D + 1;
-  const PassInfo info = *t.info_target;
-  int rows_before = 0;                               // walking sequences in earlier chunks
-  for (int base = 0; base < t.B; base += kWalkThreads) {
-    const int b = base + tid;
-    const bool in = b < t.B;
-    const size_t fb = (size_t)b * Nw;
-    if (round == 0) {
-      if (in) {
-        const int n = t.final_n[b];
-        for (int i = 0; i < Nw; ++i) t.node_argmax[fb + i] = -1;
-        if (out.path)
-          for (int w = 0; w < width; ++w) out.path[(size_t)b * width + w] = w == 0 ? 0 : -1;
-        t.walk_cur[b] = 0;
-        t.walk_len[b] = 0;
-        t.walk_active[b] = n > 0;
-        if (n <= 0) {
-          if (out.accept_len) out.accept_len[b] = 0;
-          if (out.next_token) out.next_token[b] = -1;
-        }
-      }
-      continue;
+  if (b >= t.B) return;
+  const size_t fb = (size_t)b * Nw;
+  const int n = t.final_n[b];
+  if (round == 0) {
+    for (int i = 0; i < Nw; ++i) t.node_argmax[fb + i] = -1;
+    if (out.path)
+      for (int w = 0; w < width; ++w) out.path[(size_t)b * width + w] = w == 0 ? 0 : -1;
+    t.walk_cur[b] = 0;
+    t.walk_len[b] = 0;
+    t.walk_active[b] = n > 0;
+    if (n <= 0) {
+      if (out.accept_len) out.accept_len[b] = 0;
+      if (out.next_token) out.next_token[b] = -1;
     }
-    const int was = in ? t.walk_active[b] : 0;
-    // the row number of this sequence in the pass: walking sequences before it
-    int inc = was;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(kFull, inc, o);
-      if (lane >= o) inc += v;
-    }
-    __syncthreads();
-    if (lane == 31) s_warp[warp] = inc;
-    __syncthreads();
-    if (tid == 0) {
-      int run = 0;
-      for (int w = 0; w < kWalkThreads / 32; ++w) { const int v = s_warp[w]; s_warp[w] = run; run += v; }
-      s_warp[kWalkThreads / 32] = run;
-    }
-    __syncthreads();
-    const int a = rows_before + s_warp[warp] + inc - was;
-    rows_before += s_warp[kWalkThreads / 32];
-    if (!was) continue;
-
-    unsigned long long best = 0ull;
-    if (gathered) {                                    // equal logits in two shards: the larger key is the lower token id
-      for (int sh = 0; sh < n_shards; ++sh) {
-        const unsigned long long k = gathered[(size_t)sh * t.B + b];
-        best = k > best ? k : best;
-      }
-    } else {
-      const long long first_vec = (long long)a * info.vec_per_row;
-      const int c_first = (int)(first_vec / info.span);
-      const int c_last = (int)((first_vec + info.vec_per_row - 1) / info.span);
-      int n_splits = c_last - c_first + 1;
-      if (n_splits > t.max_splits_tgt) {
-        n_splits = t.max_splits_tgt;
-        atomicOr(&t.status[b], C2T_ST_INTERNAL);
-      }
-      for (int sp = 0; sp < n_splits; ++sp) {
-        const unsigned long long k = t.part_best[(size_t)a * t.max_splits_tgt + sp];
-        best = k > best ? k : best;
-      }
-    }
-    const int want = best ? key_token(best) : -1;
-    const int n = t.final_n[b];
-    int cur = t.walk_cur[b], len = t.walk_len[b];
-    t.node_argmax[fb + cur] = want;
-    int found = -1;
-    if (len + 1 < width)
-      for (int c = cur + 1; c < n; ++c)
-        if (t.final_parent[fb + c] == cur && t.final_token[fb + c] == want) { found = c; break; }
-    if (found >= 0) {
-      ++len;
-      t.walk_cur[b] = found;
-      t.walk_len[b] = len;
-      if (out.path) out.path[(size_t)b * width + len] = found;
-    } else {
-      t.walk_active[b] = 0;
-      if (out.accept_len) out.accept_len[b] = len;
-      if (out.next_token) out.next_token[b] = want;
-    }
+    return;
+  }
+  if (!t.walk_active[b]) return;
+  unsigned long long best = 0ull;                      // equal logits in two shards: the larger key is the lower token id
+#pragma unroll 4
+  for (int sh = 0; sh < n_shards; ++sh) {
+    const unsigned long long k = gathered[(size_t)sh * t.B + b];
+    best = k > best ? k : best;
+  }
+  const int want = best ? key_token(best) : -1;
+  int cur = t.walk_cur[b], len = t.walk_len[b];
+  t.node_argmax[fb + cur] = want;
+  int found = -1;
+  if (len + 1 < width)
+    for (int c = cur + 1; c < n; ++c)
+      if (t.final_parent[fb + c] == cur && t.final_token[fb + c] == want) { found = c; break; }
+  if (found >= 0) {
+    ++len;
+    t.walk_cur[b] = found;
+    t.walk_len[b] = len;
+    if (out.path) out.path[(size_t)b * width + len] = found;
+  } else {
+    t.walk_active[b] = 0;
+    if (out.accept_len) out.accept_len[b] = len;
+    if (out.next_token) out.next_token[b] = want;
   }
 }
 
 // After an arg-max pass over one token range of the walking sequences' current rows: per sequence the best key of
-// that range with the token id made global (0 for a sequence that has stopped), for c2t_lazy_argmax_shard.  The
-// pass numbered the walking sequences in sequence order; the scan here does the same.
+// that range with the token id made global (0 for a sequence that has stopped), for c2t_lazy_argmax_shard.
 __global__ void __launch_bounds__(kWalkThreads) export_lazy_best_kernel(TreeState t, int tok_base, unsigned long long *out) {
-  __shared__ int s_warp[kWalkThreads / 32 + 1];
   chain_enter();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const PassInfo info = *t.info_target;
-  int rows_before = 0;
-  for (int base = 0; base < t.B; base += kWalkThreads) {
-    const int b = base + tid;
-    const int was = b < t.B ? t.walk_active[b] : 0;
-    int inc = was;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(kFull, inc, o);
-      if (lane >= o) inc += v;
-    }
-    __syncthreads();
-    if (lane == 31) s_warp[warp] = inc;
-    __syncthreads();
-    if (tid == 0) {
-      int run = 0;
-      for (int w = 0; w < kWalkThreads / 32; ++w) { const int v = s_warp[w]; s_warp[w] = run; run += v; }
-      s_warp[kWalkThreads / 32] = run;
-    }
-    __syncthreads();
-    const int a = rows_before + s_warp[warp] + inc - was;
-    rows_before += s_warp[kWalkThreads / 32];
-    if (b >= t.B) continue;
-    unsigned long long key = 0ull;
-    if (was) {
-      const unsigned long long best = row_best_key(t, info, b, a);
-      if (best) key = (best & 0xFFFFFFFF00000000ull) | (0xFFFFFFFFu - (uint32_t)(key_token(best) + tok_base));
-    }
-    out[b] = key;
-  }
+  const int b = blockIdx.x * kWalkThreads + threadIdx.x;
+  if (b >= t.B) return;
+  const unsigned long long best = take_best(t, b);
+  out[b] = best ? (best & 0xFFFFFFFF00000000ull) | (0xFFFFFFFFu - (uint32_t)(key_token(best) + tok_base)) : 0ull;
 }
 
 }  // namespace
@@ -515,9 +449,9 @@ cudaError_t launch_dense_mask(const TreeState &t, void *out, int out_dtype, int6
   const dim3 grid((t.Nw + kMaskRows - 1) / kMaskRows, t.B);
   const size_t smem = (size_t)t.Nw * sizeof(int) + (size_t)kMaskRows * ((t.Nw + 31) / 32) * sizeof(unsigned);    // (at most 40 KB)
   if (out_dtype == C2T_F32)                          // the values as raw words: +0 and -inf
-    return launch_chained(dense_mask_kernel<unsigned>, grid, dim3(kMaskRows * 32), smem, s, t, reinterpret_cast<unsigned *>(out),
+    return launch_chained(dense_mask_kernel<unsigned>, grid, dim3(kMaskThreads), smem, s, t, reinterpret_cast<unsigned *>(out),
                           (long long)kv_len, 0xFF800000u);
-  return launch_chained(dense_mask_kernel<unsigned short>, grid, dim3(kMaskRows * 32), smem, s, t, reinterpret_cast<unsigned short *>(out),
+  return launch_chained(dense_mask_kernel<unsigned short>, grid, dim3(kMaskThreads), smem, s, t, reinterpret_cast<unsigned short *>(out),
                         (long long)kv_len, (unsigned short)0xFF80);
 }
 
@@ -526,11 +460,11 @@ cudaError_t launch_lazy_walk_round(const TreeState &t, int round, const c2t_acce
   c2t_accept_out o;
   memset(&o, 0, sizeof o);
   if (out) o = *out;
-  return launch_chained(lazy_walk_round_kernel, dim3(1), dim3(kWalkThreads), 0, s, t, round, o, gathered, n_shards);
+  return launch_chained(lazy_walk_round_kernel, dim3((t.B + kWalkThreads - 1) / kWalkThreads), dim3(kWalkThreads), 0, s, t, round, o, gathered, n_shards);
 }
 
 cudaError_t launch_export_lazy_best(const TreeState &t, int vocab_begin, unsigned long long *out, cudaStream_t s) {
-  return launch_chained(export_lazy_best_kernel, dim3(1), dim3(kWalkThreads), 0, s, t, vocab_begin, out);
+  return launch_chained(export_lazy_best_kernel, dim3((t.B + kWalkThreads - 1) / kWalkThreads), dim3(kWalkThreads), 0, s, t, vocab_begin, out);
 }
 
 cudaError_t launch_begin_step(const TreeState &t, const int32_t *root_tok, const int32_t *prefix_len,
@@ -575,7 +509,7 @@ cudaError_t launch_build_verify(const TreeState &t, const c2t_verify *out, cudaS
 }
 
 cudaError_t launch_export_best(const TreeState &t, int vocab_begin, unsigned long long *out, cudaStream_t s) {
-  return launch_chained(export_best_kernel, dim3(t.B), dim3(kTreeThreads), 0, s, t, vocab_begin, out);
+  return launch_chained(export_best_kernel, dim3((unsigned)(((size_t)t.B * t.Nw + kTreeThreads - 1) / kTreeThreads)), dim3(kTreeThreads), 0, s, t, vocab_begin, out);
 }
 
 cudaError_t launch_accept_walk(const TreeState &t, const c2t_accept_out *out, const unsigned long long *gathered,

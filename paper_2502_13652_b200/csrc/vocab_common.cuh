@@ -148,30 +148,5 @@ __device__ __forceinline__ int find_sequence(const int *s_off, int B, int a) {
   return lo;
 }
 
-struct Partition {
-  int n_rows, vec_per_row, v_full;
-  long long span, start, end;
-};
-
-template <int VEC>
-__device__ __forceinline__ Partition make_partition(const PassParams &p, int n_rows) {
-  Partition pt;
-  pt.n_rows = n_rows;
-  pt.vec_per_row = (p.V + VEC - 1) / VEC;
-  pt.v_full = p.V / VEC;
-  long long W = (long long)n_rows * pt.vec_per_row;
-  long long span = (W + gridDim.x - 1) / gridDim.x;
-  pt.span = span < kMinSpanVectors ? kMinSpanVectors : span;
-  pt.start = (long long)blockIdx.x * pt.span;
-  pt.end = pt.start + pt.span < W ? pt.start + pt.span : W;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    p.info->n_rows = n_rows;
-    p.info->vec_per_row = pt.vec_per_row;
-    p.info->span = pt.span;
-  }
-  return pt;
-}
-
-
 }  // namespace
 }  // namespace c2t
