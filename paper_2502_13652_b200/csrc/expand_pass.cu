@@ -567,16 +567,20 @@ __device__ __forceinline__ void complete_keys(const PassParams &p, PairShared *w
       }
       mask |= (unsigned long long)m << (32 * h);
     }
-    for (;;) {
-      const unsigned bal = __ballot_sync(kFull, mask != 0ull);
-      if (!bal || n_list > kListCap) break;
-      const int pos = n_list + __popc(bal & ((1u << lane) - 1u));
-      if (mask) {
-        const int bit = __ffsll((long long)mask) - 1, chunk = 2 * (c0 + ((bit & 32) >> 1) + (bit & 15)) + ((bit >> 4) & 1);
-        if (pos < kListCap) ws->list[pos] = chunk < rs.nc ? chunk * 32 + lane : -1;
-      }
+    const int mine = __popcll(mask);
+    int upto = mine;                                // places in lane order
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(kFull, upto, o);
+      if (lane >= o) upto += v;
+    }
+    int pos = n_list + upto - mine;
+    n_list += __shfl_sync(kFull, upto, 31);
+    while (mask) {
+      const int bit = __ffsll((long long)mask) - 1, chunk = 2 * (c0 + ((bit & 32) >> 1) + (bit & 15)) + ((bit >> 4) & 1);
+      if (pos < kListCap) ws->list[pos] = chunk < rs.nc ? chunk * 32 + lane : -1;
+      ++pos;
       mask &= mask - 1ull;
-      n_list += __popc(bal);
     }
   }
   __syncwarp();
@@ -957,12 +961,14 @@ __global__ void __launch_bounds__(kExpandThreads, 1) expand_prune_kernel(const _
   if (threadIdx.x >= kStreamWarps * 32) stage_classifier(t, s_w, threadIdx.x - kStreamWarps * 32, kExpandThreads - kStreamWarps * 32);   // (written at init)
   chain_enter();
   expand_pass_body<BF16, false>(p, s_dyn);
-  __threadfence();                                   // this CTA's row results, before its ticket
   __syncthreads();
-  if (threadIdx.x == 0) s_ticket = atomicAdd(t.ticket, 1u);
+  if (threadIdx.x == 0) {
+    __threadfence();                                 // this CTA's row results (seen at the barrier), before its ticket
+    s_ticket = atomicAdd(t.ticket, 1u);
+    __threadfence();                                 // the other CTAs' results, after their tickets
+  }
   __syncthreads();
   if (s_ticket != gridDim.x - 1) return;
-  __threadfence();                                   // the other CTAs' results, after their tickets
   if (threadIdx.x == 0) *t.ticket = 0u;              // for the next launch
   // the pass's shared memory is free now
   PruneShared &sh = *reinterpret_cast<PruneShared *>(s_dyn);

@@ -162,7 +162,7 @@ struct PruneShared {
   int rowfault[C2T_MAX_FRONTIER];
   unsigned long long ckey[kMaxCand];           // confidence of every candidate as an orderable integer, 0 for a dropped one
   int count[32];                               // candidates added and selected, per 32
-  unsigned char sel[kMaxCand];
+  short before[kMaxCand];                      // survivors that come before a candidate
 };
 // ... and with gathered records, behind it:
 struct GatherShared {
@@ -295,26 +295,26 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
   }
 
   // ---- second pruning: the F survivors that come first under (C desc, index asc); a warp counts what comes before a
-  // candidate, every lane with four of the keys in registers
+  // candidate, four of the keys in every lane's registers (up to 128 candidates at a time)
   if (n_keep > F) {
-    for (int c0 = warp; c0 < nc; c0 += kNW) {
-      const unsigned long long kc = sh.ckey[c0];
-      int before = 0;
-      for (int o0 = 0; o0 < nc; o0 += 128) {
+    for (int o0 = 0; o0 < nc; o0 += 128) {
+      unsigned long long ko[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int o = o0 + q * 32 + lane;
-          const unsigned long long ko = o < nc ? sh.ckey[o] : 0ull;
-          before += ko > kc || (ko == kc && o < c0);
-        }
+      for (int q = 0; q < 4; ++q) ko[q] = o0 + q * 32 + lane < nc ? sh.ckey[o0 + q * 32 + lane] : 0ull;
+#pragma unroll 4
+      for (int c0 = warp; c0 < nc; c0 += kNW) {
+        const unsigned long long kc = sh.ckey[c0];
+        int before = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) before += ko[q] >= kc + (o0 + q * 32 + lane < c0 ? 0 : 1);   // (a key is never all ones)
+        before = __reduce_add_sync(kFullMask, before);
+        if (lane == 0) sh.before[c0] = (short)(o0 == 0 ? before : sh.before[c0] + before);
       }
-      before = __reduce_add_sync(kFullMask, before);
-      if (lane == 0) sh.sel[c0] = kc != 0ull && before < F;
     }
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < kRounds; ++r)
-      if (tid + r * NT < nc) sel[r] = sh.sel[tid + r * NT];
+      if (tid + r * NT < nc) sel[r] = keep[r] && sh.before[tid + r * NT] < F;
   }
 
   // ---- stable compaction in candidate order; append to the tree, emit the frontier
