@@ -983,12 +983,16 @@ size_t topm_pool_vectors(size_t batch, size_t rows_per_seq, int vocab, int elem_
   return n < 0x7FFFFFFFu ? n : 0x7FFFFFFFu;          // records hold 32-bit positions
 }
 
+// A row's floor is the highest of its segments' (up to some forty), and a low place among 32 lane maxima scatters widely: with
+// M = 500 of 128256 the place for 3 M elements is the 11th and most rows were read again (1320 us per eight levels of 40 rows
+// of fp32; at the 24th or beyond 369).
+constexpr int kTopmLeastPlace = 24;
 int topm_floor_place(int vocab, int elem_bytes, int M) {
   const int vec = 16 / elem_bytes;
   const int vec_per_row = (vocab + vec - 1) / vec, head = vec_per_row < 256 ? vec_per_row : 256;
   const double per_lane = (double)head * vec / 32.0, share = 3.0 * M / vocab;
   const int place = share >= 1.0 ? 31 : (int)ceil(32.0 * (1.0 - pow(1.0 - share, per_lane)));
-  return place < 1 ? 1 : (place > 31 ? 31 : place);
+  return place < kTopmLeastPlace ? kTopmLeastPlace : (place > 31 ? 31 : place);
 }
 
 int row_chunks(int vocab, int elem_bytes) {
