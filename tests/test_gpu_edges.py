@@ -1,0 +1,153 @@
+"""GPU parity at the edges of the kernels' tiles and dispatch rules: chunks of the expand pass, the K for which it takes its
+bound from half columns, its selection in order, the sizes of the lazy walk's clusters, the rerank of large trees, the short
+and long rows of the arg-max pass, the mask's 16-byte vectors, the host step's two ways to its target rows."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2502_13652_b200 as c2t
+from parity_util import gen_inputs, make_configs, run_and_compare
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2502_13652_b200 import build
+    build.build()
+    oracle.build()
+
+
+def step(B, V, D, K, F, N, beta, dtype, draft=None, **kw):
+    ocfg, gcfg = make_configs(B, V, D, K, F, N, beta, dtype, **kw)
+    dr, target, root, prefix = gen_inputs(B, V, D, F, c2t.c2t_final_width(gcfg), dtype)
+    pad = -(-V // 8) * 8
+
+    def rows(t):                                       # rows on 16-byte boundaries
+        buf = torch.zeros(t.shape[0], t.shape[1], pad, dtype=dtype, device="cuda")
+        buf[:, :, :V] = t.cuda()
+        return buf[:, :, :V]
+
+    dr = draft if draft is not None else dr
+    rep = run_and_compare(ocfg, gcfg, dr, target, root, prefix, draft_dev=[rows(t) for t in dr], target_dev=rows(target))
+    assert rep.status_bits == 0
+
+
+# a chunk is 256 vectors: 2048 bf16 or 1024 fp32 tokens; two chunks share a word of cells; 12 warps stream
+@pytest.mark.parametrize("dtype,chunk", [(torch.bfloat16, 2048), (torch.float32, 1024)])
+@pytest.mark.parametrize("V", ["7", "1-1", "1", "1+1", "2+5", "3", "12+1", "64", "65-3"])
+def test_vocabulary_around_chunk_edges(dtype, chunk, V):
+    n, plus = (V + "+0").split("+")[:2] if "+" in V else ((V.split("-")[0], "-" + V.split("-")[1]) if "-" in V else (V, "0"))
+    v = 7 if V == "7" else int(n) * chunk + int(plus)
+    step(3, v, 3, 4, 5, 14, 0.0, dtype, classifier="identity")
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("K", [16, 17, 32])
+def test_widths_of_the_selection(dtype, K):
+    step(2, 9000, 2, K, 3, 20, 0.0, dtype, classifier="identity")
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_rows_with_more_candidates_than_the_pool(dtype):
+    """Well over a hundred equal largest values in scattered cells: more than the pool of a row holds, so the row is taken in
+    token order.  Such a row's candidates have the probability 1 / count, and with equal counts in two rows children of
+    different rows would tie to 1e-6, where either order is right; the counts here differ by 4 % or more from row to row."""
+    B, V, F, D = 2, 24000, 4, 2
+    g = torch.Generator().manual_seed(3)
+    draft = []
+    for _ in range(D):
+        x = torch.randn(B, F, V, generator=g)
+        for b in range(B):
+            for j in range(F):
+                x[b, j, ::80 + 9 * (F * b + j)] = 20.0
+        draft.append(x.to(dtype))
+    step(B, V, D, 6, F, 12, 0.0, dtype, draft=draft, classifier="identity")
+
+
+@pytest.mark.parametrize("dtype,V", [(torch.bfloat16, 8200), (torch.float32, 4100), (torch.bfloat16, 40003), (torch.float32, 16389)])
+@pytest.mark.parametrize("B", [1, 37, 75, 149])
+def test_lazy_walk_equals_the_walk_over_all_rows(B, V, dtype):
+    """Clusters of 8, 8 or 4, 2 and 1 CTAs per sequence on a chip of 148 SMs; short and long, whole and ragged rows."""
+    D, K, F, N = 3, 4, 3, 9
+    _, gcfg = make_configs(B, V, D, K, F, N, 0.0, dtype, classifier="identity")
+    ctx = c2t.Context(gcfg)
+    pad = -(-V // 8) * 8
+    g = torch.Generator(device="cuda").manual_seed(B)
+    draft = [torch.randn(B, F, pad, device="cuda", generator=g).to(dtype)[:, :, :V] for _ in range(D)]
+    target = torch.randn(B, ctx.Nw, pad, device="cuda", generator=g).to(dtype)[:, :, :V]
+    zeros = torch.zeros(B, dtype=torch.int32, device="cuda")
+    ctx.decode_step(draft, target, zeros, zeros)
+    ver = {k: v.cpu() for k, v in ctx.verify.items()}
+    for b in range(B):                                  # a path of every length, the last token near the row's end
+        row = [int(x) for x in ver["retrieve"][b, b % int(ver["n_leaves"][b])] if x >= 0][:1 + b % (D + 1)]
+        for here, nxt in zip(row, row[1:]):
+            target[b, here, int(ver["tokens"][b, nxt])] = 50.0
+        target[b, row[-1], V - 1] = 60.0
+    ctx.c2t_accept(target)
+    torch.cuda.synchronize()
+    want = {k: v.clone() for k, v in ctx.accepted.items()}
+    amax = ctx.c2t_get_view()["node_argmax"].clone()
+    assert torch.equal(amax.cpu(), target.float().cpu().max(dim=2).indices.to(torch.int32)[:, :ctx.Nw].where(
+        torch.arange(ctx.Nw)[None, :] < ver["n_nodes"][:, None], torch.tensor(-1, dtype=torch.int32)))
+    assert int(want["accept_len"].max()) >= min(B - 1, D - 1)
+    ctx.c2t_accept_lazy(target)
+    torch.cuda.synchronize()
+    for k, v in want.items():
+        assert torch.equal(ctx.accepted[k], v), k
+    on_path = torch.zeros_like(amax, dtype=torch.bool)
+    path = want["path"].long()
+    on_path.scatter_(1, path.clamp(min=0), True)
+    assert torch.equal(ctx.c2t_get_view()["node_argmax"], torch.where(on_path, amax, -1))
+    ctx.close()
+
+
+@pytest.mark.parametrize("N,wstd", [(20, 0.1), (400, 0.1), (20, 0.0), (1, 0.1)])
+def test_rerank_of_a_large_tree(N, wstd):
+    """511 nodes (more than a warp ranks one by one), with distinct confidences and with all of them equal."""
+    step(2, 3000, 6, 10, 10, N, 0.0, torch.float32, tree_add="all", wstd=wstd)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("kv", [1, 7, 40, 133, 256])
+def test_mask_vectors(dtype, kv):
+    """Rows that start on every alignment, end inside the prefix, inside the tree and behind it."""
+    B, V, D, K, F, N = 3, 2000, 4, 4, 4, 13
+    _, gcfg = make_configs(B, V, D, K, F, N, 0.0, torch.bfloat16, classifier="identity")
+    ctx = c2t.Context(gcfg)
+    draft = [torch.randn(B, F, V, device="cuda").to(torch.bfloat16) for _ in range(D)]
+    prefix = torch.tensor([0, 33, 128], dtype=torch.int32)
+    ctx.c2t_begin_step(torch.zeros(B, dtype=torch.int32, device="cuda"), prefix.cuda())
+    for l in range(D):
+        ctx.c2t_expand_level(l, draft[l]); ctx.c2t_prune(l)
+    ctx.c2t_prune(c2t.FINAL); ctx.c2t_build_verify()
+    out = torch.full((B, ctx.Nw, kv), 7.0, dtype=dtype, device="cuda")
+    ctx.c2t_dense_mask(out)
+    bits = ctx.verify["mask_bits"].cpu().numpy()
+    got = out.float().cpu().numpy()
+    for b in range(B):
+        for i in range(ctx.Nw):
+            on = [c < prefix[b] or (c - prefix[b] < 64 and int(bits[b, i, 0]) >> int(c - prefix[b]) & 1) for c in range(kv)]
+            assert np.array_equal(got[b, i], np.where(np.array(on, dtype=bool), 0.0, -np.inf)), (b, i)
+    ctx.close()
+
+
+@pytest.mark.parametrize("pinned", [True, False])
+@pytest.mark.parametrize("N", [16, 3])
+def test_host_step_ways(pinned, N):
+    """Target rows read from the pinned buffer by the walk, or copied; two staging buffers for the levels, or one (N < F)."""
+    B, V, D, K, F = 3, 4096, 4, 5, 4
+    _, gcfg = make_configs(B, V, D, K, F, N, 0.3, torch.bfloat16)
+    draft, target, root, prefix = gen_inputs(B, V, D, F, c2t.c2t_final_width(gcfg), torch.bfloat16)
+    ctx = c2t.Context(gcfg)
+    ctx.decode_step([t.cuda() for t in draft], target.cuda(), root.cuda(), prefix.cuda())
+    torch.cuda.synchronize()
+    want = {k: v.cpu().clone() for k, v in list(ctx.verify.items())[:2] + list(ctx.accepted.items())}
+    stage, results = ctx.host_step_buffers()
+    pin = (lambda t: t.pin_memory()) if pinned else (lambda t: t.contiguous())
+    for _ in range(2):
+        ctx.c2t_decode_step_host([pin(t) for t in draft], pin(target), root, prefix, results, stage)
+        for k, w in want.items():
+            assert torch.equal(results[k], w), k
+    ctx.close()
