@@ -316,9 +316,10 @@ int c2t_accept_gathered(c2t_ctx *ctx, const uint64_t *keys_dev, int32_t n_shards
  * sequence and depth, accept_len + 1 rows per sequence instead of all n_nodes.  Arguments,
  * layout, outputs and error codes are those of c2t_accept; accept_len, path and next_token are
  * identical to c2t_accept's.  The node_argmax view (c2t_get_view) is filled for the nodes on the
- * accepted path only, -1 elsewhere.  Issues 2*(D+1)+1 short launches whatever the accept
- * lengths turn out to be (the host never waits for the device); rounds in which no sequence is
- * still walking read nothing.  Must follow c2t_prune(C2T_FINAL).
+ * accepted path only, -1 elsewhere.  One launch: every sequence is walked by a cluster of thread
+ * blocks of its own, without waiting for the others or for the host.  target_logits_dev may also be
+ * pinned host memory as the device sees it: the few rows visited are read in place.
+ * Must follow c2t_prune(C2T_FINAL).
  */
 int c2t_accept_lazy(c2t_ctx *ctx, const void *target_logits_dev, int64_t seq_stride,
                     int64_t row_stride, const c2t_accept_out *out, void *stream);
@@ -365,17 +366,16 @@ int c2t_lazy_step_gathered(c2t_ctx *ctx, int round, const uint64_t *keys_dev, in
  *
  * Limits and rules:
  *   - rows <= C2T_STATIC_MAX_ROWS and vocab <= C2T_STATIC_MAX_VOCAB; larger sizes are refused
- *     with C2T_ERANGE.  The array takes about 2.1 MB on every GPU that loads the library,
+ *     with C2T_ERANGE.  The array takes 48 KB on every GPU that loads the library,
  *     until the process ends;
  *   - the first call on a device looks the array's device address up (cudaGetSymbolAddress,
  *     with that device current) and reads the SM count; make that first call once at start-up,
  *     before any stream capture begins;
- *   - the call only enqueues kernels on `stream`; it never calls cudaMalloc, cudaFree or any
+ *   - the call only enqueues one kernel on `stream`; it never calls cudaMalloc, cudaFree or any
  *     allocating routine.  Work is done on the device that is current when it is called;
- *   - all calls on a device share the one array and it keeps the last call's contents (the
- *     call clears what it is about to use): two calls whose kernels can overlap on the GPU -
- *     different streams, or different host threads without ordering - race on it.  Issue them
- *     on one stream, or order them with events.
+ *   - all calls on a device share the one array, which is all zeros between calls: two calls whose
+ *     kernels can overlap on the GPU - different streams, or different host threads without
+ *     ordering - race on it.  Issue them on one stream, or order them with events.
  */
 #define C2T_STATIC_MAX_ROWS  4096
 #define C2T_STATIC_MAX_VOCAB 262144
@@ -434,10 +434,13 @@ size_t c2t_host_step_ints(const c2t_config *cfg);
 
 /*
  * One whole decode step (all the calls listed at the top) with inputs and results in HOST
- * memory: copies each level's draft logits and the target logits to the caller's device
- * staging buffers on `stream`, runs the step, copies the results back and waits for
- * `stream`.  Level 0 copies only slot 0 of each sequence (the root's row).  Exists so that
- * an end-to-end figure including the transfers can be measured through the library.
+ * memory, results back when it returns.  The levels' draft logits are copied to the staging buffers
+ * ahead of the kernels, on a stream that the context makes at the first call (both staging buffers
+ * serve the levels in turn); level 0 copies only slot 0 of each sequence (the root's row).  If
+ * target_logits_host is pinned, the acceptance walk reads the rows it visits from it in place
+ * (c2t_accept_lazy; node_argmax holds the nodes on the path); else all rows are copied to
+ * target_stage_dev.  Exists so that an end-to-end figure including the transfers can be measured
+ * through the library.
  */
 int c2t_decode_step_host(c2t_ctx *ctx, const c2t_host_step *io, void *stream);
 
