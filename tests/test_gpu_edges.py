@@ -49,6 +49,12 @@ def test_widths_of_the_selection(dtype, K):
     step(2, 9000, 2, K, 3, 20, 0.0, dtype, classifier="identity")
 
 
+@pytest.mark.parametrize("B,K,F", [(1, 7, 7), (15, 10, 10)])
+def test_few_frontier_nodes_with_long_rows(B, K, F):
+    """A row lies in many chunks and its records must stay clear of the classifier's weights behind them."""
+    step(B, 128256, 3, K, F, 40, 0.5, torch.float32)
+
+
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 def test_rows_with_more_candidates_than_the_pool(dtype):
     """Well over a hundred equal largest values in scattered cells: more than the pool of a row holds, so the row is taken in
