@@ -258,6 +258,7 @@ int c2t_init(const c2t_config *cfg, void *workspace_dev, size_t workspace_bytes,
   if (e == cudaSuccess) e = cudaMemset(t.status, 0, sizeof(uint32_t) * cfg->batch);
   if (e == cudaSuccess) e = cudaMemset(t.ticket, 0, sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(t.best, 0, sizeof(unsigned long long) * cfg->batch * t.Nw);
+  if (e == cudaSuccess && t.topm_done) e = cudaMemset(t.topm_done, 0, sizeof(int32_t) * cfg->batch * cfg->frontier_cap);
   if (e == cudaSuccess) e = cudaMemset(t.row_done, 0, sizeof(int32_t) * cfg->batch * cfg->frontier_cap);
   if (e != cudaSuccess) { cudaGetLastError(); delete ctx; return C2T_ECUDA; }
   *out = ctx;
@@ -298,18 +299,19 @@ int c2t_expand_level(c2t_ctx *ctx, int level, const void *logits_dev, int64_t se
   const TreeState &t = ctx->t;
   PassParams p = expand_params(t, level, logits_dev, seq_stride, row_stride, t.V);
   const bool truncated = t.entropy_top_m > 0 && t.entropy_top_m < t.V;   // Eq. 3: the sums over the M most probable tokens
-  if (truncated) { p.topm_pool = t.topm_pool; p.topm_pool_vecs = t.topm_pool_vecs; p.topm_seg = t.topm_seg; p.topm_place = t.topm_place; }
+  const bool set_aside = truncated && t.topm_place > 0;
+  if (set_aside) { p.topm_pool = t.topm_pool; p.topm_pool_vecs = t.topm_pool_vecs; p.topm_seg = t.topm_seg; p.topm_place = t.topm_place; }
   if (launch_expand_pass(p, ctx->cfg.dtype, ctx->grid_expand, (cudaStream_t)stream) != cudaSuccess)
     return C2T_ECUDA;
   ctx->launches += 1;
   if (truncated) {
     // from the vectors the pass set aside; then, for the rows where those did not suffice, from the rows themselves
-    if (launch_topm_finish(t.entropy_top_m, t.F, t.B, p.counts, t, t.topm, ctx->cfg.dtype, (cudaStream_t)stream) != cudaSuccess)
+    if (set_aside && launch_topm_finish(t.entropy_top_m, t.F, t.B, p.counts, t, t.topm, ctx->cfg.dtype, (cudaStream_t)stream) != cudaSuccess)
       return C2T_ECUDA;
     if (launch_topm_entropy(logits_dev, seq_stride, row_stride, t.V, t.entropy_top_m, t.F, t.B, p.counts, t, t.topm,
                             t.topm_done, ctx->grid_expand, ctx->cfg.dtype, (cudaStream_t)stream) != cudaSuccess)
       return C2T_ECUDA;
-    ctx->launches += 2;
+    ctx->launches += set_aside ? 2 : 1;
   }
   ctx->expanded = 1;
   return C2T_OK;

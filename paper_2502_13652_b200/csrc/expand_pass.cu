@@ -991,6 +991,9 @@ int topm_floor_place(int vocab, int elem_bytes, int M) {
   const int vec = 16 / elem_bytes;
   const int vec_per_row = (vocab + vec - 1) / vec, head = vec_per_row < 256 ? vec_per_row : 256;
   const double per_lane = (double)head * vec / 32.0, share = 3.0 * M / vocab;
+  // The lowest place reaches a share 1 - (1 / 32)^(1 / per_lane) of the row (5 % for bf16, 10 % for fp32).  Where that is hardly M
+  // elements nothing is set aside, and the rows are read again at once: 8192 bf16 tokens with M = 1000, say.
+  if ((1.0 - pow(1.0 / 32.0, 1.0 / per_lane)) * vocab < 1.5 * M) return 0;
   const int place = share >= 1.0 ? 31 : (int)ceil(32.0 * (1.0 - pow(1.0 - share, per_lane)));
   return place < kTopmLeastPlace ? kTopmLeastPlace : (place > 31 ? 31 : place);
 }

@@ -13,8 +13,8 @@
 // highest floor among the row's segments, the M largest are among them.  The rows are not read again.
 //   topm_entropy_kernel, a persistent grid, takes the rows that kernel could not serve and reads them
 // once more.  Fast path: the row maximum is known from the expand pass; one sweep copies the elements
-// within two top key bytes of it to shared memory and the selection runs on those.  General path (that
-// guess failed too): a radix select over the row in up to five sweeps (the row stays in L2); the top
+// within two top key bytes of it to shared memory (or all elements, if those are too few and the row fits) and the selection runs on
+// those.  General path (neither served): a radix select over the row in up to five sweeps (the row stays in L2); the top
 // byte is counted in registers from the maximum's bin downwards, the later bytes with a 256-bin
 // histogram in shared memory over the elements that still match.
 #include "vocab_common.cuh"
@@ -224,20 +224,25 @@ __device__ __forceinline__ void topm_entropy_row(const void *logits, long long s
   const int sweeps = (vpr + kTopmThreads - 1) / kTopmThreads;     // the same trip count for every thread
   const uint32_t lo = BF16 ? kLowestBf16x2 : __float_as_uint(kLowestF32);
 
-  // ---- fast path: ONE sweep.  The maximum is known from the expand pass; the M-th largest value
-  // almost always lies within two top key bytes below the maximum's (a factor 64 to 256 in value), so
-  // the elements from there upwards are copied to shared memory and the selection runs on them alone;
-  // rows where that guess fails (fewer than M such elements, or more than fit) take the general path.
+  // ---- fast path.  The maximum is known from the expand pass; the M-th largest value often lies within two top key bytes
+  // below the maximum's (a factor 64 to 256 in value), so the elements from there upwards are copied to shared memory and the
+  // selection runs on them alone.  Where that is fewer than M and the row fits, all its elements are copied: a row
+  // of 8192 with M = 1000 took 88 us on the general path, which is left to long rows where the guess fails (fewer than M
+  // such elements, or more than fit) and to rows with fewer than M finite elements.
   if (M < V) {
     const unsigned long long top = aux.rows[(size_t)b * F + j].top;
     const uint32_t top_key = (uint32_t)(top >> 32);
     const int d0 = (int)(top_key >> 24);
     const float mf = key_value(top);
-    if (tid == 0) { s_win[0] = 0u; s_win[1] = 0u; s_found = 0; }
-    __syncthreads();
-    const float floor1 = __uint_as_float(f32_from_orderable((uint32_t)(d0 >= 2 ? d0 - 2 : 0) << 24));   // smallest value of byte d0-2
-    // (uniform; the floor must stay above -2^127, the value that pads a ragged vector)
-    if (top != 0ull && d0 >= 2 && mf < INFINITY && floor1 > kLowestF32) {
+    const float guess = __uint_as_float(f32_from_orderable((uint32_t)(d0 >= 2 ? d0 - 2 : 0) << 24));   // smallest value of byte d0-2
+    if (tid == 0) { s_win[0] = 0u; s_found = 0; }
+    for (int whole = 0; whole < 2; ++whole) {
+      // (uniform; the floor must stay above -2^127, the value that pads a ragged vector)
+      if (top == 0ull || !(mf < INFINITY) || (whole ? V > kTopmCand : d0 < 2 || !(guess > kLowestF32))) continue;
+      const float floor1 = whole ? kTopmLowestFloor : guess;
+      __syncthreads();
+      if (tid == 0) s_win[1] = 0u;
+      __syncthreads();
       for (int it0 = 0; it0 < sweeps; it0 += kTopmBatch) {
         uint4 qb[kTopmBatch];
 #pragma unroll
@@ -537,7 +542,8 @@ struct TopmCollected {
 constexpr int kFinishThreads = 512;
 constexpr int kFinishCand = 8192;      // keys of a row that fit in shared memory (several CTAs per SM)
 constexpr int kFinishSegs = 256;       // chunks of a row the kernel handles
-constexpr int kFinishBatch = 4;        // independent 16-byte loads a thread keeps in flight
+constexpr int kFinishBatch = 6;        // independent 16-byte loads a thread keeps in flight: 3072 vectors, as a rule all of a row's, in one
+                                       // trip (4: two trips; six levels of 160 rows of 128256 bf16 306 us, with 6 295)
 constexpr int kFinishMulti = 512;      // vectors of a row with more than one candidate that the list holds
 
 // How many elements of a vector are at or above a floor (a floor that is an element's value, or kTopmLowestFloor).
@@ -572,7 +578,7 @@ __global__ void __launch_bounds__(kFinishThreads) topm_finish_kernel(int M, int 
   __shared__ int s_first[kFinishSegs], s_start[kFinishSegs + 1];
   __shared__ unsigned long long s_top;
   __shared__ float s_floor;
-  __shared__ int s_ok;
+  __shared__ int s_ok, s_total;
   const int b = blockIdx.y, j = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
   chain_enter();
   int n = counts[b];
@@ -580,7 +586,8 @@ __global__ void __launch_bounds__(kFinishThreads) topm_finish_kernel(int M, int 
   if (j >= n) return;
   const PassInfo info = *aux.info;
   const int a = aux.row_off[b] + j;
-  // ---- the row's segments: warp 0, several chunks of the row per lane.  In the pass a CTA has cta_chunks chunks, its warps equal
+  // ---- the row's segments, closed up, by warp 0, a chunk of the row per lane (a row has about a
+  // dozen segments; a list of its 63 chunks, most of them empty, cost every thread a walk through it: 312 -> 306 us).  In the pass a CTA has cta_chunks chunks, its warps equal
   // parts of those in order; a segment begins with the row, with a CTA's range or with a warp's part.
   const int nc = info.row_chunks, n_seg = nc < kFinishSegs ? nc : kFinishSegs;
   if (tid < 32) {
@@ -589,44 +596,52 @@ __global__ void __launch_bounds__(kFinishThreads) topm_finish_kernel(int M, int 
     const int per_cta = info.cta_chunks, part = (per_cta + kExpandWarps - 1) / kExpandWarps;
     float floor = kTopmLowestFloor;
     bool ok = nc <= kFinishSegs;
-    int cnt[PER], sum = 0;
+    TopmSegment rec[PER];
+    unsigned starts[PER];
 #pragma unroll
-    for (int h = 0; h < PER; ++h) {
-      const int ch = lane * PER + h;
-      cnt[h] = 0;
-      if (ch < n_seg) {
+    for (int h = 0; h < PER; ++h) {                  // (all loads before the first use)
+      const int ch = h * 32 + lane;
+      starts[h] = 0u;
+      if (h * 32 < n_seg) {                          // (uniform)
         const int u = a * nc + ch, cta = u / per_cta, at = u - cta * per_cta;
-        if (ch == 0 || at % part == 0) {
-          const TopmSegment rec = col.seg[cta * kExpandWarps + at / part + a];
-          ok = ok && rec.n >= 0;
-          floor = fmaxf(floor, rec.floor);
-          cnt[h] = rec.n > 0 ? rec.n : 0;
-          s_first[ch] = rec.first;
-        }
+        const bool first = ch < n_seg && (ch == 0 || at % part == 0);
+        if (first) rec[h] = col.seg[cta * kExpandWarps + at / part + a];
+        starts[h] = __ballot_sync(kFull, first);
       }
-      sum += cnt[h];
     }
-    int inc = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(kFull, inc, o);
-      if (lane >= o) inc += v;
-    }
-    int run = inc - sum;
+    int n_list = 0, run = 0;                         // segments, and vectors in them, so far
 #pragma unroll
     for (int h = 0; h < PER; ++h) {
-      run += cnt[h];
-      s_start[lane * PER + h + 1] = run;
+      if (h * 32 >= n_seg) break;
+      const bool first = (starts[h] >> lane) & 1u;
+      int inc = 0;
+      if (first) {
+        ok = ok && rec[h].n >= 0;
+        floor = fmaxf(floor, rec[h].floor);
+        inc = rec[h].n > 0 ? rec[h].n : 0;
+      }
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += v;
+      }
+      if (first) {
+        const int at = n_list + __popc(starts[h] & ((1u << lane) - 1u));
+        s_first[at] = rec[h].first;
+        s_start[at + 1] = run + inc;
+      }
+      n_list += __popc(starts[h]);
+      run += __shfl_sync(kFull, inc, 31);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) floor = fmaxf(floor, __shfl_xor_sync(kFull, floor, o));
     ok = __all_sync(kFull, ok);
-    if (lane == 0) { s_start[0] = 0; s_top = top; s_floor = floor; s_ok = ok; s_count = 0u; s_multi_n = 0u; }
+    if (lane == 0) { s_start[0] = 0; s_total = run; s_top = top; s_floor = floor; s_ok = ok; s_count = 0u; s_multi_n = 0u; }
   }
   __syncthreads();
   const float mf = key_value(s_top);
   const float floor = s_floor;
-  const int total = s_start[n_seg];
+  const int total = s_total;
   if (s_ok && s_top != 0ull && mf < INFINITY) {      // (uniform)
     // A thread takes a vector at a time.  Nearly every vector holds exactly one element at or above the floor, and
     // that element is the vector's maximum: two packed operations per word give the count and the maximum without

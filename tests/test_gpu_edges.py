@@ -55,6 +55,13 @@ def test_few_frontier_nodes_with_long_rows(B, K, F):
     step(B, 128256, 3, K, F, 40, 0.5, torch.float32)
 
 
+@pytest.mark.parametrize("dtype,V,M", [(torch.bfloat16, 8192, 1000), (torch.float32, 4099, 700), (torch.bfloat16, 32768, 4000),
+                                       (torch.float32, 32768, 7000), (torch.bfloat16, 32776, 5000), (torch.bfloat16, 1003, 1002)])
+def test_truncated_entropy_of_rows_read_again(dtype, V, M):
+    """M so large that nothing is set aside: rows that fit in shared memory as a whole, up to the last that does, and the next."""
+    step(3, V, 3, 4, 3, 10, 0.0, dtype, M=M)
+
+
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 def test_rows_with_more_candidates_than_the_pool(dtype):
     """Well over a hundred equal largest values in scattered cells: more than the pool of a row holds, so the row is taken in
