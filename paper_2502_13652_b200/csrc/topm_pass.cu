@@ -587,8 +587,8 @@ __global__ void __launch_bounds__(kFinishThreads) topm_finish_kernel(int M, int 
   const PassInfo info = *aux.info;
   const int a = aux.row_off[b] + j;
   // ---- the row's segments, closed up, by warp 0, a chunk of the row per lane (a row has about a
-  // dozen segments; a list of its 63 chunks, most of them empty, cost every thread a walk through it: 312 -> 306 us).  In the pass a CTA has cta_chunks chunks, its warps equal
-  // parts of those in order; a segment begins with the row, with a CTA's range or with a warp's part.
+  // dozen segments; a list of its 63 chunks, most of them empty, cost every thread a walk through it: 312 -> 306 us).  In the pass a CTA has
+  // cta_chunks chunks, its warps equal parts of those in order; a segment begins with the row, with a CTA's range or with a warp's part.
   const int nc = info.row_chunks, n_seg = nc < kFinishSegs ? nc : kFinishSegs;
   if (tid < 32) {
     constexpr int PER = kFinishSegs / 32;
