@@ -434,7 +434,9 @@ def run_cuda(args) -> None:
     e2e_ms = max_over_ranks(e2e_ms, dist, dev)
     assert torch.equal(results["accept_len"], accept_len) and torch.equal(results["n_nodes"], n_nodes)
     eb = 2
-    h2d = B * V * eb + (D - 1) * B * F * V * eb + B * Nw * V * eb + 2 * B * 4
+    # the draft levels are copied; of the target rows the walk reads those it visits, in place
+    target_rows = int((results["accept_len"] + 1).sum())
+    h2d = B * V * eb + (D - 1) * B * F * V * eb + target_rows * V * eb + 2 * B * 4
     d2h = 4 * (B + B * Nw + B + B * (D + 1) + B)
 
     if rank != 0:
