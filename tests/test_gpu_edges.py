@@ -164,3 +164,45 @@ def test_host_step_ways(pinned, N):
         for k, w in want.items():
             assert torch.equal(results[k], w), k
     ctx.close()
+
+
+def far_rows(kind, B, F, V, dtype, seed):
+    """Rows whose warps first meet values far below the rest: a head of -80, then a body near -11, then one peak; or a body 60 to
+    69 above the head and a peak of 1e9."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    noise = torch.rand(B, F, V, device="cuda", generator=g)
+    if kind == "masked_head":
+        x = -11.2 + 0.1 * noise
+        x[:, :, :2 * V // 5] = -80.0
+        x[:, :, V - 3000:] = -90.0
+        x[:, :, V - 1500] = 8.5
+    else:
+        x = 60.0 + 9.0 * noise
+        x[:, :, :2 * V // 5] = noise[:, :, :2 * V // 5]
+        x[:, :, V - 1500] = 1e9
+    return x.to(dtype)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("kind", ["masked_head", "jump"])
+def test_rows_with_a_head_far_below_the_rest(dtype, kind):
+    """Enough chunks per row and rows per CTA that a warp meets all three parts; the sums of the body must survive the peak."""
+    B, V = 160, 65536 if dtype == torch.float32 else 131072
+    ocfg, gcfg = make_configs(B, V, 1, 10, 1, 0, 0.0, dtype, classifier="identity")
+    _, target, root, prefix = gen_inputs(1, V, 1, 1, c2t.c2t_final_width(gcfg), dtype)
+    rep = run_and_compare(ocfg, gcfg, None, None, root.expand(B).contiguous(), prefix.expand(B).contiguous(), seqs=[0, 9, 77, 159],
+                          draft_dev=[far_rows(kind, B, 1, V, dtype, 3)], target_dev=target.cuda().expand(B, -1, -1).contiguous())
+    assert rep.status_bits == 0
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("scale", [4.0, 8.0])
+def test_error_of_probabilities_and_entropies(dtype, scale):
+    """One level of whole rows.  A weight 2^t carries the error of `ex2.approx` (2^-22 at most) and the rounding of t (2^-25 for the
+    t in [-1, 0] of the largest ones), fp32 additions 2^-24 a few times over: 4e-7 in a probability.  An entropy is ln(1 + S) plus a sum
+    of weights times their logarithm, each with that error: 1e-6."""
+    B, V = 16, 128256
+    ocfg, gcfg = make_configs(B, V, 1, 10, 10, 12, 0.0, dtype)
+    draft, target, root, prefix = gen_inputs(B, V, 1, 10, c2t.c2t_final_width(gcfg), dtype, scale=scale, device="cuda")
+    rep = run_and_compare(ocfg, gcfg, None, None, root, prefix, draft_dev=draft, target_dev=target)
+    assert rep.status_bits == 0 and rep.max_rel_p < 4e-7 and rep.max_rel_H < 1e-6
