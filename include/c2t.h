@@ -76,9 +76,10 @@ typedef enum { C2T_ADD_FRONTIER = 0, C2T_ADD_ALL_SURVIVORS = 1 } c2t_tree_add;
 #define C2T_ST_POSINF_LOGIT  2u
 #define C2T_ST_ALL_NEGINF    4u
 #define C2T_ST_TREE_OVERFLOW 8u
-/* The library caught itself outside its own bounds: a row has more partial records than the workspace
- * was carved for, or (in a build with -DC2T_DEBUG_BOUNDS) an index check failed.  The access is
- * clamped or skipped, never made; the sequence's results are unspecified.  Never set by data. */
+/* The library caught itself: a bounded wait inside the expand pass ran out (the row is given up and its
+ * candidates dropped), or, in a build with -DC2T_DEBUG_BOUNDS, an index check failed (the access is skipped,
+ * never made).  The results of the sequence in this step are unspecified; later steps are not affected.
+ * Never set by data. */
 #define C2T_ST_INTERNAL      16u
 
 /*

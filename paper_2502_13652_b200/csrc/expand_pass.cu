@@ -706,13 +706,36 @@ __device__ __forceinline__ void complete_sums(const PassParams &p, const CtaRang
   __syncwarp();
 }
 
-// The CTA's part of a row shared with others is done: is the row complete?  (By one lane; the others' records are visible to it afterwards.)
-__device__ __forceinline__ bool count_shared(const PassParams &p, int a, int chunks, int nc) {
+// What becomes of a row once a CTA has done its part of it, or given up waiting for that part.
+enum RowState { kRowWaits, kRowComplete, kRowBroken };
+
+// The CTA's part of a row shared with others: is it the last?  (By one lane; the others' records are visible to it afterwards.)
+// A part that was given up is counted too, so that the count comes back to zero and the row is known to be broken.
+constexpr unsigned kBrokenPart = 1u << 23;           // above any row's chunks; the parts of a row are at most a grid's 256 CTAs
+__device__ __forceinline__ RowState count_shared(const PassParams &p, int a, int chunks, int nc, bool ok) {
   __threadfence();                                   // the CTA's records, before its count
-  if (atomicAdd(&p.row_done[a], chunks) + chunks != nc) return false;
+  const unsigned part = (unsigned)chunks + (ok ? 0u : kBrokenPart);
+  const unsigned total = atomicAdd(reinterpret_cast<unsigned *>(&p.row_done[a]), part) + part;
+  if ((total & (kBrokenPart - 1u)) != (unsigned)nc) return kRowWaits;
   p.row_done[a] = 0;                                 // for the next launch
   __threadfence();                                   // the other CTAs' records, after their counts
-  return true;
+  return total == (unsigned)nc ? kRowComplete : kRowBroken;
+}
+
+// The result of a row that was given up: no candidates, and the fault that says so.
+__device__ __forceinline__ void give_up_row(const PassParams &p, int b, int j) {
+  const int lane = threadIdx.x & 31;
+  const size_t slot = (size_t)b * p.rows_per_seq_max + j;
+  for (int i = lane; i < p.K; i += 32) p.row_keys[slot * p.K + i] = 0ull;
+  if (lane == 0) {
+    RowResult r;
+    r.M = r.S = r.T = r.L = r.H = 0.0;
+    r.top = 0ull;
+    r.n_valid = 0;
+    r.fault = C2T_ST_INTERNAL;
+    p.rows[slot] = r;
+  }
+  __syncwarp();
 }
 
 // ---------------------------------------------------------------- truncated entropy (Eq. 3): setting candidates aside
@@ -892,18 +915,18 @@ __device__ __forceinline__ void stream(const PassParams &p, CtaShared *cs, const
 __device__ __forceinline__ void pair_barrier(int pair) { asm volatile("bar.sync %0, 64;" ::"r"(1 + pair) : "memory"); }
 
 // Until all records of a task are written; false if the wait ran out.
-constexpr int kTaskWaitLimit = 1 << 22;               // tries of a task's barrier before a pair gives up (and says so)
-__device__ __forceinline__ bool wait_task(unsigned long long *bar_ptr) {
+__device__ __forceinline__ bool wait_task(unsigned long long *bar_ptr, int limit) {
   const uint32_t bar = (uint32_t)__cvta_generic_to_shared(bar_ptr);
   uint32_t done = 0u;
-  for (int i = 0; i < kTaskWaitLimit && !done; ++i)
+  for (int i = 0; i < limit && !done; ++i)
     asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                  : "=r"(done) : "r"(bar) : "memory");
   return done != 0u;
 }
 
 // A pair's work: the CTA's tasks, one after the other.  A row inside the range is complete when its records are; a
-// shared one if this CTA's part of it was the last.
+// shared one if this CTA's part of it was the last.  A row whose records do not come in time is given up: it gets a result
+// that faults its sequence, and nothing of it stays behind for later rows or launches.
 template <bool BF16, bool TOPM>
 __device__ __forceinline__ void complete(const PassParams &p, CtaShared *cs, const int *s_off, const RowShape<BF16> &rs, const CtaRange<TOPM> &cr) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pair = warp >> 1, role = warp & 1;
@@ -912,11 +935,12 @@ __device__ __forceinline__ void complete(const PassParams &p, CtaShared *cs, con
   for (;;) {
     if (role == 0 && lane == 0) {
       const int k = atomicAdd(&cs->task, 1);
-      int go = 0;
+      RowState go = kRowWaits;
       if (k < n_tasks) {
         const int a = cr.task_row(k);
-        if (!wait_task(cs->bars() + k)) { if (p.status) atomicOr(p.status, C2T_ST_INTERNAL); }
-        else go = (a >= cr.in0 && a < cr.in1) || count_shared(p, a, cr.task_chunks(a), rs.nc);
+        const bool ok = wait_task(cs->bars() + k, p.wait_limit);
+        if (a >= cr.in0 && a < cr.in1) go = ok ? kRowComplete : kRowBroken;
+        else go = count_shared(p, a, cr.task_chunks(a), rs.nc, ok);
       }
       cs->task_of[pair] = k;
       cs->flag[pair] = go;
@@ -925,9 +949,11 @@ __device__ __forceinline__ void complete(const PassParams &p, CtaShared *cs, con
     const int k = cs->task_of[pair], go = cs->flag[pair];
     pair_barrier(pair);
     if (k >= n_tasks) break;
-    if (!go) continue;
+    if (go == kRowWaits) continue;
     const int a = cr.task_row(k), b = find_sequence(s_off, p.B, a);
-    if (role == 0) complete_keys<BF16>(p, &cs->scratch[pair], a, b, a - s_off[b]);
+    if (go == kRowBroken) {
+      if (role == 0) give_up_row(p, b, a - s_off[b]);
+    } else if (role == 0) complete_keys<BF16>(p, &cs->scratch[pair], a, b, a - s_off[b]);
     else complete_sums<BF16, TOPM>(p, cr, a, b, a - s_off[b]);
   }
 }
@@ -1022,8 +1048,20 @@ int row_chunks(int vocab, int elem_bytes) {
   return ((vocab + vec - 1) / vec + kChunkVecs - 1) / kChunkVecs;
 }
 
-// the launch's shared memory
+// tries of a task's barrier before a pair gives up
+constexpr int kTaskWaitLimit = 1 << 22;
+#ifdef C2T_DEBUG_BOUNDS
+extern "C" {
+int c2t_debug_task_wait_limit = kTaskWaitLimit;      // tests let the wait run out
+}
+#define C2T_TASK_WAIT_LIMIT c2t_debug_task_wait_limit
+#else
+#define C2T_TASK_WAIT_LIMIT kTaskWaitLimit
+#endif
+
+// the launch's shared memory and limits
 static size_t plan_shared(PassParams &p, int grid) {
+  p.wait_limit = C2T_TASK_WAIT_LIMIT;
   p.cta_tasks = (int)((long long)p.B * p.rows_per_seq_max / grid) + 4;       // rows inside a CTA's range, and the two it shares
   return sizeof(CtaShared) + (size_t)p.cta_tasks * sizeof(unsigned long long) + ((size_t)p.B + 1) * sizeof(int);
 }

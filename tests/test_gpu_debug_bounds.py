@@ -51,3 +51,57 @@ def test_parity_cases_under_index_checks():
     out = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=900)
     assert out.returncode == 0, out.stdout[-2000:] + out.stderr[-4000:]
     assert "debug-bounds cases ok" in out.stdout
+
+
+GIVE_UP = r"""
+import ctypes, sys, torch
+sys.path.insert(0, {root!r}); sys.path.insert(0, {tests!r})
+import paper_2502_13652_b200 as c2t
+from parity_util import gen_inputs, make_configs
+assert c2t.LIB_PATH.endswith("libc2t_debug.so")
+limit = ctypes.c_int.in_dll(c2t.lib(), "c2t_debug_task_wait_limit")
+usual = limit.value
+# rows shared by several CTAs and rows inside one; expand and prune in one launch, in two, with candidates set aside
+for B, V, F, dtype, M in [(1, 32000, 4, torch.float32, 0), (2, 70000, 8, torch.bfloat16, 0), (5, 40000, 8, torch.float32, 0),
+                          (96, 4096, 10, torch.bfloat16, 0), (6, 32000, 8, torch.bfloat16, 64)]:
+    D, K, N = 4, 6, 20
+    _, cfg = make_configs(B, V, D, K, F, N, 0.3, dtype, M=M)
+    draft, target, root, prefix = gen_inputs(B, V, D, F, c2t.c2t_final_width(cfg), dtype)
+    draft = [t.cuda() for t in draft]; target = target.cuda(); root = root.cuda(); prefix = prefix.cuda()
+    ctx = c2t.Context(cfg)
+
+    def step(*limits):                                 # one per level
+        ctx.c2t_begin_step(root, prefix)
+        for l in range(D):
+            limit.value = limits[l]
+            ctx.c2t_expand_prune_level(l, draft[l])
+        limit.value = usual
+        ctx.c2t_prune(c2t.FINAL); ctx.c2t_build_verify(); ctx.c2t_accept(target)
+        out = [v.cpu().clone() for v in list(ctx.verify.values()) + list(ctx.accepted.values())]
+        return out, ctx.c2t_status()[1]
+
+    out, status = step(0, usual, usual, usual)         # on a new workspace: every row of level 0 is given up
+    assert all(s == c2t.ST_INTERNAL for s in status), status
+    assert (out[0] == 1).all(), out[0]                 # the roots alone
+    want, status = step(*[usual] * D)
+    assert not any(status) and int(want[0].max()) > 1, status
+    out, status = step(usual, usual, 0, usual)         # in the middle of a step
+    assert all(s == c2t.ST_INTERNAL for s in status), status
+    step(usual, 1, 2, usual)                           # whatever runs out here
+    out, status = step(*[usual] * D)
+    assert not any(status)
+    for a, b in zip(out, want):
+        assert torch.equal(a, b)
+    ctx.close()
+print("given-up rows ok")
+"""
+
+
+def test_a_wait_that_runs_out_ends_with_its_step():
+    """Rows whose records do not come in time are reported as C2T_ST_INTERNAL, and the next step on the same workspace is right."""
+    from paper_2502_13652_b200 import build
+    env = dict(os.environ, C2T_LIBRARY=build.build(debug_bounds=True))
+    code = GIVE_UP.format(root=ROOT, tests=os.path.join(ROOT, "tests"))
+    out = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=900)
+    assert out.returncode == 0, out.stdout[-2000:] + out.stderr[-4000:]
+    assert "given-up rows ok" in out.stdout
