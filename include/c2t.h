@@ -367,16 +367,17 @@ int c2t_lazy_step_gathered(c2t_ctx *ctx, int round, const uint64_t *keys_dev, in
  *
  * Limits and rules:
  *   - rows <= C2T_STATIC_MAX_ROWS and vocab <= C2T_STATIC_MAX_VOCAB; larger sizes are refused
- *     with C2T_ERANGE.  The array takes 48 KB on every GPU that loads the library,
+ *     with C2T_ERANGE.  The array takes 8 KB on every GPU that loads the library,
  *     until the process ends;
  *   - the first call on a device looks the array's device address up (cudaGetSymbolAddress,
  *     with that device current) and reads the SM count; make that first call once at start-up,
  *     before any stream capture begins;
  *   - the call only enqueues one kernel on `stream`; it never calls cudaMalloc, cudaFree or any
  *     allocating routine.  Work is done on the device that is current when it is called;
- *   - all calls on a device share the one array, which is all zeros between calls: two calls whose
- *     kernels can overlap on the GPU - different streams, or different host threads without
- *     ordering - race on it.  Issue them on one stream, or order them with events.
+ *   - all calls on a device share the one array: two calls whose kernels can overlap on the GPU -
+ *     different streams, or different host threads without ordering - race on it.  Issue them on
+ *     one stream, or order them with events.  An overlap spoils the results of the calls that
+ *     overlap, not those of later calls.
  */
 #define C2T_STATIC_MAX_ROWS  4096
 #define C2T_STATIC_MAX_VOCAB 262144

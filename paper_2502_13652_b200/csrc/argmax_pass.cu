@@ -110,29 +110,32 @@ __global__ void __launch_bounds__(kPassThreads, kPassCtasPerSm) argmax_pass_kern
   }
 }
 
-// Rows a * row_stride of a matrix, in equal spans, one per CTA.  A row that lies in one span is answered by that CTA; the pieces
-// of a row cut between CTAs meet in best[row] (atomic maximum) and done[row] (vectors seen; both 0 between calls), and the CTA
-// that completes the count answers and puts the zeros back: no launch before this one to clear anything, none after it to
-// gather.  256 rows of 128256 bf16 values: 23.9 -> 14.9 us per call (66 MB); a span per warp makes it 18 pieces to a row, with
-// two fences each, and 19.4 us.
+// Rows a * row_stride of a matrix, in equal spans, one per CTA.  A row that lies in one span is answered by that CTA; of a row
+// cut between CTAs each leaves its best key, and the CTA that finishes last answers those rows: no launch before this one to
+// clear anything, none after it to gather.  The keys are written before they are read in every call.  What one call leaves for the
+// next is the ticket: it counts modulo the grid, which is the same for all calls of a device, so that it is 0 after any number of
+// whole calls, also when some of them overlapped.  256 rows of 128256 bf16 values (66 MB): 15.1 us;
+// with keys and counts per row that the last CTA of a row puts back to zero 14.8, with a launch to clear and one to gather 23.9.
 constexpr int kMinSpanVectors = 1024;  // a CTA never gets fewer 16-byte vectors than this
 template <bool BF16>
 __global__ void __launch_bounds__(kPassThreads, kPassCtasPerSm) row_argmax_kernel(const char *logits, long long row_bytes, int rows, int V,
-                                                                                 unsigned long long *best, int *done, int32_t *out) {
+                                                                                 ArgmaxPieces *pieces, unsigned *ticket, int32_t *out) {
   using VT = Vec<BF16>;
-  __shared__ unsigned long long s_best[kWarps];
+  __shared__ unsigned long long s_best[kWarps], s_key[kMaxArgmaxCtas];
+  __shared__ bool s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  static_assert(kMaxArgmaxCtas <= kPassThreads, "a thread per CTA");
   chain_enter();
   const int vpr = (V + VT::N - 1) / VT::N, v_full = V / VT::N;
-  const long long total = (long long)rows * vpr;
-  long long span = (total + gridDim.x - 1) / gridDim.x;
+  const int total = rows * vpr;                      // (at most 4096 * 65536)
+  int span = (total + (int)gridDim.x - 1) / (int)gridDim.x;
   if (span < kMinSpanVectors) span = kMinSpanVectors;
-  long long pos = (long long)blockIdx.x * span;
-  const long long end = pos + span < total ? pos + span : total;
-  int a = (int)(pos / vpr), v0 = (int)(pos - (long long)a * vpr);
+  int pos = (int)blockIdx.x * span;
+  const int end = pos + span < total ? pos + span : total;
+  int a = pos / vpr, v0 = pos - a * vpr;
+  ArgmaxPieces mine = {0ull, 0ull};                  // (thread 0)
   for (; pos < end; ++a, v0 = 0) {
-    const long long left = end - pos;
-    const int seg = left < (long long)(vpr - v0) ? (int)left : vpr - v0, v1 = v0 + seg;
+    const int seg = end - pos < vpr - v0 ? end - pos : vpr - v0, v1 = v0 + seg;
     const char *row = logits + (size_t)a * row_bytes;
     BestVector<BF16> bv;
     bv.clear();
@@ -150,22 +153,39 @@ __global__ void __launch_bounds__(kPassThreads, kPassCtasPerSm) row_argmax_kerne
     __syncthreads();
     if (warp == 0) key = warp_best(lane < kWarps ? s_best[lane] : 0ull);
     __syncthreads();
-    if (tid == 0) {
-      bool whole = seg == vpr;
-      if (!whole) {
-        if (key) atomicMax(&best[a], key);
-        __threadfence();
-        whole = atomicAdd(&done[a], seg) + seg == vpr;
-        if (whole) {
-          __threadfence();
-          key = atomicExch(&best[a], 0ull);
-          done[a] = 0;
-        }
-      }
-      if (whole) out[a] = key ? key_token(key) : -1;
+    if (seg == vpr) {
+      if (tid == 0) out[a] = key ? key_token(key) : -1;
+    } else if (v0 > 0) {
+      mine.first = key;                              // (the row began in another CTA's span)
+    } else {
+      mine.last = key;
     }
     pos += seg;
   }
+  if (tid == 0) {
+    pieces[blockIdx.x] = mine;
+    unsigned turn;                                   // released: this CTA's pieces; acquired: those of the CTAs before it
+    asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;" : "=r"(turn) : "l"(ticket), "r"(gridDim.x - 1) : "memory");
+    s_last = turn == gridDim.x - 1;
+  }
+  // CTA c = tid, meanwhile: the row that begins in its span and goes on behind it; the CTA in which the row of its first vector begins
+  const int c0 = tid * span, c1 = c0 + span < total ? c0 + span : total;
+  const bool live = tid < (int)gridDim.x && c0 < total;
+  int cut = -1, owner = -1;
+  if (live) {
+    const int r0 = (c1 - 1) / vpr, f0 = c0 / vpr * vpr;
+    if (r0 * vpr >= c0 && (r0 + 1) * vpr > c1) cut = r0;
+    if (f0 < c0) owner = f0 / span;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  ArgmaxPieces p = {0ull, 0ull};
+  if (live) { p.first = __ldcg(&pieces[tid].first); p.last = __ldcg(&pieces[tid].last); }
+  s_key[tid] = p.last;
+  __syncthreads();
+  if (owner >= 0) atomicMax(&s_key[owner], p.first);
+  __syncthreads();
+  if (cut >= 0) out[cut] = s_key[tid] ? key_token(s_key[tid]) : -1;
 }
 
 // ---------------------------------------------------------------- lazy acceptance
@@ -272,12 +292,12 @@ cudaError_t launch_argmax_pass(const PassParams &p, int dtype, int grid, cudaStr
   return launch_chained(long_rows ? argmax_pass_kernel<false, 4> : argmax_pass_kernel<false, 8>, dim3(grid), dim3(kPassThreads), 0, s, p);
 }
 
-cudaError_t launch_row_argmax(const void *logits, int64_t row_stride, int rows, int V, int dtype, unsigned long long *best, int *done,
+cudaError_t launch_row_argmax(const void *logits, int64_t row_stride, int rows, int V, int dtype, ArgmaxPieces *pieces, unsigned *ticket,
                               int32_t *out, int grid, cudaStream_t s) {
   const char *base = reinterpret_cast<const char *>(logits);
   if (dtype == C2T_BF16)
-    return launch_chained(row_argmax_kernel<true>, dim3(grid), dim3(kPassThreads), 0, s, base, (long long)row_stride * 2, rows, V, best, done, out);
-  return launch_chained(row_argmax_kernel<false>, dim3(grid), dim3(kPassThreads), 0, s, base, (long long)row_stride * 4, rows, V, best, done, out);
+    return launch_chained(row_argmax_kernel<true>, dim3(grid), dim3(kPassThreads), 0, s, base, (long long)row_stride * 2, rows, V, pieces, ticket, out);
+  return launch_chained(row_argmax_kernel<false>, dim3(grid), dim3(kPassThreads), 0, s, base, (long long)row_stride * 4, rows, V, pieces, ticket, out);
 }
 
 static size_t lazy_smem(int Nw) { return 2 * (size_t)Nw * sizeof(int); }

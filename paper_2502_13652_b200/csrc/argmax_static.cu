@@ -11,13 +11,13 @@ constexpr int kStaticMaxRows = C2T_STATIC_MAX_ROWS;
 constexpr int kStaticMaxVocab = C2T_STATIC_MAX_VOCAB;
 constexpr int kMaxDevices = 64;
 
-// What the CTAs that read pieces of one row meet in; all zeros between calls (and when the library is loaded).
+// What the CTAs of a call leave for the one that finishes last.
 struct StaticScratch {
-  unsigned long long best[kStaticMaxRows];                    // best key so far
-  int32_t done[kStaticMaxRows];                               // vectors seen
+  ArgmaxPieces pieces[kMaxArgmaxCtas];
+  unsigned ticket;                                            // 0 between calls (and when the library is loaded)
 };
 
-// The scratch itself.  Every GPU that loads the library holds these 48 KB until the process exits.
+// The scratch itself.  Every GPU that loads the library holds these 8 KB until the process exits.
 static __device__ __align__(256) unsigned char g_static_scratch[sizeof(StaticScratch)];
 
 // Host side: the array's name is only a handle here; the device address comes from
@@ -57,13 +57,13 @@ extern "C" int c2t_row_argmax_static(const void *logits_dev, int32_t rows, int32
         return C2T_ECUDA;
       }
       g_dev[dev].scratch = static_cast<StaticScratch *>(ptr);
-      g_dev[dev].grid = sms * kPassCtasPerSm;
+      g_dev[dev].grid = sms * kPassCtasPerSm < kMaxArgmaxCtas ? sms * kPassCtasPerSm : kMaxArgmaxCtas;
     }
     pd = g_dev[dev];
   }
 
-  if (launch_row_argmax(logits_dev, row_stride, rows, vocab, dtype, pd.scratch->best, pd.scratch->done, argmax_dev, pd.grid,
-                        (cudaStream_t)stream) != cudaSuccess)
+  if (launch_row_argmax(logits_dev, row_stride, rows, vocab, dtype, pd.scratch->pieces, &pd.scratch->ticket, argmax_dev,
+                        pd.grid, (cudaStream_t)stream) != cudaSuccess)
     return C2T_ECUDA;                                         // (address arithmetic on device pointers, never dereferenced here)
   return C2T_OK;
 }

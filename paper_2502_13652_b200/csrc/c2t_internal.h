@@ -176,8 +176,13 @@ int row_chunks(int vocab, int elem_bytes);   // chunks of a row of the expand pa
 cudaError_t prepare_expand_pass();   // once per device: opt in to the kernel's shared-memory size
 cudaError_t launch_expand_pass(PassParams p, int dtype, int grid, cudaStream_t s);
 cudaError_t launch_argmax_pass(const PassParams &p, int dtype, int grid, cudaStream_t s);
-// arg-max of every row of a matrix; best, done: [rows] device scratch, zeros between calls
-cudaError_t launch_row_argmax(const void *logits, int64_t row_stride, int rows, int V, int dtype, unsigned long long *best, int *done,
+// arg-max of every row of a matrix; pieces: [grid] device scratch, a CTA's best keys of the rows it shares with the CTA before it
+// (first) and behind it (last); ticket: 0 between calls, which all have the same grid of at most kMaxArgmaxCtas
+constexpr int kMaxArgmaxCtas = kPassThreads;
+struct ArgmaxPieces {
+  unsigned long long first, last;
+};
+cudaError_t launch_row_argmax(const void *logits, int64_t row_stride, int rows, int V, int dtype, ArgmaxPieces *pieces, unsigned *ticket,
                               int32_t *out, int grid, cudaStream_t s);
 struct TreeState;
 cudaError_t prepare_accept_lazy();   // once per device

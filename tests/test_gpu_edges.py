@@ -206,3 +206,33 @@ def test_error_of_probabilities_and_entropies(dtype, scale):
     draft, target, root, prefix = gen_inputs(B, V, 1, 10, c2t.c2t_final_width(gcfg), dtype, scale=scale, device="cuda")
     rep = run_and_compare(ocfg, gcfg, None, None, root, prefix, draft_dev=draft, target_dev=target)
     assert rep.status_bits == 0 and rep.max_rel_p < 4e-7 and rep.max_rel_H < 1e-6
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_static_argmax_of_cut_rows_and_after_an_overlap(dtype):
+    """Rows cut between thread blocks in every way: one row over many of them, rows that begin or end with a span, whole rows between
+    two cut ones, rows shorter than a span.  Then calls on two streams that may overlap: what they return is undefined, what
+    later calls return is not."""
+    vec = 8 if dtype == torch.bfloat16 else 4
+    g = torch.Generator(device="cuda").manual_seed(2)
+    shapes = [(1, 262144), (1, 5), (3, 1024 * vec), (7, 1536 * vec), (40, 128256), (297, 1023 * vec + 3), (4096, 1000)]
+
+    def check():
+        for rows, V in shapes:
+            x = torch.randn(rows, -(-V // 8) * 8, device="cuda", generator=g).to(dtype)[:, :V]
+            at = torch.randint(0, V, (rows,), device="cuda", generator=g)
+            x[torch.arange(rows, device="cuda"), at] = 9.0
+            out = torch.full((rows,), -7, dtype=torch.int32, device="cuda")
+            c2t.c2t_row_argmax_static(x, out)
+            assert torch.equal(out, at.to(torch.int32)), (rows, V)
+
+    check()
+    x = torch.randn(64, 128256, device="cuda", generator=g).to(dtype)
+    outs = [torch.zeros(64, dtype=torch.int32, device="cuda") for _ in range(2)]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    for _ in range(50):
+        for s, o in zip(streams, outs):
+            c2t.c2t_row_argmax_static(x, o, s)
+    torch.cuda.synchronize()
+    check()
