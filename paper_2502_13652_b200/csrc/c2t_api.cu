@@ -260,6 +260,8 @@ int c2t_init(const c2t_config *cfg, void *workspace_dev, size_t workspace_bytes,
   if (e == cudaSuccess) e = cudaMemset(t.best, 0, sizeof(unsigned long long) * cfg->batch * t.Nw);
   if (e == cudaSuccess && t.topm_done) e = cudaMemset(t.topm_done, 0, sizeof(int32_t) * cfg->batch * cfg->frontier_cap);
   if (e == cudaSuccess) e = cudaMemset(t.row_done, 0, sizeof(int32_t) * cfg->batch * cfg->frontier_cap);
+  // all of this is on the default stream, which the stream of the first step need not wait for
+  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
   if (e != cudaSuccess) { cudaGetLastError(); delete ctx; return C2T_ECUDA; }
   *out = ctx;
   return C2T_OK;

@@ -236,3 +236,28 @@ def test_static_argmax_of_cut_rows_and_after_an_overlap(dtype):
             c2t.c2t_row_argmax_static(x, o, s)
     torch.cuda.synchronize()
     check()
+
+
+@pytest.mark.parametrize("classifier", ["mlp", "identity"])
+def test_first_step_on_a_stream_of_its_own(classifier):
+    """The default stream is busy when the context is made; the first step runs on a stream that does not wait for it."""
+    B, V, D, K, F, N = 2, 32000, 3, 5, 4, 12
+    _, gcfg = make_configs(B, V, D, K, F, N, 0.0, torch.float32, classifier=classifier)
+    draft, target, root, prefix = gen_inputs(B, V, D, F, c2t.c2t_final_width(gcfg), torch.float32)
+    draft = [t.cuda() for t in draft]; target = target.cuda(); root = root.cuda(); prefix = prefix.cuda()
+    side = torch.cuda.Stream()
+    outs = []
+    for busy in (False, True):
+        torch.full((64 << 20,), -1, dtype=torch.int32, device="cuda")              # (the next workspace is not all zeros)
+        torch.cuda.synchronize()
+        if busy:
+            torch.cuda._sleep(100_000_000)
+        ctx = c2t.Context(gcfg)
+        with torch.cuda.stream(side):
+            ctx.decode_step(draft, target, root, prefix)
+        torch.cuda.synchronize()
+        assert ctx.c2t_status()[0] == 0
+        outs.append([v.clone() for v in list(ctx.verify.values()) + list(ctx.accepted.values())])
+        ctx.close()
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)

@@ -1,0 +1,59 @@
+"""The host side of the library over a runtime that only writes down its calls (tests/fake_cuda.cpp): the order of clears, copies,
+waits and launches, and what is left behind by a call that fails.  No GPU."""
+import ctypes as C
+import os
+import subprocess
+
+import pytest
+
+import paper_2502_13652_b200 as c2t
+from paper_2502_13652_b200 import binding
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+STREAM = 0x77                                           # the caller's stream
+LEGACY = 0x1                                            # cudaStreamLegacy
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("fake") / "libc2t_fake.so")
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-w", "-Wl,-Bsymbolic", "-I", os.path.join(CUDA, "include"), "-I",
+                           os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_2502_13652_b200", "csrc"), "-o", so,
+                           os.path.join(ROOT, "tests", "fake_cuda.cpp")])
+    L = C.CDLL(so)
+    L.fake_log.restype = C.c_char_p
+    L.c2t_workspace_bytes.restype = L.c2t_host_step_ints.restype = C.c_size_t
+    L.fake_reset()
+    return L
+
+
+def config(B=3, V=4096, D=4, K=5, F=4, N=16, M=0, classifier=c2t.CLS_IDENTITY_JOINT, device=0):
+    return binding.c2t_config(B, V, c2t.F32, D, K, F, N, 0.0, M, classifier, 0, None, None, None, None, 0, device)
+
+
+def calls(L):
+    return [line.split() for line in L.fake_log().decode().splitlines()]
+
+
+class Ctx:
+    def __init__(self, L, **kw):
+        self.L, self.cfg = L, config(**kw)
+        L.fake_reset()
+        n = L.c2t_workspace_bytes(C.byref(self.cfg))
+        self.mem = C.create_string_buffer(n + 512)
+        base = (C.addressof(self.mem) + 255) & ~255
+        self.h = C.c_void_p()
+        assert L.c2t_init(C.byref(self.cfg), C.c_void_p(base), C.c_size_t(n), C.byref(self.h)) == c2t.OK
+
+    def close(self):
+        self.L.c2t_destroy(self.h)
+
+
+def test_init_waits_for_its_clears(lib):
+    """A first step may run on a stream that does not wait for the default one."""
+    ctx = Ctx(lib)
+    log = calls(lib)
+    last = max(i for i, c in enumerate(log) if c[0] in ("memset", "memcpy"))
+    assert ["sync", hex(LEGACY)] in log[last + 1:] or ["sync", "(nil)"] in log[last + 1:], log
+    ctx.close()
