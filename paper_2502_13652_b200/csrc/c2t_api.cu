@@ -17,6 +17,7 @@ struct c2t_ctx {
   int shard_vocab;       // tokens of that shard
   int finalized;         // 1 after c2t_prune(C2T_FINAL)
   int started;
+  int keys_unread;       // 1 between an arg-max pass and the launch that reads its keys and puts the zeros back
   int64_t launches;
   size_t elem_bytes;
   // c2t_decode_step_host only (made at its first call): its copies run ahead on a stream of their own
@@ -177,6 +178,17 @@ PassParams argmax_params(const TreeState &t, const void *logits, int64_t seq_str
   p.best = t.best;
   p.n_slots = (int64_t)t.B * t.Nw;
   return p;
+}
+
+// The arg-max pass.  It takes the largest of a row's keys and of what is in its place; the launch behind it reads the places and
+// leaves zeros.  Where that launch failed after an earlier pass, its keys are cleared first.
+cudaError_t argmax_pass(c2t_ctx *ctx, const PassParams &p, cudaStream_t s) {
+  if (ctx->keys_unread) {
+    const cudaError_t e = cudaMemsetAsync(p.best, 0, sizeof(unsigned long long) * (size_t)p.n_slots, s);
+    if (e != cudaSuccess) return e;
+  }
+  ctx->keys_unread = 1;
+  return launch_argmax_pass(p, ctx->cfg.dtype, ctx->grid, s);
 }
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
@@ -434,9 +446,9 @@ int c2t_accept(c2t_ctx *ctx, const void *target_logits_dev, int64_t seq_stride, 
     return C2T_EALIGN;
   const TreeState &t = ctx->t;
   const PassParams p = argmax_params(t, target_logits_dev, seq_stride, row_stride, t.V, false);
-  if (launch_argmax_pass(p, ctx->cfg.dtype, ctx->grid, (cudaStream_t)stream) != cudaSuccess)
-    return C2T_ECUDA;
+  if (argmax_pass(ctx, p, (cudaStream_t)stream) != cudaSuccess) return C2T_ECUDA;
   if (launch_accept_walk(t, out, nullptr, 0, (cudaStream_t)stream) != cudaSuccess) return C2T_ECUDA;
+  ctx->keys_unread = 0;
   ctx->launches += 2;
   return C2T_OK;
 }
@@ -453,11 +465,11 @@ int c2t_argmax_shard(c2t_ctx *ctx, const void *target_logits_dev, int64_t seq_st
     return C2T_EALIGN;
   const TreeState &t = ctx->t;
   const PassParams p = argmax_params(t, target_logits_dev, seq_stride, row_stride, vocab_count, false);
-  if (launch_argmax_pass(p, ctx->cfg.dtype, ctx->grid, (cudaStream_t)stream) != cudaSuccess)
-    return C2T_ECUDA;
+  if (argmax_pass(ctx, p, (cudaStream_t)stream) != cudaSuccess) return C2T_ECUDA;
   if (launch_export_best(t, vocab_begin, reinterpret_cast<unsigned long long *>(keys_dev), (cudaStream_t)stream) !=
       cudaSuccess)
     return C2T_ECUDA;
+  ctx->keys_unread = 0;
   ctx->launches += 2;
   return C2T_OK;
 }
@@ -509,9 +521,10 @@ int c2t_lazy_argmax_shard(c2t_ctx *ctx, const void *target_logits_dev, int64_t s
   const TreeState &t = ctx->t;
   const PassParams p = argmax_params(t, target_logits_dev, seq_stride, row_stride, vocab_count, true);
   cudaStream_t s = (cudaStream_t)stream;
-  if (launch_argmax_pass(p, ctx->cfg.dtype, ctx->grid, s) != cudaSuccess) return C2T_ECUDA;
+  if (argmax_pass(ctx, p, s) != cudaSuccess) return C2T_ECUDA;
   if (launch_export_lazy_best(t, vocab_begin, reinterpret_cast<unsigned long long *>(keys_dev), s) != cudaSuccess)
     return C2T_ECUDA;
+  ctx->keys_unread = 0;
   ctx->launches += 2;
   return C2T_OK;
 }

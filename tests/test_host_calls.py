@@ -57,3 +57,32 @@ def test_init_waits_for_its_clears(lib):
     last = max(i for i, c in enumerate(log) if c[0] in ("memset", "memcpy"))
     assert ["sync", hex(LEGACY)] in log[last + 1:] or ["sync", "(nil)"] in log[last + 1:], log
     ctx.close()
+
+
+def arg_max_calls(L, ctx, buf):
+    keys, big = C.c_void_p(buf), C.c_int64(4096)
+    h, s = ctx.h, C.c_void_p(STREAM)
+    return {"accept": lambda: L.c2t_accept(h, keys, big, big, None, s),
+            "argmax_shard": lambda: L.c2t_argmax_shard(h, keys, big, big, 4096, 0, keys, s),
+            "lazy_argmax_shard": lambda: L.c2t_lazy_argmax_shard(h, keys, big, big, 4096, 0, keys, s)}
+
+
+@pytest.mark.parametrize("second", ["accept", "argmax_shard", "lazy_argmax_shard"])
+@pytest.mark.parametrize("first,kernel", [("accept", "accept_walk"), ("argmax_shard", "export_best"), ("lazy_argmax_shard", "export_lazy_best")])
+def test_keys_of_an_arg_max_that_nobody_read(lib, first, kernel, second):
+    """An arg-max pass takes the largest of what is there; if the launch that reads its keys failed, they must go before the next."""
+    ctx = Ctx(lib)
+    buf = (C.addressof(ctx.mem) + 255) & ~255
+    assert lib.c2t_begin_step(ctx.h, C.c_void_p(buf), C.c_void_p(buf), C.c_void_p(STREAM)) == c2t.OK
+    assert lib.c2t_prune(ctx.h, c2t.FINAL, None, C.c_void_p(STREAM)) == c2t.OK
+    call = arg_max_calls(lib, ctx, buf)
+    lib.fake_fail(kernel.encode(), 1)
+    assert call[first]() == c2t.ECUDA
+    lib.fake_reset()
+    assert call[second]() == c2t.OK
+    names = [c[0] for c in calls(lib)]
+    assert names[:2] == ["memset_async", "argmax"], names
+    lib.fake_reset()
+    assert call[second]() == c2t.OK
+    assert "memset_async" not in [c[0] for c in calls(lib)]           # once
+    ctx.close()
