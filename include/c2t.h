@@ -436,13 +436,15 @@ size_t c2t_host_step_ints(const c2t_config *cfg);
 
 /*
  * One whole decode step (all the calls listed at the top) with inputs and results in HOST
- * memory, results back when it returns.  The levels' draft logits are copied to the staging buffers
- * ahead of the kernels, on a stream that the context makes at the first call (both staging buffers
- * serve the levels in turn); level 0 copies only slot 0 of each sequence (the root's row).  If
- * target_logits_host is pinned, the acceptance walk reads the rows it visits from it in place
- * (c2t_accept_lazy; node_argmax holds the nodes on the path); else all rows are copied to
- * target_stage_dev.  Exists so that an end-to-end figure including the transfers can be measured
- * through the library.
+ * memory: copies each level's draft logits and the target logits to the caller's device staging
+ * buffers, runs the step, copies the results back and waits for them.  Level 0 copies only slot 0 of
+ * each sequence (the root's row).  The copies run ahead of the kernels, ordered behind the earlier work
+ * of `stream`, on a stream that the context makes at the first call; until the target rows come both
+ * staging buffers serve the levels in turn.  When the call returns, draft_stage_dev holds the last level's
+ * rows, target_stage_dev the target rows, node_argmax (c2t_get_view) the arg-max of every node.  Exists so
+ * that an end-to-end figure including the transfers can be measured through the library.  (Where the
+ * logits that the walk does not visit need not cross the host link, make the calls one by one and give
+ * c2t_accept_lazy the pinned buffer.)
  */
 int c2t_decode_step_host(c2t_ctx *ctx, const c2t_host_step *io, void *stream);
 

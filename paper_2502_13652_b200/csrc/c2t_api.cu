@@ -610,16 +610,13 @@ int c2t_decode_step_host(c2t_ctx *ctx, const c2t_host_step *io, void *stream) {
   }
   cudaStream_t cs = ctx->copy_stream;
   // The step is bound by the host link, so it is kept busy: the levels' rows are copied ahead of the kernels into the two
-  // staging buffers in turn (the target's is free until the walk; it holds a level's rows if Nw >= F), and of the target
-  // logits only the rows on the accepted path cross the link, read by the walk itself from the pinned buffer.
-  // 8 sequences, 32000 tokens, bf16: 1512 -> 828 us per step (72 -> 38 MB; copies and kernels took turns before).
-  void *stage[2] = {io->draft_stage_dev, Nw >= F ? io->target_stage_dev : io->draft_stage_dev};
-  const int bufs = Nw >= F ? 2 : 1;
-  cudaPointerAttributes where;
-  const char *target = nullptr;                  // the target logits as the device sees them
-  if (cudaPointerGetAttributes(&where, io->target_logits_host) != cudaSuccess) cudaGetLastError();
-  else if (where.type == cudaMemoryTypeHost && aligned16(where.devicePointer) && (V * eb) % 16 == 0)
-    target = reinterpret_cast<const char *>(where.devicePointer);
+  // staging buffers in turn (the target's is free until the target rows come, and holds a level's rows if Nw >= F), the last level's
+  // into its own; the target rows follow them.  8 sequences, 32000 tokens, bf16: 1512 -> 1309 us per step, 67 MB over a link of 55 GB/s.
+  // (With the walk reading the rows it visits from the pinned buffer in place 821 us, but then neither the arg-max of the other
+  // nodes nor the staged target rows are there, which this call has always left behind; c2t_accept_lazy takes such a buffer.)
+  void *stage[2] = {io->draft_stage_dev, io->target_stage_dev};
+  const bool two = Nw >= F;
+  bool used[2] = {false, false};
 
   C2T_CUDA(cudaEventRecord(ctx->entered, s));    // (earlier work of the stream may still use the staging buffers)
   C2T_CUDA(cudaStreamWaitEvent(cs, ctx->entered, 0));
@@ -627,8 +624,9 @@ int c2t_decode_step_host(c2t_ctx *ctx, const c2t_host_step *io, void *stream) {
   C2T_CUDA(cudaMemcpyAsync(prefix, io->prefix_len_host, B * 4, cudaMemcpyHostToDevice, s));
   C2T_CALL(c2t_begin_step(ctx, root, prefix, s));
   for (size_t l = 0; l < D; ++l) {
-    const int i = (int)(l % bufs);
-    if (l >= (size_t)bufs) C2T_CUDA(cudaStreamWaitEvent(cs, ctx->consumed[i], 0));
+    const int i = two ? (int)((D - 1 - l) & 1) : 0;
+    if (used[i]) C2T_CUDA(cudaStreamWaitEvent(cs, ctx->consumed[i], 0));
+    used[i] = true;
     if (l == 0)   // only the root's row of each sequence is ever read at level 0
       C2T_CUDA(cudaMemcpy2DAsync(stage[i], F * V * eb, io->draft_logits_host[0], F * V * eb, V * eb, B, cudaMemcpyHostToDevice, cs));
     else
@@ -641,13 +639,11 @@ int c2t_decode_step_host(c2t_ctx *ctx, const c2t_host_step *io, void *stream) {
   }
   C2T_CALL(c2t_prune(ctx, C2T_FINAL, nullptr, s));
   C2T_CALL(c2t_build_verify(ctx, &vo, s));
-  if (target) {
-    C2T_CALL(c2t_lazy_begin(ctx, &ao, s));
-    C2T_CALL(c2t_accept_lazy(ctx, target, (int64_t)(Nw * V), (int64_t)V, &ao, s));
-  } else {                                       // the buffer is not pinned: by a copy of all rows
-    C2T_CUDA(cudaMemcpyAsync(io->target_stage_dev, io->target_logits_host, B * Nw * V * eb, cudaMemcpyHostToDevice, s));
-    C2T_CALL(c2t_accept(ctx, io->target_stage_dev, (int64_t)(Nw * V), (int64_t)V, &ao, s));
-  }
+  if (used[1]) C2T_CUDA(cudaStreamWaitEvent(cs, ctx->consumed[1], 0));
+  C2T_CUDA(cudaMemcpyAsync(io->target_stage_dev, io->target_logits_host, B * Nw * V * eb, cudaMemcpyHostToDevice, cs));
+  C2T_CUDA(cudaEventRecord(ctx->copied[1], cs));
+  C2T_CUDA(cudaStreamWaitEvent(s, ctx->copied[1], 0));
+  C2T_CALL(c2t_accept(ctx, io->target_stage_dev, (int64_t)(Nw * V), (int64_t)V, &ao, s));
   if (io->n_nodes_host) C2T_CUDA(cudaMemcpyAsync(io->n_nodes_host, vo.n_nodes, B * 4, cudaMemcpyDeviceToHost, s));
   if (io->tokens_host) C2T_CUDA(cudaMemcpyAsync(io->tokens_host, vo.tokens, B * Nw * 4, cudaMemcpyDeviceToHost, s));
   if (io->accept_len_host) C2T_CUDA(cudaMemcpyAsync(io->accept_len_host, ao.accept_len, B * 4, cudaMemcpyDeviceToHost, s));

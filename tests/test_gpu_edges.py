@@ -1,6 +1,6 @@
 """GPU parity at the edges of the kernels' tiles and dispatch rules: chunks of the expand pass, the K for which it takes its
 bound from half columns, its selection in order, the sizes of the lazy walk's clusters, the rerank of large trees, the short
-and long rows of the arg-max pass, the mask's 16-byte vectors, the host step's two ways to its target rows."""
+and long rows of the arg-max pass, the mask's 16-byte vectors, the host step."""
 import numpy as np
 import pytest
 import torch
@@ -149,7 +149,7 @@ def test_mask_vectors(dtype, kv):
 @pytest.mark.parametrize("pinned", [True, False])
 @pytest.mark.parametrize("N", [16, 3])
 def test_host_step_ways(pinned, N):
-    """Target rows read from the pinned buffer by the walk, or copied; two staging buffers for the levels, or one (N < F)."""
+    """Pinned or pageable host buffers; two staging buffers for the levels, or one (N < F)."""
     B, V, D, K, F = 3, 4096, 4, 5, 4
     _, gcfg = make_configs(B, V, D, K, F, N, 0.3, torch.bfloat16)
     draft, target, root, prefix = gen_inputs(B, V, D, F, c2t.c2t_final_width(gcfg), torch.bfloat16)
@@ -261,3 +261,30 @@ def test_first_step_on_a_stream_of_its_own(classifier):
         ctx.close()
     for a, b in zip(*outs):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("pinned", [True, False])
+@pytest.mark.parametrize("B,M,N", [(1, 0, 16), (2, 0, 3), (3, 64, 16), (5, 0, 16)])
+def test_host_step_leaves_what_the_calls_leave(B, M, N, pinned):
+    """One and two sequences, the truncated entropy, a budget below the frontier: results, the arg-max of every final node and the
+    staged rows are those of the calls one by one, whatever memory the rows come from."""
+    V, D, K, F = 8192, 4, 5, 4
+    _, gcfg = make_configs(B, V, D, K, F, N, 0.3, torch.bfloat16, M=M)
+    draft, target, root, prefix = gen_inputs(B, V, D, F, c2t.c2t_final_width(gcfg), torch.bfloat16)
+    ctx = c2t.Context(gcfg)
+    view = ctx.c2t_get_view()
+    ctx.decode_step([t.cuda() for t in draft], target.cuda(), root.cuda(), prefix.cuda())
+    want = {k: v.cpu().clone() for k, v in list(ctx.verify.items())[:2] + list(ctx.accepted.items())}
+    amax = view["node_argmax"].clone()
+    assert int((amax >= 0).sum()) == int(want["n_nodes"].sum())
+    stage, results = ctx.host_step_buffers()
+    pin = (lambda t: t.pin_memory()) if pinned else (lambda t: t.contiguous())
+    for _ in range(2):
+        view["node_argmax"].fill_(-7)
+        torch.cuda.synchronize()
+        ctx.c2t_decode_step_host([pin(t) for t in draft], pin(target), root, prefix, results, stage)
+        for k, w in want.items():
+            assert torch.equal(results[k], w), k
+        assert torch.equal(view["node_argmax"], amax)
+        assert torch.equal(stage["target"].cpu(), target) and torch.equal(stage["draft"].cpu(), draft[D - 1])
+    ctx.close()

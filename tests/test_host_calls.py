@@ -86,3 +86,60 @@ def test_keys_of_an_arg_max_that_nobody_read(lib, first, kernel, second):
     assert call[second]() == c2t.OK
     assert "memset_async" not in [c[0] for c in calls(lib)]           # once
     ctx.close()
+
+
+def host_step(L, ctx, alias=None):
+    """Issues a c2t_decode_step_host; returns its code and the staging ranges.  alias: bytes from the draft stage's start to the
+    target stage's (default: apart)."""
+    B, F, V, D = ctx.cfg.batch, ctx.cfg.frontier_cap, ctx.cfg.vocab, ctx.cfg.max_depth
+    rows, tgt = B * F * V * 4, B * L.c2t_final_width(C.byref(ctx.cfg)) * V * 4
+    draft = 0x10000000
+    target = draft + (0x8000000 if alias is None else alias)
+    ints = C.create_string_buffer(L.c2t_host_step_ints(C.byref(ctx.cfg)) * 4 + 64)
+    host = C.create_string_buffer(64)
+    at = (C.addressof(host) + 15) & ~15
+    arr = (C.c_void_p * D)(*[at] * D)
+    io = binding.c2t_host_step(arr, at, at, at, draft, target, (C.addressof(ints) + 15) & ~15, None, None, None, None, None)
+    rc = L.c2t_decode_step_host(ctx.h, C.byref(io), C.c_void_p(STREAM))
+    return rc, (draft, draft + rows), (target, target + tgt)
+
+
+def races(log, stages):
+    """Accesses to the staging buffers that nothing orders: (earlier, later) pairs of log lines.  A copy writes its range, a launch
+    with a pointer reads the stage that begins there."""
+    knows, events, touched, bad = {}, {}, [], []
+    for i, c in enumerate(log):
+        if c[0] == "record":
+            events[c[1]] = set(knows.setdefault(c[2], set()))
+        elif c[0] == "wait":
+            knows.setdefault(c[1], set()).update(events.get(c[2], ()))
+        elif c[0] == "copy" or (c[0] in ("expand", "argmax", "topm_entropy") and c[2] != "(nil)"):
+            stream, lo = (c[3], int(c[1], 16)) if c[0] == "copy" else (c[1], int(c[2], 16))
+            hi = lo + int(c[2]) if c[0] == "copy" else next((e for b, e in stages if b == lo), lo)
+            mine = knows.setdefault(stream, set())
+            for j, a, b, writes in touched:
+                if a < hi and lo < b and (writes or c[0] == "copy") and j not in mine:
+                    bad.append((log[j], c))
+            touched.append((i, lo, hi, c[0] == "copy"))
+            mine.add(i)
+    return bad
+
+
+@pytest.mark.parametrize("D", [1, 2, 4])
+@pytest.mark.parametrize("N", [16, 3])
+def test_host_step_leaves_its_rows_in_the_staging_buffers(lib, D, N):
+    """The last level's rows in the one, all target rows in the other, and the arg-max of every node's row is taken."""
+    ctx = Ctx(lib, D=D, N=N)
+    lib.fake_reset()
+    rc, draft, target = host_step(lib, ctx)
+    assert rc == c2t.OK
+    log = calls(lib)
+    into = {hex(draft[0]): [], hex(target[0]): []}
+    for c in log:
+        if c[0] == "copy" and c[1] in into:
+            into[c[1]].append(int(c[2]))
+    assert into[hex(draft[0])][-1] == draft[1] - draft[0] and into[hex(target[0])][-1] == target[1] - target[0]
+    assert [c[2] for c in log if c[0] == "argmax"] == [hex(target[0])]
+    assert sum(c[0] == "expand" for c in log) == D
+    assert not races(log, (draft, target))
+    ctx.close()
