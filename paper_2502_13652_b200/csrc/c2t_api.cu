@@ -615,7 +615,9 @@ int c2t_decode_step_host(c2t_ctx *ctx, const c2t_host_step *io, void *stream) {
   // (With the walk reading the rows it visits from the pinned buffer in place 821 us, but then neither the arg-max of the other
   // nodes nor the staged target rows are there, which this call has always left behind; c2t_accept_lazy takes such a buffer.)
   void *stage[2] = {io->draft_stage_dev, io->target_stage_dev};
-  const bool two = Nw >= F;
+  const uintptr_t d0 = reinterpret_cast<uintptr_t>(stage[0]), t0 = reinterpret_cast<uintptr_t>(stage[1]);
+  const bool apart = d0 + B * F * V * eb <= t0 || t0 + B * Nw * V * eb <= d0;     // (one buffer may serve as both)
+  const bool two = Nw >= F && apart;
   bool used[2] = {false, false};
 
   C2T_CUDA(cudaEventRecord(ctx->entered, s));    // (earlier work of the stream may still use the staging buffers)
@@ -639,7 +641,7 @@ int c2t_decode_step_host(c2t_ctx *ctx, const c2t_host_step *io, void *stream) {
   }
   C2T_CALL(c2t_prune(ctx, C2T_FINAL, nullptr, s));
   C2T_CALL(c2t_build_verify(ctx, &vo, s));
-  if (used[1]) C2T_CUDA(cudaStreamWaitEvent(cs, ctx->consumed[1], 0));
+  if (used[1] || !apart) C2T_CUDA(cudaStreamWaitEvent(cs, ctx->consumed[used[1]], 0));
   C2T_CUDA(cudaMemcpyAsync(io->target_stage_dev, io->target_logits_host, B * Nw * V * eb, cudaMemcpyHostToDevice, cs));
   C2T_CUDA(cudaEventRecord(ctx->copied[1], cs));
   C2T_CUDA(cudaStreamWaitEvent(s, ctx->copied[1], 0));

@@ -143,3 +143,14 @@ def test_host_step_leaves_its_rows_in_the_staging_buffers(lib, D, N):
     assert sum(c[0] == "expand" for c in log) == D
     assert not races(log, (draft, target))
     ctx.close()
+
+
+@pytest.mark.parametrize("alias", [0, 4096, 16 * 3 * 4 * 4096, -4096])
+def test_host_step_with_staging_buffers_that_overlap(lib, alias):
+    """One buffer for both stages, or two that share a part: a copy must not meet the kernel that still reads there."""
+    ctx = Ctx(lib)
+    lib.fake_reset()
+    rc, draft, target = host_step(lib, ctx, alias=alias)
+    assert rc == c2t.OK
+    assert not races(calls(lib), (draft, target))
+    ctx.close()
