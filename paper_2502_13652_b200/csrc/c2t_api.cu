@@ -191,6 +191,12 @@ cudaError_t argmax_pass(c2t_ctx *ctx, const PassParams &p, cudaStream_t s) {
   return launch_argmax_pass(p, ctx->cfg.dtype, ctx->grid, s);
 }
 
+// Waits for a stream on the way out, unless told that there is nothing left to wait for.
+struct WaitOnExit {
+  cudaStream_t stream;
+  ~WaitOnExit() { if (stream) cudaStreamSynchronize(stream); }
+};
+
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 }  // namespace
@@ -609,6 +615,7 @@ int c2t_decode_step_host(c2t_ctx *ctx, const c2t_host_step *io, void *stream) {
     ctx->copy_stream = cs;
   }
   cudaStream_t cs = ctx->copy_stream;
+  WaitOnExit copies{cs};                         // (a call that fails in the middle: its copies use the caller's buffers)
   // The step is bound by the host link, so it is kept busy: the levels' rows are copied ahead of the kernels into the two
   // staging buffers in turn (the target's is free until the target rows come, and holds a level's rows if Nw >= F), the last level's
   // into its own; the target rows follow them.  8 sequences, 32000 tokens, bf16: 1512 -> 1309 us per step, 67 MB over a link of 55 GB/s.
@@ -652,6 +659,7 @@ int c2t_decode_step_host(c2t_ctx *ctx, const c2t_host_step *io, void *stream) {
   if (io->path_host) C2T_CUDA(cudaMemcpyAsync(io->path_host, ao.path, B * (D + 1) * 4, cudaMemcpyDeviceToHost, s));
   if (io->next_token_host) C2T_CUDA(cudaMemcpyAsync(io->next_token_host, ao.next_token, B * 4, cudaMemcpyDeviceToHost, s));
   C2T_CUDA(cudaStreamSynchronize(s));
+  copies.stream = nullptr;                       // (every copy has a kernel behind it)
 #undef C2T_CUDA
 #undef C2T_CALL
   return C2T_OK;

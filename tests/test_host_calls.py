@@ -154,3 +154,23 @@ def test_host_step_with_staging_buffers_that_overlap(lib, alias):
     assert rc == c2t.OK
     assert not races(calls(lib), (draft, target))
     ctx.close()
+
+
+@pytest.mark.parametrize("call,at", [("expand", 1), ("expand", 3), ("prune", 2), ("copy", 4), ("copy", 6), ("record", 3), ("wait", 4),
+                                     ("final_prune", 1), ("argmax", 1), ("accept_walk", 1), ("sync", 1)])
+def test_host_step_that_fails_waits_for_its_copies(lib, call, at):
+    """The copies run on a stream that the caller does not have, from and to the caller's buffers."""
+    ctx = Ctx(lib)
+    assert host_step(lib, ctx)[0] == c2t.OK
+    lib.fake_reset()
+    lib.fake_fail(call.encode(), at)
+    rc = host_step(lib, ctx)[0]
+    assert rc == c2t.ECUDA
+    log = calls(lib)
+    own = {c[3] for c in log if c[0] == "copy"} - {hex(STREAM)}
+    assert len(own) == 1
+    last = max(i for i, c in enumerate(log) if c[0] == "copy" and c[3] in own)
+    assert ["sync", own.pop()] in log[last + 1:], log
+    lib.fake_reset()
+    assert host_step(lib, ctx)[0] == c2t.OK             # and the context is still good
+    ctx.close()
