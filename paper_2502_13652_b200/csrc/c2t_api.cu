@@ -191,6 +191,36 @@ cudaError_t argmax_pass(c2t_ctx *ctx, const PassParams &p, cudaStream_t s) {
   return launch_argmax_pass(p, ctx->cfg.dtype, ctx->grid, s);
 }
 
+// The stream of c2t_decode_step_host's copies and its events, on the context's device: all of them or none.
+void drop_copy_stream(c2t_ctx *ctx) {
+  cudaEvent_t *events[] = {&ctx->entered, &ctx->copied[0], &ctx->copied[1], &ctx->consumed[0], &ctx->consumed[1]};
+  for (cudaEvent_t *e : events) {
+    if (*e) cudaEventDestroy(*e);
+    *e = nullptr;
+  }
+  if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
+  ctx->copy_stream = nullptr;
+}
+
+cudaError_t make_copy_stream(c2t_ctx *ctx) {
+  int current = 0;
+  cudaError_t e = cudaGetDevice(&current);
+  if (e == cudaSuccess && current != ctx->cfg.device) e = cudaSetDevice(ctx->cfg.device);
+  if (e != cudaSuccess) return e;
+  cudaEvent_t *events[] = {&ctx->entered, &ctx->copied[0], &ctx->copied[1], &ctx->consumed[0], &ctx->consumed[1]};
+  for (cudaEvent_t *ev : events) {
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+    if (e != cudaSuccess) *ev = nullptr;
+  }
+  if (e == cudaSuccess) {
+    e = cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking);
+    if (e != cudaSuccess) ctx->copy_stream = nullptr;
+  }
+  if (e != cudaSuccess) drop_copy_stream(ctx);
+  if (current != ctx->cfg.device) cudaSetDevice(current);
+  return e;
+}
+
 // Waits for a stream on the way out, unless told that there is nothing left to wait for.
 struct WaitOnExit {
   cudaStream_t stream;
@@ -286,11 +316,7 @@ int c2t_init(const c2t_config *cfg, void *workspace_dev, size_t workspace_bytes,
 }
 
 void c2t_destroy(c2t_ctx *ctx) {
-  if (ctx && ctx->copy_stream) {
-    cudaStreamDestroy(ctx->copy_stream);
-    cudaEventDestroy(ctx->entered);
-    for (int i = 0; i < 2; ++i) { cudaEventDestroy(ctx->copied[i]); cudaEventDestroy(ctx->consumed[i]); }
-  }
+  if (ctx) drop_copy_stream(ctx);
   delete ctx;
 }
 
@@ -604,16 +630,7 @@ int c2t_decode_step_host(c2t_ctx *ctx, const c2t_host_step *io, void *stream) {
 
 #define C2T_CUDA(x) do { if ((x) != cudaSuccess) { cudaGetLastError(); return C2T_ECUDA; } } while (0)
 #define C2T_CALL(x) do { int rc_ = (x); if (rc_ != C2T_OK) return rc_; } while (0)
-  if (!ctx->copy_stream) {
-    cudaStream_t cs;
-    C2T_CUDA(cudaEventCreateWithFlags(&ctx->entered, cudaEventDisableTiming));
-    for (int i = 0; i < 2; ++i) {
-      C2T_CUDA(cudaEventCreateWithFlags(&ctx->copied[i], cudaEventDisableTiming));
-      C2T_CUDA(cudaEventCreateWithFlags(&ctx->consumed[i], cudaEventDisableTiming));
-    }
-    C2T_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-    ctx->copy_stream = cs;
-  }
+  if (!ctx->copy_stream) C2T_CUDA(make_copy_stream(ctx));
   cudaStream_t cs = ctx->copy_stream;
   WaitOnExit copies{cs};                         // (a call that fails in the middle: its copies use the caller's buffers)
   // The step is bound by the host link, so it is kept busy: the levels' rows are copied ahead of the kernels into the two

@@ -174,3 +174,26 @@ def test_host_step_that_fails_waits_for_its_copies(lib, call, at):
     lib.fake_reset()
     assert host_step(lib, ctx)[0] == c2t.OK             # and the context is still good
     ctx.close()
+
+
+@pytest.mark.parametrize("fail", [None] + [("create_event", i) for i in range(1, 6)] + [("create_stream", 1)])
+def test_host_step_makes_its_stream_once_on_the_device_of_the_context(lib, fail):
+    """Whatever device is current, and however often making them fails."""
+    ctx = Ctx(lib, device=2)
+    lib.fake_reset()
+    lib.cudaSetDevice(5)
+    events, streams = lib.fake_events(), lib.fake_streams()
+    if fail:
+        lib.fake_fail(fail[0].encode(), fail[1])
+        assert host_step(lib, ctx)[0] == c2t.ECUDA
+        assert (lib.fake_events(), lib.fake_streams()) == (events, streams)
+    for _ in range(2):
+        assert host_step(lib, ctx)[0] == c2t.OK
+    assert (lib.fake_events(), lib.fake_streams()) == (events + 5, streams + 1)
+    made = [c for c in calls(lib) if c[0].startswith("create")]
+    assert all(c[3] == "2" for c in made), made
+    device = C.c_int()
+    lib.cudaGetDevice(C.byref(device))
+    assert device.value == 5
+    ctx.close()
+    assert (lib.fake_events(), lib.fake_streams()) == (events, streams)
