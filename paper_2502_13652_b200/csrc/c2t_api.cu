@@ -102,7 +102,6 @@ size_t carve(const c2t_config *c, void *base, TreeState *t) {
   s.tree_logP = w.take<double>(B * cap);
   s.tree_C = w.take<double>(B * cap);
   s.tree_Chat = w.take<double>(B * cap);
-  s.remap = w.take<int32_t>(B * cap);
   s.cand_n = w.take<int32_t>(B);
   s.cand_token = w.take<int32_t>(B * F * K);
   s.cand_flags = w.take<int32_t>(B * F * K);

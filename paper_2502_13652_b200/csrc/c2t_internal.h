@@ -205,7 +205,6 @@ struct TreeState {
   int32_t *tree_n;             // [B]
   int32_t *tree_token, *tree_parent, *tree_level;   // [B, cap]
   double *tree_logP, *tree_C, *tree_Chat;           // [B, cap]
-  int32_t *remap;              // [B, cap] scratch of the rerank
   // candidates of the last level
   int32_t *cand_n;             // [B]
   int32_t *cand_token, *cand_flags;                 // [B, F*K]

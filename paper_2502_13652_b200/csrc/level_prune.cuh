@@ -17,30 +17,6 @@ __device__ __forceinline__ double warp_sum(double v) {
   return __shfl_sync(kFullMask, v, 0);
 }
 
-// Exclusive scan of one int per thread over a CTA of NT threads; returns the exclusive prefix, *total = sum.
-template <int NT>
-__device__ int block_exclusive_scan(int v, int *s_warp /*[NT/32+1]*/, int *total) {
-  constexpr int kTreeWarps = NT / 32;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int inc = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int t = __shfl_up_sync(kFullMask, inc, o);
-    if (lane >= o) inc += t;
-  }
-  __syncthreads();
-  if (lane == 31) s_warp[warp] = inc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int run = 0;
-    for (int w = 0; w < kTreeWarps; ++w) { int t = s_warp[w]; s_warp[w] = run; run += t; }
-    s_warp[kTreeWarps] = run;
-  }
-  __syncthreads();
-  *total = s_warp[kTreeWarps];
-  return s_warp[warp] + inc - v;
-}
-
 // ---------------------------------------------------------------- a level ---
 
 // The classifier's weights in shared memory, as doubles (a conversion per use costs more than the arithmetic): per hidden
