@@ -98,7 +98,8 @@ typedef struct {
   float   threshold;      /* beta; a node is kept iff C >= beta                           */
   int32_t entropy_top_m;  /* M of Eq. 3: entropy over the M most probable tokens, their
                              probabilities not renormalised; 0 (or M >= V) = exact, Eq. 2.
-                             M > 0 adds a pool of a third of [B, F, V] to the workspace     */
+                             M > 0 adds a pool of a third of [B, F, V] to the workspace,
+                             unless M is so large that all rows are read twice anyway       */
   int32_t classifier;     /* c2t_classifier                                               */
   int32_t hidden;         /* h                                                            */
   const float *w1;        /* HOST [h*3] row-major, features in the order (P, H, d)        */

@@ -129,11 +129,12 @@ size_t carve(const c2t_config *c, void *base, TreeState *t) {
   const size_t segs = B * F + (size_t)kMaxSms * kExpandWarps;
   s.n_segs = (int64_t)segs;
   s.n_chunks = (int64_t)(B * F * row_chunks(c->vocab, eb));
-  if (c->entropy_top_m > 0 && c->entropy_top_m < c->vocab) {   // the expand pass sets Eq. 3's candidates aside
+  const bool truncated = c->entropy_top_m > 0 && c->entropy_top_m < c->vocab;
+  if (truncated) s.topm_done = w.take<int32_t>(B * F);
+  if (truncated && topm_floor_place(c->vocab, eb, c->entropy_top_m) > 0) {     // the expand pass sets Eq. 3's candidates aside
     s.topm_pool_vecs = (long long)topm_pool_vectors(B, F, c->vocab, eb);
     s.topm_pool = w.take<uint4>((size_t)s.topm_pool_vecs);
     s.topm_seg = w.take<TopmSegment>(segs);
-    s.topm_done = w.take<int32_t>(B * F);
   }
   s.rows = w.take<RowResult>(B * F);
   s.row_keys = w.take<unsigned long long>(B * F * K);

@@ -197,3 +197,17 @@ def test_host_step_makes_its_stream_once_on_the_device_of_the_context(lib, fail)
     assert device.value == 5
     ctx.close()
     assert (lib.fake_events(), lib.fake_streams()) == (events, streams)
+
+
+def test_workspace_has_no_pool_where_nothing_is_set_aside(lib):
+    """With M so large that the floors cannot hold M elements (here: more than a quarter of the row) the rows are read again."""
+    def size(M):
+        cfg = config(B=16, V=32768, F=8, M=M)
+        return lib.c2t_workspace_bytes(C.byref(cfg))
+    pool = 16 * 8 * 32768 * 4 // 48 * 16
+    assert size(1000) - size(0) > pool
+    assert size(12000) - size(0) < 4096
+    ctx = Ctx(lib, M=2000)
+    view = binding.c2t_view()
+    assert lib.c2t_get_view(ctx.h, C.byref(view)) == c2t.OK and view.topm_from_pass
+    ctx.close()
