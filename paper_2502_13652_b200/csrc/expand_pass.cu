@@ -690,10 +690,10 @@ __device__ __forceinline__ void complete_sums(const PassParams &p, const CtaRang
   equals = __reduce_add_sync(kFull, equals);
   if (lane == 0) {
     // sums of e^(t kBack) from those of 2^t, to first order (sum 2^t t^2 taken as U^2 / S: the weight lies close together)
-    if (S > 0.0) {
-      const double S2 = S + kShort * U;
-      U += kShort * U * U / S;
-      S = S2;
+    if (S > 1e-30) {
+      const double short_of = kShort * U;
+      U += short_of * (double)__fdividef((float)U, (float)S);
+      S += short_of;
     }
     const double Sn = S * scale + (double)(equals - 1), Tn = scale * (kBack * U + g * S);
     RowResult *r = p.rows + (size_t)b * p.rows_per_seq_max + j;
