@@ -139,7 +139,9 @@ size_t carve(const c2t_config *c, void *base, TreeState *t) {
   s.rows = w.take<RowResult>(B * F);
   s.row_keys = w.take<unsigned long long>(B * F * K);
   s.row_done = w.take<int32_t>(B * F);
-  s.cells = w.take<uint32_t>(B * F * ((row_chunks(c->vocab, eb) + 1) / 2) * 32);
+  const size_t cells = B * F * ((row_chunks(c->vocab, eb) + 1) / 2) * 32;
+  s.cells = w.take<uint32_t>(cells);
+  if (eb == 4) s.cell_low = w.take<uint32_t>(cells);
   s.sums = w.take<SumRecord>((size_t)s.n_chunks);
   s.best = w.take<unsigned long long>(B * Nw);
   s.w1 = w.take<float>(3 * C2T_MAX_HIDDEN);
@@ -161,7 +163,7 @@ PassParams expand_params(const TreeState &t, int level, const void *logits, int6
   p.info = t.info_draft;
   p.row_off = t.row_off_draft;
   p.rows = t.rows; p.row_keys = t.row_keys; p.row_done = t.row_done;
-  p.cells = t.cells; p.sums = t.sums;
+  p.cells = t.cells; p.cell_low = t.cell_low; p.sums = t.sums;
   p.n_chunks = t.n_chunks; p.n_segs = t.n_segs;
   return p;
 }

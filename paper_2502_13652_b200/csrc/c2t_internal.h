@@ -134,7 +134,7 @@ struct PassParams {
   RowResult *rows;                  // [B, F]
   unsigned long long *row_keys;     // [B, F, K] the row's K largest keys, sorted descending, 0-padded
   int32_t *row_done;                // [B * F] finished chunks of a row shared by several CTAs; 0 between launches
-  uint32_t *cells;                  // [row, two chunks, 32] lane maxima (expand_pass.cu)
+  uint32_t *cells, *cell_low;       // [row, two chunks, 32] lane maxima, rounded; fp32: their lower halves (expand_pass.cu)
   SumRecord *sums;                  // [chunk] at a warp's last chunk of a row
   int64_t n_chunks, n_segs;
   int32_t cta_tasks;                // barriers in a CTA's shared memory (set at launch)
@@ -228,7 +228,7 @@ struct TreeState {
   RowResult *rows;                 // the expand pass: see PassParams
   unsigned long long *row_keys;
   int32_t *row_done;
-  uint32_t *cells;
+  uint32_t *cells, *cell_low;
   SumRecord *sums;
   int64_t n_chunks, n_segs;
   unsigned long long *best;        // [B, Nw] best key per row of the last arg-max pass; zeros between passes

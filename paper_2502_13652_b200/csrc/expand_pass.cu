@@ -279,11 +279,16 @@ __device__ __forceinline__ void load_group(uint4 (&q)[4], const uint4 *src, int 
 }
 
 // Cells are bf16, fp32 maxima rounded towards -inf: the floor taken from them is still reached by K elements, and a cell
-// with an element that reaches the floor still reaches it.
+// with an element that reaches the floor still reaches it.  The lower halves of fp32 maxima are kept apart, for select_in_order.
 __device__ __forceinline__ uint32_t cell_bits(float x, bool exact) {
   uint32_t b = __float_as_uint(x);
   if (!exact && (b & 0x80000000u)) b += 0xFFFFu;      // (a negative value: towards the larger magnitude)
   return b >> 16;
+}
+
+// the maximum of an fp32 cell from its rounded and its lower half
+__device__ __forceinline__ float whole_cell(uint32_t cell, uint32_t low) {
+  return __uint_as_float(((cell & 0x8000u) && low ? cell - 1u : cell) << 16 | low);
 }
 
 // How the launch cut the rows, as one CTA sees it.  CTA i has chunks [i per_cta, (i + 1) per_cta) of the rows laid end to end.
@@ -406,44 +411,65 @@ __device__ __noinline__ int rank_pool(PairShared *ws, int n, int K) {
   return K;
 }
 
-// Rows whose K largest do not come out of a short list (many equal values, few values): the chunks in order, elements
-// in token order 32 at a time, against a filter that rises.
+// Which of N values of a lane reach x in any lane, as bits.
+template <int N>
+__device__ __forceinline__ unsigned reached(const float (&v)[N], float x) {
+  unsigned bits = 0u;
+#pragma unroll
+  for (int i = 0; i < N; ++i) bits |= (unsigned)__any_sync(kFull, v[i] >= x) << i;
+  return bits;
+}
+
+// Rows whose K largest do not come out of a short list (many equal values, few values, most of the row masked): the chunks whose
+// maxima reach a filter, in order, elements in token order 32 at a time; the filter rises to just above the K-th value.  The maxima are
+// taken whole here: with the rounded ones every chunk of a masked fp32 row stays in question (four levels of 320 rows of
+// 128256 values, six of them finite: 2085 us, so 223).
 template <bool BF16>
 __device__ __noinline__ int select_in_order(const PassParams &p, PairShared *ws, const char *row, int a, float floor) {
+  constexpr int kWords = 8;                         // words of cells of a lane at a time
+  constexpr int kBatch = 16;                        // elements of a lane in flight
   const RowShape<BF16> rs(p.V);
   const int lane = threadIdx.x & 31, K = p.K;
   int have = 0;                                     // keys kept in pool[0 .. K)
   float thr = floor;
-  constexpr int kBatch = 8;                         // elements of a lane in flight
-  for (int w = 0; w < rs.words; ++w) {
-    const uint32_t two = p.cells[((size_t)a * rs.words + w) * 32 + lane];
-    // a cell is below the largest value it stands for by less than a bf16 step
-    const float cell = fmaxf(__uint_as_float(two << 16), __uint_as_float(two & 0xFFFF0000u));
-    const float most = BF16 ? cell : __uint_as_float(f32_from_orderable(f32_orderable(__float_as_uint(cell)) + 0xFFFFu));
-    if (!__any_sync(kFull, most >= thr)) continue;
-    const int t1 = (w + 1) * 2 * kChunkVecs * Vec<BF16>::N;
-    const int end = t1 < p.V ? t1 : p.V;
-    for (int t0 = w * 2 * kChunkVecs * Vec<BF16>::N; t0 < end; t0 += 32 * kBatch) {
-      float x[kBatch];
-      bool any = false;
+  for (int w0 = 0; w0 < rs.words; w0 += kWords) {
+    uint32_t two[kWords], low[kWords];
+    float most[kWords];
 #pragma unroll
-      for (int i = 0; i < kBatch; ++i) {
-        const int tok = t0 + i * 32 + lane;
-        x[i] = tok < end ? element<BF16>(row, tok) : -INFINITY;
-        any = any || x[i] >= thr;
-      }
-      if (!__any_sync(kFull, any)) continue;
+    for (int i = 0; i < kWords; ++i) {
+      const size_t at = ((size_t)a * rs.words + w0 + i) * 32 + lane;
+      two[i] = w0 + i < rs.words ? p.cells[at] : 0xFF80FF80u;
+      low[i] = !BF16 && w0 + i < rs.words ? p.cell_low[at] : 0u;
+    }
 #pragma unroll
-      for (int i = 0; i < kBatch; ++i) {
-        const unsigned long long key = x[i] >= thr ? make_key(x[i], (uint32_t)(t0 + i * 32 + lane)) : 0ull;
-        const bool in = key != 0ull && (have < K || key > ws->pool[K - 1]);
-        const unsigned mask = __ballot_sync(kFull, in);
-        if (mask) {
-          __syncwarp();
-          if (in) ws->pool[have + __popc(mask & ((1u << lane) - 1u))] = key;
-          __syncwarp();
-          have = rank_pool(ws, have + __popc(mask), K);
-          if (have == K) thr = just_above(key_value(ws->pool[K - 1]));   // later tokens of the K-th value lose the tie
+    for (int i = 0; i < kWords; ++i) most[i] = fmaxf(whole_cell(two[i] & 0xFFFFu, low[i] & 0xFFFFu), whole_cell(two[i] >> 16, low[i] >> 16));
+    unsigned left = (1u << kWords) - 1u;
+    for (unsigned hit; (hit = reached(most, thr) & left) != 0u;) {
+      const int w = w0 + __ffs(hit) - 1;
+      left &= ~((2u << (w - w0)) - 1u);
+      const int t1 = (w + 1) * 2 * kChunkVecs * Vec<BF16>::N, end = t1 < p.V ? t1 : p.V;
+      for (int t0 = w * 2 * kChunkVecs * Vec<BF16>::N; t0 < end; t0 += 32 * kBatch) {
+        float x[kBatch];
+        bool any = false;
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+          const int tok = t0 + i * 32 + lane;
+          x[i] = tok < end ? element<BF16>(row, tok) : -INFINITY;
+          any = any || x[i] >= thr;
+        }
+        if (!__any_sync(kFull, any)) continue;
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+          const unsigned long long key = x[i] >= thr ? make_key(x[i], (uint32_t)(t0 + i * 32 + lane)) : 0ull;
+          const bool in = key != 0ull && (have < K || key > ws->pool[K - 1]);
+          const unsigned mask = __ballot_sync(kFull, in);
+          if (mask) {
+            __syncwarp();
+            if (in) ws->pool[have + __popc(mask & ((1u << lane) - 1u))] = key;
+            __syncwarp();
+            have = rank_pool(ws, have + __popc(mask), K);
+            if (have == K) thr = just_above(key_value(ws->pool[K - 1]));   // later tokens of the K-th value lose the tie
+          }
         }
       }
     }
@@ -884,8 +910,14 @@ __device__ __forceinline__ void stream(const PassParams &p, CtaShared *cs, const
     fresh = !more || na != a;
     if (C2T_IN_BOUNDS(u, p.n_chunks, p.status)) {
       uint32_t *word = p.cells + ((size_t)a * rs.words + (ch >> 1)) * 32 + lane;
-      if (ch + 1 == rs.nc && !(ch & 1)) *word = cell_bits(cv, BF16) | (kLowestBf16x2 & 0xFFFF0000u);     // (no second cell)
-      else reinterpret_cast<unsigned short *>(word)[ch & 1] = (unsigned short)cell_bits(cv, BF16);
+      uint32_t *low = BF16 ? nullptr : p.cell_low + (word - p.cells);
+      if (ch + 1 == rs.nc && !(ch & 1)) {            // (no second cell)
+        *word = cell_bits(cv, BF16) | (kLowestBf16x2 & 0xFFFF0000u);
+        if (!BF16) *low = __float_as_uint(cv) & 0xFFFFu;
+      } else {
+        reinterpret_cast<unsigned short *>(word)[ch & 1] = (unsigned short)cell_bits(cv, BF16);
+        if (!BF16) reinterpret_cast<unsigned short *>(low)[ch & 1] = (unsigned short)__float_as_uint(cv);
+      }
       if (fresh) write_record(p.sums + u, ls);
     }
     if (fresh) {

@@ -288,3 +288,32 @@ def test_host_step_leaves_what_the_calls_leave(B, M, N, pinned):
         assert torch.equal(view["node_argmax"], amax)
         assert torch.equal(stage["target"].cpu(), target) and torch.equal(stage["draft"].cpu(), draft[D - 1])
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("mask", [float("-inf"), torch.finfo(torch.float32).min, -1e9, -10000.0, 0.0, 7.0])
+@pytest.mark.parametrize("V", [4096, 30000, 33 * 1024 + 5])
+def test_rows_of_one_value_but_for_a_few(dtype, mask, V):
+    """The K-th largest is the value that fills the row: the lowest tokens that hold it, and before them what lies above it, also by
+    less than a bf16 step (an fp32 cell is rounded to one) and in the row's last chunk."""
+    B, K = 6, 10
+    x = torch.full((B, 1, V), mask)
+    g = torch.Generator().manual_seed(1)
+    for b in range(B):
+        at = torch.randperm(V, generator=g)[:b + 3]
+        x[b, 0, at] = 20.0 + torch.arange(b + 3)
+        if mask > -1e30 and dtype == torch.float32:     # just above, early and late
+            x[b, 0, V - 1 - 700 * b] = torch.nextafter(torch.tensor(mask), torch.tensor(100.0)) + abs(mask) * 1e-6
+            x[b, 0, 2 * b] = torch.nextafter(torch.tensor(mask), torch.tensor(100.0))
+    ocfg, gcfg = make_configs(B, V, 1, K, 1, 0, 0.0, dtype, classifier="identity")
+    _, target, root, prefix = gen_inputs(B, V, 1, 1, c2t.c2t_final_width(gcfg), dtype)
+    pad = -(-V // 8) * 8
+
+    def rows(t):
+        buf = torch.zeros(B, t.shape[1], pad, dtype=dtype, device="cuda")
+        buf[:, :, :V] = t.cuda()
+        return buf[:, :, :V]
+
+    x = x.to(dtype)
+    rep = run_and_compare(ocfg, gcfg, [x], target, root, prefix, draft_dev=[rows(x)], target_dev=rows(target))
+    assert rep.status_bits == 0
