@@ -10,7 +10,9 @@ K=F=10, budget 60, threshold 0.5 (640 logits rows of 256 512 bytes per full leve
     python bench.py --impl reference [--steps K] [--warmup W]      the CPU oracle on a bounded sample
 
 For N > 1 launch through torch.distributed.run: every rank owns its own B sequences (weak
-scaling, no collective on the data path).  Rank 0 prints one JSON line.
+scaling, no collective on the data path).  Rank 0 prints one JSON line of at most 3 KB and writes what else was
+measured (the other configurations, the ablation sweep, planted paths, further levels) to build/bench_details.json
+(--details PATH).
 """
 from __future__ import annotations
 
@@ -141,6 +143,36 @@ def max_over_ranks(value: float, dist=None, device="cpu") -> float:
 def whole_job_levels_per_second(world: int, batch_per_rank: int, depth: int, ms_per_step: float) -> float:
     """Sequence-levels per second of the whole job: every rank advances its own sequences (weak scaling)."""
     return world * batch_per_rank * depth / (ms_per_step * 1e-3)
+
+
+MAX_LINE = 3000
+
+
+def rounded(x, digits: int = 6):
+    """The same object with floats cut to significant digits."""
+    if isinstance(x, dict):
+        return {k: rounded(v, digits) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [rounded(v, digits) for v in x]
+    return float(f"{x:.{digits}g}") if isinstance(x, float) else x
+
+
+def emit(line: dict, details: dict, path: str) -> str:
+    """Writes the details to `path` (the line names it, or None if it cannot be written) and returns the line's text."""
+    try:
+        os.makedirs(os.path.dirname(os.path.abspath(path)), exist_ok=True)
+        with open(path, "w") as f:
+            json.dump(dict(line, details=details), f, indent=1)
+        line = dict(line, details=os.path.relpath(path, ROOT))
+    except OSError as exc:
+        print(f"bench.py: details not written: {exc}", file=sys.stderr)
+        line = dict(line, details=None)
+    line = rounded(line)
+    for spare in ("us_per_step_blocks", "us_per_step_graph", "us_per_step_lazy_accept", "details"):   # (never needed so far)
+        if len(json.dumps(line).encode()) <= MAX_LINE:
+            break
+        line.pop(spare, None)
+    return json.dumps(line)
 
 
 def make_weights(hidden):
@@ -434,9 +466,8 @@ def run_cuda(args) -> None:
     e2e_ms = max_over_ranks(e2e_ms, dist, dev)
     assert torch.equal(results["accept_len"], accept_len) and torch.equal(results["n_nodes"], n_nodes)
     eb = 2
-    # the draft levels are copied; of the target rows the walk reads those it visits, in place
-    target_rows = int((results["accept_len"] + 1).sum())
-    h2d = B * V * eb + (D - 1) * B * F * V * eb + target_rows * V * eb + 2 * B * 4
+    # the root's rows, the other levels' rows, all target rows, roots and prefix lengths
+    h2d = B * V * eb + (D - 1) * B * F * V * eb + B * Nw * V * eb + 2 * B * 4
     d2h = 4 * (B + B * Nw + B + B * (D + 1) + B)
 
     if rank != 0:
@@ -490,50 +521,40 @@ def run_cuda(args) -> None:
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": {"workload": WORKLOAD_NAME, "value_counts": "sequence-levels per second (B*D per step, all ranks)",
                    "l2": "inputs larger than L2: 1.17 GB of draft rows and 0.98 GB of target rows per step",
-                   "rows_per_level": rows_per_level, "mean_final_nodes": float(n_nodes.float().mean()),
+                   "acceptance": "c2t_accept, all target rows",
+                   "mean_final_nodes": float(n_nodes.float().mean()),
                    "mean_accept_len": float(accept_len.float().mean()), "status_bits": status,
                    "parallelism": f"dp{world} (independent sequences per rank, no collective)"},
-        "us_per_step": ms_per_step * 1e3, "us_per_level": ms_per_step * 1e3 / D,
-        "us_per_step_blocks": {"n": len(block_ms), "steps_per_block": args.steps,
-                               "median": statistics.median(block_ms) * 1e3, "min": min(block_ms) * 1e3,
-                               "max": max(block_ms) * 1e3},
-        "graph_replay": None if graph_ms_per_step is None else {
-            "us_per_step": graph_ms_per_step * 1e3,
-            "value": whole_job_levels_per_second(world, B, D, graph_ms_per_step), "unit": UNIT,
-            "note": "the step's 21 launches captured once in a CUDA graph and replayed"},
-        "lazy_accept": {"us_per_step": lazy_ms_per_step * 1e3,
-                        "value": whole_job_levels_per_second(world, B, D, lazy_ms_per_step), "unit": UNIT,
-                        "mean_accept_len": float(accept_len.float().mean()),
-                        "note": "c2t_accept_lazy: accept_len+1 target rows per sequence instead of all final nodes",
-                        "planted_paths": {
-                            "mean_accept_len": sum(planted_depth) / len(planted_depth),
-                            "target_rows_read_per_sequence": sum(planted_depth) / len(planted_depth) + 1,
-                            "us_per_step_lazy": planted["lazy"] * 1e3,
-                            "us_per_step_all_rows": planted["all_rows"] * 1e3,
-                            "note": "target arg-maxes planted along a path of each final tree"}},
-        "single_sequence": single_seq,
-        "configs": configs,
+        "us_per_step_blocks": {"n": len(block_ms), "median": statistics.median(block_ms) * 1e3,
+                               "min": min(block_ms) * 1e3, "max": max(block_ms) * 1e3},
+        "us_per_step_graph": None if graph_ms_per_step is None else graph_ms_per_step * 1e3,
+        "us_per_step_lazy_accept": lazy_ms_per_step * 1e3,
         "clocks": clocks,
         "e2e": {"value": whole_job_levels_per_second(world, B, D, e2e_ms), "unit": UNIT, "h2d_bytes_per_step": h2d,
-                "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms, "steps": e2e_steps},
+                "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms, "steps": e2e_steps,
+                "call": "c2t_decode_step_host: pinned host logits, all target rows, results back"},
         "gpu_launches": int(launches),
         "roofline": {"bound": "hbm", "kernel": "expand_pass_kernel<bf16>", "achieved": achieved, "peak": peak,
                      "unit": "GB/s", "frac": achieved / peak, "peak_kind": f"of {peak_kind}",
-                     "traffic": traffic, "traffic_unit": "DRAM bytes per launch (ncu, read + write)",
-                     "bytes_per_launch": bytes_per_launch,
-                     "avg_launch_us": avg_launch_s * 1e6,
+                     "traffic": traffic, "bytes_per_launch": bytes_per_launch, "avg_launch_us": avg_launch_s * 1e6,
                      "full_level_rows": full_rows, "full_level_gbs": full_level_gbs,
-                     "frac_of_8000": achieved / 8000.0,
-                     "us_x_sm_mhz": None if not clocks or not clocks.get("sm_mhz") else
-                     avg_launch_s * 1e6 * clocks["sm_mhz"],
-                     "fp32_logits_full_level": None if fp32_level is None else dict(
-                         fp32_level, frac=fp32_level["gbs"] / peak),
-                     "scale1_logits_full_level": None if scale1_level is None else dict(
-                         scale1_level, frac=scale1_level["gbs"] / peak, frac_of_8000=scale1_level["gbs"] / 8000.0),
-                     "truncated_entropy_full_level": topm_level},
+                     "fp32_full_level_gbs": fp32_level["gbs"] if fp32_level else None},
         "cpu_baseline": cpu_base,
     }
-    print(json.dumps(line), flush=True)
+    details = {
+        "rows_per_level": rows_per_level,
+        "lazy_accept_planted_paths": {
+            "mean_accept_len": sum(planted_depth) / len(planted_depth),
+            "target_rows_read_per_sequence": sum(planted_depth) / len(planted_depth) + 1,
+            "us_per_step_lazy": planted["lazy"] * 1e3, "us_per_step_all_rows": planted["all_rows"] * 1e3,
+            "note": "target arg-maxes planted along a path of each final tree"},
+        "fp32_logits_full_level": None if fp32_level is None else dict(fp32_level, frac=fp32_level["gbs"] / peak),
+        "scale1_logits_full_level": None if scale1_level is None else dict(scale1_level, frac=scale1_level["gbs"] / peak),
+        "truncated_entropy_full_level": topm_level,
+        "single_sequence": single_seq, "configs": configs,
+    }
+    text = emit(line, details, args.details)
+    print(text, flush=True)
     if dist is not None:
         dist.destroy_process_group()
 
@@ -822,6 +843,8 @@ def main() -> None:
     ap.add_argument("--steps", type=int, default=None)
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", choices=["cuda", "reference"], default="cuda")
+    ap.add_argument("--details", default=os.path.join(ROOT, "build", "bench_details.json"),
+                    help="where the measurements beside the line go")
     ap.add_argument("--profile", action="store_true",
                     help="small run for profiler captures: levels 0-1 of the workload plus rerank, verify "
                          "inputs and accept; no end-to-end leg, no CPU baseline")
