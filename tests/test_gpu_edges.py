@@ -51,7 +51,8 @@ def test_widths_of_the_selection(dtype, K):
 
 @pytest.mark.parametrize("B,K,F", [(1, 7, 7), (15, 10, 10)])
 def test_few_frontier_nodes_with_long_rows(B, K, F):
-    """A row lies in many chunks and its records must stay clear of the classifier's weights behind them."""
+    """A row lies in many chunks; its cells and records must stay clear of each other and of the arg-max keys behind them, which the
+    acceptance calls (compared here too) take their maxima from."""
     step(B, 128256, 3, K, F, 40, 0.5, torch.float32)
 
 
