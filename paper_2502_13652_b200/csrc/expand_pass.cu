@@ -31,10 +31,7 @@
 // precision.  The row's largest element stays out of the sums, so that they keep fp32 relative accuracy with respect to
 // "everything but the maximum" however peaked the row is: the one lane and chunk that holds it is summed again without it.
 // Everything is computed in an order that does not depend on timing, so the results are reproducible bit for bit.
-#include <math.h>
-
-#include "vocab_common.cuh"
-#include "level_prune.cuh"
+#include "row_sums.cuh"
 
 namespace c2t {
 namespace {
@@ -44,7 +41,6 @@ constexpr int kEWarps = kExpandThreads / 32;          // ... the others only com
 constexpr int kPairs = kEWarps / 2;
 constexpr int kGroups = kChunkVecs / 128;             // groups of a chunk; a lane holds 4 vectors of each, 32 apart
 constexpr int kListCap = 128;                         // cells of a row that are read again
-constexpr int kPoolCap = 128;                         // keys ranked at a time
 static_assert(kStreamWarps % 2 == 0 && kPairs <= 15, "pairs of warps, one named barrier each");
 
 // What a pair of warps needs in shared memory to complete a row.
@@ -63,108 +59,12 @@ struct CtaShared {
   __device__ unsigned long long *bars() { return reinterpret_cast<unsigned long long *>(this + 1); }
 };
 
-// ---------------------------------------------------------------- packed sums
-
-typedef unsigned long long f32x2;
-
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
-  f32x2 d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-  return d;
-}
-__device__ __forceinline__ void unpack2(f32x2 a, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a)); }
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-  f32x2 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
-// S and U of a lane: two packed accumulators each, so that consecutive additions do not wait for each other.
-struct Acc {
-  f32x2 S[2], U[2];
-  __device__ __forceinline__ void clear() { S[0] = S[1] = U[0] = U[1] = 0ull; }
-  __device__ __forceinline__ void totals(float &s, float &u) const {
-    float a, b, c, d;
-    unpack2(add2(S[0], S[1]), a, b);
-    unpack2(add2(U[0], U[1]), c, d);
-    s = a + b;
-    u = c + d;
-  }
-};
-
-__device__ __forceinline__ void acc_pair(Acc &a, int i, float x0, float x1, f32x2 scale, f32x2 c) {
-  const f32x2 t = fma2(pack2(x0, x1), scale, c);
-  float t0, t1;
-  unpack2(t, t0, t1);
-  const f32x2 e = pack2(ex2f(t0), ex2f(t1));
-  a.S[i] = add2(a.S[i], e);
-  a.U[i] = fma2(e, t, a.U[i]);
-}
-
-template <bool BF16>
-__device__ __forceinline__ void acc_vector(Acc &a, const uint4 &q, f32x2 scale, f32x2 c) {
-  float x[Vec<BF16>::N];
-  Vec<BF16>::unpack(q, x);
-#pragma unroll
-  for (int i = 0; i < Vec<BF16>::N; i += 2) acc_pair(a, (i >> 1) & 1, x[i], x[i + 1], scale, c);
-}
-
-// ---------------------------------------------------------------- maxima
-
-// A running maximum of whole vectors (NaN ignored): packed for bf16, plain for fp32.
-template <bool BF16>
-struct RunMax {
-  uint32_t v;
-  __device__ __forceinline__ void clear() { v = BF16 ? kLowestBf16x2 : __float_as_uint(kLowestF32); }
-  __device__ __forceinline__ void take(const uint4 &q) {
-    if (BF16) v = max_bf16x2(v, max_bf16x2(max_bf16x2(q.x, q.y), max_bf16x2(q.z, q.w)));
-    else v = __float_as_uint(fmaxf(__uint_as_float(v), fmaxf(fmaxf(__uint_as_float(q.x), __uint_as_float(q.y)),
-                                                             fmaxf(__uint_as_float(q.z), __uint_as_float(q.w)))));
-  }
-  __device__ __forceinline__ void take(const RunMax &o) {
-    v = BF16 ? max_bf16x2(v, o.v) : __float_as_uint(fmaxf(__uint_as_float(v), __uint_as_float(o.v)));
-  }
-  __device__ __forceinline__ float value() const {
-    return BF16 ? fmaxf(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u)) : __uint_as_float(v);
-  }
-};
-
 // the float just above a value
 __device__ __forceinline__ float just_above(float x) {
   return __uint_as_float(f32_from_orderable(f32_orderable(__float_as_uint(x)) + 1u));
 }
 
 // ---------------------------------------------------------------- a warp's sums of a row
-
-// The offset of a reference m: an integer at or below -m log2(e), and monotone, so that no value up to m has a positive t.
-__device__ __forceinline__ float offset_of(float m) { return floorf(__fmul_rd(fminf(m, 2e38f), -kLog2e)); }
-constexpr float kNoOffset = 3e38f;                    // no data yet: behind every real offset
-
-// Sums follow their offset down by d, an integer <= 0: every t by d, every weight by 2^d (0 from d = -127 on).
-struct Shift {
-  f32x2 d, f;
-  __device__ __forceinline__ explicit Shift(float by) {
-    by = fmaxf(by, -127.f);
-    const float two = __int_as_float((__float_as_int(by + 12582912.f) << 23) + 0x3F800000);      // 2^by
-    d = pack2(by, by);
-    f = pack2(two, two);
-  }
-  __device__ __forceinline__ void apply(f32x2 &S, f32x2 &U) const {
-    U = mul2(f, fma2(d, S, U));
-    S = mul2(f, S);
-  }
-};
 
 // A lane's sums of the chunks of a row that its warp streams; the chunk with the lane's largest value is kept apart.
 struct LaneSums {
@@ -215,9 +115,6 @@ struct LaneSums {
   }
 };
 
-// 2^d for an integer d <= 0
-__device__ __forceinline__ double pow2_f64(float d) { return d < -1000.f ? 0.0 : __hiloint2double((1023 + (int)d) << 20, 0); }
-
 // The lanes' sums over the warp into a record, relative to the warp's largest value.
 __device__ __forceinline__ void write_record(SumRecord *rec, LaneSums &ls) {
   const int lane = threadIdx.x & 31;
@@ -256,10 +153,6 @@ struct RowShape {
 __device__ __forceinline__ const char *row_pointer(const PassParams &p, int b, int j, size_t esz) {
   return reinterpret_cast<const char *>(p.logits) + ((size_t)b * p.seq_stride + (size_t)j * p.row_stride) * esz;
 }
-
-// the ragged last vector of a row, assembled from scalar loads
-template <bool BF16>
-__device__ __noinline__ uint4 load_ragged(const void *row, int v, int v_full, int V) { return Vec<BF16>::load(row, v, v_full, V); }
 
 // Requests group g of a chunk: src points at the lane's first vector of the chunk, nv counts the whole vectors from the
 // chunk's start on.  Vectors past them become the lowest value, which adds exactly 0 to the sums.
@@ -377,40 +270,6 @@ __device__ __forceinline__ void load_vectors(uint4 (&q)[N], const char *row, con
   for (int u = 0; u < N; ++u) Vec<BF16>::clamp(q[u]);
 }
 
-// Ranks the first n keys of the pool: the K largest move to pool[0 .. K), sorted, 0-padded.  Returns how many there are.
-__device__ __noinline__ int rank_pool(PairShared *ws, int n, int K) {
-  const int lane = threadIdx.x & 31;
-  if (n <= 32) {                                     // the usual case: a key per lane
-    const unsigned long long key = lane < n ? ws->pool[lane] : 0ull;
-    int place = 0;
-#pragma unroll 8
-    for (int r = 0; r < n; ++r) place += ws->pool[r] > key;
-    if (lane >= n) place = lane;                     // (the zeros behind the keys)
-    __syncwarp();
-    ws->pool[place] = key;
-    __syncwarp();
-    return n < K ? n : K;
-  }
-  unsigned long long mine[kPoolCap / 32];
-  int rank[kPoolCap / 32];
-#pragma unroll
-  for (int i = 0; i < kPoolCap / 32; ++i) {
-    mine[i] = i * 32 + lane < n ? ws->pool[i * 32 + lane] : 0ull;
-    rank[i] = 0;
-  }
-  for (int r = 0; r < n; ++r) {
-    const unsigned long long k = ws->pool[r];
-#pragma unroll
-    for (int i = 0; i < kPoolCap / 32; ++i) rank[i] += k > mine[i];
-  }
-  __syncwarp();
-#pragma unroll
-  for (int i = 0; i < kPoolCap / 32; ++i)
-    if (mine[i] != 0ull && rank[i] < K) ws->pool[rank[i]] = mine[i];     // (K <= 32 < n: all K places are taken)
-  __syncwarp();
-  return K;
-}
-
 // Which of N values of a lane reach x in any lane, as bits.
 template <int N>
 __device__ __forceinline__ unsigned reached(const float (&v)[N], float x) {
@@ -467,7 +326,7 @@ __device__ __noinline__ int select_in_order(const PassParams &p, PairShared *ws,
             __syncwarp();
             if (in) ws->pool[have + __popc(mask & ((1u << lane) - 1u))] = key;
             __syncwarp();
-            have = rank_pool(ws, have + __popc(mask), K);
+            have = rank_pool(ws->pool, have + __popc(mask), K);
             if (have == K) thr = just_above(key_value(ws->pool[K - 1]));   // later tokens of the K-th value lose the tie
           }
         }
@@ -623,7 +482,7 @@ __device__ __forceinline__ void complete_keys(const PassParams &p, PairShared *w
   }
   __syncwarp();
   const int n_keys = n_list <= kListCap ? gather_keys<BF16>(ws, row, rs, p.V, floor, n_list) : -1;
-  const int n_valid = n_keys >= 0 ? rank_pool(ws, n_keys, K) : select_in_order<BF16>(p, ws, row, a, floor);
+  const int n_valid = n_keys >= 0 ? rank_pool(ws->pool, n_keys, K) : select_in_order<BF16>(p, ws, row, a, floor);
   const size_t slot = (size_t)b * p.rows_per_seq_max + j;
   for (int i = lane; i < K; i += 32) p.row_keys[slot * K + i] = ws->pool[i];
   if (lane == 0) {
@@ -684,11 +543,6 @@ __device__ __forceinline__ void complete_sums(const PassParams &p, const CtaRang
     for (int e = 0; e < Vec<BF16>::N; e += 2) acc_pair(acc, (e >> 1) & 1, x[e], x[e + 1], pack2(kLog2e, kLog2e), pack2(cM, cM));
     acc.totals(s_own, u_own);
   }
-  // t = x kLog2e + cM with the fp32 constant, so x - M = t kBack + g, exactly that constant's inverse: its error of 1.3e-8 of x must
-  // not meet the exact M.  What is left is that 2^t is not e^(t kBack) but short of it by kShort t, small where the weight is.
-  const double kBack = 1.0 / (double)kLog2e, kShort = kBack - 0.69314718055994530942;
-  const double M = (double)Mf, g = -(double)cM * kBack - M, scale = exp(g);
-
   // ---- merge: all records brought to the reference of the maximum
   double S = (double)s_own, U = (double)u_own;
   for (int c0 = 0; c0 < rs.nc; c0 += 32 * kBatch) {
@@ -714,21 +568,7 @@ __device__ __forceinline__ void complete_sums(const PassParams &p, const CtaRang
   S = warp_sum(S);
   U = warp_sum(U);
   equals = __reduce_add_sync(kFull, equals);
-  if (lane == 0) {
-    // sums of e^(t kBack) from those of 2^t, to first order (sum 2^t t^2 taken as U^2 / S: the weight lies close together)
-    if (S > 1e-30) {
-      const double short_of = kShort * U;
-      U += short_of * (double)__fdividef((float)U, (float)S);
-      S += short_of;
-    }
-    const double Sn = S * scale + (double)(equals - 1), Tn = scale * (kBack * U + g * S);
-    RowResult *r = p.rows + (size_t)b * p.rows_per_seq_max + j;
-    r->M = M; r->S = Sn; r->T = Tn;
-    const double L = log1p(Sn);                     // ln sum_v e^(x_v - M); the maximum contributes the 1
-    r->L = L;
-    r->H = L - Tn / (1.0 + Sn);                     // Eq. 2 with natural log
-    r->fault = row_fault_bits(Mf, Sn, Tn);
-  }
+  if (lane == 0) write_sums(p.rows + (size_t)b * p.rows_per_seq_max + j, Mf, cM, S, U, equals);
   __syncwarp();
 }
 
