@@ -11,7 +11,7 @@ CSRC = os.path.join(_HERE, "csrc")
 INCLUDE = os.path.join(_ROOT, "include")
 LIB = os.path.join(_HERE, "libc2t.so")
 LIB_DEBUG = os.path.join(_HERE, "libc2t_debug.so")      # the same sources with -DC2T_DEBUG_BOUNDS (index checks)
-SOURCES = ["c2t_api.cu", "expand_pass.cu", "argmax_pass.cu", "topm_pass.cu", "tree_kernels.cu", "argmax_static.cu"]
+SOURCES = ["c2t_api.cu", "expand_pass.cu", "row_pass.cu", "argmax_pass.cu", "topm_pass.cu", "tree_kernels.cu", "argmax_static.cu"]
 
 
 def _newest_source() -> float:

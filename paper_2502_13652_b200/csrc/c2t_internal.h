@@ -128,6 +128,7 @@ struct PassParams {
   int64_t seq_stride, row_stride;   // elements
   int32_t V, K, B;
   int32_t rows_per_seq_max;         // F (draft) or Nw (target)
+  int32_t rows_bound;               // expand: no sequence has more active rows at this level
   const int32_t *counts;            // [B] active rows per sequence, device
   const int32_t *row_sel;           // arg-max pass only, may be null: [B] the row of sequence b to read (then counts is 0 or 1)
   uint32_t *status;                 // may be null: a status word for C2T_ST_INTERNAL (the first sequence's)
@@ -147,6 +148,10 @@ struct PassParams {
   long long topm_pool_vecs;
   int32_t topm_place;               // the floor's place among the lane maxima (topm_floor_place)
   TopmSegment *topm_seg;            // [warp + row]
+  // expand with M > 0 and the rows in registers (else null): Eq. 3's sums and which rows have them, [B, F]
+  double2 *topm_out;
+  int32_t *topm_done;
+  int32_t topm_m;
   // argmax: [B, rows_per_seq_max] best key per row, the largest of what is there and of the row's keys (0 before the pass;
   // the kernel that reads a key puts the 0 back)
   unsigned long long *best;
@@ -175,6 +180,17 @@ int topm_floor_place(int vocab, int elem_bytes, int M);
 size_t topm_pool_vectors(size_t batch, size_t rows_per_seq, int vocab, int elem_bytes);
 
 int row_chunks(int vocab, int elem_bytes);   // chunks of a row of the expand pass
+
+// ---------------------------------------------------------------- rows in registers (row_pass.cu)
+constexpr int kRowThreads = 512;
+constexpr int kRowPart = kRowThreads * 8;       // 16-byte vectors of a row that a block holds
+constexpr int kRowCluster = 8;                  // blocks of a row at most
+constexpr int kRowBlocksPerSm = 2;
+constexpr int kRowTopmList = 12288;             // keys of a row's candidates for Eq. 3, cut evenly among its blocks
+struct TreeState;
+cudaError_t prepare_row_pass();                 // once per device: opt in to the shared-memory size
+cudaError_t launch_expand_rows(const PassParams &p, int dtype, int cluster, cudaStream_t s);
+cudaError_t launch_expand_rows_prune(const PassParams &p, const TreeState &t, int level, const c2t_frontier &out, int dtype, int cluster, cudaStream_t s);
 
 cudaError_t prepare_expand_pass();   // once per device: opt in to the kernel's shared-memory size
 cudaError_t launch_expand_pass(PassParams p, int dtype, int grid, cudaStream_t s);
