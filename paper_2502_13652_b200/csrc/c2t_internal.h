@@ -188,6 +188,32 @@ constexpr int kRowCluster = 8;                  // blocks of a row at most
 constexpr int kRowBlocksPerSm = 2;
 constexpr int kRowTopmList = 12288;             // keys of a row's candidates for Eq. 3, cut evenly among its blocks
 struct TreeState;
+
+// tries of a task's barrier in the streaming pass before a pair gives up
+constexpr int kTaskWaitLimit = 1 << 22;
+#ifdef C2T_DEBUG_BOUNDS
+extern "C" int c2t_debug_task_wait_limit;       // tests let the wait run out: then every level takes the pass that waits
+#define C2T_TASK_WAIT_LIMIT c2t_debug_task_wait_limit
+#else
+#define C2T_TASK_WAIT_LIMIT kTaskWaitLimit
+#endif
+
+// The blocks per row, 0 where the level is not for that pass.
+inline int row_pass_cluster(int vocab, int elem_bytes, long long rows, int sms, int blocks) {
+  if (C2T_TASK_WAIT_LIMIT != kTaskWaitLimit) return 0;
+  const int vec = 16 / elem_bytes, vpr = (vocab + vec - 1) / vec;
+  int cluster = 1;
+  while (cluster < kRowCluster && (vpr + cluster - 1) / cluster > kRowPart) cluster *= 2;
+  if ((vpr + cluster - 1) / cluster > kRowPart || rows * cluster > blocks) return 0;
+  while (cluster < kRowCluster && 2 * cluster * rows <= sms) cluster *= 2;
+  return cluster;
+}
+// The same with Eq. 3's sums.
+inline int row_topm_cluster(int vocab, int elem_bytes, long long rows, int sms, int M) {
+  const int vec = 16 / elem_bytes;
+  if (vocab < kRowThreads * vec || 4 * M > kRowTopmList) return 0;
+  return row_pass_cluster(vocab, elem_bytes, rows, sms, 0x7FFFFFFF);
+}
 cudaError_t prepare_row_pass();                 // once per device: opt in to the shared-memory size
 cudaError_t launch_expand_rows(const PassParams &p, int dtype, int cluster, cudaStream_t s);
 cudaError_t launch_expand_rows_prune(const PassParams &p, const TreeState &t, int level, const c2t_frontier &out, int dtype, int cluster, cudaStream_t s);

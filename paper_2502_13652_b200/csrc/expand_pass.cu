@@ -920,15 +920,10 @@ int row_chunks(int vocab, int elem_bytes) {
   return ((vocab + vec - 1) / vec + kChunkVecs - 1) / kChunkVecs;
 }
 
-// tries of a task's barrier before a pair gives up
-constexpr int kTaskWaitLimit = 1 << 22;
 #ifdef C2T_DEBUG_BOUNDS
 extern "C" {
-int c2t_debug_task_wait_limit = kTaskWaitLimit;      // tests let the wait run out
+int c2t_debug_task_wait_limit = kTaskWaitLimit;
 }
-#define C2T_TASK_WAIT_LIMIT c2t_debug_task_wait_limit
-#else
-#define C2T_TASK_WAIT_LIMIT kTaskWaitLimit
 #endif
 
 // the launch's shared memory and limits
@@ -939,6 +934,8 @@ static size_t plan_shared(PassParams &p, int grid) {
 }
 
 cudaError_t prepare_expand_pass() {
+  const cudaError_t r = prepare_row_pass();
+  if (r != cudaSuccess) return r;
   const int bytes = 100 * 1024;                      // more than plan_shared asks for at the limits of a configuration
   cudaError_t e = cudaFuncSetAttribute(expand_pass_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_pass_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -949,9 +946,19 @@ cudaError_t prepare_expand_pass() {
   return e;
 }
 
+// The blocks per row of the pass in registers (row_pass.cu), or 0.
+static int rows_in_registers(const PassParams &p, int dtype, int sms) {
+  const int eb = dtype == C2T_BF16 ? 2 : 4;
+  const long long rows = (long long)p.B * p.rows_bound;
+  if (p.topm_out) return row_topm_cluster(p.V, eb, rows, sms, p.topm_m);
+  if (p.topm_pool) return 0;
+  return row_pass_cluster(p.V, eb, rows, sms, sms * kRowBlocksPerSm);
+}
+
 cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, const c2t_frontier *out, int dtype, int grid, cudaStream_t s) {
   c2t_frontier o = {nullptr, nullptr, nullptr, nullptr};
   if (out) o = *out;
+  if (const int cluster = rows_in_registers(p, dtype, grid)) return launch_expand_rows_prune(p, t, level, o, dtype, cluster, s);
   size_t smem = plan_shared(p, grid);
   if (smem < sizeof(PruneShared)) smem = sizeof(PruneShared);
   if (dtype == C2T_BF16)
@@ -960,6 +967,7 @@ cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, con
 }
 
 cudaError_t launch_expand_pass(PassParams p, int dtype, int grid, cudaStream_t s) {
+  if (const int cluster = rows_in_registers(p, dtype, grid)) return launch_expand_rows(p, dtype, cluster, s);
   const size_t smem = plan_shared(p, grid);
   const bool bf16 = dtype == C2T_BF16;
   if (p.topm_pool) {                                 // also sets the candidates of Eq. 3 aside
