@@ -182,11 +182,13 @@ size_t topm_pool_vectors(size_t batch, size_t rows_per_seq, int vocab, int elem_
 int row_chunks(int vocab, int elem_bytes);   // chunks of a row of the expand pass
 
 // ---------------------------------------------------------------- rows in registers (row_pass.cu)
-constexpr int kRowThreads = 512;
-constexpr int kRowPart = kRowThreads * 8;       // 16-byte vectors of a row that a block holds
+constexpr int kRowThreads = 512;                // threads of a block at most (or half as many)
+constexpr int kRowPart = kRowThreads * 8;       // 16-byte vectors of a row that a block of so many holds
 constexpr int kRowCluster = 8;                  // blocks of a row at most
-constexpr int kRowBlocksPerSm = 2;
 constexpr int kRowTopmList = 12288;             // keys of a row's candidates for Eq. 3, cut evenly among its blocks
+struct RowPlan {
+  int cluster, threads;                         // blocks per row (0: the level is not for that pass), threads of a block
+};
 struct TreeState;
 
 // tries of a task's barrier in the streaming pass before a pair gives up
@@ -198,25 +200,29 @@ extern "C" int c2t_debug_task_wait_limit;       // tests let the wait run out: t
 #define C2T_TASK_WAIT_LIMIT kTaskWaitLimit
 #endif
 
-// The blocks per row, 0 where the level is not for that pass.
-inline int row_pass_cluster(int vocab, int elem_bytes, long long rows, int sms, int blocks) {
-  if (C2T_TASK_WAIT_LIMIT != kTaskWaitLimit) return 0;
+// How a level is cut, if all its rows fit the chip at once (or fits is false): the smaller blocks where a row fits eight of them.
+inline RowPlan row_pass_plan(int vocab, int elem_bytes, long long rows, int sms, bool fits) {
+  RowPlan plan = {0, 0};
+  if (C2T_TASK_WAIT_LIMIT != kTaskWaitLimit) return plan;
   const int vec = 16 / elem_bytes, vpr = (vocab + vec - 1) / vec;
+  const int threads = vpr <= kRowCluster * kRowPart / 2 ? kRowThreads / 2 : kRowThreads, part = threads * 8;
   int cluster = 1;
-  while (cluster < kRowCluster && (vpr + cluster - 1) / cluster > kRowPart) cluster *= 2;
-  if ((vpr + cluster - 1) / cluster > kRowPart || rows * cluster > blocks) return 0;
+  while (cluster < kRowCluster && (vpr + cluster - 1) / cluster > part) cluster *= 2;
+  if ((vpr + cluster - 1) / cluster > part || (fits && rows * cluster > (long long)sms * (1024 / threads))) return plan;
   while (cluster < kRowCluster && 2 * cluster * rows <= sms) cluster *= 2;
-  return cluster;
+  plan.cluster = cluster;
+  plan.threads = threads;
+  return plan;
 }
 // The same with Eq. 3's sums.
-inline int row_topm_cluster(int vocab, int elem_bytes, long long rows, int sms, int M) {
+inline RowPlan row_topm_plan(int vocab, int elem_bytes, long long rows, int sms, int M) {
   const int vec = 16 / elem_bytes;
-  if (vocab < kRowThreads * vec || 4 * M > kRowTopmList) return 0;
-  return row_pass_cluster(vocab, elem_bytes, rows, sms, 0x7FFFFFFF);
+  if (vocab < kRowThreads * vec || 4 * M > kRowTopmList) return RowPlan{0, 0};
+  return row_pass_plan(vocab, elem_bytes, rows, sms, false);
 }
 cudaError_t prepare_row_pass();                 // once per device: opt in to the shared-memory size
-cudaError_t launch_expand_rows(const PassParams &p, int dtype, int cluster, cudaStream_t s);
-cudaError_t launch_expand_rows_prune(const PassParams &p, const TreeState &t, int level, const c2t_frontier &out, int dtype, int cluster, cudaStream_t s);
+cudaError_t launch_expand_rows(const PassParams &p, int dtype, RowPlan plan, cudaStream_t s);
+cudaError_t launch_expand_rows_prune(const PassParams &p, const TreeState &t, int level, const c2t_frontier &out, int dtype, RowPlan plan, cudaStream_t s);
 
 cudaError_t prepare_expand_pass();   // once per device: opt in to the kernel's shared-memory size
 cudaError_t launch_expand_pass(PassParams p, int dtype, int grid, cudaStream_t s);

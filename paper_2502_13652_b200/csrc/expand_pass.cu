@@ -946,19 +946,20 @@ cudaError_t prepare_expand_pass() {
   return e;
 }
 
-// The blocks per row of the pass in registers (row_pass.cu), or 0.
-static int rows_in_registers(const PassParams &p, int dtype, int sms) {
+// How the pass in registers (row_pass.cu) takes the level, if it does.
+static RowPlan rows_in_registers(const PassParams &p, int dtype, int sms) {
   const int eb = dtype == C2T_BF16 ? 2 : 4;
   const long long rows = (long long)p.B * p.rows_bound;
-  if (p.topm_out) return row_topm_cluster(p.V, eb, rows, sms, p.topm_m);
-  if (p.topm_pool) return 0;
-  return row_pass_cluster(p.V, eb, rows, sms, sms * kRowBlocksPerSm);
+  if (p.topm_out) return row_topm_plan(p.V, eb, rows, sms, p.topm_m);
+  if (p.topm_pool) return RowPlan{0, 0};
+  return row_pass_plan(p.V, eb, rows, sms, true);
 }
 
 cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, const c2t_frontier *out, int dtype, int grid, cudaStream_t s) {
   c2t_frontier o = {nullptr, nullptr, nullptr, nullptr};
   if (out) o = *out;
-  if (const int cluster = rows_in_registers(p, dtype, grid)) return launch_expand_rows_prune(p, t, level, o, dtype, cluster, s);
+  const RowPlan plan = rows_in_registers(p, dtype, grid);
+  if (plan.cluster) return launch_expand_rows_prune(p, t, level, o, dtype, plan, s);
   size_t smem = plan_shared(p, grid);
   if (smem < sizeof(PruneShared)) smem = sizeof(PruneShared);
   if (dtype == C2T_BF16)
@@ -967,7 +968,8 @@ cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, con
 }
 
 cudaError_t launch_expand_pass(PassParams p, int dtype, int grid, cudaStream_t s) {
-  if (const int cluster = rows_in_registers(p, dtype, grid)) return launch_expand_rows(p, dtype, cluster, s);
+  const RowPlan plan = rows_in_registers(p, dtype, grid);
+  if (plan.cluster) return launch_expand_rows(p, dtype, plan, s);
   const size_t smem = plan_shared(p, grid);
   const bool bf16 = dtype == C2T_BF16;
   if (p.topm_pool) {                                 // also sets the candidates of Eq. 3 aside

@@ -5,47 +5,44 @@
 // Such a level is a chain of latencies, not a stream: its rows arrive in one round of loads, all in flight at once.  A thread holds
 // up to 8 vectors of 16 bytes.  Nothing goes through global memory but the logits and the row's result, nothing is read twice, no row
 // waits for another, and there is no list of rows to build: block (b, j) looks at one count.
-//   Maxima of 64 groups of the row (of eight lanes, or more where the row is spread over a cluster) go to every block of the cluster; the K-th
-// largest of them is a floor that at least K elements reach, and hardly more do.  While they travel the sums are
-// taken, base 2 as in expand_pass.cu, relative to an offset from the warp's largest value but for its very largest, which
-// stays apart with its equals: so the row's maximum can be left out of the sums, which keep fp32 relative accuracy
-// with respect to "everything but the maximum" however peaked the row is.  Then the threads whose maximum reaches the floor hand
-// their elements over, the leading block ranks the keys and merges the warps' sums in double precision, in a fixed order.
+//   Maxima of 64 groups of the row or more go to every block of the cluster; the K-th largest of them is a floor that at least K elements
+// reach, and hardly more do.  While they travel the sums are taken, base 2 as in expand_pass.cu, a lane's relative to an offset from
+// its own largest value.  The row's maximum is left out of them afterwards: the lane that holds it is summed again without it, its
+// elements dealt out to the warp.  So the sums keep fp32 relative accuracy with respect to "everything but the maximum" however peaked the
+// row is.  The threads whose maximum reaches the floor hand their elements over, the leading block ranks the keys and
+// merges the warps' sums in double precision, in a fixed order.
 #include "row_sums.cuh"
 #include "topm_select.cuh"
 
 namespace c2t {
 namespace {
 
-constexpr int kRowWarps = kRowThreads / 32;
+constexpr int kMaxRowWarps = kRowThreads / 32;
 constexpr int kRowLoads = kRowPart / kRowThreads;     // vectors of a thread
-constexpr int kRowGroups = 64;                        // (at least the largest K)
-constexpr int kCtaKeys = 32;                          // keys that a block hands over
+constexpr int kRowGroups = 64;                        // at least (and at least the largest K)
+constexpr int kMaxRowGroups = kRowCluster * kMaxRowWarps;
+constexpr int kCtaKeys = 64;                          // keys that a block hands over
 constexpr int kTooMany = 1 << 20;
-static_assert(kRowGroups >= C2T_MAX_TOPK && kRowGroups == 4 * kRowWarps && kRowGroups * 8 == kRowThreads, "");
+static_assert(kRowGroups >= C2T_MAX_TOPK && kMaxRowGroups >= kRowGroups, "");
 
 struct RowShared {
-  __align__(16) float quarter[kRowGroups];            // this block's maxima over eight lanes each
-  __align__(16) float group[kRowGroups];              // the row's
-  float4 sums[kRowCluster * kRowWarps];               // in the leading block: S, U, offset, largest value of every warp
-  int equals[kRowCluster * kRowWarps];                // elements with that value
-  unsigned long long keys[kRowCluster][kCtaKeys];     // what every block hands over
-  int counts[kRowCluster];
+  __align__(16) float group[kMaxRowGroups];           // the maxima of the row's groups
+  float4 sums[kRowCluster * kMaxRowWarps];            // in the leading block: S, U, offset of every warp, and how often it holds the maximum (int bits)
+  unsigned long long keys[kRowCluster][kCtaKeys];     // in the leading block: what every block hands over
+  __align__(16) int counts[kRowCluster];              // how many
   unsigned long long pool[kPoolCap];                  // this block's keys; in the leading one then the row's
-  unsigned long long best[2][kRowCluster], warp_best[kRowWarps];
+  __align__(16) uint4 again[kMaxRowWarps][kRowLoads]; // per warp: the vectors of a lane that is summed again
+  unsigned long long best[2][kRowCluster], warp_best[kMaxRowWarps];
   unsigned floor;                                     // (orderable)
   int n;
 };
 
 // What the truncated entropy needs besides; behind it the lists of candidates (in the leading block, cut evenly among the blocks).
 struct RowTopmShared {
-  float place[kRowWarps];                             // sums over a warp's groups of eight lanes of their maxima at the place asked for
-  int place_n[kRowWarps];                             // how many there are
-  float floors[kRowCluster];                          // the same of every block
-  int floor_n[kRowCluster];
-  int n, own, counts[kRowCluster];                    // listed by this block; its warps' largest values; listed by every block
+  float2 place[kRowCluster * kMaxRowWarps];           // per warp: the sum over its groups of eight lanes of their maxima at the place asked for; how many
+  int n, counts[kRowCluster];                         // listed by this block; listed by every block
   unsigned need;
-  double sum[2 * kRowWarps];
+  double sum[2 * kMaxRowWarps];
 };
 
 // ---------------------------------------------------------------- clusters
@@ -65,6 +62,7 @@ __device__ __forceinline__ uint32_t place_in(const void *at, int r) {
 }
 __device__ __forceinline__ void put(uint32_t at, uint32_t v) { asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(v) : "memory"); }
 __device__ __forceinline__ void put(uint32_t at, unsigned long long v) { asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(at), "l"(v) : "memory"); }
+__device__ __forceinline__ void put(uint32_t at, float a, float b) { asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(at), "f"(a), "f"(b) : "memory"); }
 __device__ __forceinline__ void put(uint32_t at, float a, float b, float c, float d) {
   asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
@@ -77,23 +75,23 @@ __device__ __forceinline__ float warp_max(float v) {
 
 // ---------------------------------------------------------------- a block's part of a row
 
+template <bool BF16, int NT>
 struct RowPart {
   const char *row;
   int vpr, v_full, part, v0, v1;                      // vectors of the row, whole ones, of a block; this block's range
-  template <bool BF16>
   __device__ __forceinline__ void load(uint4 (&q)[kRowLoads], int V) const {
     const uint32_t lo = BF16 ? kLowestBf16x2 : __float_as_uint(kLowestF32);
     const int whole = v1 < v_full ? v1 : v_full;
 #pragma unroll
     for (int k = 0; k < kRowLoads; ++k) {
-      const int v = v0 + k * kRowThreads + (int)threadIdx.x;
+      const int v = v0 + k * NT + (int)threadIdx.x;
       q[k] = make_uint4(lo, lo, lo, lo);
       if (v < whole) q[k] = ldg_stream(reinterpret_cast<const uint4 *>(row) + v);
     }
     if (v1 > v_full) {                                // (uniform) the row's ragged last vector
 #pragma unroll
       for (int k = 0; k < kRowLoads; ++k)
-        if (v0 + k * kRowThreads + (int)threadIdx.x == v_full) q[k] = load_ragged<BF16>(row, v_full, v_full, V);
+        if (v0 + k * NT + (int)threadIdx.x == v_full) q[k] = load_ragged<BF16>(row, v_full, v_full, V);
     }
 #pragma unroll
     for (int k = 0; k < kRowLoads; ++k) Vec<BF16>::clamp(q[k]);
@@ -115,50 +113,40 @@ __device__ __forceinline__ float element_of(const uint4 &q, int i) {
   return BF16 ? __uint_as_float((i & 1) ? w & 0xFFFF0000u : w << 16) : __uint_as_float(w);
 }
 
-// the word with the elements equal to x replaced by the lowest value
+// The elements of vector v at or above a floor (which padding does not reach) as keys into the block's pool.  The count in shared
+// memory keeps rising when the pool is full.
 template <bool BF16>
-__device__ __forceinline__ uint32_t without(uint32_t w, float x) {
-  if (!BF16) return __uint_as_float(w) == x ? __float_as_uint(kLowestF32) : w;
-  if (__uint_as_float(w << 16) == x) w = (w & 0xFFFF0000u) | (kLowestBf16x2 & 0xFFFFu);
-  if (__uint_as_float(w & 0xFFFF0000u) == x) w = (w & 0xFFFFu) | (kLowestBf16x2 & 0xFFFF0000u);
-  return w;
-}
-
-// The elements of vector v at or above a floor as keys into the block's pool; returns how many there are (tokens past the row's end
-// do not count).  The count in shared memory keeps rising when the pool is full.
-template <bool BF16>
-__device__ __forceinline__ int hand_over(RowShared &sh, const uint4 &q, float floor, int v, int V) {
+__device__ __forceinline__ void hand_over(RowShared &sh, const uint4 &q, float floor, int v) {
   constexpr int N = Vec<BF16>::N;
   int c = 0;
 #pragma unroll
-  for (int i = 0; i < N; ++i) c += element_of<BF16>(q, i) >= floor && v * N + i < V;
+  for (int i = 0; i < N; ++i) c += element_of<BF16>(q, i) >= floor;
   int pos = atomicAdd(&sh.n, c);
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     const float x = element_of<BF16>(q, i);
-    if (x >= floor && v * N + i < V) {
+    if (x >= floor) {
       if (pos < kPoolCap) sh.pool[pos] = make_key(x, (uint32_t)(v * N + i));
       ++pos;
     }
   }
-  return c;
 }
 
 // Rows whose K largest do not come out of a short list (many equal values, few values, most of the row masked, very short rows): K rounds
 // of "the largest key below the last one" over all blocks of the cluster.  Returns the number of keys, in the leading block's pool.
-template <bool BF16>
-__device__ __noinline__ int select_by_rounds(RowShared &sh, const RowPart &rp, int V, int K, int cluster, int rank) {
+template <bool BF16, int NT>
+__device__ __noinline__ int select_by_rounds(RowShared &sh, const RowPart<BF16, NT> &rp, int V, int K, int cluster, int rank) {
   constexpr int N = Vec<BF16>::N;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint4 q[kRowLoads];
-  rp.load<BF16>(q, V);
+  rp.load(q, V);
   unsigned long long last = ~0ull;
   int r = 0;
   for (; r < K; ++r) {
     unsigned long long best = 0ull;
 #pragma unroll
     for (int k = 0; k < kRowLoads; ++k) {
-      const int v = rp.v0 + k * kRowThreads + tid;
+      const int v = rp.v0 + k * NT + tid;
       if (v >= rp.v1) continue;
       float x[N];
       Vec<BF16>::unpack(q[k], x);
@@ -177,7 +165,7 @@ __device__ __noinline__ int select_by_rounds(RowShared &sh, const RowPart &rp, i
     __syncthreads();
     if (warp == 0) {
       best = 0ull;
-      for (int w = 0; w < kRowWarps; ++w) best = sh.warp_best[w] > best ? sh.warp_best[w] : best;
+      for (int w = 0; w < NT / 32; ++w) best = sh.warp_best[w] > best ? sh.warp_best[w] : best;
       if (lane < cluster) put(place_in(&sh.best[r & 1][rank], lane), best);
     }
     __syncwarp();
@@ -190,42 +178,79 @@ __device__ __noinline__ int select_by_rounds(RowShared &sh, const RowPart &rp, i
     last = best;
   }
   __syncthreads();
-  for (int i = r + tid; i < K; i += kRowThreads) sh.pool[i] = 0ull;
+  for (int i = r + tid; i < K; i += NT) sh.pool[i] = 0ull;
   __syncthreads();
   return r;
 }
 
-// The warps' sums, merged by one warp of the leading block.
-__device__ __forceinline__ void merge_sums(RowShared &sh, RowResult *out, int warps) {
-  constexpr int kPer = kRowCluster * kRowWarps / 32;
-  const int lane = threadIdx.x & 31;
-  float4 s[kPer];
-  int eq[kPer];
-  float m = kLowestF32;
+// A warp's sums to its place in the leading block: its lanes' (s, u) relative to their offsets c, m2 the largest values they come from.
+__device__ __forceinline__ void put_sums(RowShared &sh, float s, float u, float c, float m2, int equals, int w, int cluster) {
+  const float cw = offset_of(warp_max(m2)), by = fmaxf(cw - c, -127.f);
+  const float two = __int_as_float((__float_as_int(by + 12582912.f) << 23) + 0x3F800000);      // 2^by, 0 for -127
+  u = two * fmaf(by, s, u);
+  s = two * s;
 #pragma unroll
-  for (int i = 0; i < kPer; ++i) {
-    const int w = i * 32 + lane;
-    if (w < warps) { s[i] = sh.sums[w]; eq[i] = sh.equals[w]; m = fmaxf(m, s[i].w); }
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(kFull, s, o);
+    u += __shfl_xor_sync(kFull, u, o);
   }
-  const float Mf = warp_max(m), cM = offset_of(Mf);
+  if ((threadIdx.x & 31) == 0) {
+    if (cluster > 1) put(place_in(&sh.sums[w], 0), s, u, cw, __int_as_float(equals));
+    else sh.sums[w] = make_float4(s, u, cw, __int_as_float(equals));
+  }
+  __syncwarp();
+}
+
+// The warp that holds the row's maximum Mf: each such lane (mt == Mf) summed again without it and its equals, its words dealt out to the
+// warp's lanes.
+template <bool BF16>
+__device__ __forceinline__ void sum_again(RowShared &sh, const uint4 (&q)[kRowLoads], float mt, float Mf, float s, float u, float c, int w, int cluster) {
+  const int lane = threadIdx.x & 31;
+  int equals = 0;
+  float m2 = mt;
+  for (unsigned left = __ballot_sync(kFull, mt == Mf); left; left &= left - 1u) {
+    const int owner = __ffs(left) - 1;
+    __syncwarp();
+    if (lane == owner) {
+#pragma unroll
+      for (int k = 0; k < kRowLoads; ++k) sh.again[threadIdx.x >> 5][k] = q[k];
+    }
+    __syncwarp();
+    const uint32_t word = reinterpret_cast<const uint32_t *>(sh.again[threadIdx.x >> 5])[lane];
+    float x0 = BF16 ? __uint_as_float(word << 16) : __uint_as_float(word), x1 = BF16 ? __uint_as_float(word & 0xFFFF0000u) : kLowestF32;
+    equals += (x0 == Mf) + (x1 == Mf);
+    x0 = x0 == Mf ? kLowestF32 : x0;
+    x1 = x1 == Mf ? kLowestF32 : x1;
+    const float m = warp_max(fmaxf(x0, x1)), cr = offset_of(m);
+    const float t0 = fmaf(x0, kLog2e, cr), t1 = fmaf(x1, kLog2e, cr), e0 = ex2f(t0), e1 = ex2f(t1);
+    float sr = e0 + e1, ur = fmaf(e0, t0, e1 * t1);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      sr += __shfl_xor_sync(kFull, sr, o);
+      ur += __shfl_xor_sync(kFull, ur, o);
+    }
+    if (lane == owner) { s = sr; u = ur; c = cr; m2 = m; }
+  }
+  equals = __reduce_add_sync(kFull, equals);
+  put_sums(sh, s, u, c, m2, equals, w, cluster);
+}
+
+// The warps' sums, merged by one warp of the leading block.
+__device__ __forceinline__ void merge_sums(RowShared &sh, RowResult *out, float Mf, int warps) {
+  constexpr int kPer = kRowCluster * kMaxRowWarps / 32;
+  const int lane = threadIdx.x & 31;
+  const float cM = offset_of(Mf);
   double S = 0.0, U = 0.0;
   int equals = 0;
 #pragma unroll
   for (int i = 0; i < kPer; ++i) {
     if (i * 32 + lane < warps) {
-      float d = fmaxf(cM - s[i].z, -2000.f);          // (never positive)
-      double f = pow2_f64(d);
-      S += f * (double)s[i].x;
-      U += f * ((double)s[i].y + (double)d * (double)s[i].x);
-      if (s[i].w == Mf) {
-        equals += eq[i];
-      } else {                                        // the warp's largest value is an ordinary element of the row
-        const float c = offset_of(s[i].w), t = fmaf(s[i].w, kLog2e, c), e = (float)eq[i] * ex2f(t);
-        d = fmaxf(cM - c, -2000.f);
-        f = pow2_f64(d);
-        S += f * (double)e;
-        U += f * (double)e * ((double)t + (double)d);
-      }
+      const float4 r = sh.sums[i * 32 + lane];
+      const float d = fmaxf(cM - r.z, -2000.f);       // (never positive)
+      const double f = pow2_f64(d);
+      S += f * (double)r.x;
+      U += f * ((double)r.y + (double)d * (double)r.x);
+      equals += __float_as_int(r.w);
     }
   }
   S = warp_sum(S);
@@ -239,8 +264,8 @@ __device__ __forceinline__ void merge_sums(RowShared &sh, RowResult *out, int wa
 // The floor of Eq. 3's candidates: the place-th largest of the thread maxima among eight lanes, averaged over the groups of the row.  The
 // place (topm_lane_place) is the one that about 1.5 to 2.5 M elements reach; the average has little scatter, and it does not matter
 // where in the row the large elements lie.  Here a warp's sum of them.
-__device__ __forceinline__ void place_sums(RowTopmShared &ts, float mt, int place) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ float2 place_sums(float mt, int place) {
+  const int lane = threadIdx.x & 31;
   int above = 0;
 #pragma unroll
   for (int o = 1; o < 8; ++o) {
@@ -251,8 +276,7 @@ __device__ __forceinline__ void place_sums(RowTopmShared &ts, float mt, int plac
   float v = here ? mt : 0.f;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-  const int n = __popc(__ballot_sync(kFull, here));
-  if (lane == 0) { ts.place[warp] = v; ts.place_n[warp] = n; }
+  return make_float2(v, (float)__popc(__ballot_sync(kFull, here)));
 }
 
 // The elements of this block's part at or above the floor, as keys into its part of the leading block's list.
@@ -297,6 +321,7 @@ __device__ __forceinline__ void list_candidates(RowTopmShared &ts, uint32_t list
 }
 
 // the keys of the blocks' lists, dealt out to the leading block's threads
+template <int NT>
 struct ListedKeys {
   const uint32_t *list;
   const int *counts;
@@ -304,23 +329,24 @@ struct ListedKeys {
   template <typename F>
   __device__ __forceinline__ void operator()(F f) const {
     for (int r = 0; r < cluster; ++r)
-      for (int i = threadIdx.x; i < counts[r]; i += kRowThreads) f(list[r * cap + i]);
+      for (int i = threadIdx.x; i < counts[r]; i += NT) f(list[r * cap + i]);
   }
 };
 
 // ---------------------------------------------------------------- a row
 
 // Row (b, j) by the blocks of a cluster.  True in the leading block, after the row's result is written (by its first two warps).
-template <bool BF16, bool TOPM>
+template <bool BF16, bool TOPM, int NT>
 __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, int b, int j, int cluster, int rank, RowTopmShared *ts, uint32_t *s_list) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, K = p.K;
+  constexpr int kW = NT / 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, K = p.K, warps = cluster * kW;
   if (tid == 0) {
     sh.floor = 0u;
     sh.n = 0;
-    if (TOPM) ts->n = ts->own = 0;
+    if (TOPM) ts->n = 0;
   }
   if (cluster > 1) cluster_arrive();                  // (a block's shared memory can be written once the block runs)
-  RowPart rp;
+  RowPart<BF16, NT> rp;
   rp.vpr = (p.V + Vec<BF16>::N - 1) / Vec<BF16>::N;
   rp.v_full = p.V / Vec<BF16>::N;
   rp.part = (rp.vpr + cluster - 1) / cluster;
@@ -328,189 +354,129 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
   rp.v1 = rp.v0 + rp.part < rp.vpr ? rp.v0 + rp.part : rp.vpr;
   rp.row = reinterpret_cast<const char *>(p.logits) + ((size_t)b * p.seq_stride + (size_t)j * p.row_stride) * (BF16 ? 2 : 4);
   uint4 q[kRowLoads];
-  rp.load<BF16>(q, p.V);
+  rp.load(q, p.V);
 
-  // ---- maxima: the thread's, of eight lanes, the warp's; the row's groups to every block
+  // ---- maxima: the thread's, and those of groups of `width` lanes to every block, one of them from each lane of the group
   RunMax<BF16> run;
   run.clear();
 #pragma unroll
   for (int k = 0; k < kRowLoads; ++k) run.take(q[k]);
-  const float mt = run.value(), wm = warp_max(mt);
+  const float mt = run.value();
+  const int groups = warps > kRowGroups ? warps : kRowGroups, width = 32 * warps / groups;
   float g = mt;
-#pragma unroll
-  for (int o = 1; o < 8; o <<= 1) g = fmaxf(g, __shfl_xor_sync(kFull, g, o));
-  if (TOPM) place_sums(*ts, mt, p.topm_place);
-  if ((lane & 7) == 0) (cluster > 1 ? sh.quarter : sh.group)[warp * 4 + (lane >> 3)] = g;
-  __syncthreads();
+  for (int o = 1; o < width; o <<= 1) g = fmaxf(g, __shfl_xor_sync(kFull, g, o));
+  const float2 place = TOPM ? place_sums(mt, p.topm_place) : make_float2(0.f, 0.f);
+  const int to = lane & (width - 1), at = (rank * kW + warp) * (32 / width) + lane / width;
   if (cluster > 1) {
     cluster_wait();
-    const int per = kRowGroups / cluster;
-    if (warp < cluster && lane < per) {
-      float v = kLowestF32;
-      for (int i = 0; i < cluster; ++i) v = fmaxf(v, sh.quarter[lane * cluster + i]);
-      put(place_in(&sh.group[rank * per + lane], warp), __float_as_uint(v));
-    }
-  }
-  if (TOPM && warp == kRowWarps - 1) {
-    float v = lane < kRowWarps ? ts->place[lane] : 0.f;
-    int n = lane < kRowWarps ? ts->place_n[lane] : 0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    n = __reduce_add_sync(kFull, n);
-    if (lane < cluster) {
-      put(place_in(&ts->floors[rank], lane), __float_as_uint(v));
-      put(place_in(&ts->floor_n[rank], lane), (uint32_t)n);
-    }
-  }
-  if (cluster > 1) {
+    if (to < cluster) put(place_in(&sh.group[at], to), __float_as_uint(g));
+    if (TOPM && lane < cluster) put(place_in(&ts->place[rank * kW + warp], lane), place.x, place.y);
     __syncwarp();
     cluster_arrive();
+  } else {
+    if (to == 0) sh.group[at] = g;
+    if (TOPM && lane == 0) ts->place[warp] = place;
   }
 
-  // ---- the warp's largest value and its equals apart, the sums of everything else
-  float m2 = mt;
-  int equals = 0;
-  if (mt == wm) {
-    unsigned hit = 0u;
-#pragma unroll
-    for (int k = 0; k < kRowLoads; ++k) hit |= (unsigned)(Vec<BF16>::vmax(q[k]) == wm) << k;
-    while (hit) {
-      const int at = __ffs(hit) - 1, v = rp.v0 + at * kRowThreads + tid;
-      hit &= hit - 1u;
-      uint4 t = pick(q, at);
-      if (v < rp.v1) equals += hand_over<BF16>(sh, t, wm, v, p.V);
-      t.x = without<BF16>(t.x, wm); t.y = without<BF16>(t.y, wm); t.z = without<BF16>(t.z, wm); t.w = without<BF16>(t.w, wm);
-#pragma unroll
-      for (int k = 0; k < kRowLoads; ++k)
-        if (k == at) q[k] = t;
-    }
-    run.clear();
-#pragma unroll
-    for (int k = 0; k < kRowLoads; ++k) run.take(q[k]);
-    m2 = run.value();
-  }
-  __syncwarp();
+  // ---- the sums
+  const float c = offset_of(mt);
+  float s, u;
   {
-    const float c = offset_of(warp_max(m2));
     const f32x2 scale = pack2(kLog2e, kLog2e), c2 = pack2(c, c);
     Acc acc;
     acc.clear();
 #pragma unroll
     for (int k = 0; k < kRowLoads; ++k)
-      if (k * kRowThreads < rp.part) acc_vector<BF16>(acc, q[k], scale, c2);      // (uniform)
-    float s, u;
+      if (k * NT < rp.part) acc_vector<BF16>(acc, q[k], scale, c2);      // (uniform)
     acc.totals(s, u);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s += __shfl_xor_sync(kFull, s, o);
-      u += __shfl_xor_sync(kFull, u, o);
-    }
-    equals = __reduce_add_sync(kFull, equals);
-    if (lane == 0) {
-      const int w = rank * kRowWarps + warp;
-      if (TOPM) atomicAdd(&ts->own, equals);
-      if (cluster > 1) {
-        put(place_in(&sh.sums[w], 0), s, u, c, wm);
-        put(place_in(&sh.equals[w], 0), (uint32_t)equals);
-      } else {
-        sh.sums[w] = make_float4(s, u, c, wm);
-        sh.equals[w] = equals;
-      }
-    }
-    __syncwarp();
   }
-
+  put_sums(sh, s, u, c, mt, 0, rank * kW + warp, cluster);
   if (cluster > 1) cluster_wait();
+  else __syncthreads();
+
+  // ---- the row's maximum, which stays out of them; the floor: the K-th largest of the groups' maxima, the largest value that K of them reach
+  float Mf = fmaxf(sh.group[lane], sh.group[32 + lane]);
+  if (groups > 64) Mf = fmaxf(Mf, fmaxf(sh.group[64 + lane], sh.group[96 + lane]));
+  Mf = warp_max(Mf);
+  if (__any_sync(kFull, mt == Mf)) sum_again<BF16>(sh, q, mt, Mf, s, u, c, rank * kW + warp, cluster);
+  {
+    const int team = NT / groups, member = tid & (team - 1);      // threads of a group: 2 to 8
+    const float mine = sh.group[tid / team];
+    int reach = 0;
+    for (int i = member * 4; i < groups; i += team * 4) {
+      const float4 o = *reinterpret_cast<const float4 *>(&sh.group[i]);
+      reach += (o.x >= mine) + (o.y >= mine) + (o.z >= mine) + (o.w >= mine);
+    }
+    for (int o = 1; o < team; o <<= 1) reach += __shfl_xor_sync(kFull, reach, o);
+    const unsigned top = __reduce_max_sync(kFull, reach >= K ? f32_orderable(__float_as_uint(mine)) : 0u);
+    if (lane == 0 && top) atomicMax(&sh.floor, top);
+  }
   float floor_m = 0.f;
   const int cap = TOPM ? kRowTopmList / cluster : 0;
   if (TOPM) {
-    if (cluster == 1) __syncthreads();
-    float v = 0.f;
-    int n = 0;
-    for (int r = 0; r < cluster; ++r) { v += ts->floors[r]; n += ts->floor_n[r]; }
-    floor_m = fmaxf(v / (float)(n > 0 ? n : 1), kTopmLowestFloor);    // (the same in every block; NaN: nothing is listed)
-    list_candidates<BF16>(*ts, place_in(s_list + rank * cap, 0), cap, q, floor_m);
-  }
-
-  // ---- the floor: the K-th largest of the groups' maxima, the largest value that K of them reach; eight threads per group
-  {
-    const float mine = sh.group[tid >> 3];
-    const float4 o0 = *reinterpret_cast<const float4 *>(&sh.group[(tid & 7) * 8]), o1 = *reinterpret_cast<const float4 *>(&sh.group[(tid & 7) * 8 + 4]);
-    int reach = (o0.x >= mine) + (o0.y >= mine) + (o0.z >= mine) + (o0.w >= mine) + (o1.x >= mine) + (o1.y >= mine) + (o1.z >= mine) + (o1.w >= mine);
+    float v = 0.f, n = 0.f;
+    for (int i = lane; i < warps; i += 32) { v += ts->place[i].x; n += ts->place[i].y; }
 #pragma unroll
-    for (int o = 1; o < 8; o <<= 1) reach += __shfl_xor_sync(kFull, reach, o);
-    const unsigned top = __reduce_max_sync(kFull, reach >= K ? f32_orderable(__float_as_uint(mine)) : 0u);
-    if (lane == 0 && top) atomicMax(&sh.floor, top);
+    for (int o = 16; o > 0; o >>= 1) {
+      v += __shfl_xor_sync(kFull, v, o);
+      n += __shfl_xor_sync(kFull, n, o);
+    }
+    floor_m = fmaxf(v / fmaxf(n, 1.f), kTopmLowestFloor);             // (the same in every warp; NaN: nothing is listed)
+    list_candidates<BF16>(*ts, place_in(s_list + rank * cap, 0), cap, q, floor_m);
   }
   __syncthreads();
   const float floor = __uint_as_float(f32_from_orderable(sh.floor));
   const bool live = floor > kLowestF32;               // (uniform; else fewer than K groups have data)
 
-  // ---- the elements that reach it (the warps' largest values are in the pool already)
-  if (live && m2 >= floor) {
+  // ---- the elements that reach it
+  if (live && mt >= floor) {
     unsigned hit = 0u;
 #pragma unroll
     for (int k = 0; k < kRowLoads; ++k) hit |= (unsigned)(Vec<BF16>::vmax(q[k]) >= floor) << k;
     while (hit) {
-      const int at = __ffs(hit) - 1;
+      const int k = __ffs(hit) - 1;
       hit &= hit - 1u;
-      hand_over<BF16>(sh, pick(q, at), floor, rp.v0 + at * kRowThreads + tid, p.V);
+      hand_over<BF16>(sh, pick(q, k), floor, rp.v0 + k * NT + tid);
     }
   }
   __syncthreads();
   if (warp == 0) {
-    const int n = sh.n;
-    int c = 0;
-    if (TOPM) {                                       // (the warps' largest values, the first in the pool, are in no list yet)
-      const int at = ts->n;
-      int more = 0;
-      for (int i0 = 0; i0 < n && n <= kPoolCap; i0 += 32) {
-        const bool in = i0 + lane < ts->own && key_value(sh.pool[i0 + lane]) >= floor_m;
-        const unsigned mask = __ballot_sync(kFull, in);
-        const int pos = at + more + __popc(mask & ((1u << lane) - 1u));
-        if (in && pos < cap) put(place_in(s_list + rank * cap + pos, 0), (uint32_t)(sh.pool[i0 + lane] >> 32));
-        more += __popc(mask);
-      }
-      if (lane == 0) put(place_in(&ts->counts[rank], 0), n > kPoolCap || at + more > cap ? (uint32_t)kTooMany : (uint32_t)(at + more));
-    }
-    if (!live || n > kPoolCap) {
-      c = kTooMany;
-    } else {
-      for (int i0 = 0; i0 < n; i0 += 32) {
-        const unsigned long long key = i0 + lane < n ? sh.pool[i0 + lane] : 0ull;
-        const bool in = key != 0ull && key_value(key) >= floor;
-        const unsigned mask = __ballot_sync(kFull, in);
-        const int pos = c + __popc(mask & ((1u << lane) - 1u));
-        if (in && pos < kCtaKeys) {
-          if (cluster > 1) put(place_in(&sh.keys[rank][pos], 0), key);
-          else sh.keys[0][pos] = key;
-        }
-        c += __popc(mask);
-      }
+    const int n = sh.n, c_n = !live || n > kCtaKeys ? kTooMany : n;
+    for (int i = lane; i < c_n && c_n != kTooMany; i += 32) {
+      const unsigned long long key = sh.pool[i];
+      if (cluster > 1) put(place_in(&sh.keys[rank][i], 0), key);
+      else sh.keys[0][i] = key;
     }
     if (lane < cluster) {
-      if (cluster > 1) put(place_in(&sh.counts[rank], lane), (uint32_t)c);
-      else sh.counts[0] = c;
+      if (cluster > 1) put(place_in(&sh.counts[rank], lane), (uint32_t)c_n);
+      else sh.counts[0] = c_n;
     }
+    if (TOPM && lane == 0) put(place_in(&ts->counts[rank], 0), ts->n > cap ? (uint32_t)kTooMany : (uint32_t)ts->n);
     __syncwarp();
   }
   if (cluster > 1) { cluster_arrive(); cluster_wait(); }
   else __syncthreads();
 
   // ---- the row's result
-  int total = 0, most = 0;
-  for (int r = 0; r < cluster; ++r) { total += sh.counts[r]; most = sh.counts[r] > most ? sh.counts[r] : most; }
-  const bool listed = most <= kCtaKeys && total <= kPoolCap;      // (the same in every block)
+  int upto[kRowCluster], total = 0;                   // keys up to and with block r
+#pragma unroll
+  for (int r = 0; r < kRowCluster; ++r) {
+    if (r < cluster) total += sh.counts[r];
+    upto[r] = total;
+  }
+  const bool listed = total <= kPoolCap;              // (the same in every block)
   int n_valid = 0;
-  if (!listed) n_valid = select_by_rounds<BF16>(sh, rp, p.V, K, cluster, rank);
+  if (!listed) n_valid = select_by_rounds<BF16, NT>(sh, rp, p.V, K, cluster, rank);
   if (rank != 0) return false;
   const size_t slot = (size_t)b * p.rows_per_seq_max + j;
   if (warp == 0) {
     if (listed) {
-      for (int r = 0, at = 0; r < cluster; ++r) {
-        const int c = sh.counts[r];
-        if (lane < c) sh.pool[at + lane] = sh.keys[r][lane];
-        at += c;
+      for (int i = lane; i < total; i += 32) {
+        int r = 0, before = 0;
+#pragma unroll
+        for (int k = 0; k < kRowCluster; ++k)
+          if (upto[k] <= i) { r = k + 1; before = upto[k]; }
+        sh.pool[i] = sh.keys[r][i - before];
       }
       __syncwarp();
       n_valid = rank_pool(sh.pool, total, K);
@@ -521,7 +487,7 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
       p.rows[slot].n_valid = n_valid;
     }
   } else if (warp == 1) {
-    merge_sums(sh, p.rows + slot, cluster * kRowWarps);
+    merge_sums(sh, p.rows + slot, Mf, warps);
   }
   if (TOPM) {
     __syncthreads();                                  // (the row's largest key)
@@ -530,9 +496,9 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
     const unsigned long long top = sh.pool[0];
     const bool served = n_c >= p.topm_m && n_c < kTooMany && top != 0ull && key_value(top) < INFINITY;
     if (served) {
-      const ListedKeys listed_keys = {s_list, ts->counts, cluster, cap};
-      select_and_sum<BF16, kRowThreads>(listed_keys, p.topm_m, key_value(top), f32_orderable(__float_as_uint(floor_m)), (uint32_t)(top >> 32), ts->sum,
-                                        &ts->need, &p.topm_out[slot]);
+      const ListedKeys<NT> listed_keys = {s_list, ts->counts, cluster, cap};
+      select_and_sum<BF16, NT>(listed_keys, p.topm_m, key_value(top), f32_orderable(__float_as_uint(floor_m)), (uint32_t)(top >> 32), ts->sum,
+                               &ts->need, &p.topm_out[slot]);
     }
     if (tid == 0) p.topm_done[slot] = served;
   }
@@ -542,35 +508,35 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
 // ---------------------------------------------------------------- kernels
 
 // Block x = (row slot, place in the cluster), y = sequence.
-template <bool BF16, bool TOPM>
-__global__ void __launch_bounds__(kRowThreads, 2) expand_rows_kernel(const __grid_constant__ PassParams p, int cluster) {
+template <bool BF16, bool TOPM, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) expand_rows_kernel(const __grid_constant__ PassParams p, int cluster) {
   __shared__ RowShared sh;
   extern __shared__ __align__(16) unsigned char s_topm[];
   chain_enter();
   const int b = blockIdx.y, j = (int)blockIdx.x / cluster;
   if (j >= p.counts[b]) return;
-  expand_row<BF16, TOPM>(p, sh, b, j, cluster, cluster > 1 ? cluster_rank() : 0, reinterpret_cast<RowTopmShared *>(s_topm),
+  expand_row<BF16, TOPM, NT>(p, sh, b, j, cluster, cluster > 1 ? cluster_rank() : 0, reinterpret_cast<RowTopmShared *>(s_topm),
                          reinterpret_cast<uint32_t *>(s_topm + sizeof(RowTopmShared)));
 }
 
 // Expand and prune of a level in one launch, for small batches: the cluster that finishes a sequence's last row (a count, nobody
 // waits) does the sequence's part of c2t_prune.
-template <bool BF16>
-__global__ void __launch_bounds__(kRowThreads, 1) expand_rows_prune_kernel(const __grid_constant__ PassParams p, const __grid_constant__ TreeState t,
+template <bool BF16, int NT>
+__global__ void __launch_bounds__(NT, 512 / NT) expand_rows_prune_kernel(const __grid_constant__ PassParams p, const __grid_constant__ TreeState t,
                                                                            int level, c2t_frontier out, int cluster) {
   __shared__ union { RowShared row; PruneShared prune; } sh;
   __shared__ double s_w[kWCount];
   __shared__ int s_last;
   const int rank = cluster > 1 ? cluster_rank() : 0;
   chain_release();
-  if (rank == 0) stage_classifier(t, s_w, threadIdx.x, kRowThreads);           // (written at init)
+  if (rank == 0) stage_classifier(t, s_w, threadIdx.x, NT);           // (written at init)
   chain_wait();
   const int b = blockIdx.y, j = (int)blockIdx.x / cluster;
   int n = p.counts[b];
   n = n < p.rows_per_seq_max ? n : p.rows_per_seq_max;
   if (j >= n && !(n <= 0 && j == 0)) return;
   if (n > 0) {
-    if (!expand_row<BF16, false>(p, sh.row, b, j, cluster, rank, nullptr, nullptr)) return;
+    if (!expand_row<BF16, false, NT>(p, sh.row, b, j, cluster, rank, nullptr, nullptr)) return;
     __syncthreads();                                 // the row's result, before its count
     if (threadIdx.x == 0) {
       int done;                                      // released: this row's result; acquired: those of the rows before it
@@ -582,16 +548,16 @@ __global__ void __launch_bounds__(kRowThreads, 1) expand_rows_prune_kernel(const
   } else if (rank != 0) {
     return;
   }
-  prune_level_body<kRowThreads>(t, level, out, nullptr, 0, b, sh.prune, s_w, nullptr);
+  prune_level_body<NT>(t, level, out, nullptr, 0, b, sh.prune, s_w, nullptr);
 }
 
 constexpr size_t kRowTopmBytes = sizeof(RowTopmShared) + kRowTopmList * sizeof(uint32_t);
 
 template <typename... KArgs, typename... Args>
-cudaError_t launch_rows(void (*kernel)(KArgs...), dim3 grid, int cluster, size_t smem, cudaStream_t s, Args &&...args) {
+cudaError_t launch_rows(void (*kernel)(KArgs...), dim3 grid, int threads, int cluster, size_t smem, cudaStream_t s, Args &&...args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(kRowThreads);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
@@ -608,9 +574,9 @@ cudaError_t launch_rows(void (*kernel)(KArgs...), dim3 grid, int cluster, size_t
 // The place among eight thread maxima (1 the largest) whose average value 1.5 to 2.5 M of the row's elements reach: of n elements each, a
 // share 1 - (1 - s)^n of the threads holds one of the row's share s of largest elements, and the k-th largest of eight lies at the
 // share k / 9 on average.
-int topm_lane_place(int vocab, int vec, int M, int cluster) {
+int topm_lane_place(int vocab, int vec, int M, int cluster, int threads) {
   const int vpr = (vocab + vec - 1) / vec, part = (vpr + cluster - 1) / cluster;
-  const double n = (double)vocab / cluster / (part < kRowThreads ? part : kRowThreads), s = 1.5 * M / vocab;
+  const double n = (double)vocab / cluster / (part < threads ? part : threads), s = 1.5 * M / vocab;
   const int k = s >= 1.0 ? 8 : (int)ceil(9.0 * (1.0 - pow(1.0 - s, n)));
   return k > 8 ? 8 : k;
 }
@@ -618,26 +584,35 @@ int topm_lane_place(int vocab, int vec, int M, int cluster) {
 }  // namespace
 
 cudaError_t prepare_row_pass() {
-  const cudaError_t e = cudaFuncSetAttribute(expand_rows_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowTopmBytes);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(expand_rows_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowTopmBytes);
+  const int bytes = (int)kRowTopmBytes;
+  cudaError_t e = cudaFuncSetAttribute(expand_rows_kernel<true, true, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_rows_kernel<false, true, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_rows_kernel<true, true, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_rows_kernel<false, true, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  return e;
 }
 
-cudaError_t launch_expand_rows(const PassParams &params, int dtype, int cluster, cudaStream_t s) {
+template <int NT>
+static cudaError_t launch_rows_nt(const PassParams &p, bool bf16, int cluster, cudaStream_t s) {
+  const dim3 grid(p.rows_bound * cluster, p.B);
+  if (p.topm_out)
+    return launch_rows(bf16 ? expand_rows_kernel<true, true, NT> : expand_rows_kernel<false, true, NT>, grid, NT, cluster, kRowTopmBytes, s, p, cluster);
+  return launch_rows(bf16 ? expand_rows_kernel<true, false, NT> : expand_rows_kernel<false, false, NT>, grid, NT, cluster, 0, s, p, cluster);
+}
+
+cudaError_t launch_expand_rows(const PassParams &params, int dtype, RowPlan plan, cudaStream_t s) {
   PassParams p = params;
-  const dim3 grid(p.rows_bound * cluster, p.B);
   const bool bf16 = dtype == C2T_BF16;
-  if (p.topm_out) {
-    p.topm_place = topm_lane_place(p.V, bf16 ? 8 : 4, p.topm_m, cluster);
-    return launch_rows(bf16 ? expand_rows_kernel<true, true> : expand_rows_kernel<false, true>, grid, cluster, kRowTopmBytes, s, p, cluster);
-  }
-  return launch_rows(bf16 ? expand_rows_kernel<true, false> : expand_rows_kernel<false, false>, grid, cluster, 0, s, p, cluster);
+  if (p.topm_out) p.topm_place = topm_lane_place(p.V, bf16 ? 8 : 4, p.topm_m, plan.cluster, plan.threads);
+  return plan.threads == 256 ? launch_rows_nt<256>(p, bf16, plan.cluster, s) : launch_rows_nt<512>(p, bf16, plan.cluster, s);
 }
 
-cudaError_t launch_expand_rows_prune(const PassParams &p, const TreeState &t, int level, const c2t_frontier &out, int dtype, int cluster, cudaStream_t s) {
-  const dim3 grid(p.rows_bound * cluster, p.B);
-  if (dtype == C2T_BF16) return launch_rows(expand_rows_prune_kernel<true>, grid, cluster, 0, s, p, t, level, out, cluster);
-  return launch_rows(expand_rows_prune_kernel<false>, grid, cluster, 0, s, p, t, level, out, cluster);
+cudaError_t launch_expand_rows_prune(const PassParams &p, const TreeState &t, int level, const c2t_frontier &out, int dtype, RowPlan plan, cudaStream_t s) {
+  const dim3 grid(p.rows_bound * plan.cluster, p.B);
+  const bool bf16 = dtype == C2T_BF16;
+  if (plan.threads == 256)
+    return launch_rows(bf16 ? expand_rows_prune_kernel<true, 256> : expand_rows_prune_kernel<false, 256>, grid, 256, plan.cluster, 0, s, p, t, level, out, plan.cluster);
+  return launch_rows(bf16 ? expand_rows_prune_kernel<true, 512> : expand_rows_prune_kernel<false, 512>, grid, 512, plan.cluster, 0, s, p, t, level, out, plan.cluster);
 }
 
 }  // namespace c2t
