@@ -351,20 +351,18 @@ int c2t_expand_level(c2t_ctx *ctx, int level, const void *logits_dev, int64_t se
   PassParams p = expand_params(t, level, logits_dev, seq_stride, row_stride, t.V);
   const bool truncated = t.entropy_top_m > 0 && t.entropy_top_m < t.V;   // Eq. 3: the sums over the M most probable tokens
   const bool set_aside = truncated && t.topm_place > 0;
-  const bool in_pass = set_aside && row_topm_plan(t.V, (int)ctx->elem_bytes, (long long)t.B * p.rows_bound, ctx->grid_expand, t.entropy_top_m).cluster > 0;
-  if (in_pass) { p.topm_out = t.topm; p.topm_done = t.topm_done; p.topm_m = t.entropy_top_m; }
-  else if (set_aside) { p.topm_pool = t.topm_pool; p.topm_pool_vecs = t.topm_pool_vecs; p.topm_seg = t.topm_seg; p.topm_place = t.topm_place; }
+  if (set_aside) { p.topm_pool = t.topm_pool; p.topm_pool_vecs = t.topm_pool_vecs; p.topm_seg = t.topm_seg; p.topm_place = t.topm_place; }
   if (launch_expand_pass(p, ctx->cfg.dtype, ctx->grid_expand, (cudaStream_t)stream) != cudaSuccess)
     return C2T_ECUDA;
   ctx->launches += 1;
   if (truncated) {
     // from the vectors the pass set aside; then, for the rows where those did not suffice, from the rows themselves
-    if (set_aside && !in_pass && launch_topm_finish(t.entropy_top_m, t.F, t.B, p.counts, t, t.topm, ctx->cfg.dtype, (cudaStream_t)stream) != cudaSuccess)
+    if (set_aside && launch_topm_finish(t.entropy_top_m, t.F, t.B, p.counts, t, t.topm, ctx->cfg.dtype, (cudaStream_t)stream) != cudaSuccess)
       return C2T_ECUDA;
     if (launch_topm_entropy(logits_dev, seq_stride, row_stride, t.V, t.entropy_top_m, t.F, t.B, p.counts, t, t.topm,
                             t.topm_done, ctx->grid_expand, ctx->cfg.dtype, (cudaStream_t)stream) != cudaSuccess)
       return C2T_ECUDA;
-    ctx->launches += set_aside && !in_pass ? 2 : 1;
+    ctx->launches += set_aside ? 2 : 1;
   }
   ctx->expanded = 1;
   return C2T_OK;

@@ -148,10 +148,6 @@ struct PassParams {
   long long topm_pool_vecs;
   int32_t topm_place;               // the floor's place among the lane maxima (topm_floor_place)
   TopmSegment *topm_seg;            // [warp + row]
-  // expand with M > 0 and the rows in registers (else null): Eq. 3's sums and which rows have them, [B, F]
-  double2 *topm_out;
-  int32_t *topm_done;
-  int32_t topm_m;
   // argmax: [B, rows_per_seq_max] best key per row, the largest of what is there and of the row's keys (0 before the pass;
   // the kernel that reads a key puts the 0 back)
   unsigned long long *best;
@@ -185,7 +181,6 @@ int row_chunks(int vocab, int elem_bytes);   // chunks of a row of the expand pa
 constexpr int kRowThreads = 512;                // threads of a block at most (or half as many)
 constexpr int kRowPart = kRowThreads * 8;       // 16-byte vectors of a row that a block of so many holds
 constexpr int kRowCluster = 8;                  // blocks of a row at most
-constexpr int kRowTopmList = 12288;             // keys of a row's candidates for Eq. 3, cut evenly among its blocks
 struct RowPlan {
   int cluster, threads;                         // blocks per row (0: the level is not for that pass), threads of a block
 };
@@ -200,27 +195,20 @@ extern "C" int c2t_debug_task_wait_limit;       // tests let the wait run out: t
 #define C2T_TASK_WAIT_LIMIT kTaskWaitLimit
 #endif
 
-// How a level is cut, if all its rows fit the chip at once (or fits is false): the smaller blocks where a row fits eight of them.
-inline RowPlan row_pass_plan(int vocab, int elem_bytes, long long rows, int sms, bool fits) {
+// How a level is cut, if its rows leave an SM no more than 512 threads of them: the smaller blocks where a row fits eight of them.
+inline RowPlan row_pass_plan(int vocab, int elem_bytes, long long rows, int sms) {
   RowPlan plan = {0, 0};
   if (C2T_TASK_WAIT_LIMIT != kTaskWaitLimit) return plan;
   const int vec = 16 / elem_bytes, vpr = (vocab + vec - 1) / vec;
   const int threads = vpr <= kRowCluster * kRowPart / 2 ? kRowThreads / 2 : kRowThreads, part = threads * 8;
   int cluster = 1;
   while (cluster < kRowCluster && (vpr + cluster - 1) / cluster > part) cluster *= 2;
-  if ((vpr + cluster - 1) / cluster > part || (fits && rows * cluster > (long long)sms * (1024 / threads))) return plan;
+  if ((vpr + cluster - 1) / cluster > part || rows * cluster > (long long)sms * (kRowThreads / threads)) return plan;
   while (cluster < kRowCluster && 2 * cluster * rows <= sms) cluster *= 2;
   plan.cluster = cluster;
   plan.threads = threads;
   return plan;
 }
-// The same with Eq. 3's sums.
-inline RowPlan row_topm_plan(int vocab, int elem_bytes, long long rows, int sms, int M) {
-  const int vec = 16 / elem_bytes;
-  if (vocab < kRowThreads * vec || 4 * M > kRowTopmList) return RowPlan{0, 0};
-  return row_pass_plan(vocab, elem_bytes, rows, sms, false);
-}
-cudaError_t prepare_row_pass();                 // once per device: opt in to the shared-memory size
 cudaError_t launch_expand_rows(const PassParams &p, int dtype, RowPlan plan, cudaStream_t s);
 cudaError_t launch_expand_rows_prune(const PassParams &p, const TreeState &t, int level, const c2t_frontier &out, int dtype, RowPlan plan, cudaStream_t s);
 

@@ -934,8 +934,6 @@ static size_t plan_shared(PassParams &p, int grid) {
 }
 
 cudaError_t prepare_expand_pass() {
-  const cudaError_t r = prepare_row_pass();
-  if (r != cudaSuccess) return r;
   const int bytes = 100 * 1024;                      // more than plan_shared asks for at the limits of a configuration
   cudaError_t e = cudaFuncSetAttribute(expand_pass_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_pass_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -948,11 +946,8 @@ cudaError_t prepare_expand_pass() {
 
 // How the pass in registers (row_pass.cu) takes the level, if it does.
 static RowPlan rows_in_registers(const PassParams &p, int dtype, int sms) {
-  const int eb = dtype == C2T_BF16 ? 2 : 4;
-  const long long rows = (long long)p.B * p.rows_bound;
-  if (p.topm_out) return row_topm_plan(p.V, eb, rows, sms, p.topm_m);
   if (p.topm_pool) return RowPlan{0, 0};
-  return row_pass_plan(p.V, eb, rows, sms, true);
+  return row_pass_plan(p.V, dtype == C2T_BF16 ? 2 : 4, (long long)p.B * p.rows_bound, sms);
 }
 
 cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, const c2t_frontier *out, int dtype, int grid, cudaStream_t s) {

@@ -1,6 +1,6 @@
 // The expand pass for levels of few rows: every row in the registers of one thread block, or of a cluster of up to eight, per row
 // the softmax normaliser and entropy sums and the K largest logits (ties to the lower token id), as expand_pass.cu leaves them
-//                                                        (Sec. 4.2.1, Eq. 2, Eq. 3, Sec. 4.2.2).
+//                                                        (Sec. 4.2.1, Eq. 2, Sec. 4.2.2).
 //
 // Such a level is a chain of latencies, not a stream: its rows arrive in one round of loads, all in flight at once.  A thread holds
 // up to 8 vectors of 16 bytes.  Nothing goes through global memory but the logits and the row's result, nothing is read twice, no row
@@ -12,7 +12,6 @@
 // row is.  The threads whose maximum reaches the floor hand their elements over, the leading block ranks the keys and
 // merges the warps' sums in double precision, in a fixed order.
 #include "row_sums.cuh"
-#include "topm_select.cuh"
 
 namespace c2t {
 namespace {
@@ -37,14 +36,6 @@ struct RowShared {
   int n;
 };
 
-// What the truncated entropy needs besides; behind it the lists of candidates (in the leading block, cut evenly among the blocks).
-struct RowTopmShared {
-  float2 place[kRowCluster * kMaxRowWarps];           // per warp: the sum over its groups of eight lanes of their maxima at the place asked for; how many
-  int n, counts[kRowCluster];                         // listed by this block; listed by every block
-  unsigned need;
-  double sum[2 * kMaxRowWarps];
-};
-
 // ---------------------------------------------------------------- clusters
 
 __device__ __forceinline__ int cluster_rank() {
@@ -62,7 +53,6 @@ __device__ __forceinline__ uint32_t place_in(const void *at, int r) {
 }
 __device__ __forceinline__ void put(uint32_t at, uint32_t v) { asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(v) : "memory"); }
 __device__ __forceinline__ void put(uint32_t at, unsigned long long v) { asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(at), "l"(v) : "memory"); }
-__device__ __forceinline__ void put(uint32_t at, float a, float b) { asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(at), "f"(a), "f"(b) : "memory"); }
 __device__ __forceinline__ void put(uint32_t at, float a, float b, float c, float d) {
   asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
@@ -259,91 +249,16 @@ __device__ __forceinline__ void merge_sums(RowShared &sh, RowResult *out, float 
   if (lane == 0) write_sums(out, Mf, cM, S, U, equals);
 }
 
-// ---------------------------------------------------------------- truncated entropy (Eq. 3)
-
-// The floor of Eq. 3's candidates: the place-th largest of the thread maxima among eight lanes, averaged over the groups of the row.  The
-// place (topm_lane_place) is the one that about 1.5 to 2.5 M elements reach; the average has little scatter, and it does not matter
-// where in the row the large elements lie.  Here a warp's sum of them.
-__device__ __forceinline__ float2 place_sums(float mt, int place) {
-  const int lane = threadIdx.x & 31;
-  int above = 0;
-#pragma unroll
-  for (int o = 1; o < 8; ++o) {
-    const float other = __shfl_xor_sync(kFull, mt, o);
-    above += other > mt || (other == mt && (lane ^ o) < lane);
-  }
-  const bool here = above == place - 1 && mt > kTopmLowestFloor;
-  float v = here ? mt : 0.f;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-  return make_float2(v, (float)__popc(__ballot_sync(kFull, here)));
-}
-
-// The elements of this block's part at or above the floor, as keys into its part of the leading block's list.
-template <bool BF16>
-__device__ __forceinline__ void list_candidates(RowTopmShared &ts, uint32_t list, int cap, const uint4 (&q)[kRowLoads], float floor) {
-  constexpr int N = Vec<BF16>::N;
-  const int lane = threadIdx.x & 31;
-  uint32_t c = 0u;                                    // per vector four bits
-  int mine = 0;
-#pragma unroll
-  for (int k = 0; k < kRowLoads; ++k) {
-    int n = 0;
-#pragma unroll
-    for (int i = 0; i < N; ++i) n += element_of<BF16>(q[k], i) >= floor;
-    c |= (uint32_t)n << (4 * k);
-    mine += n;
-  }
-  int upto = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(kFull, upto, o);
-    if (lane >= o) upto += v;
-  }
-  int base = 0;
-  if (lane == 31) base = atomicAdd(&ts.n, upto);
-  int pos = __shfl_sync(kFull, base, 31) + upto - mine;
-#pragma unroll
-  for (int k = 0; k < kRowLoads; ++k) {
-    const int n = (c >> (4 * k)) & 15u;
-    if (n == 1) {                                     // (nearly always: the vector's maximum)
-      if (pos < cap) put(list + 4 * pos, f32_orderable(__float_as_uint(Vec<BF16>::vmax(q[k]))));
-      ++pos;
-    } else if (n > 1) {
-#pragma unroll
-      for (int i = 0; i < N; ++i)
-        if (element_of<BF16>(q[k], i) >= floor) {
-          if (pos < cap) put(list + 4 * pos, f32_orderable(__float_as_uint(element_of<BF16>(q[k], i))));
-          ++pos;
-        }
-    }
-  }
-}
-
-// the keys of the blocks' lists, dealt out to the leading block's threads
-template <int NT>
-struct ListedKeys {
-  const uint32_t *list;
-  const int *counts;
-  int cluster, cap;
-  template <typename F>
-  __device__ __forceinline__ void operator()(F f) const {
-    for (int r = 0; r < cluster; ++r)
-      for (int i = threadIdx.x; i < counts[r]; i += NT) f(list[r * cap + i]);
-  }
-};
-
 // ---------------------------------------------------------------- a row
 
 // Row (b, j) by the blocks of a cluster.  True in the leading block, after the row's result is written (by its first two warps).
-template <bool BF16, bool TOPM, int NT>
-__device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, int b, int j, int cluster, int rank, RowTopmShared *ts, uint32_t *s_list) {
+template <bool BF16, int NT>
+__device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, int b, int j, int cluster, int rank) {
   constexpr int kW = NT / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, K = p.K, warps = cluster * kW;
   if (tid == 0) {
     sh.floor = 0u;
     sh.n = 0;
-    if (TOPM) ts->n = 0;
   }
   if (cluster > 1) cluster_arrive();                  // (a block's shared memory can be written once the block runs)
   RowPart<BF16, NT> rp;
@@ -365,17 +280,14 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
   const int groups = warps > kRowGroups ? warps : kRowGroups, width = 32 * warps / groups;
   float g = mt;
   for (int o = 1; o < width; o <<= 1) g = fmaxf(g, __shfl_xor_sync(kFull, g, o));
-  const float2 place = TOPM ? place_sums(mt, p.topm_place) : make_float2(0.f, 0.f);
   const int to = lane & (width - 1), at = (rank * kW + warp) * (32 / width) + lane / width;
   if (cluster > 1) {
     cluster_wait();
     if (to < cluster) put(place_in(&sh.group[at], to), __float_as_uint(g));
-    if (TOPM && lane < cluster) put(place_in(&ts->place[rank * kW + warp], lane), place.x, place.y);
     __syncwarp();
     cluster_arrive();
-  } else {
-    if (to == 0) sh.group[at] = g;
-    if (TOPM && lane == 0) ts->place[warp] = place;
+  } else if (to == 0) {
+    sh.group[at] = g;
   }
 
   // ---- the sums
@@ -411,19 +323,6 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
     const unsigned top = __reduce_max_sync(kFull, reach >= K ? f32_orderable(__float_as_uint(mine)) : 0u);
     if (lane == 0 && top) atomicMax(&sh.floor, top);
   }
-  float floor_m = 0.f;
-  const int cap = TOPM ? kRowTopmList / cluster : 0;
-  if (TOPM) {
-    float v = 0.f, n = 0.f;
-    for (int i = lane; i < warps; i += 32) { v += ts->place[i].x; n += ts->place[i].y; }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      v += __shfl_xor_sync(kFull, v, o);
-      n += __shfl_xor_sync(kFull, n, o);
-    }
-    floor_m = fmaxf(v / fmaxf(n, 1.f), kTopmLowestFloor);             // (the same in every warp; NaN: nothing is listed)
-    list_candidates<BF16>(*ts, place_in(s_list + rank * cap, 0), cap, q, floor_m);
-  }
   __syncthreads();
   const float floor = __uint_as_float(f32_from_orderable(sh.floor));
   const bool live = floor > kLowestF32;               // (uniform; else fewer than K groups have data)
@@ -451,7 +350,6 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
       if (cluster > 1) put(place_in(&sh.counts[rank], lane), (uint32_t)c_n);
       else sh.counts[0] = c_n;
     }
-    if (TOPM && lane == 0) put(place_in(&ts->counts[rank], 0), ts->n > cap ? (uint32_t)kTooMany : (uint32_t)ts->n);
     __syncwarp();
   }
   if (cluster > 1) { cluster_arrive(); cluster_wait(); }
@@ -489,34 +387,19 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
   } else if (warp == 1) {
     merge_sums(sh, p.rows + slot, Mf, warps);
   }
-  if (TOPM) {
-    __syncthreads();                                  // (the row's largest key)
-    int n_c = 0;
-    for (int r = 0; r < cluster; ++r) n_c += ts->counts[r];
-    const unsigned long long top = sh.pool[0];
-    const bool served = n_c >= p.topm_m && n_c < kTooMany && top != 0ull && key_value(top) < INFINITY;
-    if (served) {
-      const ListedKeys<NT> listed_keys = {s_list, ts->counts, cluster, cap};
-      select_and_sum<BF16, NT>(listed_keys, p.topm_m, key_value(top), f32_orderable(__float_as_uint(floor_m)), (uint32_t)(top >> 32), ts->sum,
-                               &ts->need, &p.topm_out[slot]);
-    }
-    if (tid == 0) p.topm_done[slot] = served;
-  }
   return true;
 }
 
 // ---------------------------------------------------------------- kernels
 
 // Block x = (row slot, place in the cluster), y = sequence.
-template <bool BF16, bool TOPM, int NT>
+template <bool BF16, int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT) expand_rows_kernel(const __grid_constant__ PassParams p, int cluster) {
   __shared__ RowShared sh;
-  extern __shared__ __align__(16) unsigned char s_topm[];
   chain_enter();
   const int b = blockIdx.y, j = (int)blockIdx.x / cluster;
   if (j >= p.counts[b]) return;
-  expand_row<BF16, TOPM, NT>(p, sh, b, j, cluster, cluster > 1 ? cluster_rank() : 0, reinterpret_cast<RowTopmShared *>(s_topm),
-                         reinterpret_cast<uint32_t *>(s_topm + sizeof(RowTopmShared)));
+  expand_row<BF16, NT>(p, sh, b, j, cluster, cluster > 1 ? cluster_rank() : 0);
 }
 
 // Expand and prune of a level in one launch, for small batches: the cluster that finishes a sequence's last row (a count, nobody
@@ -536,7 +419,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) expand_rows_prune_kernel(const _
   n = n < p.rows_per_seq_max ? n : p.rows_per_seq_max;
   if (j >= n && !(n <= 0 && j == 0)) return;
   if (n > 0) {
-    if (!expand_row<BF16, false, NT>(p, sh.row, b, j, cluster, rank, nullptr, nullptr)) return;
+    if (!expand_row<BF16, NT>(p, sh.row, b, j, cluster, rank)) return;
     __syncthreads();                                 // the row's result, before its count
     if (threadIdx.x == 0) {
       int done;                                      // released: this row's result; acquired: those of the rows before it
@@ -551,14 +434,11 @@ __global__ void __launch_bounds__(NT, 512 / NT) expand_rows_prune_kernel(const _
   prune_level_body<NT>(t, level, out, nullptr, 0, b, sh.prune, s_w, nullptr);
 }
 
-constexpr size_t kRowTopmBytes = sizeof(RowTopmShared) + kRowTopmList * sizeof(uint32_t);
-
 template <typename... KArgs, typename... Args>
-cudaError_t launch_rows(void (*kernel)(KArgs...), dim3 grid, int threads, int cluster, size_t smem, cudaStream_t s, Args &&...args) {
+cudaError_t launch_rows(void (*kernel)(KArgs...), dim3 grid, int threads, int cluster, cudaStream_t s, Args &&...args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -571,48 +451,21 @@ cudaError_t launch_rows(void (*kernel)(KArgs...), dim3 grid, int threads, int cl
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
-// The place among eight thread maxima (1 the largest) whose average value 1.5 to 2.5 M of the row's elements reach: of n elements each, a
-// share 1 - (1 - s)^n of the threads holds one of the row's share s of largest elements, and the k-th largest of eight lies at the
-// share k / 9 on average.
-int topm_lane_place(int vocab, int vec, int M, int cluster, int threads) {
-  const int vpr = (vocab + vec - 1) / vec, part = (vpr + cluster - 1) / cluster;
-  const double n = (double)vocab / cluster / (part < threads ? part : threads), s = 1.5 * M / vocab;
-  const int k = s >= 1.0 ? 8 : (int)ceil(9.0 * (1.0 - pow(1.0 - s, n)));
-  return k > 8 ? 8 : k;
-}
-
 }  // namespace
 
-cudaError_t prepare_row_pass() {
-  const int bytes = (int)kRowTopmBytes;
-  cudaError_t e = cudaFuncSetAttribute(expand_rows_kernel<true, true, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_rows_kernel<false, true, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_rows_kernel<true, true, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_rows_kernel<false, true, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  return e;
-}
-
-template <int NT>
-static cudaError_t launch_rows_nt(const PassParams &p, bool bf16, int cluster, cudaStream_t s) {
-  const dim3 grid(p.rows_bound * cluster, p.B);
-  if (p.topm_out)
-    return launch_rows(bf16 ? expand_rows_kernel<true, true, NT> : expand_rows_kernel<false, true, NT>, grid, NT, cluster, kRowTopmBytes, s, p, cluster);
-  return launch_rows(bf16 ? expand_rows_kernel<true, false, NT> : expand_rows_kernel<false, false, NT>, grid, NT, cluster, 0, s, p, cluster);
-}
-
-cudaError_t launch_expand_rows(const PassParams &params, int dtype, RowPlan plan, cudaStream_t s) {
-  PassParams p = params;
+cudaError_t launch_expand_rows(const PassParams &p, int dtype, RowPlan plan, cudaStream_t s) {
+  const dim3 grid(p.rows_bound * plan.cluster, p.B);
   const bool bf16 = dtype == C2T_BF16;
-  if (p.topm_out) p.topm_place = topm_lane_place(p.V, bf16 ? 8 : 4, p.topm_m, plan.cluster, plan.threads);
-  return plan.threads == 256 ? launch_rows_nt<256>(p, bf16, plan.cluster, s) : launch_rows_nt<512>(p, bf16, plan.cluster, s);
+  if (plan.threads == 256) return launch_rows(bf16 ? expand_rows_kernel<true, 256> : expand_rows_kernel<false, 256>, grid, 256, plan.cluster, s, p, plan.cluster);
+  return launch_rows(bf16 ? expand_rows_kernel<true, 512> : expand_rows_kernel<false, 512>, grid, 512, plan.cluster, s, p, plan.cluster);
 }
 
 cudaError_t launch_expand_rows_prune(const PassParams &p, const TreeState &t, int level, const c2t_frontier &out, int dtype, RowPlan plan, cudaStream_t s) {
   const dim3 grid(p.rows_bound * plan.cluster, p.B);
   const bool bf16 = dtype == C2T_BF16;
   if (plan.threads == 256)
-    return launch_rows(bf16 ? expand_rows_prune_kernel<true, 256> : expand_rows_prune_kernel<false, 256>, grid, 256, plan.cluster, 0, s, p, t, level, out, plan.cluster);
-  return launch_rows(bf16 ? expand_rows_prune_kernel<true, 512> : expand_rows_prune_kernel<false, 512>, grid, 512, plan.cluster, 0, s, p, t, level, out, plan.cluster);
+    return launch_rows(bf16 ? expand_rows_prune_kernel<true, 256> : expand_rows_prune_kernel<false, 256>, grid, 256, plan.cluster, s, p, t, level, out, plan.cluster);
+  return launch_rows(bf16 ? expand_rows_prune_kernel<true, 512> : expand_rows_prune_kernel<false, 512>, grid, 512, plan.cluster, s, p, t, level, out, plan.cluster);
 }
 
 }  // namespace c2t

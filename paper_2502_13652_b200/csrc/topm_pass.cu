@@ -17,7 +17,7 @@
 // those.  General path (neither served): a radix select over the row in up to five sweeps (the row stays in L2); the top
 // byte is counted in registers from the maximum's bin downwards, the later bytes with a 256-bin
 // histogram in shared memory over the elements that still match.
-#include "topm_select.cuh"
+#include "vocab_common.cuh"
 
 namespace c2t {
 namespace {
@@ -99,6 +99,112 @@ __device__ __forceinline__ void push_candidates(const uint4 &q, float floor, uin
     }
 }
 
+// Eq. 3's sums from a candidate set in shared memory that is known to hold the M largest elements of the row
+// (n_c >= M keys, the order-preserving images of the values): the M-th largest key, then the terms above it and as
+// many copies of the term at it as are still missing.  Called by all NT threads of the CTA; thread 0 writes the
+// result.
+//   The candidates lie close together (between a floor and the row maximum), so a histogram over fixed key bytes
+// would put nearly all of them in one bin, one shared-memory atomic after the other.  The bins follow the data
+// instead: kSelBins equal steps between the smallest and the largest key still in play, refined until a step is
+// one key wide (one round for bf16 rows as a rule, two or three for fp32).
+constexpr int kSelBins = 2048;
+
+// key_lo, key_hi: keys that bound the set from below and from above (the floor it was collected with, the row maximum).
+template <bool BF16, int NT>
+__device__ __forceinline__ void select_and_sum(const uint32_t *s_cand, unsigned n_c, int M, float mf, uint32_t key_lo,
+                                               uint32_t key_hi, double *s_sum, unsigned *s_need, double2 *out) {
+  __shared__ unsigned s_bins[kSelBins];
+  __shared__ unsigned s_wsum[NT / 32], s_lo, s_hi;
+  __shared__ double s_tail[2];
+  constexpr int BPT = kSelBins / NT;               // bins a thread owns when the bin with the M-th largest is looked for
+  static_assert(kSelBins % NT == 0, "whole bins per thread");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int KS = BF16 ? 16 : 0;                // bf16 images are told apart by their upper halves
+  if (key_lo == 0x80000000u) key_lo = 0x7FFFFFFFu; // a floor of +0 also admits -0, whose key is one lower
+  if (tid == 0) { s_lo = key_lo >> KS; s_hi = key_hi >> KS; *s_need = (unsigned)M; }
+  __syncthreads();
+  // ---- refine [lo, hi] around the M-th largest key
+  for (int round = 0; round < 4; ++round) {          // (32 key bits, 11 per round: three at most)
+    const uint32_t lo = s_lo, hi = s_hi;
+    const unsigned need = *s_need;
+    if (lo == hi) break;                             // (uniform) one key left: `need` copies of it are still missing
+    const uint32_t range = hi - lo;
+    const int shift = range < (uint32_t)kSelBins ? 0 : 32 - __clz(range) - 11;     // range >> shift < kSelBins
+    for (int i = tid; i < kSelBins; i += NT) s_bins[i] = 0u;
+    __syncthreads();
+    for (unsigned i = tid; i < n_c; i += NT) {
+      const uint32_t k = s_cand[i] >> KS;
+      if (k >= lo && k <= hi) atomicAdd(&s_bins[(k - lo) >> shift], 1u);
+    }
+    __syncthreads();
+    // the bin, from the top, that holds the need-th largest: thread t owns bins [t BPT, (t + 1) BPT)
+    unsigned h[BPT], mine = 0u;
+#pragma unroll
+    for (int i = 0; i < BPT; ++i) { h[i] = s_bins[tid * BPT + i]; mine += h[i]; }
+    unsigned suf = mine;                             // inclusive suffix sum over the lanes of the warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned v = __shfl_down_sync(kFull, suf, o);
+      if (lane + o < 32) suf += v;
+    }
+    if (lane == 0) s_wsum[warp] = suf;
+    __syncthreads();
+    unsigned higher = suf - mine;                    // keys in the bins of higher threads
+    for (int w = warp + 1; w < NT / 32; ++w) higher += s_wsum[w];
+    if (higher < need && higher + mine >= need) {    // exactly one thread (at least `need` keys are in play)
+      unsigned acc = higher;
+      int d = tid * BPT;
+#pragma unroll
+      for (int i = BPT - 1; i >= 0; --i) {
+        if (acc + h[i] >= need) { d = tid * BPT + i; break; }
+        acc += h[i];
+      }
+      const uint32_t new_lo = lo + ((uint32_t)d << shift);
+      const uint32_t step_top = new_lo + ((1u << shift) - 1u);
+      s_lo = new_lo;
+      s_hi = step_top < hi ? step_top : hi;
+      *s_need = need - acc;
+    }
+    __syncthreads();
+    if (shift == 0) break;                           // (uniform) the bin was one key
+  }
+  // keys above tau are all taken; of the keys equal to tau, *s_need are
+  const uint32_t tau = s_lo;
+  double Sd = 0.0, Td = 0.0;
+  for (unsigned i = tid; i < n_c; i += NT) {
+    const uint32_t key = s_cand[i];
+    if ((key >> KS) > tau) {
+      const float d = __uint_as_float(f32_from_orderable(key)) - mf;
+      const float e = ex2f(d * kLog2e);            // (the expand pass takes its exponentials the same way)
+      Sd += (double)e;
+      Td += (double)(e * d);
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    Sd += __shfl_xor_sync(kFull, Sd, o);
+    Td += __shfl_xor_sync(kFull, Td, o);
+  }
+  if (lane == 0) { s_sum[warp] = Sd; s_sum[NT / 32 + warp] = Td; }
+  if (tid == NT - 1) {                               // meanwhile: the term at tau (its double-precision exp is long)
+    // the key's value (a bf16 image's lower half is all ones for a negative value)
+    const uint32_t tk = BF16 ? (tau << 16) | ((tau >> 15) ? 0u : 0xFFFFu) : tau;
+    const double d = (double)__uint_as_float(f32_from_orderable(tk)) - (double)mf;
+    const double e = exp(d);
+    s_tail[0] = e;
+    s_tail[1] = e * d;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    double St = 0.0, Tt = 0.0;
+    for (int w = 0; w < NT / 32; ++w) { St += s_sum[w]; Tt += s_sum[NT / 32 + w]; }
+    const unsigned need = *s_need;
+    St += (double)need * s_tail[0];
+    Tt += (double)need * s_tail[1];
+    *out = make_double2(St, Tt);
+  }
+}
+
 // One row, by all threads of a CTA (s_cand: kTopmCand keys of the fast path).
 template <bool BF16>
 __device__ __forceinline__ void topm_entropy_row(const void *logits, long long seq_stride, long long row_stride, int V,
@@ -154,7 +260,7 @@ __device__ __forceinline__ void topm_entropy_row(const void *logits, long long s
       __syncthreads();
       const unsigned n_c = s_win[1];
       if (n_c >= (unsigned)M && n_c <= (unsigned)kTopmCand) {                     // (uniform)
-        select_and_sum<BF16, kTopmThreads>(flat_keys<kTopmThreads>(s_cand, n_c), M, mf, f32_orderable(__float_as_uint(floor1)), top_key, s_sum, &s_need,
+        select_and_sum<BF16, kTopmThreads>(s_cand, n_c, M, mf, f32_orderable(__float_as_uint(floor1)), top_key, s_sum, &s_need,
                                            &out[(size_t)b * F + j]);
         return;
       }
@@ -608,7 +714,7 @@ __global__ void __launch_bounds__(kFinishThreads) topm_finish_kernel(int M, int 
     __syncthreads();
     const unsigned n_c = s_count;
     if (n_multi <= (unsigned)kFinishMulti && n_c >= (unsigned)M && n_c <= (unsigned)kFinishCand) {
-      select_and_sum<BF16, kFinishThreads>(flat_keys<kFinishThreads>(s_cand, n_c), M, mf, f32_orderable(__float_as_uint(floor)), (uint32_t)(s_top >> 32),
+      select_and_sum<BF16, kFinishThreads>(s_cand, n_c, M, mf, f32_orderable(__float_as_uint(floor)), (uint32_t)(s_top >> 32),
                                            s_sum, &s_need, &out[(size_t)b * F + j]);
       if (tid == 0) col.done[(size_t)b * F + j] = 1;
       return;
