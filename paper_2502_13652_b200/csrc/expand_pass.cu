@@ -874,7 +874,7 @@ __global__ void __launch_bounds__(kExpandThreads, 1) expand_prune_kernel(const _
                                                                          c2t_frontier out) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
   __shared__ unsigned s_ticket;
-  __shared__ double s_w[kWCount];
+  __shared__ __align__(16) double s_w[kWCount];
   if (threadIdx.x >= kStreamWarps * 32) stage_classifier(t, s_w, threadIdx.x - kStreamWarps * 32, kExpandThreads - kStreamWarps * 32);   // (written at init)
   chain_enter();
   expand_pass_body<BF16, false>(p, s_dyn);

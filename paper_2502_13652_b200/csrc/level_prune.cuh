@@ -21,7 +21,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 
 // The classifier's weights in shared memory, as doubles (a conversion per use costs more than the arithmetic): per hidden
 // unit its three input weights, its bias, its output weight; w[kW0] is the output bias.
-constexpr int kWStride = 6;
+constexpr int kWStride = 6;                       // (16-byte loads)
 constexpr int kW0 = kWStride * C2T_MAX_HIDDEN;
 constexpr int kWCount = kW0 + 2;
 __device__ __forceinline__ void stage_classifier(const TreeState &t, double *w, int tid, int n_threads) {
@@ -36,15 +36,16 @@ __device__ __forceinline__ void stage_classifier(const TreeState &t, double *w, 
 
 // Confidence of one child (Eq. 4): two-layer FFN on (P, H, d), ReLU, sigmoid.
 __device__ __forceinline__ double classify(int hidden, const double *w, double P, double H, double d) {
-  double z = w[kW0];
+  double z0 = w[kW0], z1 = 0.0;                     // (two chains of additions)
 #pragma unroll 4
   for (int k = 0; k < hidden; ++k) {
-    const double *u = w + k * kWStride;
-    double a = u[3] + u[0] * P + u[1] * H + u[2] * d;
+    const double2 a01 = *reinterpret_cast<const double2 *>(w + k * kWStride), a23 = *reinterpret_cast<const double2 *>(w + k * kWStride + 2);
+    double a = a23.y + a01.x * P + a01.y * H + a23.x * d;
     if (a < 0.0) a = 0.0;
-    z += u[4] * a;
+    if (k & 1) z1 += w[k * kWStride + 4] * a;
+    else z0 += w[k * kWStride + 4] * a;
   }
-  return 1.0 / (1.0 + exp(-z));
+  return 1.0 / (1.0 + exp(-(z0 + z1)));
 }
 
 // A row's merged sums, as one warp holds them.
@@ -137,8 +138,9 @@ struct PruneShared {
   int fnode[C2T_MAX_FRONTIER];                 // tree id of every frontier node
   int rowfault[C2T_MAX_FRONTIER];
   alignas(16) unsigned long long ckey[kMaxCand + 8];   // confidence of every candidate as an orderable integer, 0 for a dropped one
+  alignas(16) unsigned chi[kMaxCand + 32];      // its upper half, zeros behind the last one
   int count[32];                               // candidates added and selected, per 32
-  short before[kMaxCand];                      // survivors that come before a candidate
+  short before[kMaxCand];                      // survivors that come before a candidate (itself among them, where the upper halves decide)
 };
 // ... and with gathered records, behind it:
 struct GatherShared {
@@ -173,6 +175,7 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
   const int K = t.K, F = t.F;
   const int cur = level & 1, nxt = cur ^ 1;
   const size_t cbase = (size_t)b * F * K, fbase = (size_t)b * F;
+  const unsigned per_k = (65536u + (unsigned)K - 1u) / (unsigned)K;       // c / K = c per_k >> 16 for c < 1024, K <= 32
 
   // ---- loads (slots past the frontier's size hold anything: kept in bounds, unused)
   int n = t.frontier_n[cur][b];
@@ -242,8 +245,9 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
     keep[r] = false;
     if (r * NT < nc) {                            // (uniform)
       if (c >= nc && c < nc + 8) sh.ckey[c] = 0ull;
+      if (tid < 32) sh.chi[nc + tid] = 0u;
       if (c < nc) {
-        const int j = c / K;
+        const int j = (int)((unsigned)c * per_k >> 16);
         float x;
         if (records) { x = gs->x[c]; tok[r] = gs->tok[c]; }
         else { x = key[r] ? key_value(key[r]) : -INFINITY; tok[r] = key[r] ? key_token(key[r]) : -1; }
@@ -260,6 +264,7 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
         // (C desc, index asc) as integer compares: an orderable image of C, 0 for a dropped candidate
         const unsigned long long cb = (unsigned long long)__double_as_longlong(C[r]);
         sh.ckey[c] = keep[r] ? (cb ^ ((cb >> 63) ? ~0ull : 0x8000000000000000ull)) : 0ull;
+        sh.chi[c] = (unsigned)(sh.ckey[c] >> 32);
         t.cand_token[cbase + c] = tok[r];
         t.cand_lp[cbase + c] = ok ? lp : NAN;
         t.cand_logP[cbase + c] = ok ? logP[r] : NAN;
@@ -271,14 +276,51 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
     sel[r] = keep[r];
   }
 
-  // ---- second pruning: the F survivors that come first under (C desc, index asc); four threads count what comes before a
-  // candidate, two keys to a load (a warp per candidate with a warp-wide sum each took 1.5 us for 128 candidates, this 0.9)
+  // ---- second pruning: the F survivors that come first under (C desc, index asc).  One to eight threads count what comes before a
+  // candidate, first by the upper halves of the keys alone, four to a load: where that leaves F candidates they are the ones.  Else
+  // some are equal in it around the cut, and the whole keys decide (below).  (By whole keys at once 0.9 us for 128 candidates.)
   if (n_keep > F) {
-    for (int c0 = 0; c0 < nc; c0 += NT / 4) {
+    int lg = 3;
+    while (lg > 0 && (nc << lg) > NT) --lg;
+    const int part = tid & ((1 << lg) - 1);
+    for (int c0 = 0; c0 < nc; c0 += NT >> lg) {
+      const int c = c0 + (tid >> lg);
+      const unsigned kc = c < nc ? sh.chi[c] : 0xFFFFFFFFu;
+      int reach = 0;                                // candidates at or above it, itself among them
+#pragma unroll 4
+      for (int o = 4 * part; o < nc; o += 4 << lg) {
+        const uint4 k = *reinterpret_cast<const uint4 *>(&sh.chi[o]);
+        reach += (k.x >= kc) + (k.y >= kc) + (k.z >= kc) + (k.w >= kc);
+      }
+      for (int m = 1; m < 1 << lg; m <<= 1) reach += __shfl_xor_sync(kFullMask, reach, m);
+      if (part == 0 && c < nc) sh.before[c] = (short)reach;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r)
+      if (tid + r * NT < nc) sel[r] = keep[r] && sh.before[tid + r * NT] <= F;
+  }
+
+  // ---- stable compaction in candidate order; append to the tree, emit the frontier
+  const bool add_all = t.tree_add == C2T_ADD_ALL_SURVIVORS;
+  unsigned add_mask[kRounds], sel_mask[kRounds];
+  auto count_up = [&] {
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) {
+      add_mask[r] = __ballot_sync(kFullMask, add_all ? keep[r] : sel[r]);
+      sel_mask[r] = __ballot_sync(kFullMask, sel[r]);
+      if (lane == 0) sh.count[r * kNW + warp] = __popc(add_mask[r]) | (__popc(sel_mask[r]) << 16);    // (each total at most 1024)
+    }
+    __syncthreads();
+    return sh.count[lane];
+  };
+  int counts = count_up(), total = __reduce_add_sync(kFullMask, counts);
+  if (n_keep > F && (total >> 16) != F) {           // (uniform)
+    for (int c0 = 0; c0 < nc; c0 += NT / 4) {       // four threads to a candidate, two keys to a load
       const int c = c0 + (tid >> 2);
       const unsigned long long kc = c < nc ? sh.ckey[c] : 0ull, kc1 = kc + 1ull;      // (a key is never all ones)
       int before = 0;
-#pragma unroll 8
+#pragma unroll 4
       for (int o = 2 * (tid & 3); o < nc; o += 8) {                                   // (zeros behind the last key)
         const ulonglong2 k = *reinterpret_cast<const ulonglong2 *>(&sh.ckey[o]);
         before += k.x >= (o < c ? kc : kc1);
@@ -292,21 +334,10 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
 #pragma unroll
     for (int r = 0; r < kRounds; ++r)
       if (tid + r * NT < nc) sel[r] = keep[r] && sh.before[tid + r * NT] < F;
-  }
-
-  // ---- stable compaction in candidate order; append to the tree, emit the frontier
-  const bool add_all = t.tree_add == C2T_ADD_ALL_SURVIVORS;
-  unsigned add_mask[kRounds], sel_mask[kRounds];
-#pragma unroll
-  for (int r = 0; r < kRounds; ++r) {
-    add_mask[r] = __ballot_sync(kFullMask, add_all ? keep[r] : sel[r]);
-    sel_mask[r] = __ballot_sync(kFullMask, sel[r]);
-    if (lane == 0) sh.count[r * kNW + warp] = __popc(add_mask[r]) | (__popc(sel_mask[r]) << 16);    // (each total at most 1024)
+    counts = count_up();
+    total = __reduce_add_sync(kFullMask, counts);
   }
   static_assert(kRounds * kNW == 32, "a count per lane");
-  __syncthreads();
-  const int counts = sh.count[lane];
-  const int total = __reduce_add_sync(kFullMask, counts);
   const int tot_add = total & 0xFFFF, tot_sel = total >> 16;
   const bool overflow = base + tot_add > t.cap;
   const size_t tb = (size_t)b * t.cap;
@@ -320,7 +351,7 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
     if (!(add_all ? keep[r] : sel[r])) continue;
     const unsigned lt = (1u << lane) - 1u;
     const int id = base + (before & 0xFFFF) + __popc(add_mask[r] & lt);
-    const int j = c / K;
+    const int j = (int)((unsigned)c * per_k >> 16);
     const double chat = C[r] < sh.fchat[j] ? C[r] : sh.fchat[j];
     if (id < t.cap) {
       t.tree_token[tb + id] = tok[r];

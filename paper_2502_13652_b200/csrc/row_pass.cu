@@ -408,7 +408,7 @@ template <bool BF16, int NT>
 __global__ void __launch_bounds__(NT, 512 / NT) expand_rows_prune_kernel(const __grid_constant__ PassParams p, const __grid_constant__ TreeState t,
                                                                            int level, c2t_frontier out, int cluster) {
   __shared__ union { RowShared row; PruneShared prune; } sh;
-  __shared__ double s_w[kWCount];
+  __shared__ __align__(16) double s_w[kWCount];
   __shared__ int s_last;
   const int rank = cluster > 1 ? cluster_rank() : 0;
   chain_release();

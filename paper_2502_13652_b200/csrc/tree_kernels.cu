@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(kExportWarps * 32) export_rows_kernel(TreeStat
 __global__ void __launch_bounds__(kTreeThreads) prune_level_kernel(TreeState t, int level, c2t_frontier out,
                                                                    const c2t_row_record *records, int n_shards) {
   extern __shared__ __align__(16) unsigned char s_prune[];
-  __shared__ double s_w[kWCount];
+  __shared__ __align__(16) double s_w[kWCount];
   PruneShared &sh = *reinterpret_cast<PruneShared *>(s_prune);
   GatherShared *gs = reinterpret_cast<GatherShared *>(s_prune + sizeof(PruneShared));
   chain_release();
@@ -91,6 +91,8 @@ __global__ void __launch_bounds__(kTreeThreads) final_prune_kernel(TreeState t) 
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const size_t tb = (size_t)b * t.cap, fb = (size_t)b * t.Nw;
   int n = t.tree_n[b];
+  int token = 0, level = 0;                                    // of node tid
+  if (tid < t.cap) { token = t.tree_token[tb + tid]; level = t.tree_level[tb + tid]; }
   for (int i = tid; i < t.cap; i += kTreeThreads) {            // (past n: anything, unused)
     const unsigned long long cb = (unsigned long long)__double_as_longlong(t.tree_Chat[tb + i]);
     s_score[i] = cb ^ ((cb >> 63) ? ~0ull : 0x8000000000000000ull);
@@ -179,9 +181,9 @@ __global__ void __launch_bounds__(kTreeThreads) final_prune_kernel(TreeState t) 
     if (m < 0 || m >= t.Nw) continue;
     const int par = s_parent[i];
     t.final_src[fb + m] = i;
-    t.final_token[fb + m] = t.tree_token[tb + i];
+    t.final_token[fb + m] = i == tid ? token : t.tree_token[tb + i];
     t.final_parent[fb + m] = par < 0 ? -1 : s_remap[par];
-    t.final_level[fb + m] = t.tree_level[tb + i];
+    t.final_level[fb + m] = i == tid ? level : t.tree_level[tb + i];
   }
   for (int m = n_final + tid; m < t.Nw; m += kTreeThreads) {
     t.final_src[fb + m] = -1;
@@ -285,6 +287,8 @@ __global__ void __launch_bounds__(kTreeThreads) accept_walk_kernel(TreeState t, 
   const int n = t.final_n[b], Nw = t.Nw, width = t.D + 1;
   const size_t fb = (size_t)b * Nw;
   int *want = s_walk, *next = s_walk + Nw;
+  int parent = -1, token = 0;                                  // of node 1 + tid
+  if (1 + tid < Nw) { parent = t.final_parent[fb + 1 + tid]; token = t.final_token[fb + 1 + tid]; }
   if (out.path)
     for (int k = tid; k < width; k += kTreeThreads) out.path[(size_t)b * width + k] = k == 0 ? 0 : -1;
   for (int i = tid; i < Nw; i += kTreeThreads) {
@@ -305,8 +309,8 @@ __global__ void __launch_bounds__(kTreeThreads) accept_walk_kernel(TreeState t, 
   }
   __syncthreads();
   for (int c = 1 + tid; c < n; c += kTreeThreads) {
-    const int par = t.final_parent[fb + c];
-    if (par >= 0 && t.final_token[fb + c] == want[par]) atomicMin(&next[par], c);
+    if (c != 1 + tid) { parent = t.final_parent[fb + c]; token = t.final_token[fb + c]; }
+    if (parent >= 0 && token == want[parent]) atomicMin(&next[parent], c);
   }
   __syncthreads();
   if (tid != 0) return;
