@@ -417,6 +417,26 @@ typedef struct {
 } c2t_view;
 int c2t_get_view(c2t_ctx *ctx, c2t_view *out);
 
+/* A whole decode step on device logits. */
+typedef struct {
+  const int32_t *root_tok_dev, *prefix_len_dev;      /* as for c2t_begin_step                       */
+  const void *const *draft_logits_dev;               /* HOST array of D pointers, one per level     */
+  const int64_t *draft_strides;                      /* HOST [D, 2]: seq_stride, row_stride         */
+  const void *target_logits_dev;
+  int64_t target_seq_stride, target_row_stride;
+  const c2t_frontier *frontier;                      /* outputs, each may be NULL                   */
+  const c2t_verify *verify;
+  const c2t_accept_out *accept;
+} c2t_step;
+
+/*
+ * c2t_begin_step, c2t_expand_prune_level for all D levels, c2t_prune(C2T_FINAL), c2t_build_verify and c2t_accept, in this
+ * order, as one call: the same launches, the same results, without a caller's overhead between them.  For callers that have the
+ * logits of all levels at hand (a draft model that runs between the levels needs the single calls).  Stops at
+ * the first call that fails and returns its code.
+ */
+int c2t_decode_step(c2t_ctx *ctx, const c2t_step *step, void *stream);
+
 /* Host-side description of a whole decode step fed from host memory. */
 typedef struct {
   const void *const *draft_logits_host; /* [D] pointers, each [B, F, V] contiguous, pinned  */

@@ -610,6 +610,17 @@ int c2t_get_view(c2t_ctx *ctx, c2t_view *v) {
   return C2T_OK;
 }
 
+int c2t_decode_step(c2t_ctx *ctx, const c2t_step *step, void *stream) {
+  if (!ctx || !step || !step->draft_logits_dev || !step->draft_strides) return C2T_EINVAL;
+  int rc = c2t_begin_step(ctx, step->root_tok_dev, step->prefix_len_dev, stream);
+  for (int l = 0; l < ctx->cfg.max_depth && rc == C2T_OK; ++l)
+    rc = c2t_expand_prune_level(ctx, l, step->draft_logits_dev[l], step->draft_strides[2 * l], step->draft_strides[2 * l + 1], step->frontier, stream);
+  if (rc == C2T_OK) rc = c2t_prune(ctx, C2T_FINAL, nullptr, stream);
+  if (rc == C2T_OK) rc = c2t_build_verify(ctx, step->verify, stream);
+  if (rc == C2T_OK) rc = c2t_accept(ctx, step->target_logits_dev, step->target_seq_stride, step->target_row_stride, step->accept, stream);
+  return rc;
+}
+
 int c2t_decode_step_host(c2t_ctx *ctx, const c2t_host_step *io, void *stream) {
   if (!ctx || !io || !io->draft_logits_host || !io->target_logits_host || !io->root_tok_host ||
       !io->prefix_len_host || !io->draft_stage_dev || !io->target_stage_dev || !io->int_stage_dev)
