@@ -152,15 +152,20 @@ size_t carve(const c2t_config *c, void *base, TreeState *t) {
   return (w.off + 255) & ~(size_t)255;
 }
 
+// no sequence has more active rows at this level
+int rows_bound(const TreeState &t, int level) {
+  long long bound = 1;
+  for (int l = 0; l < level && bound < t.F; ++l) bound *= t.K;
+  return bound < t.F ? (int)bound : t.F;
+}
+
 // the expand pass of a level over rows of `vocab` tokens (the whole vocabulary, or one shard of it)
 PassParams expand_params(const TreeState &t, int level, const void *logits, int64_t seq_stride, int64_t row_stride, int vocab) {
   PassParams p;
   memset(&p, 0, sizeof p);
   p.logits = logits; p.seq_stride = seq_stride; p.row_stride = row_stride;
   p.V = vocab; p.K = t.K; p.B = t.B; p.rows_per_seq_max = t.F;
-  long long bound = 1;
-  for (int l = 0; l < level && bound < t.F; ++l) bound *= t.K;
-  p.rows_bound = bound < t.F ? (int)bound : t.F;
+  p.rows_bound = rows_bound(t, level);
   p.counts = t.frontier_n[level & 1];
   p.status = t.status;
   p.info = t.info_draft;
@@ -390,7 +395,10 @@ int c2t_expand_prune_level(c2t_ctx *ctx, int level, const void *logits_dev, int6
                            const c2t_frontier *out, void *stream) {
   if (!ctx || !logits_dev) return C2T_EINVAL;
   const TreeState &t = ctx->t;
-  if (t.B > C2T_FUSED_MAX_BATCH || (t.entropy_top_m > 0 && t.entropy_top_m < t.V)) {
+  // one launch where a level is small: few sequences, or the rows in registers
+  const bool small = t.B <= C2T_FUSED_MAX_BATCH ||
+                     row_pass_plan(t.V, (int)ctx->elem_bytes, (long long)t.B * rows_bound(t, level), ctx->grid_expand).cluster > 0;
+  if (!small || (t.entropy_top_m > 0 && t.entropy_top_m < t.V)) {
     const int rc = c2t_expand_level(ctx, level, logits_dev, seq_stride, row_stride, stream);
     return rc != C2T_OK ? rc : c2t_prune(ctx, level, out, stream);
   }

@@ -251,16 +251,20 @@ __device__ __forceinline__ void merge_sums(RowShared &sh, RowResult *out, float 
 
 // ---------------------------------------------------------------- a row
 
-// Row (b, j) by the blocks of a cluster.  True in the leading block, after the row's result is written (by its first two warps).
+// Before the kernel waits for its predecessor: this block's shared memory can be written once the block runs.
+__device__ __forceinline__ void open_row(RowShared &sh, int cluster) {
+  if (threadIdx.x == 0) {
+    sh.floor = 0u;
+    sh.n = 0;
+  }
+  if (cluster > 1) cluster_arrive();
+}
+
+// Row (b, j) by the blocks of a cluster, after open_row and the wait for it.  True in the leading block, after the row's result is written (by its first two warps).
 template <bool BF16, int NT>
 __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, int b, int j, int cluster, int rank) {
   constexpr int kW = NT / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, K = p.K, warps = cluster * kW;
-  if (tid == 0) {
-    sh.floor = 0u;
-    sh.n = 0;
-  }
-  if (cluster > 1) cluster_arrive();                  // (a block's shared memory can be written once the block runs)
   RowPart<BF16, NT> rp;
   rp.vpr = (p.V + Vec<BF16>::N - 1) / Vec<BF16>::N;
   rp.v_full = p.V / Vec<BF16>::N;
@@ -282,7 +286,6 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
   for (int o = 1; o < width; o <<= 1) g = fmaxf(g, __shfl_xor_sync(kFull, g, o));
   const int to = lane & (width - 1), at = (rank * kW + warp) * (32 / width) + lane / width;
   if (cluster > 1) {
-    cluster_wait();
     if (to < cluster) put(place_in(&sh.group[at], to), __float_as_uint(g));
     __syncwarp();
     cluster_arrive();
@@ -310,7 +313,6 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
   float Mf = fmaxf(sh.group[lane], sh.group[32 + lane]);
   if (groups > 64) Mf = fmaxf(Mf, fmaxf(sh.group[64 + lane], sh.group[96 + lane]));
   Mf = warp_max(Mf);
-  if (__any_sync(kFull, mt == Mf)) sum_again<BF16>(sh, q, mt, Mf, s, u, c, rank * kW + warp, cluster);
   {
     const int team = NT / groups, member = tid & (team - 1);      // threads of a group: 2 to 8
     const float mine = sh.group[tid / team];
@@ -352,6 +354,7 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
     }
     __syncwarp();
   }
+  if (__any_sync(kFull, mt == Mf)) sum_again<BF16>(sh, q, mt, Mf, s, u, c, rank * kW + warp, cluster);
   if (cluster > 1) { cluster_arrive(); cluster_wait(); }
   else __syncthreads();
 
@@ -396,13 +399,17 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
 template <bool BF16, int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT) expand_rows_kernel(const __grid_constant__ PassParams p, int cluster) {
   __shared__ RowShared sh;
-  chain_enter();
+  chain_release();
+  open_row(sh, cluster);
   const int b = blockIdx.y, j = (int)blockIdx.x / cluster;
-  if (j >= p.counts[b]) return;
+  chain_wait();
+  const int n = p.counts[b];
+  if (cluster > 1) cluster_wait();
+  if (j >= n) return;
   expand_row<BF16, NT>(p, sh, b, j, cluster, cluster > 1 ? cluster_rank() : 0);
 }
 
-// Expand and prune of a level in one launch, for small batches: the cluster that finishes a sequence's last row (a count, nobody
+// Expand and prune of a level in one launch: the cluster that finishes a sequence's last row (a count, nobody
 // waits) does the sequence's part of c2t_prune.
 template <bool BF16, int NT>
 __global__ void __launch_bounds__(NT, 512 / NT) expand_rows_prune_kernel(const __grid_constant__ PassParams p, const __grid_constant__ TreeState t,
@@ -412,10 +419,12 @@ __global__ void __launch_bounds__(NT, 512 / NT) expand_rows_prune_kernel(const _
   __shared__ int s_last;
   const int rank = cluster > 1 ? cluster_rank() : 0;
   chain_release();
+  open_row(sh.row, cluster);
   if (rank == 0) stage_classifier(t, s_w, threadIdx.x, NT);           // (written at init)
-  chain_wait();
   const int b = blockIdx.y, j = (int)blockIdx.x / cluster;
+  chain_wait();
   int n = p.counts[b];
+  if (cluster > 1) cluster_wait();
   n = n < p.rows_per_seq_max ? n : p.rows_per_seq_max;
   if (j >= n && !(n <= 0 && j == 0)) return;
   if (n > 0) {
