@@ -889,7 +889,8 @@ __global__ void __launch_bounds__(kExpandThreads, 1) expand_prune_kernel(const _
   if (threadIdx.x == 0) *t.ticket = 0u;              // for the next launch
   // the pass's shared memory is free now
   PruneShared &sh = *reinterpret_cast<PruneShared *>(s_dyn);
-  for (int b = 0; b < t.B; ++b) prune_level_body<kExpandThreads>(t, level, out, nullptr, 0, b, sh, s_w, nullptr);
+#pragma unroll 1
+  for (int b = 0; b < t.B; ++b) prune_level_body<kExpandThreads, kMaxCand / kExpandThreads, false>(t, level, out, nullptr, 0, b, sh, s_w, nullptr);
 }
 
 }  // namespace

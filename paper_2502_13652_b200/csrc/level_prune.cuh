@@ -38,12 +38,16 @@ __device__ __forceinline__ void stage_classifier(const TreeState &t, double *w, 
   if (tid == 0) w[kW0] = (double)t.b2[0];
 }
 
+// One copy of exp for all its callers in a kernel.  The kernels here are chains that run through their code once, and what code costs
+// then is fetching it: about 400 cycles for a jump over something that is not in the instruction caches yet.
+__device__ __noinline__ double exp_shared(double x) { return exp(x); }
+
 // Confidence of one child (Eq. 4): two-layer FFN on (P, H, d), ReLU, sigmoid.
 //   The hidden units are taken kBatch at a time, without a branch and with all of a batch's loads first: one after the other they are a
 // chain of loads, additions and a comparison each (89 cycles per unit; the classification of a level 1.3 -> 0.6 us).
 __device__ __forceinline__ double classify(int hidden, const double *w, double P, double H, double d) {
   double z[kHiddenBatch] = {w[kW0], 0.0, 0.0, 0.0};
-#pragma unroll 2
+#pragma unroll 1
   for (int k0 = 0; k0 < hidden; k0 += kHiddenBatch) {            // (units of weight 0 behind the last one)
     double2 a01[kHiddenBatch], a23[kHiddenBatch];
     double v[kHiddenBatch];
@@ -60,7 +64,7 @@ __device__ __forceinline__ double classify(int hidden, const double *w, double P
       z[i] = fma(v[i], a < 0.0 ? 0.0 : a, z[i]);
     }
   }
-  return 1.0 / (1.0 + exp(-((z[0] + z[1]) + (z[2] + z[3]))));
+  return 1.0 / (1.0 + exp_shared(-((z[0] + z[1]) + (z[2] + z[3]))));
 }
 
 // A row's merged sums, as one warp holds them.
@@ -177,17 +181,40 @@ __device__ __forceinline__ void row_stats(const TreeState &t, const RowResult &r
   if (r.fault) atomicOr(&t.status[b], r.fault);
 }
 
+// The candidates that come before each one under (C desc, index asc), by their whole keys.  Called by all threads; ends with a barrier.
+template <int NT>
+__device__ __noinline__ void rank_whole_keys(PruneShared &sh, int nc) {
+  const int tid = threadIdx.x;
+  for (int c0 = 0; c0 < nc; c0 += NT / 4) {       // four threads to a candidate, two keys to a load
+    const int c = c0 + (tid >> 2);
+    const unsigned long long kc = c < nc ? sh.ckey[c] : 0ull, kc1 = kc + 1ull;      // (a key is never all ones)
+    int before = 0;
+#pragma unroll 4
+    for (int o = 2 * (tid & 3); o < nc; o += 8) {                                   // (zeros behind the last key)
+      const ulonglong2 k = *reinterpret_cast<const ulonglong2 *>(&sh.ckey[o]);
+      before += k.x >= (o < c ? kc : kc1);
+      before += k.y >= (o + 1 < c ? kc : kc1);
+    }
+    before += __shfl_xor_sync(kFullMask, before, 1);
+    before += __shfl_xor_sync(kFullMask, before, 2);
+    if ((tid & 3) == 0 && c < nc) sh.before[c] = (short)before;
+  }
+  __syncthreads();
+}
+
 // NT: threads of the CTA; b: the sequence; w: the classifier's staged weights.  records == nullptr: the rows come from
 // this context's own expand pass; else from gathered records of n_shards shards (gs: room for their merge).
 //   The work is a chain of dependent steps over at most F K candidates, on the critical path of every level, so it is short
 // in steps rather than in operations: every global load whose address does not depend on another is issued at the top
 // (frontier nodes carry their log-probabilities and path confidences with them for that), a thread keeps its
-// candidates in registers, the cap ranks a candidate with a whole warp, and the compaction needs one barrier.
-// Eight levels of 64 sequences: 323 -> 314 us (expand and prune).
-template <int NT>
-__device__ void prune_level_body(const TreeState &t, int level, const c2t_frontier &out, const c2t_row_record *records,
-                                 int n_shards, int b, PruneShared &sh, const double *w, GatherShared *gs) {
-  constexpr int kRounds = kMaxCand / NT, kNW = NT / 32;        // candidates per thread; warps
+// candidates in registers, the cap ranks a candidate with several threads, and the compaction needs one barrier.
+// Eight levels of 64 sequences: 323 -> 314 us (expand and prune).  And it is short in code, which is cold whenever a level's last block is
+// on another SM than the last level's: a candidate per thread where that is enough (ROUNDS 1), what is rarely needed in functions of its
+// own, loops that are not unrolled.
+template <int NT, int ROUNDS, bool GATHERED>
+__device__ __forceinline__ void prune_level_body(const TreeState &t, int level, const c2t_frontier &out, const c2t_row_record *records,
+                                                 int n_shards, int b, PruneShared &sh, const double *w, GatherShared *gs) {
+  constexpr int kRounds = ROUNDS, kNW = NT / 32;               // candidates per thread; warps
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int K = t.K, F = t.F;
   const int cur = level & 1, nxt = cur ^ 1;
@@ -201,12 +228,12 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
 #pragma unroll
   for (int r = 0; r < kRounds; ++r) {
     const int c = tid + r * NT;
-    key[r] = !records && c < F * K ? __ldcg(&t.row_keys[cbase + c]) : 0ull;
+    key[r] = !GATHERED && c < F * K ? __ldcg(&t.row_keys[cbase + c]) : 0ull;
   }
   const int jr = tid - (NT - 64), jf = tid - (NT - 32);        // the last two warps fetch the rows' and the frontier's data
   RowResult row;
   double2 sm = make_double2(0.0, 0.0);
-  if (!records && jr >= 0 && jr < F) {
+  if (!GATHERED && jr >= 0 && jr < F) {
     row = t.rows[fbase + jr];
     if (t.entropy_top_m > 0) sm = t.topm[fbase + jr];
   }
@@ -227,7 +254,7 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
     return;
   }
   __syncthreads();                                // (a CTA that serves several sequences: the last one's reads are done)
-  if (!records) {
+  if (!GATHERED) {
     if (jr >= 0 && jr < n) row_stats(t, row, sm, b, jr, sh);
   } else {
     for (int j = warp; j < n; j += kNW) {
@@ -266,16 +293,16 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
       if (c < nc) {
         const int j = (int)((unsigned)c * per_k >> 16);
         float x;
-        if (records) { x = gs->x[c]; tok[r] = gs->tok[c]; }
+        if (GATHERED) { x = gs->x[c]; tok[r] = gs->tok[c]; }
         else { x = key[r] ? key_value(key[r]) : -INFINITY; tok[r] = key[r] ? key_token(key[r]) : -1; }
         const bool ok = tok[r] >= 0 && !sh.rowfault[j];
         const double lp = (x > kNegInfAsFinite) ? ((double)x - sh.rowM[j]) - sh.rowL[j] : -INFINITY;
         logP[r] = sh.flogP[j] + lp;                                             // Eq. 1 in log space
-        const double P = exp(logP[r]);
+        const double P = exp_shared(logP[r]);
         const double H = sh.rowH[j];
         if (!ok) C[r] = NAN;
         else if (t.classifier == C2T_CLS_IDENTITY_JOINT) C[r] = P;
-        else if (t.classifier == C2T_CLS_IDENTITY_COND) C[r] = exp(lp);
+        else if (t.classifier == C2T_CLS_IDENTITY_COND) C[r] = exp_shared(lp);
         else C[r] = classify(t.hidden, w, P, H, (double)level);
         keep[r] = ok && C[r] >= (double)t.beta;                                 // first pruning
         // (C desc, index asc) as integer compares: an orderable image of C, 0 for a dropped candidate
@@ -303,8 +330,9 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
       const int c = c0 + tid / kParts;
       const unsigned kc = c < nc ? sh.chi[c] : 0xFFFFFFFFu;
       int reach = 0;                                // candidates at or above it, itself among them
+#pragma unroll 1
       for (int o = 0; o < nc; o += kCapBlock) {
-#pragma unroll
+#pragma unroll 1
         for (int i0 = 0; i0 < kLoads; i0 += 8) {
           uint4 k[8];
 #pragma unroll
@@ -341,32 +369,18 @@ __device__ void prune_level_body(const TreeState &t, int level, const c2t_fronti
       if (lane == 0) sh.count[r * kNW + warp] = __popc(add_mask[r]) | (__popc(sel_mask[r]) << 16);    // (each total at most 1024)
     }
     __syncthreads();
-    return sh.count[lane];
+    return lane < kRounds * kNW ? sh.count[lane] : 0;
   };
   int counts = count_up(), total = __reduce_add_sync(kFullMask, counts);
   if (n_keep > F && (total >> 16) != F) {           // (uniform)
-    for (int c0 = 0; c0 < nc; c0 += NT / 4) {       // four threads to a candidate, two keys to a load
-      const int c = c0 + (tid >> 2);
-      const unsigned long long kc = c < nc ? sh.ckey[c] : 0ull, kc1 = kc + 1ull;      // (a key is never all ones)
-      int before = 0;
-#pragma unroll 4
-      for (int o = 2 * (tid & 3); o < nc; o += 8) {                                   // (zeros behind the last key)
-        const ulonglong2 k = *reinterpret_cast<const ulonglong2 *>(&sh.ckey[o]);
-        before += k.x >= (o < c ? kc : kc1);
-        before += k.y >= (o + 1 < c ? kc : kc1);
-      }
-      before += __shfl_xor_sync(kFullMask, before, 1);
-      before += __shfl_xor_sync(kFullMask, before, 2);
-      if ((tid & 3) == 0 && c < nc) sh.before[c] = (short)before;
-    }
-    __syncthreads();
+    rank_whole_keys<NT>(sh, nc);
 #pragma unroll
     for (int r = 0; r < kRounds; ++r)
       if (tid + r * NT < nc) sel[r] = keep[r] && sh.before[tid + r * NT] < F;
     counts = count_up();
     total = __reduce_add_sync(kFullMask, counts);
   }
-  static_assert(kRounds * kNW == 32, "a count per lane");
+  static_assert(kRounds * kNW <= 32, "a count per lane");
   const int tot_add = total & 0xFFFF, tot_sel = total >> 16;
   const bool overflow = base + tot_add > t.cap;
   const size_t tb = (size_t)b * t.cap;

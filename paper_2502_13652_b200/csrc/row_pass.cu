@@ -174,7 +174,7 @@ __device__ __noinline__ int select_by_rounds(RowShared &sh, const RowPart<BF16, 
 }
 
 // A warp's sums to its place in the leading block: its lanes' (s, u) relative to their offsets c, m2 the largest values they come from.
-__device__ __forceinline__ void put_sums(RowShared &sh, float s, float u, float c, float m2, int equals, int w, int cluster) {
+__device__ __noinline__ void put_sums(RowShared &sh, float s, float u, float c, float m2, int equals, int w, int cluster) {
   const float cw = offset_of(warp_max(m2)), by = fmaxf(cw - c, -127.f);
   const float two = __int_as_float((__float_as_int(by + 12582912.f) << 23) + 0x3F800000);      // 2^by, 0 for -127
   u = two * fmaf(by, s, u);
@@ -191,38 +191,23 @@ __device__ __forceinline__ void put_sums(RowShared &sh, float s, float u, float 
   __syncwarp();
 }
 
-// The warp that holds the row's maximum Mf: each such lane (mt == Mf) summed again without it and its equals, its words dealt out to the
-// warp's lanes.
+// One lane's vectors, in sh.again, summed again without the row's maximum and its equals, by the whole warp.
 template <bool BF16>
-__device__ __forceinline__ void sum_again(RowShared &sh, const uint4 (&q)[kRowLoads], float mt, float Mf, float s, float u, float c, int w, int cluster) {
-  const int lane = threadIdx.x & 31;
-  int equals = 0;
-  float m2 = mt;
-  for (unsigned left = __ballot_sync(kFull, mt == Mf); left; left &= left - 1u) {
-    const int owner = __ffs(left) - 1;
-    __syncwarp();
-    if (lane == owner) {
+__device__ __noinline__ void sum_again(RowShared &sh, float Mf, float *s, float *u, float *c, float *m2, int *equals) {
+  const uint32_t word = reinterpret_cast<const uint32_t *>(sh.again[threadIdx.x >> 5])[threadIdx.x & 31];
+  float x0 = BF16 ? __uint_as_float(word << 16) : __uint_as_float(word), x1 = BF16 ? __uint_as_float(word & 0xFFFF0000u) : kLowestF32;
+  *equals += (x0 == Mf) + (x1 == Mf);
+  x0 = x0 == Mf ? kLowestF32 : x0;
+  x1 = x1 == Mf ? kLowestF32 : x1;
+  const float m = warp_max(fmaxf(x0, x1)), cr = offset_of(m);
+  const float t0 = fmaf(x0, kLog2e, cr), t1 = fmaf(x1, kLog2e, cr), e0 = ex2f(t0), e1 = ex2f(t1);
+  float sr = e0 + e1, ur = fmaf(e0, t0, e1 * t1);
 #pragma unroll
-      for (int k = 0; k < kRowLoads; ++k) sh.again[threadIdx.x >> 5][k] = q[k];
-    }
-    __syncwarp();
-    const uint32_t word = reinterpret_cast<const uint32_t *>(sh.again[threadIdx.x >> 5])[lane];
-    float x0 = BF16 ? __uint_as_float(word << 16) : __uint_as_float(word), x1 = BF16 ? __uint_as_float(word & 0xFFFF0000u) : kLowestF32;
-    equals += (x0 == Mf) + (x1 == Mf);
-    x0 = x0 == Mf ? kLowestF32 : x0;
-    x1 = x1 == Mf ? kLowestF32 : x1;
-    const float m = warp_max(fmaxf(x0, x1)), cr = offset_of(m);
-    const float t0 = fmaf(x0, kLog2e, cr), t1 = fmaf(x1, kLog2e, cr), e0 = ex2f(t0), e1 = ex2f(t1);
-    float sr = e0 + e1, ur = fmaf(e0, t0, e1 * t1);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      sr += __shfl_xor_sync(kFull, sr, o);
-      ur += __shfl_xor_sync(kFull, ur, o);
-    }
-    if (lane == owner) { s = sr; u = ur; c = cr; m2 = m; }
+  for (int o = 16; o > 0; o >>= 1) {
+    sr += __shfl_xor_sync(kFull, sr, o);
+    ur += __shfl_xor_sync(kFull, ur, o);
   }
-  equals = __reduce_add_sync(kFull, equals);
-  put_sums(sh, s, u, c, m2, equals, w, cluster);
+  *s = sr; *u = ur; *c = cr; *m2 = m;
 }
 
 // The warps' sums, merged by one warp of the leading block.
@@ -354,7 +339,23 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
     }
     __syncwarp();
   }
-  if (__any_sync(kFull, mt == Mf)) sum_again<BF16>(sh, q, mt, Mf, s, u, c, rank * kW + warp, cluster);
+  if (unsigned left = __ballot_sync(kFull, mt == Mf)) {      // the warp that holds the maximum: such lanes again without it
+    float m2 = mt, cs = c;
+    int equals = 0;
+    for (; left; left &= left - 1u) {
+      const bool mine = lane == __ffs(left) - 1;
+      __syncwarp();
+      if (mine) {
+#pragma unroll
+        for (int k = 0; k < kRowLoads; ++k) sh.again[warp][k] = q[k];
+      }
+      __syncwarp();
+      float sr, ur, cr, mr;
+      sum_again<BF16>(sh, Mf, &sr, &ur, &cr, &mr, &equals);
+      if (mine) { s = sr; u = ur; cs = cr; m2 = mr; }
+    }
+    put_sums(sh, s, u, cs, m2, __reduce_add_sync(kFull, equals), rank * kW + warp, cluster);
+  }
   if (cluster > 1) { cluster_arrive(); cluster_wait(); }
   else __syncthreads();
 
@@ -411,7 +412,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) expand_rows_kernel(const __grid
 
 // Expand and prune of a level in one launch: the cluster that finishes a sequence's last row (a count, nobody
 // waits) does the sequence's part of c2t_prune.
-template <bool BF16, int NT>
+template <bool BF16, int NT, int ROUNDS>
 __global__ void __launch_bounds__(NT, 512 / NT) expand_rows_prune_kernel(const __grid_constant__ PassParams p, const __grid_constant__ TreeState t,
                                                                            int level, c2t_frontier out, int cluster) {
   __shared__ union { RowShared row; PruneShared prune; } sh;
@@ -440,7 +441,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) expand_rows_prune_kernel(const _
   } else if (rank != 0) {
     return;
   }
-  prune_level_body<NT>(t, level, out, nullptr, 0, b, sh.prune, s_w, nullptr);
+  prune_level_body<NT, ROUNDS, false>(t, level, out, nullptr, 0, b, sh.prune, s_w, nullptr);
 }
 
 template <typename... KArgs, typename... Args>
@@ -472,9 +473,14 @@ cudaError_t launch_expand_rows(const PassParams &p, int dtype, RowPlan plan, cud
 cudaError_t launch_expand_rows_prune(const PassParams &p, const TreeState &t, int level, const c2t_frontier &out, int dtype, RowPlan plan, cudaStream_t s) {
   const dim3 grid(p.rows_bound * plan.cluster, p.B);
   const bool bf16 = dtype == C2T_BF16;
-  if (plan.threads == 256)
-    return launch_rows(bf16 ? expand_rows_prune_kernel<true, 256> : expand_rows_prune_kernel<false, 256>, grid, 256, plan.cluster, s, p, t, level, out, plan.cluster);
-  return launch_rows(bf16 ? expand_rows_prune_kernel<true, 512> : expand_rows_prune_kernel<false, 512>, grid, 512, plan.cluster, s, p, t, level, out, plan.cluster);
+  const bool small = t.F * t.K <= plan.threads;       // a candidate per thread
+  constexpr int k256 = kMaxCand / 256, k512 = kMaxCand / 512;
+  const auto kernel = plan.threads == 256
+                          ? (bf16 ? (small ? expand_rows_prune_kernel<true, 256, 1> : expand_rows_prune_kernel<true, 256, k256>)
+                                  : (small ? expand_rows_prune_kernel<false, 256, 1> : expand_rows_prune_kernel<false, 256, k256>))
+                          : (bf16 ? (small ? expand_rows_prune_kernel<true, 512, 1> : expand_rows_prune_kernel<true, 512, k512>)
+                                  : (small ? expand_rows_prune_kernel<false, 512, 1> : expand_rows_prune_kernel<false, 512, k512>));
+  return launch_rows(kernel, grid, plan.threads, plan.cluster, s, p, t, level, out, plan.cluster);
 }
 
 }  // namespace c2t

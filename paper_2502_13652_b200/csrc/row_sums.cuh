@@ -123,7 +123,7 @@ __device__ __noinline__ uint4 load_ragged(const void *row, int v, int v_full, in
 // weight is.
 __device__ __forceinline__ void write_sums(RowResult *r, float Mf, float cM, double S, double U, int equals) {
   const double kBack = 1.0 / (double)kLog2e, kShort = kBack - 0.69314718055994530942;
-  const double M = (double)Mf, g = -(double)cM * kBack - M, scale = exp(g);
+  const double M = (double)Mf, g = -(double)cM * kBack - M, scale = exp_shared(g);
   // sums of e^(t kBack) from those of 2^t, to first order (sum 2^t t^2 taken as U^2 / S: the weight lies close together)
   if (S > 1e-30) {
     const double short_of = kShort * U;

@@ -61,7 +61,9 @@ __global__ void __launch_bounds__(kExportWarps * 32) export_rows_kernel(TreeStat
   }
 }
 
-// records == nullptr: the rows come from this context's own expand pass; else from gathered records of n_shards shards
+// ROUNDS: candidates of a thread at most; GATHERED: the rows come from gathered records of n_shards shards, not from this context's own
+// expand pass
+template <int ROUNDS, bool GATHERED>
 __global__ void __launch_bounds__(kTreeThreads) prune_level_kernel(TreeState t, int level, c2t_frontier out,
                                                                    const c2t_row_record *records, int n_shards) {
   extern __shared__ __align__(16) unsigned char s_prune[];
@@ -71,8 +73,9 @@ __global__ void __launch_bounds__(kTreeThreads) prune_level_kernel(TreeState t, 
   chain_release();
   stage_classifier(t, s_w, threadIdx.x, kTreeThreads);   // (written at init, not by the chain: while the expand pass is finishing)
   chain_wait();
-  prune_level_body<kTreeThreads>(t, level, out, records, n_shards, blockIdx.x, sh, s_w, gs);
+  prune_level_body<kTreeThreads, ROUNDS, GATHERED>(t, level, out, records, n_shards, blockIdx.x, sh, s_w, gs);
 }
+constexpr int kPruneRounds = kMaxCand / kTreeThreads;
 
 // ---------------------------------------------------------------- rerank ----
 
@@ -486,7 +489,10 @@ cudaError_t launch_prune_level(const TreeState &t, int level, const c2t_frontier
                                int n_shards, cudaStream_t s) {
   c2t_frontier o = {nullptr, nullptr, nullptr, nullptr};
   if (out) o = *out;
-  return launch_chained(prune_level_kernel, dim3(t.B), dim3(kTreeThreads), sizeof(PruneShared) + (records ? sizeof(GatherShared) : 0),
+  const bool small = t.F * t.K <= kTreeThreads;
+  const auto kernel = records ? (small ? prune_level_kernel<1, true> : prune_level_kernel<kPruneRounds, true>)
+                              : (small ? prune_level_kernel<1, false> : prune_level_kernel<kPruneRounds, false>);
+  return launch_chained(kernel, dim3(t.B), dim3(kTreeThreads), sizeof(PruneShared) + (records ? sizeof(GatherShared) : 0),
                         s, t, level, o, records, n_shards);
 }
 
@@ -494,8 +500,9 @@ cudaError_t launch_prune_level(const TreeState &t, int level, const c2t_frontier
 static size_t final_smem(int cap) { return (size_t)cap * (sizeof(unsigned long long) + 2 * sizeof(int)); }
 
 cudaError_t prepare_tree_kernels() {
-  cudaError_t e = cudaFuncSetAttribute(prune_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(PruneShared) + sizeof(GatherShared)));
+  const int gather = (int)(sizeof(PruneShared) + sizeof(GatherShared));
+  cudaError_t e = cudaFuncSetAttribute(prune_level_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, gather);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(prune_level_kernel<kPruneRounds, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, gather);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(final_prune_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)final_smem(C2T_MAX_TREE));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(build_verify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 3 * C2T_MAX_TREE * (int)sizeof(int));
   if (e == cudaSuccess) e = cudaFuncSetAttribute(accept_walk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * C2T_MAX_TREE * (int)sizeof(int));
