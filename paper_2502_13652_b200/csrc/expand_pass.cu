@@ -588,22 +588,6 @@ __device__ __forceinline__ RowState count_shared(const PassParams &p, int a, int
   return total == (unsigned)nc ? kRowComplete : kRowBroken;
 }
 
-// The result of a row that was given up: no candidates, and the fault that says so.
-__device__ __forceinline__ void give_up_row(const PassParams &p, int b, int j) {
-  const int lane = threadIdx.x & 31;
-  const size_t slot = (size_t)b * p.rows_per_seq_max + j;
-  for (int i = lane; i < p.K; i += 32) p.row_keys[slot * p.K + i] = 0ull;
-  if (lane == 0) {
-    RowResult r;
-    r.M = r.S = r.T = r.L = r.H = 0.0;
-    r.top = 0ull;
-    r.n_valid = 0;
-    r.fault = C2T_ST_INTERNAL;
-    p.rows[slot] = r;
-  }
-  __syncwarp();
-}
-
 // ---------------------------------------------------------------- truncated entropy (Eq. 3): setting candidates aside
 
 // Where a warp puts the vectors whose largest element reaches its segment's floor (ballot-ranked places in stream

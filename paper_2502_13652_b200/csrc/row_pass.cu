@@ -25,6 +25,7 @@ constexpr int kTooMany = 1 << 20;
 static_assert(kRowGroups >= C2T_MAX_TOPK && kMaxRowGroups >= kRowGroups, "");
 
 struct RowShared {
+  unsigned long long maxima_in, results_in;           // transaction barriers: all groups' maxima; everything for the row's result
   __align__(16) float group[kMaxRowGroups];           // the maxima of the row's groups
   float4 sums[kRowCluster * kMaxRowWarps];            // in the leading block: S, U, offset of every warp, and how often it holds the maximum (int bits)
   unsigned long long keys[kRowCluster][kCtaKeys];     // in the leading block: what every block hands over
@@ -51,10 +52,31 @@ __device__ __forceinline__ uint32_t place_in(const void *at, int r) {
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"((uint32_t)__cvta_generic_to_shared(at)), "r"(r));
   return to;
 }
-__device__ __forceinline__ void put(uint32_t at, uint32_t v) { asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(at), "r"(v) : "memory"); }
 __device__ __forceinline__ void put(uint32_t at, unsigned long long v) { asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(at), "l"(v) : "memory"); }
-__device__ __forceinline__ void put(uint32_t at, float a, float b, float c, float d) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+// The same with its bytes counted by a transaction barrier of the block that it goes to: the receiver waits for the data, and nobody for
+// the stores to be acknowledged (a cluster barrier with release semantics did: 0.5 us after the maxima, 0.7 us before the result).
+__device__ __forceinline__ void send(uint32_t at, uint32_t v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(at), "r"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void send(uint32_t at, unsigned long long v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(at), "l"(v), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void send(uint32_t at, float a, float b, float c, float d, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+               ::"r"(at), "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(__float_as_uint(c)), "r"(__float_as_uint(d)), "r"(bar) : "memory");
+}
+// an arrival at a block's barrier that announces bytes to it
+__device__ __forceinline__ void announce(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+// false if the wait ran out
+__device__ __forceinline__ bool wait_bar(const unsigned long long *bar) {
+  const uint32_t at = (uint32_t)__cvta_generic_to_shared(bar);
+  uint32_t done = 0u;
+  for (int i = 0; i < kTaskWaitLimit && !done; ++i)
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done) : "r"(at) : "memory");
+  return done != 0u;
 }
 
 __device__ __forceinline__ float warp_max(float v) {
@@ -173,9 +195,10 @@ __device__ __noinline__ int select_by_rounds(RowShared &sh, const RowPart<BF16, 
   return r;
 }
 
-// A warp's sums to its place in the leading block: its lanes' (s, u) relative to their offsets c, m2 the largest values they come from.
-__device__ __noinline__ void put_sums(RowShared &sh, float s, float u, float c, float m2, int equals, int w, int cluster) {
-  const float cw = offset_of(warp_max(m2)), by = fmaxf(cw - c, -127.f);
+// A warp's sums, from its lanes' (s, u) relative to their offsets c; m2 the largest values they come from: in lane 0, relative to cw.
+__device__ __forceinline__ void warp_sums(float &s, float &u, float c, float m2, float &cw) {
+  cw = offset_of(warp_max(m2));
+  const float by = fmaxf(cw - c, -127.f);
   const float two = __int_as_float((__float_as_int(by + 12582912.f) << 23) + 0x3F800000);      // 2^by, 0 for -127
   u = two * fmaf(by, s, u);
   s = two * s;
@@ -184,11 +207,6 @@ __device__ __noinline__ void put_sums(RowShared &sh, float s, float u, float c, 
     s += __shfl_xor_sync(kFull, s, o);
     u += __shfl_xor_sync(kFull, u, o);
   }
-  if ((threadIdx.x & 31) == 0) {
-    if (cluster > 1) put(place_in(&sh.sums[w], 0), s, u, cw, __int_as_float(equals));
-    else sh.sums[w] = make_float4(s, u, cw, __int_as_float(equals));
-  }
-  __syncwarp();
 }
 
 // One lane's vectors, in sh.again, summed again without the row's maximum and its equals, by the whole warp.
@@ -241,7 +259,15 @@ __device__ __forceinline__ void open_row(RowShared &sh, int cluster) {
   if (threadIdx.x == 0) {
     sh.floor = 0u;
     sh.n = 0;
+    if (cluster > 1) {
+      const uint32_t maxima = (uint32_t)__cvta_generic_to_shared(&sh.maxima_in), results = (uint32_t)__cvta_generic_to_shared(&sh.results_in);
+      const int warps = cluster * (int)(blockDim.x >> 5), groups = warps > kRowGroups ? warps : kRowGroups;
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n\tmbarrier.init.shared::cta.b64 [%1], %2;\n\tfence.mbarrier_init.release.cluster;"
+                   ::"r"(maxima), "r"(results), "r"(cluster) : "memory");
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(maxima), "r"(groups * 4) : "memory");
+    }
   }
+  __syncwarp();
   if (cluster > 1) cluster_arrive();
 }
 
@@ -271,9 +297,7 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
   for (int o = 1; o < width; o <<= 1) g = fmaxf(g, __shfl_xor_sync(kFull, g, o));
   const int to = lane & (width - 1), at = (rank * kW + warp) * (32 / width) + lane / width;
   if (cluster > 1) {
-    if (to < cluster) put(place_in(&sh.group[at], to), __float_as_uint(g));
-    __syncwarp();
-    cluster_arrive();
+    if (to < cluster) send(place_in(&sh.group[at], to), __float_as_uint(g), place_in(&sh.maxima_in, to));
   } else if (to == 0) {
     sh.group[at] = g;
   }
@@ -290,8 +314,10 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
       if (k * NT < rp.part) acc_vector<BF16>(acc, q[k], scale, c2);      // (uniform)
     acc.totals(s, u);
   }
-  put_sums(sh, s, u, c, mt, 0, rank * kW + warp, cluster);
-  if (cluster > 1) cluster_wait();
+  float sw = s, uw = u, cw;
+  warp_sums(sw, uw, c, mt, cw);
+  bool ok = true;
+  if (cluster > 1) ok = wait_bar(&sh.maxima_in);
   else __syncthreads();
 
   // ---- the row's maximum, which stays out of them; the floor: the K-th largest of the groups' maxima, the largest value that K of them reach
@@ -328,20 +354,28 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
   __syncthreads();
   if (warp == 0) {
     const int n = sh.n, c_n = !live || n > kCtaKeys ? kTooMany : n;
-    for (int i = lane; i < c_n && c_n != kTooMany; i += 32) {
-      const unsigned long long key = sh.pool[i];
-      if (cluster > 1) put(place_in(&sh.keys[rank][i], 0), key);
-      else sh.keys[0][i] = key;
-    }
-    if (lane < cluster) {
-      if (cluster > 1) put(place_in(&sh.counts[rank], lane), (uint32_t)c_n);
-      else sh.counts[0] = c_n;
+    const int handed = c_n == kTooMany ? 0 : c_n;
+    if (cluster > 1) {
+      if (lane < cluster) {
+        const uint32_t bar = place_in(&sh.results_in, lane);
+        announce(bar, lane == 0 ? (uint32_t)(4 + kW * 16 + handed * 8) : 4u);
+        send(place_in(&sh.counts[rank], lane), (uint32_t)c_n, bar);
+      }
+      const uint32_t bar = place_in(&sh.results_in, 0);
+      for (int i = lane; i < handed; i += 32) send(place_in(&sh.keys[rank][i], 0), sh.pool[i], bar);
+    } else {
+      for (int i = lane; i < handed; i += 32) sh.keys[0][i] = sh.pool[i];
+      if (lane == 0) sh.counts[0] = c_n;
     }
     __syncwarp();
   }
-  if (unsigned left = __ballot_sync(kFull, mt == Mf)) {      // the warp that holds the maximum: such lanes again without it
+
+  // ---- the warps' sums; the warp that holds the maximum: such lanes again without it
+  int equals = 0;
+  if (unsigned left = __ballot_sync(kFull, mt == Mf)) {
     float m2 = mt, cs = c;
-    int equals = 0;
+    sw = s;
+    uw = u;
     for (; left; left &= left - 1u) {
       const bool mine = lane == __ffs(left) - 1;
       __syncwarp();
@@ -352,12 +386,27 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
       __syncwarp();
       float sr, ur, cr, mr;
       sum_again<BF16>(sh, Mf, &sr, &ur, &cr, &mr, &equals);
-      if (mine) { s = sr; u = ur; cs = cr; m2 = mr; }
+      if (mine) { sw = sr; uw = ur; cs = cr; m2 = mr; }
     }
-    put_sums(sh, s, u, cs, m2, __reduce_add_sync(kFull, equals), rank * kW + warp, cluster);
+    warp_sums(sw, uw, cs, m2, cw);
+    equals = __reduce_add_sync(kFull, equals);
   }
-  if (cluster > 1) { cluster_arrive(); cluster_wait(); }
-  else __syncthreads();
+  if (lane == 0) {
+    float4 *record = &sh.sums[rank * kW + warp];
+    if (cluster > 1) send(place_in(record, 0), sw, uw, cw, __int_as_float(equals), place_in(&sh.results_in, 0));
+    else *record = make_float4(sw, uw, cw, __int_as_float(equals));
+  }
+  __syncwarp();
+  if (cluster > 1) {
+    if (__syncthreads_or(!(ok && wait_bar(&sh.results_in)))) {        // (nothing of the kind is expected) the row is given up
+      cluster_arrive();
+      cluster_wait();                                 // (blocks that have ended count)
+      if (rank == 0 && warp == 0) give_up_row(p, b, j);
+      return rank == 0;
+    }
+  } else {
+    __syncthreads();
+  }
 
   // ---- the row's result
   int upto[kRowCluster], total = 0;                   // keys up to and with block r
@@ -415,7 +464,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) expand_rows_kernel(const __grid
 template <bool BF16, int NT, int ROUNDS>
 __global__ void __launch_bounds__(NT, 512 / NT) expand_rows_prune_kernel(const __grid_constant__ PassParams p, const __grid_constant__ TreeState t,
                                                                            int level, c2t_frontier out, int cluster) {
-  __shared__ union { RowShared row; PruneShared prune; } sh;
+  __shared__ union {
+    RowShared row;
+    struct { unsigned long long barriers[2]; PruneShared prune; } then;       // (barriers keep their place)
+  } sh;
   __shared__ __align__(16) double s_w[kWCount];
   __shared__ int s_last;
   const int rank = cluster > 1 ? cluster_rank() : 0;
@@ -441,7 +493,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) expand_rows_prune_kernel(const _
   } else if (rank != 0) {
     return;
   }
-  prune_level_body<NT, ROUNDS, false>(t, level, out, nullptr, 0, b, sh.prune, s_w, nullptr);
+  prune_level_body<NT, ROUNDS, false>(t, level, out, nullptr, 0, b, sh.then.prune, s_w, nullptr);
 }
 
 template <typename... KArgs, typename... Args>

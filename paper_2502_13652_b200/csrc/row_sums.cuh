@@ -138,6 +138,22 @@ __device__ __forceinline__ void write_sums(RowResult *r, float Mf, float cM, dou
   r->fault = row_fault_bits(Mf, Sn, Tn);
 }
 
+// The result of a row that was given up: no candidates, and the fault that says so.
+__device__ __forceinline__ void give_up_row(const PassParams &p, int b, int j) {
+  const int lane = threadIdx.x & 31;
+  const size_t slot = (size_t)b * p.rows_per_seq_max + j;
+  for (int i = lane; i < p.K; i += 32) p.row_keys[slot * p.K + i] = 0ull;
+  if (lane == 0) {
+    RowResult r;
+    r.M = r.S = r.T = r.L = r.H = 0.0;
+    r.top = 0ull;
+    r.n_valid = 0;
+    r.fault = C2T_ST_INTERNAL;
+    p.rows[slot] = r;
+  }
+  __syncwarp();
+}
+
 constexpr int kPoolCap = 128;                       // keys ranked at a time
 
 // Ranks the first n keys of the pool: the K largest move to pool[0 .. K), sorted, 0-padded.  Returns how many there are.
