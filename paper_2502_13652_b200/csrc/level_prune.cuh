@@ -67,13 +67,6 @@ __device__ __forceinline__ double classify(int hidden, const double *w, double P
   return 1.0 / (1.0 + exp_shared(-((z[0] + z[1]) + (z[2] + z[3]))));
 }
 
-// Confidence of a child under the configured classifier, from the logarithms of its joint and its own probability.
-__device__ __noinline__ double confidence(int classifier, int hidden, const double *w, double logP, double lp, double H, double d) {
-  if (classifier == C2T_CLS_IDENTITY_COND) return exp_shared(lp);
-  const double P = exp_shared(logP);
-  return classifier == C2T_CLS_IDENTITY_JOINT ? P : classify(hidden, w, P, H, d);
-}
-
 // A row's merged sums, as one warp holds them.
 struct RowMerge {
   double M, S, T;              // row maximum; sums over every other element of e^(x - M) and e^(x - M)(x - M)
@@ -210,8 +203,7 @@ __device__ __noinline__ void rank_whole_keys(PruneShared &sh, int nc) {
 }
 
 // NT: threads of the CTA; b: the sequence; w: the classifier's staged weights.  records == nullptr: the rows come from
-// this context's own expand pass; else from gathered records of n_shards shards (gs: room for their merge).  rehearse: the same way over made-up
-// candidates, without a global access, for a kernel that still waits for its predecessor: its code is in the caches when it counts.
+// this context's own expand pass; else from gathered records of n_shards shards (gs: room for their merge).
 //   The work is a chain of dependent steps over at most F K candidates, on the critical path of every level, so it is short
 // in steps rather than in operations: every global load whose address does not depend on another is issued at the top
 // (frontier nodes carry their log-probabilities and path confidences with them for that), a thread keeps its
@@ -221,7 +213,7 @@ __device__ __noinline__ void rank_whole_keys(PruneShared &sh, int nc) {
 // own, loops that are not unrolled.
 template <int NT, int ROUNDS, bool GATHERED>
 __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, const c2t_frontier &out, const c2t_row_record *records,
-                                                 int n_shards, int b, PruneShared &sh, const double *w, GatherShared *gs, bool rehearse = false) {
+                                                 int n_shards, int b, PruneShared &sh, const double *w, GatherShared *gs) {
   constexpr int kRounds = ROUNDS, kNW = NT / 32;               // candidates per thread; warps
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int K = t.K, F = t.F;
@@ -230,30 +222,24 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
   const unsigned per_k = (65536u + (unsigned)K - 1u) / (unsigned)K;       // c / K = c per_k >> 16 for c < 1024, K <= 32
 
   // ---- loads (slots past the frontier's size hold anything: kept in bounds, unused)
-  int n = F, base = 0;
-  if (!rehearse) {
-    n = t.frontier_n[cur][b];
-    base = t.tree_n[b];
-  }
+  int n = t.frontier_n[cur][b];
+  const int base = t.tree_n[b];
   unsigned long long key[kRounds];
 #pragma unroll
   for (int r = 0; r < kRounds; ++r) {
     const int c = tid + r * NT;
-    key[r] = 0ull;
-    if (!GATHERED && !rehearse && c < F * K) key[r] = __ldcg(&t.row_keys[cbase + c]);
+    key[r] = !GATHERED && c < F * K ? __ldcg(&t.row_keys[cbase + c]) : 0ull;
   }
   const int jr = tid - (NT - 64), jf = tid - (NT - 32);        // the last two warps fetch the rows' and the frontier's data
   RowResult row;
-  row.M = row.S = row.L = row.H = 0.0;
-  row.fault = 0u;
   double2 sm = make_double2(0.0, 0.0);
-  if (!GATHERED && !rehearse && jr >= 0 && jr < F) {
+  if (!GATHERED && jr >= 0 && jr < F) {
     row = t.rows[fbase + jr];
     if (t.entropy_top_m > 0) sm = t.topm[fbase + jr];
   }
   int fnode = 0;
   double flogP = 0.0, fchat = 0.0;
-  if (!rehearse && jf >= 0 && jf < F) {
+  if (jf >= 0 && jf < F) {
     fnode = t.frontier_node[cur][fbase + jf];
     flogP = t.frontier_logP[cur][fbase + jf];
     fchat = t.frontier_chat[cur][fbase + jf];
@@ -270,7 +256,7 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
   __syncthreads();                                // (a CTA that serves several sequences: the last one's reads are done)
   if (!GATHERED) {
     if (jr >= 0 && jr < n) row_stats(t, row, sm, b, jr, sh);
-  } else if (!rehearse) {
+  } else {
     for (int j = warp; j < n; j += kNW) {
       uint32_t shard_faults = 0u;
       const RowMerge m = merge_row_records(t, records, n_shards, b, j, K, &gs->x[j * K], &gs->tok[j * K], &shard_faults, gs->stage[warp]);
@@ -312,20 +298,22 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
         const bool ok = tok[r] >= 0 && !sh.rowfault[j];
         const double lp = (x > kNegInfAsFinite) ? ((double)x - sh.rowM[j]) - sh.rowL[j] : -INFINITY;
         logP[r] = sh.flogP[j] + lp;                                             // Eq. 1 in log space
+        const double P = exp_shared(logP[r]);
         const double H = sh.rowH[j];
-        C[r] = ok ? confidence(t.classifier, t.hidden, w, logP[r], lp, H, (double)level) : NAN;
-        keep[r] = (ok && C[r] >= (double)t.beta) || rehearse;                   // first pruning
+        if (!ok) C[r] = NAN;
+        else if (t.classifier == C2T_CLS_IDENTITY_JOINT) C[r] = P;
+        else if (t.classifier == C2T_CLS_IDENTITY_COND) C[r] = exp_shared(lp);
+        else C[r] = classify(t.hidden, w, P, H, (double)level);
+        keep[r] = ok && C[r] >= (double)t.beta;                                 // first pruning
         // (C desc, index asc) as integer compares: an orderable image of C, 0 for a dropped candidate
         const unsigned long long cb = (unsigned long long)__double_as_longlong(C[r]);
-        sh.ckey[c] = keep[r] ? (rehearse ? (unsigned long long)(c + 1) << 32 : cb ^ ((cb >> 63) ? ~0ull : 0x8000000000000000ull)) : 0ull;
+        sh.ckey[c] = keep[r] ? (cb ^ ((cb >> 63) ? ~0ull : 0x8000000000000000ull)) : 0ull;
         sh.chi[c] = (unsigned)(sh.ckey[c] >> 32);
-        if (!rehearse) {
-          t.cand_token[cbase + c] = tok[r];
-          t.cand_lp[cbase + c] = ok ? lp : NAN;
-          t.cand_logP[cbase + c] = ok ? logP[r] : NAN;
-          t.cand_H[cbase + c] = ok ? H : NAN;
-          t.cand_C[cbase + c] = C[r];
-        }
+        t.cand_token[cbase + c] = tok[r];
+        t.cand_lp[cbase + c] = ok ? lp : NAN;
+        t.cand_logP[cbase + c] = ok ? logP[r] : NAN;
+        t.cand_H[cbase + c] = ok ? H : NAN;
+        t.cand_C[cbase + c] = C[r];
       }
       n_keep += __syncthreads_count(keep[r]);
     }
@@ -401,7 +389,7 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
     const int c = tid + r * NT;
     if (r * NT >= nc) break;                      // (uniform)
     const int before = __reduce_add_sync(kFullMask, lane < r * kNW + warp ? counts : 0);
-    if (c >= nc || rehearse) continue;
+    if (c >= nc) continue;
     t.cand_flags[cbase + c] = (keep[r] ? 1 : 0) | (sel[r] ? 2 : 0);
     if (!(add_all ? keep[r] : sel[r])) continue;
     const unsigned lt = (1u << lane) - 1u;
@@ -427,7 +415,7 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
       if (out.parent_slot) out.parent_slot[fbase + slot] = j;
     }
   }
-  if (tid == 0 && !rehearse) {
+  if (tid == 0) {
     const int next_n = overflow ? 0 : tot_sel;
     t.tree_n[b] = overflow ? t.cap : base + tot_add;
     t.frontier_n[nxt][b] = next_n;

@@ -470,7 +470,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) expand_rows_prune_kernel(const _
   } sh;
   __shared__ __align__(16) double s_w[kWCount];
   __shared__ int s_last;
-  __shared__ volatile double s_rehearsed;
   const int rank = cluster > 1 ? cluster_rank() : 0;
   chain_release();
   open_row(sh.row, cluster);
@@ -483,8 +482,6 @@ __global__ void __launch_bounds__(NT, 512 / NT) expand_rows_prune_kernel(const _
   if (j >= n && !(n <= 0 && j == 0)) return;
   if (n > 0) {
     if (!expand_row<BF16, NT>(p, sh.row, b, j, cluster, rank)) return;
-    // while two warps write the row's result: the classifier's code into the caches
-    if (threadIdx.x >= NT - 32) s_rehearsed = confidence(t.classifier, t.hidden, s_w, -1.0, -1.0, 1.0, 0.0);
     __syncthreads();                                 // the row's result, before its count
     if (threadIdx.x == 0) {
       int done;                                      // released: this row's result; acquired: those of the rows before it

@@ -72,12 +72,8 @@ __global__ void __launch_bounds__(kTreeThreads) prune_level_kernel(TreeState t, 
   GatherShared *gs = reinterpret_cast<GatherShared *>(s_prune + sizeof(PruneShared));
   chain_release();
   stage_classifier(t, s_w, threadIdx.x, kTreeThreads);   // (written at init, not by the chain: while the expand pass is finishing)
-  // once without a global access while the expand pass is finishing, once in earnest
-#pragma unroll 1
-  for (int pass = 0; pass < 2; ++pass) {
-    if (pass == 1) chain_wait();
-    prune_level_body<kTreeThreads, ROUNDS, GATHERED>(t, level, out, records, n_shards, blockIdx.x, sh, s_w, gs, pass == 0);
-  }
+  chain_wait();
+  prune_level_body<kTreeThreads, ROUNDS, GATHERED>(t, level, out, records, n_shards, blockIdx.x, sh, s_w, gs);
 }
 constexpr int kPruneRounds = kMaxCand / kTreeThreads;
 
