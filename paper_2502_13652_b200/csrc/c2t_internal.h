@@ -142,6 +142,7 @@ struct PassParams {
   SumRecord *sums;                  // [chunk] at a warp's last chunk of a row
   int64_t n_chunks, n_segs;
   int32_t cta_tasks;                // barriers in a CTA's shared memory (set at launch)
+  int32_t near_cells;               // where the cells of a CTA's own rows begin in its shared memory, 0: in the workspace (set at launch)
   int32_t wait_limit;               // tries of such a barrier (set at launch)
   // expand with M > 0 (else null): the pool of candidate vectors, cut evenly among the warps, and a record per segment
   uint4 *topm_pool;

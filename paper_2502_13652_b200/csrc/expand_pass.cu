@@ -240,6 +240,14 @@ struct CtaRange {
   }
 };
 
+// The cells of a row: in shared memory where there is room for those of all rows inside the CTA's range (`near`, else null), in the
+// workspace for a row that it shares.  fp32 rows only: eight levels of 320 rows of 128256 tokens (with the acceptance) 403 -> 397 us; the
+// bf16 stream, which has no time to spare, loses by the other kind of store (640 rows 465 -> 468).
+template <bool BF16, bool TOPM>
+__device__ __forceinline__ uint32_t *cells_of_row(const PassParams &p, uint32_t *near, const CtaRange<TOPM> &cr, const RowShape<BF16> &rs, int a) {
+  return near && a >= cr.in0 && a < cr.in1 ? near + (size_t)(a - cr.in0) * rs.words * 32 : p.cells + (size_t)a * rs.words * 32;
+}
+
 // ---------------------------------------------------------------- completing a row
 
 // vector k of the lane's 8 in a chunk
@@ -284,7 +292,7 @@ __device__ __forceinline__ unsigned reached(const float (&v)[N], float x) {
 // taken whole here: with the rounded ones every chunk of a masked fp32 row stays in question (four levels of 320 rows of
 // 128256 values, six of them finite: 2085 us, so 223).
 template <bool BF16>
-__device__ __noinline__ int select_in_order(const PassParams &p, PairShared *ws, const char *row, int a, float floor) {
+__device__ __noinline__ int select_in_order(const PassParams &p, PairShared *ws, const char *row, const uint32_t *cells, int a, float floor) {
   constexpr int kWords = 8;                         // words of cells of a lane at a time
   constexpr int kBatch = 16;                        // elements of a lane in flight
   const RowShape<BF16> rs(p.V);
@@ -297,7 +305,7 @@ __device__ __noinline__ int select_in_order(const PassParams &p, PairShared *ws,
 #pragma unroll
     for (int i = 0; i < kWords; ++i) {
       const size_t at = ((size_t)a * rs.words + w0 + i) * 32 + lane;
-      two[i] = w0 + i < rs.words ? p.cells[at] : 0xFF80FF80u;
+      two[i] = w0 + i < rs.words ? cells[(w0 + i) * 32 + lane] : 0xFF80FF80u;
       low[i] = !BF16 && w0 + i < rs.words ? p.cell_low[at] : 0u;
     }
 #pragma unroll
@@ -394,12 +402,12 @@ __device__ __forceinline__ int gather_keys(PairShared *ws, const char *row, cons
 
 // The K largest.
 template <bool BF16>
-__device__ __forceinline__ void complete_keys(const PassParams &p, PairShared *ws, int a, int b, int j) {
+__device__ __forceinline__ void complete_keys(const PassParams &p, PairShared *ws, const uint32_t *row_cells, int a, int b, int j) {
   constexpr int kBatch = 32;                        // words of its column that a lane holds at a time: 64 chunks
   const RowShape<BF16> rs(p.V);
   const int lane = threadIdx.x & 31, K = p.K;
   const char *row = row_pointer(p, b, j, BF16 ? 2 : 4);
-  const uint32_t *cells = p.cells + (size_t)a * rs.words * 32 + lane;
+  const uint32_t *cells = row_cells + lane;
   uint32_t v[kBatch], cm2 = kLowestBf16x2;
 #pragma unroll
   for (int i = 0; i < kBatch; ++i) v[i] = i < rs.words ? cells[i * 32] : kLowestBf16x2;
@@ -482,7 +490,7 @@ __device__ __forceinline__ void complete_keys(const PassParams &p, PairShared *w
   }
   __syncwarp();
   const int n_keys = n_list <= kListCap ? gather_keys<BF16>(ws, row, rs, p.V, floor, n_list) : -1;
-  const int n_valid = n_keys >= 0 ? rank_pool(ws->pool, n_keys, K) : select_in_order<BF16>(p, ws, row, a, floor);
+  const int n_valid = n_keys >= 0 ? rank_pool(ws->pool, n_keys, K) : select_in_order<BF16>(p, ws, row, row_cells, a, floor);
   const size_t slot = (size_t)b * p.rows_per_seq_max + j;
   for (int i = lane; i < K; i += 32) p.row_keys[slot * K + i] = ws->pool[i];
   if (lane == 0) {
@@ -654,7 +662,7 @@ __device__ __forceinline__ float stream_chunk(uint4 (&q)[kGroups][4], const uint
 
 // One warp's stream: every kStreamWarps-th chunk of the CTA's work order (TOPM: a contiguous part of it).
 template <bool BF16, bool TOPM>
-__device__ __forceinline__ void stream(const PassParams &p, CtaShared *cs, const int *s_off, const RowShape<BF16> &rs, const CtaRange<TOPM> &cr) {
+__device__ __forceinline__ void stream(const PassParams &p, CtaShared *cs, const int *s_off, uint32_t *near, const RowShape<BF16> &rs, const CtaRange<TOPM> &cr) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = cr.u1 - cr.u0, step = TOPM ? 1 : kStreamWarps;
   int i = TOPM ? warp * cr.part : warp;
@@ -733,8 +741,8 @@ __device__ __forceinline__ void stream(const PassParams &p, CtaShared *cs, const
     const int u = a * rs.nc + ch;
     fresh = !more || na != a;
     if (C2T_IN_BOUNDS(u, p.n_chunks, p.status)) {
-      uint32_t *word = p.cells + ((size_t)a * rs.words + (ch >> 1)) * 32 + lane;
-      uint32_t *low = BF16 ? nullptr : p.cell_low + (word - p.cells);
+      uint32_t *word = cells_of_row(p, near, cr, rs, a) + (ch >> 1) * 32 + lane;
+      uint32_t *low = BF16 ? nullptr : p.cell_low + ((size_t)a * rs.words + (ch >> 1)) * 32 + lane;
       if (ch + 1 == rs.nc && !(ch & 1)) {            // (no second cell)
         *word = cell_bits(cv, BF16) | (kLowestBf16x2 & 0xFFFF0000u);
         if (!BF16) *low = __float_as_uint(cv) & 0xFFFFu;
@@ -784,7 +792,7 @@ __device__ __forceinline__ bool wait_task(unsigned long long *bar_ptr, int limit
 // shared one if this CTA's part of it was the last.  A row whose records do not come in time is given up: it gets a result
 // that faults its sequence, and nothing of it stays behind for later rows or launches.
 template <bool BF16, bool TOPM>
-__device__ __forceinline__ void complete(const PassParams &p, CtaShared *cs, const int *s_off, const RowShape<BF16> &rs, const CtaRange<TOPM> &cr) {
+__device__ __forceinline__ void complete(const PassParams &p, CtaShared *cs, const int *s_off, uint32_t *near, const RowShape<BF16> &rs, const CtaRange<TOPM> &cr) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pair = warp >> 1, role = warp & 1;
   const int n_tasks = cr.n_tasks();
   pair_barrier(pair);                                // (both have done with streaming)
@@ -809,7 +817,7 @@ __device__ __forceinline__ void complete(const PassParams &p, CtaShared *cs, con
     const int a = cr.task_row(k), b = find_sequence(s_off, p.B, a);
     if (go == kRowBroken) {
       if (role == 0) give_up_row(p, b, a - s_off[b]);
-    } else if (role == 0) complete_keys<BF16>(p, &cs->scratch[pair], a, b, a - s_off[b]);
+    } else if (role == 0) complete_keys<BF16>(p, &cs->scratch[pair], cells_of_row(p, near, cr, rs, a), a, b, a - s_off[b]);
     else complete_sums<BF16, TOPM>(p, cr, a, b, a - s_off[b]);
   }
 }
@@ -819,6 +827,7 @@ template <bool BF16, bool TOPM>
 __device__ __forceinline__ void expand_pass_body(const PassParams &p, unsigned char *s_dyn) {
   CtaShared *cs = reinterpret_cast<CtaShared *>(s_dyn);
   int *s_off = reinterpret_cast<int *>(cs->bars() + p.cta_tasks);
+  uint32_t *near = !BF16 && p.near_cells ? reinterpret_cast<uint32_t *>(s_dyn + p.near_cells) : nullptr;
   const int n_rows = build_row_offsets(p.counts, p.B, p.rows_per_seq_max, s_off);
   const RowShape<BF16> rs(p.V);
   const CtaRange<TOPM> cr(rs.nc, n_rows * rs.nc);
@@ -837,9 +846,9 @@ __device__ __forceinline__ void expand_pass_body(const PassParams &p, unsigned c
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(cr.task_records(cr.task_row(k))) : "memory");
   }
   if (threadIdx.x == kExpandThreads - 1) cs->task = 0;
-  if (threadIdx.x < kStreamWarps * 32) stream<BF16, TOPM>(p, cs, s_off, rs, cr);
+  if (threadIdx.x < kStreamWarps * 32) stream<BF16, TOPM>(p, cs, s_off, near, rs, cr);
   else __syncthreads();
-  complete<BF16, TOPM>(p, cs, s_off, rs, cr);
+  complete<BF16, TOPM>(p, cs, s_off, near, rs, cr);
 }
 
 template <bool BF16, bool TOPM>
@@ -912,14 +921,19 @@ int c2t_debug_task_wait_limit = kTaskWaitLimit;
 #endif
 
 // the launch's shared memory and limits
-static size_t plan_shared(PassParams &p, int grid) {
+constexpr size_t kPassSharedBytes = 100 * 1024;        // more than plan_shared's fixed part at the limits of a configuration
+static size_t plan_shared(PassParams &p, int elem_bytes, int grid) {
   p.wait_limit = C2T_TASK_WAIT_LIMIT;
   p.cta_tasks = (int)((long long)p.B * p.rows_per_seq_max / grid) + 4;       // rows inside a CTA's range, and the two it shares
-  return sizeof(CtaShared) + (size_t)p.cta_tasks * sizeof(unsigned long long) + ((size_t)p.B + 1) * sizeof(int);
+  const size_t fixed = sizeof(CtaShared) + (size_t)p.cta_tasks * sizeof(unsigned long long) + ((size_t)p.B + 1) * sizeof(int);
+  const long long nc = row_chunks(p.V, elem_bytes), per_cta = ((long long)p.B * p.rows_per_seq_max * nc + grid - 1) / grid;
+  const size_t at = (fixed + 127) & ~(size_t)127, cells = (size_t)(per_cta / nc + 1) * ((nc + 1) / 2) * 128;
+  p.near_cells = elem_bytes == 4 && at + cells <= kPassSharedBytes ? (int)at : 0;
+  return p.near_cells ? at + cells : fixed;
 }
 
 cudaError_t prepare_expand_pass() {
-  const int bytes = 100 * 1024;                      // more than plan_shared asks for at the limits of a configuration
+  const int bytes = (int)kPassSharedBytes;
   cudaError_t e = cudaFuncSetAttribute(expand_pass_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_pass_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_pass_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -940,7 +954,7 @@ cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, con
   if (out) o = *out;
   const RowPlan plan = rows_in_registers(p, dtype, grid);
   if (plan.cluster) return launch_expand_rows_prune(p, t, level, o, dtype, plan, s);
-  size_t smem = plan_shared(p, grid);
+  size_t smem = plan_shared(p, dtype == C2T_BF16 ? 2 : 4, grid);
   if (smem < sizeof(PruneShared)) smem = sizeof(PruneShared);
   if (dtype == C2T_BF16)
     return launch_chained(expand_prune_kernel<true>, dim3(grid), dim3(kExpandThreads), smem, s, p, t, level, o);
@@ -950,7 +964,7 @@ cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, con
 cudaError_t launch_expand_pass(PassParams p, int dtype, int grid, cudaStream_t s) {
   const RowPlan plan = rows_in_registers(p, dtype, grid);
   if (plan.cluster) return launch_expand_rows(p, dtype, plan, s);
-  const size_t smem = plan_shared(p, grid);
+  const size_t smem = plan_shared(p, dtype == C2T_BF16 ? 2 : 4, grid);
   const bool bf16 = dtype == C2T_BF16;
   if (p.topm_pool) {                                 // also sets the candidates of Eq. 3 aside
     if (bf16) return launch_chained(expand_pass_kernel<true, true>, dim3(grid), dim3(kExpandThreads), smem, s, p);

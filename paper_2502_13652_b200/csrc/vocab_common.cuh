@@ -109,29 +109,35 @@ struct Vec {
   }
 };
 
-// Exclusive prefix sums of the clamped per-sequence row counts into s_off[0..B]; returns the total.
+// Exclusive prefix sums of the clamped per-sequence row counts into s_off[0..B]; returns the total.  By one warp, four counts of a lane in
+// flight, with one barrier: every level begins with it.
 __device__ int build_row_offsets(const int32_t *counts, int B, int cap, int *s_off) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  for (int i = tid; i < B; i += blockDim.x) {
-    int c = counts[i];
-    s_off[i + 1] = c < 0 ? 0 : (c > cap ? cap : c);
-  }
-  if (tid == 0) s_off[0] = 0;
-  __syncthreads();
-  if (tid < 32) {
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 32) {
     int carry = 0;
-    for (int base = 1; base <= B; base += 32) {
-      int i = base + lane;
-      int v = i <= B ? s_off[i] : 0;
+    for (int base = 0; base < B; base += 128) {
+      int v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = base + u * 32 + lane, c = i < B ? counts[i] : 0;
+        v[u] = c < 0 ? 0 : (c > cap ? cap : c);
+      }
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        int t = __shfl_up_sync(kFull, v, o);
-        if (lane >= o) v += t;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int t = __shfl_up_sync(kFull, v[u], o);
+          if (lane >= o) v[u] += t;
+        }
       }
-      v += carry;
-      if (i <= B) s_off[i] = v;
-      carry = __shfl_sync(kFull, v, 31);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = base + u * 32 + lane;
+        if (i < B) s_off[i + 1] = v[u] + carry;
+        carry += __shfl_sync(kFull, v[u], 31);
+      }
     }
+    if (lane == 0) s_off[0] = 0;
   }
   __syncthreads();
   return s_off[B];
