@@ -305,7 +305,7 @@ __device__ __noinline__ int select_in_order(const PassParams &p, PairShared *ws,
 #pragma unroll
     for (int i = 0; i < kWords; ++i) {
       const size_t at = ((size_t)a * rs.words + w0 + i) * 32 + lane;
-      two[i] = w0 + i < rs.words ? cells[(w0 + i) * 32 + lane] : 0xFF80FF80u;
+      two[i] = w0 + i < rs.words ? (BF16 ? p.cells[at] : cells[(w0 + i) * 32 + lane]) : 0xFF80FF80u;
       low[i] = !BF16 && w0 + i < rs.words ? p.cell_low[at] : 0u;
     }
 #pragma unroll
@@ -407,7 +407,7 @@ __device__ __forceinline__ void complete_keys(const PassParams &p, PairShared *w
   const RowShape<BF16> rs(p.V);
   const int lane = threadIdx.x & 31, K = p.K;
   const char *row = row_pointer(p, b, j, BF16 ? 2 : 4);
-  const uint32_t *cells = row_cells + lane;
+  const uint32_t *cells = (BF16 ? p.cells + (size_t)a * rs.words * 32 : row_cells) + lane;
   uint32_t v[kBatch], cm2 = kLowestBf16x2;
 #pragma unroll
   for (int i = 0; i < kBatch; ++i) v[i] = i < rs.words ? cells[i * 32] : kLowestBf16x2;
@@ -741,8 +741,9 @@ __device__ __forceinline__ void stream(const PassParams &p, CtaShared *cs, const
     const int u = a * rs.nc + ch;
     fresh = !more || na != a;
     if (C2T_IN_BOUNDS(u, p.n_chunks, p.status)) {
-      uint32_t *word = cells_of_row(p, near, cr, rs, a) + (ch >> 1) * 32 + lane;
-      uint32_t *low = BF16 ? nullptr : p.cell_low + ((size_t)a * rs.words + (ch >> 1)) * 32 + lane;
+      uint32_t *word = p.cells + ((size_t)a * rs.words + (ch >> 1)) * 32 + lane;
+      uint32_t *low = BF16 ? nullptr : p.cell_low + (word - p.cells);
+      if (!BF16) word = cells_of_row(p, near, cr, rs, a) + (ch >> 1) * 32 + lane;
       if (ch + 1 == rs.nc && !(ch & 1)) {            // (no second cell)
         *word = cell_bits(cv, BF16) | (kLowestBf16x2 & 0xFFFF0000u);
         if (!BF16) *low = __float_as_uint(cv) & 0xFFFFu;
@@ -817,7 +818,7 @@ __device__ __forceinline__ void complete(const PassParams &p, CtaShared *cs, con
     const int a = cr.task_row(k), b = find_sequence(s_off, p.B, a);
     if (go == kRowBroken) {
       if (role == 0) give_up_row(p, b, a - s_off[b]);
-    } else if (role == 0) complete_keys<BF16>(p, &cs->scratch[pair], cells_of_row(p, near, cr, rs, a), a, b, a - s_off[b]);
+    } else if (role == 0) complete_keys<BF16>(p, &cs->scratch[pair], BF16 ? nullptr : cells_of_row(p, near, cr, rs, a), a, b, a - s_off[b]);
     else complete_sums<BF16, TOPM>(p, cr, a, b, a - s_off[b]);
   }
 }
