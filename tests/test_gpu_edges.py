@@ -318,3 +318,71 @@ def test_rows_of_one_value_but_for_a_few(dtype, mask, V):
     x = x.to(dtype)
     rep = run_and_compare(ocfg, gcfg, [x], target, root, prefix, draft_dev=[rows(x)], target_dev=rows(target))
     assert rep.status_bits == 0
+
+
+# Rows in registers: a block of 256 threads holds 2048 vectors of 16 bytes, eight of them 16384; beyond that blocks of 512, up to 32768;
+# longer rows are streamed.
+@pytest.mark.parametrize("dtype,V", [(torch.bfloat16, 16384), (torch.bfloat16, 16385), (torch.bfloat16, 131072), (torch.bfloat16, 131073),
+                                     (torch.float32, 8191), (torch.float32, 8193), (torch.float32, 65537), (torch.float32, 131072),
+                                     (torch.float32, 131073)])
+def test_rows_around_a_block_of_registers(dtype, V):
+    step(1, V, 2, 3, 3, 6, 0.0, dtype, classifier="identity")
+
+
+@pytest.mark.parametrize("dtype,chunk", [(torch.bfloat16, 2048), (torch.float32, 1024)])
+@pytest.mark.parametrize("n,plus", [(1, -1), (1, 1), (2, 5), (12, 1)])
+def test_streamed_rows_around_chunk_edges(dtype, chunk, n, plus):
+    """Level 1 has 320 rows, too many for the registers (296 blocks): cut into chunks and streamed."""
+    step(160, n * chunk + plus, 2, 2, 2, 4, 0.0, dtype, classifier="identity")
+
+
+@pytest.mark.parametrize("B", [2, 60])
+def test_cap_between_confidences_with_equal_upper_halves(B):
+    """Sixteen children one unit in the last place of their fp32 logits apart (1e-6 in their probabilities): the upper 32 bits of
+    neighbouring confidences are equal, so the frontier cap in their middle goes by the whole keys."""
+    V, F, D = 9000, 8, 2
+    g = torch.Generator().manual_seed(5)
+    draft = []
+    for _ in range(D):
+        x = torch.randn(B, F, V, generator=g)
+        for b in range(B):
+            for j in range(F):
+                at = torch.randperm(V, generator=g)[:16]
+                x[b, j, at] = 10.0 + 0.31 * j + torch.arange(16) * 2.0 ** -20
+        draft.append(x)
+    step(B, V, D, 16, F, 12, 0.0, torch.float32, draft=draft, classifier="identity")
+
+
+@pytest.mark.parametrize("B,V,dtype", [(1, 32000, torch.float32), (5, 9001, torch.bfloat16), (40, 20000, torch.bfloat16)])
+def test_step_in_one_call_equals_single_calls(B, V, dtype):
+    """c2t_decode_step (levels in one launch, or streamed and pruned) against separate expand and prune calls: bit for bit."""
+    D, K, F, N = 4, 6, 9, 30
+    _, cfg = make_configs(B, V, D, K, F, N, 0.3, dtype)
+    pad = -(-V // 8) * 8
+    draft, target, root, prefix = gen_inputs(B, V, D, F, c2t.c2t_final_width(cfg), dtype)
+
+    def rows(t):
+        buf = torch.zeros(t.shape[0], t.shape[1], pad, dtype=dtype, device="cuda")
+        buf[:, :, :V] = t.cuda()
+        return buf[:, :, :V]
+
+    draft = [rows(t) for t in draft]; target = rows(target); root = root.cuda(); prefix = prefix.cuda()
+    ctx = c2t.Context(cfg)
+    got = []
+    for single in (False, True):
+        if single:
+            ctx.c2t_begin_step(root, prefix)
+            for l in range(D):
+                ctx.c2t_expand_level(l, draft[l]); ctx.c2t_prune(l)
+            ctx.c2t_prune(c2t.FINAL); ctx.c2t_build_verify(); ctx.c2t_accept(target)
+        else:
+            ctx.decode_step(draft, target, root, prefix)
+        torch.cuda.synchronize()
+        v = ctx.c2t_get_view()
+        live = torch.arange(ctx.cap, device="cuda")[None, :] < v["tree_n"][:, None]
+        got.append([t.clone() for t in list(ctx.verify.values()) + list(ctx.accepted.values()) + list(ctx.frontier.values())] +
+                   [v["tree_n"].clone(), torch.where(live, v["tree_logP"], 0.0), torch.where(live, v["tree_C"], 0.0)])
+    assert ctx.c2t_status()[0] == 0 and int(got[0][-3].max()) > 1
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+    ctx.close()
