@@ -24,10 +24,17 @@ constexpr int kCtaKeys = 64;                          // keys that a block hands
 constexpr int kTooMany = 1 << 20;
 static_assert(kRowGroups >= C2T_MAX_TOPK && kMaxRowGroups >= kRowGroups, "");
 
+// A warp's sums, relative to an integer offset, and how often it holds the row's maximum.
+struct alignas(16) RowSums {
+  double S, U;
+  float offset;
+  int equals;
+};
+
 struct RowShared {
   unsigned long long maxima_in, results_in;           // transaction barriers: all groups' maxima; everything for the row's result
   __align__(16) float group[kMaxRowGroups];           // the maxima of the row's groups
-  float4 sums[kRowCluster * kMaxRowWarps];            // in the leading block: S, U, offset of every warp, and how often it holds the maximum (int bits)
+  RowSums sums[kRowCluster * kMaxRowWarps];           // in the leading block
   unsigned long long keys[kRowCluster][kCtaKeys];     // in the leading block: what every block hands over
   __align__(16) int counts[kRowCluster];              // how many
   unsigned long long pool[kPoolCap];                  // this block's keys; in the leading one then the row's
@@ -61,9 +68,8 @@ __device__ __forceinline__ void send(uint32_t at, uint32_t v, uint32_t bar) {
 __device__ __forceinline__ void send(uint32_t at, unsigned long long v, uint32_t bar) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(at), "l"(v), "r"(bar) : "memory");
 }
-__device__ __forceinline__ void send(uint32_t at, float a, float b, float c, float d, uint32_t bar) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
-               ::"r"(at), "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(__float_as_uint(c)), "r"(__float_as_uint(d)), "r"(bar) : "memory");
+__device__ __forceinline__ void send(uint32_t at, unsigned long long a, unsigned long long b, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(at), "l"(a), "l"(b), "r"(bar) : "memory");
 }
 // an arrival at a block's barrier that announces bytes to it
 __device__ __forceinline__ void announce(uint32_t bar, uint32_t bytes) {
@@ -195,18 +201,23 @@ __device__ __noinline__ int select_by_rounds(RowShared &sh, const RowPart<BF16, 
   return r;
 }
 
-// A warp's sums, from its lanes' (s, u) relative to their offsets c; m2 the largest values they come from: in lane 0, relative to cw.
-__device__ __forceinline__ void warp_sums(float &s, float &u, float c, float m2, float &cw) {
-  cw = offset_of(warp_max(m2));
-  const float by = fmaxf(cw - c, -127.f);
-  const float two = __int_as_float((__float_as_int(by + 12582912.f) << 23) + 0x3F800000);      // 2^by, 0 for -127
-  u = two * fmaf(by, s, u);
-  s = two * s;
+// A warp's sums, from its lanes' (s, u) relative to their offsets c; m2 the largest values they come from.  In double precision: a row's
+// sums are mostly a few large elements, which fp32 would round five more times (32000 tokens, scale 4: 1.1e-8 r.m.s. in a probability, so
+// rounded 1.6e-8).
+__device__ __forceinline__ RowSums warp_sums(float s, float u, float c, float m2) {
+  RowSums r;
+  r.offset = offset_of(warp_max(m2));
+  r.equals = 0;
+  const float by = fmaxf(r.offset - c, -2000.f);      // (never positive)
+  const double f = pow2_f64(by);
+  r.S = f * (double)s;
+  r.U = f * ((double)u + (double)by * (double)s);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    s += __shfl_xor_sync(kFull, s, o);
-    u += __shfl_xor_sync(kFull, u, o);
+    r.S += __shfl_xor_sync(kFull, r.S, o);
+    r.U += __shfl_xor_sync(kFull, r.U, o);
   }
+  return r;
 }
 
 // One lane's vectors, in sh.again, summed again without the row's maximum and its equals, by the whole warp.
@@ -238,12 +249,12 @@ __device__ __forceinline__ void merge_sums(RowShared &sh, RowResult *out, float 
 #pragma unroll
   for (int i = 0; i < kPer; ++i) {
     if (i * 32 + lane < warps) {
-      const float4 r = sh.sums[i * 32 + lane];
-      const float d = fmaxf(cM - r.z, -2000.f);       // (never positive)
+      const RowSums r = sh.sums[i * 32 + lane];
+      const float d = fmaxf(cM - r.offset, -2000.f);  // (never positive)
       const double f = pow2_f64(d);
-      S += f * (double)r.x;
-      U += f * ((double)r.y + (double)d * (double)r.x);
-      equals += __float_as_int(r.w);
+      S += f * r.S;
+      U += f * (r.U + (double)d * r.S);
+      equals += r.equals;
     }
   }
   S = warp_sum(S);
@@ -314,8 +325,7 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
       if (k * NT < rp.part) acc_vector<BF16>(acc, q[k], scale, c2);      // (uniform)
     acc.totals(s, u);
   }
-  float sw = s, uw = u, cw;
-  warp_sums(sw, uw, c, mt, cw);
+  RowSums sums = warp_sums(s, u, c, mt);
   bool ok = true;
   if (cluster > 1) ok = wait_bar(&sh.maxima_in);
   else __syncthreads();
@@ -358,7 +368,7 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
     if (cluster > 1) {
       if (lane < cluster) {
         const uint32_t bar = place_in(&sh.results_in, lane);
-        announce(bar, lane == 0 ? (uint32_t)(4 + kW * 16 + handed * 8) : 4u);
+        announce(bar, lane == 0 ? (uint32_t)(4 + kW * 24 + handed * 8) : 4u);
         send(place_in(&sh.counts[rank], lane), (uint32_t)c_n, bar);
       }
       const uint32_t bar = place_in(&sh.results_in, 0);
@@ -371,11 +381,9 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
   }
 
   // ---- the warps' sums; the warp that holds the maximum: such lanes again without it
-  int equals = 0;
   if (unsigned left = __ballot_sync(kFull, mt == Mf)) {
-    float m2 = mt, cs = c;
-    sw = s;
-    uw = u;
+    float m2 = mt, cs = c, sw = s, uw = u;
+    int equals = 0;
     for (; left; left &= left - 1u) {
       const bool mine = lane == __ffs(left) - 1;
       __syncwarp();
@@ -388,13 +396,18 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
       sum_again<BF16>(sh, Mf, &sr, &ur, &cr, &mr, &equals);
       if (mine) { sw = sr; uw = ur; cs = cr; m2 = mr; }
     }
-    warp_sums(sw, uw, cs, m2, cw);
-    equals = __reduce_add_sync(kFull, equals);
+    sums = warp_sums(sw, uw, cs, m2);
+    sums.equals = __reduce_add_sync(kFull, equals);
   }
   if (lane == 0) {
-    float4 *record = &sh.sums[rank * kW + warp];
-    if (cluster > 1) send(place_in(record, 0), sw, uw, cw, __int_as_float(equals), place_in(&sh.results_in, 0));
-    else *record = make_float4(sw, uw, cw, __int_as_float(equals));
+    RowSums *record = &sh.sums[rank * kW + warp];
+    if (cluster > 1) {
+      const uint32_t bar = place_in(&sh.results_in, 0);
+      send(place_in(record, 0), (unsigned long long)__double_as_longlong(sums.S), (unsigned long long)__double_as_longlong(sums.U), bar);
+      send(place_in(&record->offset, 0), (unsigned long long)(uint32_t)sums.equals << 32 | __float_as_uint(sums.offset), bar);
+    } else {
+      *record = sums;
+    }
   }
   __syncwarp();
   if (cluster > 1) {
