@@ -137,7 +137,8 @@ struct PassParams {
   // expand: results per row, and what the warps that stream a row leave for the pair that completes it
   RowResult *rows;                  // [B, F]
   unsigned long long *row_keys;     // [B, F, K] the row's K largest keys, sorted descending, 0-padded
-  int32_t *row_done;                // [B * F] finished chunks of a row shared by several CTAs; 0 between launches
+  int32_t *row_done;                // [B * F] finished chunks of a row shared by several CTAs (rows in registers: [b F] finished rows of sequence b);
+                                    // 0 between launches
   uint32_t *cells, *cell_low;       // [row, two chunks, 32] lane maxima, rounded; fp32: their lower halves (expand_pass.cu)
   SumRecord *sums;                  // [chunk] at a warp's last chunk of a row
   int64_t n_chunks, n_segs;
