@@ -177,7 +177,7 @@ int c2t_prune(c2t_ctx *ctx, int level, const c2t_frontier *out, void *stream);
 /*
  * c2t_expand_level(level, ...) followed by c2t_prune(level, out), as one call (Sec. 4.2.1, Eq. 1-2, Eq. 4,
  * Alg. 1, Sec. 4.2.2: the same operations, the same results bit for bit).  For batches of at most
- * C2T_FUSED_MAX_BATCH sequences (the paper's own operating point is one sequence), and for levels whose rows all
+ * C2T_FUSED_MAX_BATCH sequences (the paper's own operating point is one sequence), and for levels of long rows that all
  * fit the chip's registers at once, it is ONE kernel launch:
  * the thread block that finishes the vocabulary pass (of a sequence) last does the per-sequence work, which halves the
  * launch-to-launch latency that bounds such a step.  Larger levels, and contexts with entropy_top_m > 0,

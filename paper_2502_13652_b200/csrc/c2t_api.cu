@@ -159,6 +159,8 @@ int rows_bound(const TreeState &t, int level) {
   return bound < t.F ? (int)bound : t.F;
 }
 
+constexpr long long kFusedRowBytes = 32768;            // half of what a block of 512 threads holds
+
 // the expand pass of a level over rows of `vocab` tokens (the whole vocabulary, or one shard of it)
 PassParams expand_params(const TreeState &t, int level, const void *logits, int64_t seq_stride, int64_t row_stride, int vocab) {
   PassParams p;
@@ -395,9 +397,11 @@ int c2t_expand_prune_level(c2t_ctx *ctx, int level, const void *logits_dev, int6
                            const c2t_frontier *out, void *stream) {
   if (!ctx || !logits_dev) return C2T_EINVAL;
   const TreeState &t = ctx->t;
-  // one launch where a level is small: few sequences, or the rows in registers
+  // One launch where a level is small: few sequences, or long rows in registers (80 rows of 32000 bf16 tokens: 14.3 us a level in two
+  // launches, 12.8 in one).  Short rows, and candidates for which a block's threads do not suffice, leave the pruning too much of the time.
+  const RowPlan rows = row_pass_plan(t.V, (int)ctx->elem_bytes, (long long)t.B * rows_bound(t, level), ctx->grid_expand);
   const bool small = t.B <= C2T_FUSED_MAX_BATCH ||
-                     row_pass_plan(t.V, (int)ctx->elem_bytes, (long long)t.B * rows_bound(t, level), ctx->grid_expand).cluster > 0;
+                     (rows.cluster > 0 && t.V * (long long)ctx->elem_bytes >= kFusedRowBytes && t.F * t.K <= rows.threads);
   if (!small || (t.entropy_top_m > 0 && t.entropy_top_m < t.V)) {
     const int rc = c2t_expand_level(ctx, level, logits_dev, seq_stride, row_stride, stream);
     return rc != C2T_OK ? rc : c2t_prune(ctx, level, out, stream);
