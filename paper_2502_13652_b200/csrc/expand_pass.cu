@@ -240,12 +240,12 @@ struct CtaRange {
   }
 };
 
-// The cells of a row: in shared memory where there is room for those of all rows inside the CTA's range (`near`, else null), in the
-// workspace for a row that it shares.  fp32 rows only: eight levels of 320 rows of 128256 tokens (with the acceptance) 403 -> 397 us; the
-// bf16 stream, which has no time to spare, loses by the other kind of store (640 rows 465 -> 468).
+// NEAR: the cells of a row inside the CTA's range are in shared memory, those of a row that it shares in the workspace.  For fp32 rows where a
+// CTA has two rows or more: eight levels of 320 rows of 128256 tokens (with the acceptance) 403 -> 396 us; 90 rows of 23862, all of them
+// shared, 111 -> 120.  The bf16 stream, which has no time to spare, loses by the other kind of store (640 rows 465 -> 468).
 template <bool BF16, bool TOPM>
 __device__ __forceinline__ uint32_t *cells_of_row(const PassParams &p, uint32_t *near, const CtaRange<TOPM> &cr, const RowShape<BF16> &rs, int a) {
-  return near && a >= cr.in0 && a < cr.in1 ? near + (size_t)(a - cr.in0) * rs.words * 32 : p.cells + (size_t)a * rs.words * 32;
+  return a >= cr.in0 && a < cr.in1 ? near + (size_t)(a - cr.in0) * rs.words * 32 : p.cells + (size_t)a * rs.words * 32;
 }
 
 // ---------------------------------------------------------------- completing a row
@@ -291,7 +291,7 @@ __device__ __forceinline__ unsigned reached(const float (&v)[N], float x) {
 // maxima reach a filter, in order, elements in token order 32 at a time; the filter rises to just above the K-th value.  The maxima are
 // taken whole here: with the rounded ones every chunk of a masked fp32 row stays in question (four levels of 320 rows of
 // 128256 values, six of them finite: 2085 us, so 223).
-template <bool BF16>
+template <bool BF16, bool NEAR>
 __device__ __noinline__ int select_in_order(const PassParams &p, PairShared *ws, const char *row, const uint32_t *cells, int a, float floor) {
   constexpr int kWords = 8;                         // words of cells of a lane at a time
   constexpr int kBatch = 16;                        // elements of a lane in flight
@@ -305,7 +305,7 @@ __device__ __noinline__ int select_in_order(const PassParams &p, PairShared *ws,
 #pragma unroll
     for (int i = 0; i < kWords; ++i) {
       const size_t at = ((size_t)a * rs.words + w0 + i) * 32 + lane;
-      two[i] = w0 + i < rs.words ? (BF16 ? p.cells[at] : cells[(w0 + i) * 32 + lane]) : 0xFF80FF80u;
+      two[i] = w0 + i < rs.words ? (NEAR ? cells[(w0 + i) * 32 + lane] : p.cells[at]) : 0xFF80FF80u;
       low[i] = !BF16 && w0 + i < rs.words ? p.cell_low[at] : 0u;
     }
 #pragma unroll
@@ -401,13 +401,13 @@ __device__ __forceinline__ int gather_keys(PairShared *ws, const char *row, cons
 // is a chain of dependent steps, so loads are issued in batches, as early as their addresses are known.
 
 // The K largest.
-template <bool BF16>
+template <bool BF16, bool NEAR>
 __device__ __forceinline__ void complete_keys(const PassParams &p, PairShared *ws, const uint32_t *row_cells, int a, int b, int j) {
   constexpr int kBatch = 32;                        // words of its column that a lane holds at a time: 64 chunks
   const RowShape<BF16> rs(p.V);
   const int lane = threadIdx.x & 31, K = p.K;
   const char *row = row_pointer(p, b, j, BF16 ? 2 : 4);
-  const uint32_t *cells = (BF16 ? p.cells + (size_t)a * rs.words * 32 : row_cells) + lane;
+  const uint32_t *cells = (NEAR ? row_cells : p.cells + (size_t)a * rs.words * 32) + lane;
   uint32_t v[kBatch], cm2 = kLowestBf16x2;
 #pragma unroll
   for (int i = 0; i < kBatch; ++i) v[i] = i < rs.words ? cells[i * 32] : kLowestBf16x2;
@@ -490,7 +490,7 @@ __device__ __forceinline__ void complete_keys(const PassParams &p, PairShared *w
   }
   __syncwarp();
   const int n_keys = n_list <= kListCap ? gather_keys<BF16>(ws, row, rs, p.V, floor, n_list) : -1;
-  const int n_valid = n_keys >= 0 ? rank_pool(ws->pool, n_keys, K) : select_in_order<BF16>(p, ws, row, row_cells, a, floor);
+  const int n_valid = n_keys >= 0 ? rank_pool(ws->pool, n_keys, K) : select_in_order<BF16, NEAR>(p, ws, row, row_cells, a, floor);
   const size_t slot = (size_t)b * p.rows_per_seq_max + j;
   for (int i = lane; i < K; i += 32) p.row_keys[slot * K + i] = ws->pool[i];
   if (lane == 0) {
@@ -661,7 +661,7 @@ __device__ __forceinline__ float stream_chunk(uint4 (&q)[kGroups][4], const uint
 }
 
 // One warp's stream: every kStreamWarps-th chunk of the CTA's work order (TOPM: a contiguous part of it).
-template <bool BF16, bool TOPM>
+template <bool BF16, bool TOPM, bool NEAR>
 __device__ __forceinline__ void stream(const PassParams &p, CtaShared *cs, const int *s_off, uint32_t *near, const RowShape<BF16> &rs, const CtaRange<TOPM> &cr) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = cr.u1 - cr.u0, step = TOPM ? 1 : kStreamWarps;
@@ -743,7 +743,7 @@ __device__ __forceinline__ void stream(const PassParams &p, CtaShared *cs, const
     if (C2T_IN_BOUNDS(u, p.n_chunks, p.status)) {
       uint32_t *word = p.cells + ((size_t)a * rs.words + (ch >> 1)) * 32 + lane;
       uint32_t *low = BF16 ? nullptr : p.cell_low + (word - p.cells);
-      if (!BF16) word = cells_of_row(p, near, cr, rs, a) + (ch >> 1) * 32 + lane;
+      if (NEAR) word = cells_of_row(p, near, cr, rs, a) + (ch >> 1) * 32 + lane;
       if (ch + 1 == rs.nc && !(ch & 1)) {            // (no second cell)
         *word = cell_bits(cv, BF16) | (kLowestBf16x2 & 0xFFFF0000u);
         if (!BF16) *low = __float_as_uint(cv) & 0xFFFFu;
@@ -792,7 +792,7 @@ __device__ __forceinline__ bool wait_task(unsigned long long *bar_ptr, int limit
 // A pair's work: the CTA's tasks, one after the other.  A row inside the range is complete when its records are; a
 // shared one if this CTA's part of it was the last.  A row whose records do not come in time is given up: it gets a result
 // that faults its sequence, and nothing of it stays behind for later rows or launches.
-template <bool BF16, bool TOPM>
+template <bool BF16, bool TOPM, bool NEAR>
 __device__ __forceinline__ void complete(const PassParams &p, CtaShared *cs, const int *s_off, uint32_t *near, const RowShape<BF16> &rs, const CtaRange<TOPM> &cr) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pair = warp >> 1, role = warp & 1;
   const int n_tasks = cr.n_tasks();
@@ -818,17 +818,17 @@ __device__ __forceinline__ void complete(const PassParams &p, CtaShared *cs, con
     const int a = cr.task_row(k), b = find_sequence(s_off, p.B, a);
     if (go == kRowBroken) {
       if (role == 0) give_up_row(p, b, a - s_off[b]);
-    } else if (role == 0) complete_keys<BF16>(p, &cs->scratch[pair], BF16 ? nullptr : cells_of_row(p, near, cr, rs, a), a, b, a - s_off[b]);
+    } else if (role == 0) complete_keys<BF16, NEAR>(p, &cs->scratch[pair], NEAR ? cells_of_row(p, near, cr, rs, a) : nullptr, a, b, a - s_off[b]);
     else complete_sums<BF16, TOPM>(p, cr, a, b, a - s_off[b]);
   }
 }
 
 // The pass itself: what every warp of the grid does.
-template <bool BF16, bool TOPM>
+template <bool BF16, bool TOPM, bool NEAR>
 __device__ __forceinline__ void expand_pass_body(const PassParams &p, unsigned char *s_dyn) {
   CtaShared *cs = reinterpret_cast<CtaShared *>(s_dyn);
   int *s_off = reinterpret_cast<int *>(cs->bars() + p.cta_tasks);
-  uint32_t *near = !BF16 && p.near_cells ? reinterpret_cast<uint32_t *>(s_dyn + p.near_cells) : nullptr;
+  uint32_t *near = NEAR ? reinterpret_cast<uint32_t *>(s_dyn + p.near_cells) : nullptr;
   const int n_rows = build_row_offsets(p.counts, p.B, p.rows_per_seq_max, s_off);
   const RowShape<BF16> rs(p.V);
   const CtaRange<TOPM> cr(rs.nc, n_rows * rs.nc);
@@ -847,16 +847,16 @@ __device__ __forceinline__ void expand_pass_body(const PassParams &p, unsigned c
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(cr.task_records(cr.task_row(k))) : "memory");
   }
   if (threadIdx.x == kExpandThreads - 1) cs->task = 0;
-  if (threadIdx.x < kStreamWarps * 32) stream<BF16, TOPM>(p, cs, s_off, near, rs, cr);
+  if (threadIdx.x < kStreamWarps * 32) stream<BF16, TOPM, NEAR>(p, cs, s_off, near, rs, cr);
   else __syncthreads();
-  complete<BF16, TOPM>(p, cs, s_off, near, rs, cr);
+  complete<BF16, TOPM, NEAR>(p, cs, s_off, near, rs, cr);
 }
 
-template <bool BF16, bool TOPM>
+template <bool BF16, bool TOPM, bool NEAR>
 __global__ void __launch_bounds__(kExpandThreads, 1) expand_pass_kernel(const __grid_constant__ PassParams p) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
   chain_enter();
-  expand_pass_body<BF16, TOPM>(p, s_dyn);
+  expand_pass_body<BF16, TOPM, NEAR>(p, s_dyn);
 }
 
 // Expand and prune of a level in one launch, for small batches: the CTA that finishes last (an atomic ticket, nobody
@@ -871,7 +871,7 @@ __global__ void __launch_bounds__(kExpandThreads, 1) expand_prune_kernel(const _
   __shared__ __align__(16) double s_w[kWCount];
   if (threadIdx.x >= kStreamWarps * 32) stage_classifier(t, s_w, threadIdx.x - kStreamWarps * 32, kExpandThreads - kStreamWarps * 32);   // (written at init)
   chain_enter();
-  expand_pass_body<BF16, false>(p, s_dyn);
+  expand_pass_body<BF16, false, false>(p, s_dyn);
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();                                 // this CTA's row results (seen at the barrier), before its ticket
@@ -923,22 +923,23 @@ int c2t_debug_task_wait_limit = kTaskWaitLimit;
 
 // the launch's shared memory and limits
 constexpr size_t kPassSharedBytes = 100 * 1024;        // more than plan_shared's fixed part at the limits of a configuration
-static size_t plan_shared(PassParams &p, int elem_bytes, int grid) {
+static size_t plan_shared(PassParams &p, int elem_bytes, int grid, bool near) {
   p.wait_limit = C2T_TASK_WAIT_LIMIT;
   p.cta_tasks = (int)((long long)p.B * p.rows_per_seq_max / grid) + 4;       // rows inside a CTA's range, and the two it shares
   const size_t fixed = sizeof(CtaShared) + (size_t)p.cta_tasks * sizeof(unsigned long long) + ((size_t)p.B + 1) * sizeof(int);
   const long long nc = row_chunks(p.V, elem_bytes), per_cta = ((long long)p.B * p.rows_per_seq_max * nc + grid - 1) / grid;
   const size_t at = (fixed + 127) & ~(size_t)127, cells = (size_t)(per_cta / nc + 1) * ((nc + 1) / 2) * 128;
-  p.near_cells = elem_bytes == 4 && at + cells <= kPassSharedBytes ? (int)at : 0;
+  p.near_cells = near && elem_bytes == 4 && per_cta >= 2 * nc && at + cells <= kPassSharedBytes ? (int)at : 0;
   return p.near_cells ? at + cells : fixed;
 }
 
 cudaError_t prepare_expand_pass() {
   const int bytes = (int)kPassSharedBytes;
-  cudaError_t e = cudaFuncSetAttribute(expand_pass_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_pass_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_pass_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_pass_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaError_t e = cudaFuncSetAttribute(expand_pass_kernel<true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_pass_kernel<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_pass_kernel<true, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_pass_kernel<false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_pass_kernel<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_prune_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(expand_prune_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   return e;
@@ -955,7 +956,7 @@ cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, con
   if (out) o = *out;
   const RowPlan plan = rows_in_registers(p, dtype, grid);
   if (plan.cluster) return launch_expand_rows_prune(p, t, level, o, dtype, plan, s);
-  size_t smem = plan_shared(p, dtype == C2T_BF16 ? 2 : 4, grid);
+  size_t smem = plan_shared(p, dtype == C2T_BF16 ? 2 : 4, grid, false);
   if (smem < sizeof(PruneShared)) smem = sizeof(PruneShared);
   if (dtype == C2T_BF16)
     return launch_chained(expand_prune_kernel<true>, dim3(grid), dim3(kExpandThreads), smem, s, p, t, level, o);
@@ -965,14 +966,15 @@ cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, con
 cudaError_t launch_expand_pass(PassParams p, int dtype, int grid, cudaStream_t s) {
   const RowPlan plan = rows_in_registers(p, dtype, grid);
   if (plan.cluster) return launch_expand_rows(p, dtype, plan, s);
-  const size_t smem = plan_shared(p, dtype == C2T_BF16 ? 2 : 4, grid);
+  const size_t smem = plan_shared(p, dtype == C2T_BF16 ? 2 : 4, grid, !p.topm_pool);
   const bool bf16 = dtype == C2T_BF16;
   if (p.topm_pool) {                                 // also sets the candidates of Eq. 3 aside
-    if (bf16) return launch_chained(expand_pass_kernel<true, true>, dim3(grid), dim3(kExpandThreads), smem, s, p);
-    return launch_chained(expand_pass_kernel<false, true>, dim3(grid), dim3(kExpandThreads), smem, s, p);
+    if (bf16) return launch_chained(expand_pass_kernel<true, true, false>, dim3(grid), dim3(kExpandThreads), smem, s, p);
+    return launch_chained(expand_pass_kernel<false, true, false>, dim3(grid), dim3(kExpandThreads), smem, s, p);
   }
-  if (bf16) return launch_chained(expand_pass_kernel<true, false>, dim3(grid), dim3(kExpandThreads), smem, s, p);
-  return launch_chained(expand_pass_kernel<false, false>, dim3(grid), dim3(kExpandThreads), smem, s, p);
+  if (p.near_cells) return launch_chained(expand_pass_kernel<false, false, true>, dim3(grid), dim3(kExpandThreads), smem, s, p);
+  if (bf16) return launch_chained(expand_pass_kernel<true, false, false>, dim3(grid), dim3(kExpandThreads), smem, s, p);
+  return launch_chained(expand_pass_kernel<false, false, false>, dim3(grid), dim3(kExpandThreads), smem, s, p);
 }
 
 }  // namespace c2t
