@@ -149,15 +149,6 @@ __device__ RowMerge merge_row_records(const TreeState &t, const c2t_row_record *
   return m;
 }
 
-// 32 bits of a confidence's key: six of its exponent (from 2^-63 up) and 26 of its mantissa, in the same order; 1 for anything smaller.  (Its upper
-// half has 20 of the mantissa: the confidences of a classifier that says about the same of all children were often equal in it.)
-__device__ __forceinline__ unsigned short_key(unsigned long long key) {
-  constexpr unsigned long long kLeast = 0x8000000000000000ull | (unsigned long long)(1023 - 63) << 52;
-  if (key < kLeast) return 1u;
-  const unsigned long long k = ((key - kLeast) >> 26) + 1ull;
-  return k < 0xFFFFFFFFull ? (unsigned)k : 0xFFFFFFFFu;
-}
-
 constexpr int kCapBlock = 128;                 // keys that the frontier cap compares with at a time
 static_assert(kMaxCand % kCapBlock == 0, "");
 // The shared memory of prune_level_body.
@@ -168,9 +159,9 @@ struct PruneShared {
   int fnode[C2T_MAX_FRONTIER];                 // tree id of every frontier node
   int rowfault[C2T_MAX_FRONTIER];
   alignas(16) unsigned long long ckey[kMaxCand + 8];   // confidence of every candidate as an orderable integer, 0 for a dropped one
-  alignas(16) unsigned chi[kMaxCand];           // its short key, 0 for a dropped one, zeros behind the last one up to a whole block of kCapBlock
+  alignas(16) unsigned chi[kMaxCand];           // its upper half, zeros behind the last one up to a whole block of kCapBlock
   int count[32];                               // candidates added and selected, per 32
-  short before[kMaxCand];                      // survivors that come before a candidate (itself among them, where the short keys decide)
+  short before[kMaxCand];                      // survivors that come before a candidate (itself among them, where the upper halves decide)
 };
 // ... and with gathered records, behind it:
 struct GatherShared {
@@ -317,7 +308,7 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
         // (C desc, index asc) as integer compares: an orderable image of C, 0 for a dropped candidate
         const unsigned long long cb = (unsigned long long)__double_as_longlong(C[r]);
         sh.ckey[c] = keep[r] ? (cb ^ ((cb >> 63) ? ~0ull : 0x8000000000000000ull)) : 0ull;
-        sh.chi[c] = keep[r] ? short_key(sh.ckey[c]) : 0u;
+        sh.chi[c] = (unsigned)(sh.ckey[c] >> 32);
         t.cand_token[cbase + c] = tok[r];
         t.cand_lp[cbase + c] = ok ? lp : NAN;
         t.cand_logP[cbase + c] = ok ? logP[r] : NAN;
@@ -330,8 +321,8 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
   }
 
   // ---- second pruning: the F survivors that come first under (C desc, index asc).  kParts threads count what comes before a
-  // candidate, first by the short keys alone, four to a load: where that leaves F candidates they are the ones.  Else
-  // some are equal around the cut, and the whole keys decide (below).
+  // candidate, first by the upper halves of the keys alone, four to a load: where that leaves F candidates they are the ones.  Else
+  // some are equal in it around the cut, and the whole keys decide (below).
   if (n_keep > F) {
     constexpr int kParts = NT >= 512 ? 4 : 2, kLoads = kCapBlock / kParts / 4;
     const int part = tid % kParts;

@@ -337,18 +337,18 @@ def test_streamed_rows_around_chunk_edges(dtype, chunk, n, plus):
 
 
 @pytest.mark.parametrize("B", [2, 60])
-def test_cap_between_confidences_with_equal_short_keys(B):
-    """Sixteen children one unit in the last place of their fp32 logits apart (7e-9 in their probabilities): the 26 mantissa bits by which the
-    frontier cap compares first leave neighbours equal (1.5e-8), so the cap in their middle goes by the whole keys."""
+def test_cap_between_confidences_with_equal_upper_halves(B):
+    """Sixteen children one unit in the last place of their fp32 logits apart (1e-6 in their probabilities): the upper 32 bits of
+    neighbouring confidences are equal, so the frontier cap in their middle goes by the whole keys."""
     V, F, D = 9000, 8, 2
     g = torch.Generator().manual_seed(5)
     draft = []
     for _ in range(D):
-        x = torch.randn(B, F, V, generator=g) * 0.1 - 6.0
+        x = torch.randn(B, F, V, generator=g)
         for b in range(B):
             for j in range(F):
                 at = torch.randperm(V, generator=g)[:16]
-                x[b, j, at] = 0.0625 + torch.arange(16) * 2.0 ** -27
+                x[b, j, at] = 10.0 + 0.31 * j + torch.arange(16) * 2.0 ** -20
         draft.append(x)
     step(B, V, D, 16, F, 12, 0.0, torch.float32, draft=draft, classifier="identity")
 
