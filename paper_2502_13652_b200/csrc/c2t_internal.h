@@ -188,10 +188,10 @@ struct RowPlan {
 };
 struct TreeState;
 
-// tries of a task's barrier in the streaming pass before a pair gives up
+// tries of a barrier in shared memory before the row is given up
 constexpr int kTaskWaitLimit = 1 << 22;
 #ifdef C2T_DEBUG_BOUNDS
-extern "C" int c2t_debug_task_wait_limit;       // tests let the wait run out: then every level takes the pass that waits
+extern "C" int c2t_debug_task_wait_limit;       // tests let the wait run out: then every level takes a pass that waits
 #define C2T_TASK_WAIT_LIMIT c2t_debug_task_wait_limit
 #else
 #define C2T_TASK_WAIT_LIMIT kTaskWaitLimit
@@ -204,19 +204,19 @@ extern "C" int c2t_debug_task_wait_limit;       // tests let the wait run out: t
 // holds two such clusters only while all its SMs are free).
 inline RowPlan row_pass_plan(int vocab, int elem_bytes, long long rows, int sms) {
   RowPlan plan = {0, 0};
-  if (C2T_TASK_WAIT_LIMIT != kTaskWaitLimit) return plan;
   const int vec = 16 / elem_bytes, vpr = (vocab + vec - 1) / vec;
   const int threads = vpr <= kRowCluster * kRowPart / 2 ? kRowThreads / 2 : kRowThreads, part = threads * 8;
   int cluster = 1;
   while (cluster < kRowCluster && (vpr + cluster - 1) / cluster > part) cluster *= 2;
   if ((vpr + cluster - 1) / cluster > part || rows * cluster > (long long)sms * (kRowThreads / threads)) return plan;
   while (cluster < kRowCluster && 2 * cluster * rows <= sms) cluster *= 2;
+  if (C2T_TASK_WAIT_LIMIT != kTaskWaitLimit && cluster == 1) return plan;      // (nothing waits there)
   plan.cluster = cluster;
   plan.threads = threads;
   return plan;
 }
-cudaError_t launch_expand_rows(const PassParams &p, int dtype, RowPlan plan, cudaStream_t s);
-cudaError_t launch_expand_rows_prune(const PassParams &p, const TreeState &t, int level, const c2t_frontier &out, int dtype, RowPlan plan, cudaStream_t s);
+cudaError_t launch_expand_rows(PassParams p, int dtype, RowPlan plan, cudaStream_t s);
+cudaError_t launch_expand_rows_prune(PassParams p, const TreeState &t, int level, const c2t_frontier &out, int dtype, RowPlan plan, cudaStream_t s);
 
 cudaError_t prepare_expand_pass();   // once per device: opt in to the kernel's shared-memory size
 cudaError_t launch_expand_pass(PassParams p, int dtype, int grid, cudaStream_t s);

@@ -25,7 +25,8 @@ constexpr int kRowLoads = kRowPart / kRowThreads;     // vectors of a thread
 constexpr int kRowGroups = 64;                        // at least (and at least the largest K)
 constexpr int kMaxRowGroups = kRowCluster * kMaxRowWarps;
 constexpr int kCtaKeys = 64;                          // keys that a block hands over
-constexpr int kTooMany = 1 << 20;
+constexpr int kTooMany = 1 << 20, kGivenUp = 1 << 24;  // instead of a count: not handed over; the block gives the row up
+constexpr unsigned long long kNotPut = ~0ull;         // no block's best key
 static_assert(kRowGroups >= C2T_MAX_TOPK && kMaxRowGroups >= kRowGroups, "");
 
 // A warp's sums, relative to an integer offset, and how often it holds the row's maximum.
@@ -45,7 +46,7 @@ struct RowShared {
   __align__(16) uint4 again[kMaxRowWarps][kRowLoads]; // per warp: the vectors of a lane that is summed again
   unsigned long long best[2][kRowCluster], warp_best[kMaxRowWarps];
   unsigned floor;                                     // (orderable)
-  int n;
+  int n, lost;
 };
 
 // ---------------------------------------------------------------- clusters
@@ -80,10 +81,10 @@ __device__ __forceinline__ void announce(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 // false if the wait ran out
-__device__ __forceinline__ bool wait_bar(const unsigned long long *bar) {
+__device__ __forceinline__ bool wait_bar(const unsigned long long *bar, int limit) {
   const uint32_t at = (uint32_t)__cvta_generic_to_shared(bar);
   uint32_t done = 0u;
-  for (int i = 0; i < kTaskWaitLimit && !done; ++i)
+  for (int i = 0; i < limit && !done; ++i)
     asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                  : "=r"(done) : "r"(at) : "memory");
   return done != 0u;
@@ -155,7 +156,8 @@ __device__ __forceinline__ void hand_over(RowShared &sh, const uint4 &q, float f
 }
 
 // Rows whose K largest do not come out of a short list (many equal values, few values, most of the row masked, very short rows): K rounds
-// of "the largest key below the last one" over all blocks of the cluster.  Returns the number of keys, in the leading block's pool.
+// of "the largest key below the last one" over all blocks of the cluster.  Returns the number of keys, in the leading block's pool, or
+// (in every block that is here) -1 if a block has given the row up: it does not put a key in the first round.
 template <bool BF16, int NT>
 __device__ __noinline__ int select_by_rounds(RowShared &sh, const RowPart<BF16, NT> &rp, int V, int K, int cluster, int rank) {
   constexpr int N = Vec<BF16>::N;
@@ -195,7 +197,8 @@ __device__ __noinline__ int select_by_rounds(RowShared &sh, const RowPart<BF16, 
     cluster_wait();
     best = 0ull;
     for (int i = 0; i < cluster; ++i) best = sh.best[r & 1][i] > best ? sh.best[r & 1][i] : best;
-    if (best == 0ull) break;                          // (the same in every block)
+    if (best == kNotPut && r == 0) return -1;         // (the same in every block that is here)
+    if (best == 0ull) break;                          // (likewise)
     if (tid == 0) sh.pool[r] = best;
     last = best;
   }
@@ -269,11 +272,23 @@ __device__ __forceinline__ void merge_sums(RowShared &sh, RowResult *out, float 
 
 // ---------------------------------------------------------------- a row
 
+// A block whose wait for the row's result ran out: it knows neither what the others handed over nor what they do now.  They are done, or
+// in the first round of select_by_rounds, or here.  Either way the next cluster barrier is reached by all of them (those that have
+// ended count), and behind it all that they send to this block is on its way: it stays until that has arrived.
+__device__ __noinline__ void leave_row(const RowShared &sh) {
+  cluster_arrive();
+  cluster_wait();
+  wait_bar(&sh.maxima_in, kTaskWaitLimit);
+  wait_bar(&sh.results_in, kTaskWaitLimit);
+  __syncthreads();
+}
+
 // Before the kernel waits for its predecessor: this block's shared memory can be written once the block runs.
 __device__ __forceinline__ void open_row(RowShared &sh, int cluster) {
+  if (threadIdx.x < kRowCluster) sh.best[0][threadIdx.x] = (int)threadIdx.x < cluster ? kNotPut : 0ull;
   if (threadIdx.x == 0) {
     sh.floor = 0u;
-    sh.n = 0;
+    sh.n = sh.lost = 0;
     if (cluster > 1) {
       const uint32_t maxima = (uint32_t)__cvta_generic_to_shared(&sh.maxima_in), results = (uint32_t)__cvta_generic_to_shared(&sh.results_in);
       const int warps = cluster * (int)(blockDim.x >> 5), groups = warps > kRowGroups ? warps : kRowGroups;
@@ -330,9 +345,11 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
     acc.totals(s, u);
   }
   RowSums sums = warp_sums(s, u, c, mt);
-  bool ok = true;
-  if (cluster > 1) ok = wait_bar(&sh.maxima_in);
-  else __syncthreads();
+  if (cluster > 1) {
+    if (!wait_bar(&sh.maxima_in, p.wait_limit)) sh.lost = 1;       // (nothing of the kind is expected) the block gives the row up
+  } else {
+    __syncthreads();
+  }
 
   // ---- the row's maximum, which stays out of them; the floor: the K-th largest of the groups' maxima, the largest value that K of them reach
   float Mf = fmaxf(sh.group[lane], sh.group[32 + lane]);
@@ -367,8 +384,8 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
   }
   __syncthreads();
   if (warp == 0) {
-    const int n = sh.n, c_n = !live || n > kCtaKeys ? kTooMany : n;
-    const int handed = c_n == kTooMany ? 0 : c_n;
+    const int n = sh.n, c_n = sh.lost ? kGivenUp : !live || n > kCtaKeys ? kTooMany : n;
+    const int handed = c_n < kTooMany ? c_n : 0;
     if (cluster > 1) {
       if (lane < cluster) {
         const uint32_t bar = place_in(&sh.results_in, lane);
@@ -415,9 +432,8 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
   }
   __syncwarp();
   if (cluster > 1) {
-    if (__syncthreads_or(!(ok && wait_bar(&sh.results_in)))) {        // (nothing of the kind is expected) the row is given up
-      cluster_arrive();
-      cluster_wait();                                 // (blocks that have ended count)
+    if (__syncthreads_or(!wait_bar(&sh.results_in, p.wait_limit))) {
+      leave_row(sh);
       if (rank == 0 && warp == 0) give_up_row(p, b, j);
       return rank == 0;
     }
@@ -432,9 +448,17 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
     if (r < cluster) total += sh.counts[r];
     upto[r] = total;
   }
-  const bool listed = total <= kPoolCap;              // (the same in every block)
+  const bool listed = total <= kPoolCap;              // (the same in every block that is here)
   int n_valid = 0;
-  if (!listed) n_valid = select_by_rounds<BF16, NT>(sh, rp, p.V, K, cluster, rank);
+  if (!listed) {
+    n_valid = -1;
+    if (total < kGivenUp) n_valid = select_by_rounds<BF16, NT>(sh, rp, p.V, K, cluster, rank);
+    else wait_bar(&sh.maxima_in, kTaskWaitLimit);     // (what is on its way to a block arrives before it ends)
+    if (n_valid < 0) {
+      if (rank == 0 && warp == 0) give_up_row(p, b, j);
+      return rank == 0;
+    }
+  }
   if (rank != 0) return false;
   const size_t slot = (size_t)b * p.rows_per_seq_max + j;
   if (warp == 0) {
@@ -532,14 +556,16 @@ cudaError_t launch_rows(void (*kernel)(KArgs...), dim3 grid, int threads, int cl
 
 }  // namespace
 
-cudaError_t launch_expand_rows(const PassParams &p, int dtype, RowPlan plan, cudaStream_t s) {
+cudaError_t launch_expand_rows(PassParams p, int dtype, RowPlan plan, cudaStream_t s) {
+  p.wait_limit = C2T_TASK_WAIT_LIMIT;
   const dim3 grid(p.rows_bound * plan.cluster, p.B);
   const bool bf16 = dtype == C2T_BF16;
   if (plan.threads == 256) return launch_rows(bf16 ? expand_rows_kernel<true, 256> : expand_rows_kernel<false, 256>, grid, 256, plan.cluster, s, p, plan.cluster);
   return launch_rows(bf16 ? expand_rows_kernel<true, 512> : expand_rows_kernel<false, 512>, grid, 512, plan.cluster, s, p, plan.cluster);
 }
 
-cudaError_t launch_expand_rows_prune(const PassParams &p, const TreeState &t, int level, const c2t_frontier &out, int dtype, RowPlan plan, cudaStream_t s) {
+cudaError_t launch_expand_rows_prune(PassParams p, const TreeState &t, int level, const c2t_frontier &out, int dtype, RowPlan plan, cudaStream_t s) {
+  p.wait_limit = C2T_TASK_WAIT_LIMIT;
   const dim3 grid(p.rows_bound * plan.cluster, p.B);
   const bool bf16 = dtype == C2T_BF16;
   const bool small = t.F * t.K <= plan.threads;       // a candidate per thread

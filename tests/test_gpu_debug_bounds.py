@@ -57,16 +57,21 @@ GIVE_UP = r"""
 import ctypes, sys, torch
 sys.path.insert(0, {root!r}); sys.path.insert(0, {tests!r})
 import paper_2502_13652_b200 as c2t
-from parity_util import gen_inputs, make_configs
+from parity_util import gen_inputs, make_configs, special_rows
 assert c2t.LIB_PATH.endswith("libc2t_debug.so")
 limit = ctypes.c_int.in_dll(c2t.lib(), "c2t_debug_task_wait_limit")
 usual = limit.value
-# rows shared by several CTAs and rows inside one; expand and prune in one launch, in two, with candidates set aside
-for B, V, F, dtype, M in [(1, 32000, 4, torch.float32, 0), (2, 70000, 8, torch.bfloat16, 0), (5, 40000, 8, torch.float32, 0),
-                          (96, 4096, 10, torch.bfloat16, 0), (6, 32000, 8, torch.bfloat16, 64)]:
+# rows shared by several CTAs and rows inside one; expand and prune in one launch, in two, with candidates set aside; the rows of a level
+# streamed or in the registers of clusters, there also rows whose largest are found in rounds over all blocks
+for B, V, F, dtype, M, kind in [(1, 32000, 4, torch.float32, 0, ""), (2, 70000, 8, torch.bfloat16, 0, ""), (5, 40000, 8, torch.float32, 0, ""),
+                                (96, 4096, 10, torch.bfloat16, 0, ""), (6, 32000, 8, torch.bfloat16, 64, ""),
+                                (2, 128256, 20, torch.bfloat16, 0, ""), (40, 40000, 8, torch.float32, 0, ""),
+                                (3, 70000, 5, torch.float32, 0, "two_valued"), (6, 30000, 2, torch.bfloat16, 0, "two_valued")]:
     D, K, N = 4, 6, 20
-    _, cfg = make_configs(B, V, D, K, F, N, 0.3, dtype, M=M)
+    _, cfg = make_configs(B, V, D, K, F, N, 0.3 if not kind else 0.0, dtype, M=M)
     draft, target, root, prefix = gen_inputs(B, V, D, F, c2t.c2t_final_width(cfg), dtype)
+    if kind:
+        draft = [special_rows(kind, B, F, V, dtype) for _ in range(D)]
     draft = [t.cuda() for t in draft]; target = target.cuda(); root = root.cuda(); prefix = prefix.cuda()
     ctx = c2t.Context(cfg)
 
@@ -87,12 +92,23 @@ for B, V, F, dtype, M in [(1, 32000, 4, torch.float32, 0), (2, 70000, 8, torch.b
     assert not any(status) and int(want[0].max()) > 1, status
     out, status = step(usual, usual, 0, usual)         # in the middle of a step
     assert all(s == c2t.ST_INTERNAL for s in status), status
-    step(usual, 1, 2, usual)                           # whatever runs out here
+    for few in ((usual, 1, 2, usual), (3, 8, 20, 50)):  # whatever runs out here
+        step(*few)
     out, status = step(*[usual] * D)
     assert not any(status)
     for a, b in zip(out, want):
         assert torch.equal(a, b)
     ctx.close()
+# levels of these shapes are in registers, one launch each; they stay there when the limit is changed
+ctx = c2t.Context(make_configs(5, 40000, 4, 6, 8, 20, 0.3, torch.float32)[1])
+x = torch.zeros(5, 8, 40000, device="cuda"); ints = torch.zeros(5, dtype=torch.int32, device="cuda")
+for limit.value in (usual, 0):
+    ctx.c2t_begin_step(ints, ints)
+    n = ctx.c2t_launch_count()
+    ctx.c2t_expand_prune_level(0, x)
+    assert ctx.c2t_launch_count() == n + 1, limit.value
+    assert all(s == (c2t.ST_INTERNAL if limit.value == 0 else 0) for s in ctx.c2t_status()[1])
+ctx.close()
 print("given-up rows ok")
 """
 
