@@ -208,42 +208,35 @@ __device__ __noinline__ int select_by_rounds(RowShared &sh, const RowPart<BF16, 
   return r;
 }
 
-// A warp's sums, from its lanes' (s, u) relative to their offsets c; m2 the largest values they come from.  In double precision: a row's
-// sums are mostly a few large elements, which fp32 would round five more times (32000 tokens, scale 4: 1.1e-8 r.m.s. in a probability, so
-// rounded 1.6e-8).
-__device__ __forceinline__ RowSums warp_sums(float s, float u, float c, float m2) {
-  RowSums r;
-  r.offset = offset_of(warp_max(m2));
-  r.equals = 0;
+// Sums (s, u) relative to an offset c, onto a warp's, which have an offset of at most that.  In double precision, as all sums over lanes
+// are: a row's sums are mostly a few large elements, which fp32 would round five more times (32000 tokens, scale 4: 1.1e-8 r.m.s. in a
+// probability, so rounded 1.6e-8).
+__device__ __forceinline__ void add_sums(RowSums &r, float s, float u, float c) {
   const float by = fmaxf(r.offset - c, -2000.f);      // (never positive)
   const double f = pow2_f64(by);
-  r.S = f * (double)s;
-  r.U = f * ((double)u + (double)by * (double)s);
+  r.S += f * (double)s;
+  r.U += f * ((double)u + (double)by * (double)s);
+}
+
+__device__ __forceinline__ void sum_lanes(RowSums &r) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     r.S += __shfl_xor_sync(kFull, r.S, o);
     r.U += __shfl_xor_sync(kFull, r.U, o);
   }
-  return r;
 }
 
-// One lane's vectors, in sh.again, summed again without the row's maximum and its equals, by the whole warp.
+// One lane's vectors, in sh.again, summed again without the row's maximum and its equals: a word by every lane of the warp.
 template <bool BF16>
-__device__ __noinline__ void sum_again(RowShared &sh, float Mf, float *s, float *u, float *c, float *m2, int *equals) {
+__device__ __forceinline__ void sum_again(RowShared &sh, float Mf, RowSums &r) {
   const uint32_t word = reinterpret_cast<const uint32_t *>(sh.again[threadIdx.x >> 5])[threadIdx.x & 31];
   float x0 = BF16 ? __uint_as_float(word << 16) : __uint_as_float(word), x1 = BF16 ? __uint_as_float(word & 0xFFFF0000u) : kLowestF32;
-  *equals += (x0 == Mf) + (x1 == Mf);
+  r.equals += (x0 == Mf) + (x1 == Mf);
   x0 = x0 == Mf ? kLowestF32 : x0;
   x1 = x1 == Mf ? kLowestF32 : x1;
-  const float m = warp_max(fmaxf(x0, x1)), cr = offset_of(m);
-  const float t0 = fmaf(x0, kLog2e, cr), t1 = fmaf(x1, kLog2e, cr), e0 = ex2f(t0), e1 = ex2f(t1);
-  float sr = e0 + e1, ur = fmaf(e0, t0, e1 * t1);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    sr += __shfl_xor_sync(kFull, sr, o);
-    ur += __shfl_xor_sync(kFull, ur, o);
-  }
-  *s = sr; *u = ur; *c = cr; *m2 = m;
+  const float c = offset_of(warp_max(fmaxf(x0, x1)));
+  const float t0 = fmaf(x0, kLog2e, c), t1 = fmaf(x1, kLog2e, c), e0 = ex2f(t0), e1 = ex2f(t1);
+  add_sums(r, BF16 ? e0 + e1 : e0, BF16 ? fmaf(e0, t0, e1 * t1) : e0 * t0, c);
 }
 
 // The warps' sums, merged by one warp of the leading block.
@@ -344,7 +337,9 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
       if (k * NT < rp.part) acc_vector<BF16>(acc, q[k], scale, c2);      // (uniform)
     acc.totals(s, u);
   }
-  RowSums sums = warp_sums(s, u, c, mt);
+  RowSums sums = {0.0, 0.0, offset_of(warp_max(mt)), 0};
+  add_sums(sums, s, u, c);
+  sum_lanes(sums);
   if (cluster > 1) {
     if (!wait_bar(&sh.maxima_in, p.wait_limit)) sh.lost = 1;       // (nothing of the kind is expected) the block gives the row up
   } else {
@@ -403,22 +398,19 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
 
   // ---- the warps' sums; the warp that holds the maximum: such lanes again without it
   if (unsigned left = __ballot_sync(kFull, mt == Mf)) {
-    float m2 = mt, cs = c, sw = s, uw = u;
-    int equals = 0;
+    sums = {0.0, 0.0, offset_of(Mf), 0};
+    if (mt != Mf) add_sums(sums, s, u, c);
     for (; left; left &= left - 1u) {
-      const bool mine = lane == __ffs(left) - 1;
       __syncwarp();
-      if (mine) {
+      if (lane == __ffs(left) - 1) {
 #pragma unroll
         for (int k = 0; k < kRowLoads; ++k) sh.again[warp][k] = q[k];
       }
       __syncwarp();
-      float sr, ur, cr, mr;
-      sum_again<BF16>(sh, Mf, &sr, &ur, &cr, &mr, &equals);
-      if (mine) { sw = sr; uw = ur; cs = cr; m2 = mr; }
+      sum_again<BF16>(sh, Mf, sums);
     }
-    sums = warp_sums(sw, uw, cs, m2);
-    sums.equals = __reduce_add_sync(kFull, equals);
+    sum_lanes(sums);
+    sums.equals = __reduce_add_sync(kFull, sums.equals);
   }
   if (lane == 0) {
     RowSums *record = &sh.sums[rank * kW + warp];

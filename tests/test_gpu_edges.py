@@ -386,3 +386,31 @@ def test_step_in_one_call_equals_single_calls(B, V, dtype):
     for a, b in zip(*got):
         assert torch.equal(a, b)
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_equal_values_in_the_lane_of_the_maximum(dtype):
+    """A row in registers whose finite values all belong to one thread (vectors 256 apart): the maximum, which it sums again without, and
+    n equal others.  A weight may be off by what `ex2.approx` is, but n equal weights are n times one of them: the lane's elements are
+    added in fp32 two at a time, which is exact here, and else in fp64."""
+    V = 131072 if dtype == torch.bfloat16 else 65536   # eight blocks of 256 threads with 8 vectors each
+    vec = 8 if dtype == torch.bfloat16 else 4
+    _, cfg = make_configs(1, V, 1, 4, 1, 0, 0.0, dtype, classifier="identity")
+    ctx = c2t.Context(cfg)
+    record = ctx.new_row_records()[0]
+    zero = torch.zeros(1, dtype=torch.int32, device="cuda")
+    at = torch.tensor([2048 * 2 + 256 * k + 7 for k in range(8)])[:, None] * vec + torch.arange(vec)
+    at = at.flatten().cuda()
+    S = {}
+    for n in [1, 3, 7, 13, 21, 31] + [47, 63] * (vec == 8):
+        x = torch.full((1, 1, V), float("-inf"), dtype=dtype, device="cuda")
+        x[0, 0, at[1:1 + n]] = 1.6875
+        x[0, 0, at[0]] = 3.0
+        ctx.c2t_begin_step(zero, zero)
+        ctx.c2t_expand_level_shard(0, x)
+        ctx.c2t_export_row_records(0, 0, record)
+        S[n] = float(record[0, 0, 8:16].cpu().view(torch.float64))
+    ctx.close()
+    assert abs(S[1] / np.exp(-1.3125) - 1) < 5e-7
+    for n in S:
+        assert abs(S[n] / (n * S[1]) - 1) < 1e-13, (n, S[n] / (n * S[1]) - 1)
