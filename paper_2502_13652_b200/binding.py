@@ -484,6 +484,22 @@ class Context:
             out[name] = self.workspace[off:off + n * esz].view(dt).view(shape)
         return out
 
+    def c2t_decode_step(self, draft_levels: Sequence[torch.Tensor], target: torch.Tensor,
+                        root_tok: torch.Tensor, prefix_len: torch.Tensor, stream=None) -> None:
+        """The whole step in one call of the library; all levels are looked at before the first launch."""
+        assert root_tok.dtype == torch.int32 and prefix_len.dtype == torch.int32
+        assert root_tok.is_cuda and prefix_len.is_cuda and root_tok.numel() == self.B == prefix_len.numel()
+        pointers, strides = (C.c_void_p * self.D)(), (C.c_int64 * (2 * self.D))()
+        rows = [draft_levels[level] for level in range(self.D)] + [target]
+        for level, t in enumerate(rows):
+            assert t.is_cuda and t.dtype == self.cfg.torch_dtype and t.dim() == 3
+            assert t.shape[0] == self.B and t.shape[2] == self.V and t.stride(2) == 1
+            if level < self.D:
+                pointers[level], strides[2 * level], strides[2 * level + 1] = t.data_ptr(), t.stride(0), t.stride(1)
+        step = c2t_step(root_tok.data_ptr(), prefix_len.data_ptr(), pointers, strides, target.data_ptr(), target.stride(0),
+                        target.stride(1), C.pointer(self._frontier_c), C.pointer(self._verify_c), C.pointer(self._accept_c))
+        _check(lib().c2t_decode_step(self._h, C.byref(step), _stream(stream)), "c2t_decode_step")
+
     def c2t_decode_step_host(self, draft_host: Sequence[torch.Tensor], target_host: torch.Tensor,
                              root_host: torch.Tensor, prefix_host: torch.Tensor, results: dict,
                              stage: dict, stream=None) -> None:
@@ -514,19 +530,19 @@ class Context:
     # -- convenience: the call sequence of one decode step on device tensors ---------------
     def decode_step(self, draft_levels: Sequence[torch.Tensor], target: torch.Tensor,
                     root_tok: torch.Tensor, prefix_len: torch.Tensor, stream=None) -> None:
-        assert root_tok.dtype == torch.int32 and prefix_len.dtype == torch.int32
-        assert root_tok.is_cuda and prefix_len.is_cuda and root_tok.numel() == self.B == prefix_len.numel()
-        D, B, V, dtype = self.D, self.B, self.V, self.cfg.torch_dtype
-        pointers, strides = (C.c_void_p * D)(), (C.c_int64 * (2 * D))()
-        for l in range(D):
-            t = draft_levels[l]
+        """A level's rows are looked up when the levels before it have been launched: the device has work at once, and the
+        sequence may run a draft model on the emitted frontier."""
+        L, h, s = lib(), self._h, _stream(stream)
+        B, V, dtype = self.B, self.V, self.cfg.torch_dtype
+        self.c2t_begin_step(root_tok, prefix_len, s)
+        expand_prune, out = L.c2t_expand_prune_level, C.byref(self._frontier_c)
+        for level in range(self.D):
+            t = draft_levels[level]
+            assert t.is_cuda and t.dtype == dtype and t.dim() == 3
             n, _, v = t.shape
             seq, row, one = t.stride()
-            assert t.is_cuda and t.dtype == dtype and n == B and v == V and one == 1
-            pointers[l], strides[2 * l], strides[2 * l + 1] = t.data_ptr(), seq, row
-        n, _, v = target.shape
-        seq, row, one = target.stride()
-        assert target.is_cuda and target.dtype == dtype and n == B and v == V and one == 1
-        step = c2t_step(root_tok.data_ptr(), prefix_len.data_ptr(), pointers, strides, target.data_ptr(), seq, row,
-                        C.pointer(self._frontier_c), C.pointer(self._verify_c), C.pointer(self._accept_c))
-        _check(lib().c2t_decode_step(self._h, C.byref(step), _stream(stream)), "c2t_decode_step")
+            assert n == B and v == V and one == 1
+            _check(expand_prune(h, level, t.data_ptr(), seq, row, out, s), "c2t_expand_prune_level")
+        self.c2t_prune(FINAL, s)
+        self.c2t_build_verify(s)
+        self.c2t_accept(target, s)

@@ -369,8 +369,10 @@ def test_step_in_one_call_equals_single_calls(B, V, dtype):
     draft = [rows(t) for t in draft]; target = rows(target); root = root.cuda(); prefix = prefix.cuda()
     ctx = c2t.Context(cfg)
     got = []
-    for single in (False, True):
-        if single:
+    for single in (False, True, None):
+        if single is None:
+            ctx.c2t_decode_step(draft, target, root, prefix)
+        elif single:
             ctx.c2t_begin_step(root, prefix)
             for l in range(D):
                 ctx.c2t_expand_level(l, draft[l]); ctx.c2t_prune(l)
@@ -383,8 +385,8 @@ def test_step_in_one_call_equals_single_calls(B, V, dtype):
         got.append([t.clone() for t in list(ctx.verify.values()) + list(ctx.accepted.values()) + list(ctx.frontier.values())] +
                    [v["tree_n"].clone(), torch.where(live, v["tree_logP"], 0.0), torch.where(live, v["tree_C"], 0.0)])
     assert ctx.c2t_status()[0] == 0 and int(got[0][-3].max()) > 1
-    for a, b in zip(*got):
-        assert torch.equal(a, b)
+    for a, b, c in zip(*got):
+        assert torch.equal(a, b) and torch.equal(a, c)
     ctx.close()
 
 

@@ -211,3 +211,47 @@ def test_workspace_has_no_pool_where_nothing_is_set_aside(lib):
     view = binding.c2t_view()
     assert lib.c2t_get_view(ctx.h, C.byref(view)) == c2t.OK and view.topm_from_pass
     ctx.close()
+
+
+class Rows:
+    """As much of a CUDA tensor as a call's checks look at."""
+    is_cuda, dtype = True, c2t.Config(1, 8).torch_dtype
+
+    def __init__(self, *shape):
+        self.shape = shape
+
+    def dim(self):
+        return len(self.shape)
+
+    def stride(self, i=None):
+        s = (self.shape[1] * self.shape[2], self.shape[2], 1)
+        return s if i is None else s[i]
+
+    def data_ptr(self):
+        return 4096
+
+
+def test_decode_step_launches_a_level_before_it_looks_at_the_next(monkeypatch):
+    """The device has work while the rest is looked at, and a sequence of levels may run a draft model on the frontier emitted so far."""
+    import torch
+    log = []
+
+    class Recorder:
+        def __getattr__(self, name):
+            return lambda *a: log.append((name,) + (tuple(a[1:2]) if "expand" in name or name == "c2t_prune" else ())) or 0
+
+    class Levels:
+        def __getitem__(self, level):
+            log.append(("rows", level))
+            return Rows(2, 4, 64)
+
+    monkeypatch.setattr(binding, "lib", lambda: recorder)
+    recorder = Recorder()
+    ctx = object.__new__(binding.Context)
+    ctx.cfg, ctx._h, ctx.B, ctx.D, ctx.V = c2t.Config(2, 64), None, 2, 3, 64
+    ctx._frontier_c, ctx._verify_c, ctx._accept_c = binding.c2t_frontier(), binding.c2t_verify(), binding.c2t_accept_out()
+    ints = Rows(1, 1, 2)
+    ints.dtype, ints.numel = torch.int32, lambda: 2
+    ctx.decode_step(Levels(), Rows(2, 5, 64), ints, ints, stream=0)
+    assert log == [("c2t_begin_step",)] + [x for l in range(3) for x in (("rows", l), ("c2t_expand_prune_level", l))] + \
+        [("c2t_prune", c2t.FINAL), ("c2t_build_verify",), ("c2t_accept",)]
