@@ -399,7 +399,7 @@ int c2t_expand_prune_level(c2t_ctx *ctx, int level, const void *logits_dev, int6
   const TreeState &t = ctx->t;
   // One launch where a level is small: few sequences, or long rows in registers (80 rows of 32000 bf16 tokens: 14.3 us a level in two
   // launches, 12.8 in one).  Short rows, and candidates for which a block's threads do not suffice, leave the pruning too much of the time.
-  const RowPlan rows = row_pass_plan(t.V, (int)ctx->elem_bytes, (long long)t.B * rows_bound(t, level), ctx->grid_expand);
+  const RowPlan rows = row_pass_plan(t.V, (int)ctx->elem_bytes, (long long)t.B * rows_bound(t, level), t.K, ctx->grid_expand);
   const bool small = t.B <= C2T_FUSED_MAX_BATCH ||
                      (rows.cluster > 0 && t.V * (long long)ctx->elem_bytes >= kFusedRowBytes && t.F * t.K <= rows.threads);
   if (!small || (t.entropy_top_m > 0 && t.entropy_top_m < t.V)) {

@@ -202,14 +202,19 @@ extern "C" int c2t_debug_task_wait_limit;       // tests let the wait run out: t
 // 256 threads take 8 us more than streamed, 32 of fp32 in 256 blocks of 512 6 us more; 80 rows of 32000 in 160 blocks 4 us less per level.
 // Blocks of 512 threads in clusters of eight where those of 256 would do: 16 rows of 128256 19 us per level instead of 14 (a GPC
 // holds two such clusters only while all its SMs are free).
-inline RowPlan row_pass_plan(int vocab, int elem_bytes, long long rows, int sms) {
+// And only rows that give data to 1.5 K of the groups whose maxima make the floor, so that few elements reach the K-th of those;
+// for the same reason no more blocks to a row than it has vectors for their threads.  With less data the K largest are found in rounds:
+// five levels of 3 sequences of 1000 bf16 tokens, K = 10, with eight blocks to a row 123 us, with one 45 (streamed 52); of one sequence of
+// 500, K = 16, 139 us, streamed 58.
+inline RowPlan row_pass_plan(int vocab, int elem_bytes, long long rows, int K, int sms) {
   RowPlan plan = {0, 0};
   const int vec = 16 / elem_bytes, vpr = (vocab + vec - 1) / vec;
   const int threads = vpr <= kRowCluster * kRowPart / 2 ? kRowThreads / 2 : kRowThreads, part = threads * 8;
+  if (vpr < 6 * K) return plan;                         // (a group of a single block is four of its threads)
   int cluster = 1;
   while (cluster < kRowCluster && (vpr + cluster - 1) / cluster > part) cluster *= 2;
   if ((vpr + cluster - 1) / cluster > part || rows * cluster > (long long)sms * (kRowThreads / threads)) return plan;
-  while (cluster < kRowCluster && 2 * cluster * rows <= sms) cluster *= 2;
+  while (cluster < kRowCluster && 2 * cluster * rows <= sms && vpr >= 2 * cluster * threads) cluster *= 2;
   if (C2T_TASK_WAIT_LIMIT != kTaskWaitLimit && cluster == 1) return plan;      // (nothing waits there)
   plan.cluster = cluster;
   plan.threads = threads;

@@ -948,7 +948,7 @@ cudaError_t prepare_expand_pass() {
 // How the pass in registers (row_pass.cu) takes the level, if it does.
 static RowPlan rows_in_registers(const PassParams &p, int dtype, int sms) {
   if (p.topm_pool) return RowPlan{0, 0};
-  return row_pass_plan(p.V, dtype == C2T_BF16 ? 2 : 4, (long long)p.B * p.rows_bound, sms);
+  return row_pass_plan(p.V, dtype == C2T_BF16 ? 2 : 4, (long long)p.B * p.rows_bound, p.K, sms);
 }
 
 cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, const c2t_frontier *out, int dtype, int grid, cudaStream_t s) {

@@ -103,3 +103,9 @@ cudaError_t launch_export_best(const TreeState &, int, unsigned long long *, cud
 cudaError_t launch_lazy_walk_round(const TreeState &, int, const c2t_accept_out *, const unsigned long long *, int, cudaStream_t s) { return launched("lazy_walk", s); }
 cudaError_t launch_export_lazy_best(const TreeState &, int, unsigned long long *, cudaStream_t s) { return launched("export_lazy_best", s); }
 }  // namespace c2t
+
+extern "C" void fake_row_plan(int vocab, int elem_bytes, long long rows, int K, int sms, int *cluster, int *threads) {
+  const c2t::RowPlan plan = c2t::row_pass_plan(vocab, elem_bytes, rows, K, sms);
+  *cluster = plan.cluster;
+  *threads = plan.threads;
+}

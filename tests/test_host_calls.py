@@ -255,3 +255,27 @@ def test_decode_step_launches_a_level_before_it_looks_at_the_next(monkeypatch):
     ctx.decode_step(Levels(), Rows(2, 5, 64), ints, ints, stream=0)
     assert log == [("c2t_begin_step",)] + [x for l in range(3) for x in (("rows", l), ("c2t_expand_prune_level", l))] + \
         [("c2t_prune", c2t.FINAL), ("c2t_build_verify",), ("c2t_accept",)]
+
+
+@pytest.mark.parametrize("elem", [2, 4])
+@pytest.mark.parametrize("K", [1, 4, 10, 16, 32])
+def test_rows_in_registers_have_data_for_the_floor(lib, elem, K):
+    """The floor is the K-th largest maximum of 64 groups of threads (or as many as there are warps).  Where fewer than K groups have data
+    it is no floor at all, and where hardly more have most of the row may reach it: then the K largest are found in K rounds."""
+    cluster, threads = C.c_int(), C.c_int()
+    taken = set()
+    for V in list(range(1, 3000, 53)) + [2003, 4000, 8000, 16000, 16384, 16385, 32000, 65536, 65537, 128256, 131072, 262144]:
+        for rows in (1, 2, 3, 5, 9, 12, 18, 37, 74, 148, 296, 297):
+            lib.fake_row_plan(V, elem, C.c_longlong(rows), K, 148, C.byref(cluster), C.byref(threads))
+            if not cluster.value:
+                continue
+            taken.add(V)
+            c, t = cluster.value, threads.value
+            vectors = -(-V * elem // 16)
+            part = -(-vectors // c)
+            assert part <= 8 * t and rows * c * t <= 148 * 512
+            groups = max(64, c * t // 32)
+            width = c * t // groups                     # threads of a group
+            with_data = sum(-(-min(t, max(0, min(part, vectors - r * part))) // width) for r in range(c))
+            assert with_data >= min(groups, 1.5 * K), (V, rows, c, t, with_data)
+    assert {4000, 16000, 32000, 65536} <= taken
