@@ -164,10 +164,10 @@ __device__ __noinline__ int select_by_rounds(RowShared &sh, const RowPart<BF16, 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint4 q[kRowLoads];
   rp.load(q, V);
-  unsigned long long last = ~0ull;
+  unsigned long long last = ~0ull, best = 0ull;
   int r = 0;
   for (; r < K; ++r) {
-    unsigned long long best = 0ull;
+    best = 0ull;
 #pragma unroll
     for (int k = 0; k < kRowLoads; ++k) {
       const int v = rp.v0 + k * NT + tid;
@@ -197,11 +197,11 @@ __device__ __noinline__ int select_by_rounds(RowShared &sh, const RowPart<BF16, 
     cluster_wait();
     best = 0ull;
     for (int i = 0; i < cluster; ++i) best = sh.best[r & 1][i] > best ? sh.best[r & 1][i] : best;
-    if (best == kNotPut && r == 0) return -1;         // (the same in every block that is here)
-    if (best == 0ull) break;                          // (likewise)
+    if (best + 1ull <= 1ull) break;                   // nothing left, or not put (the same in every block that is here)
     if (tid == 0) sh.pool[r] = best;
     last = best;
   }
+  if (best == kNotPut) return -1;                     // (that was the first round)
   __syncthreads();
   for (int i = r + tid; i < K; i += NT) sh.pool[i] = 0ull;
   __syncthreads();
