@@ -43,7 +43,7 @@ __device__ __forceinline__ void stage_classifier(const TreeState &t, double *w, 
 __device__ __noinline__ double exp_shared(double x) { return exp(x); }
 
 // Confidence of one child (Eq. 4): two-layer FFN on (P, H, d), ReLU, sigmoid.
-//   The hidden units are taken kBatch at a time, without a branch and with all of a batch's loads first: one after the other they are a
+//   The hidden units are taken kHiddenBatch at a time, without a branch and with all of a batch's loads first: one after the other they are a
 // chain of loads, additions and a comparison each (89 cycles per unit; the classification of a level 1.3 -> 0.6 us).
 __device__ __forceinline__ double classify(int hidden, const double *w, double P, double H, double d) {
   double z[kHiddenBatch] = {w[kW0], 0.0, 0.0, 0.0};
@@ -158,10 +158,11 @@ struct PruneShared {
   double fchat[C2T_MAX_FRONTIER];              // its smallest confidence on the path from the root
   int fnode[C2T_MAX_FRONTIER];                 // tree id of every frontier node
   int rowfault[C2T_MAX_FRONTIER];
-  alignas(16) unsigned long long ckey[kMaxCand + 8];   // confidence of every candidate as an orderable integer, 0 for a dropped one
+  alignas(16) unsigned long long ckey[kMaxCand + 2];   // confidence of every candidate as an orderable integer, 0 for a dropped one
   alignas(16) unsigned chi[kMaxCand];           // its upper half, zeros behind the last one up to a whole block of kCapBlock
   int count[32];                               // candidates added and selected, per 32
-  short before[kMaxCand];                      // survivors that come before a candidate (itself among them, where the upper halves decide)
+  int next, n_equal;                           // first_of_equals: the smallest reach above the cap, candidates that have it
+  short reach[kMaxCand];                       // survivors whose upper halves are at or above a candidate's
 };
 // ... and with gathered records, behind it:
 struct GatherShared {
@@ -181,25 +182,47 @@ __device__ __forceinline__ void row_stats(const TreeState &t, const RowResult &r
   if (r.fault) atomicOr(&t.status[b], r.fault);
 }
 
-// The candidates that come before each one under (C desc, index asc), by their whole keys.  Called by all threads; ends with a barrier.
-template <int NT>
-__device__ __noinline__ void rank_whole_keys(PruneShared &sh, int nc) {
-  const int tid = threadIdx.x;
-  for (int c0 = 0; c0 < nc; c0 += NT / 4) {       // four threads to a candidate, two keys to a load
-    const int c = c0 + (tid >> 2);
-    const unsigned long long kc = c < nc ? sh.ckey[c] : 0ull, kc1 = kc + 1ull;      // (a key is never all ones)
+// Where the upper halves leave less than F selected: the candidates of the next larger reach, all with the same upper half, share the room that
+// is left by lower half and index.  `have` are selected; kept: which of the thread's candidates survive (a bit per round).  Returns
+// which of them are among the first.  Called by all threads (sh.n_equal and sh.next are as at the level's start).
+template <int NT, int ROUNDS>
+__device__ __noinline__ unsigned first_of_equals(PruneShared &sh, unsigned kept, int have, int F) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  unsigned least = 0x7FFFu;
+#pragma unroll
+  for (int r = 0; r < ROUNDS; ++r) {
+    const unsigned reach = kept >> r & 1u ? (unsigned)sh.reach[tid + r * NT] : 0u;
+    if (reach > (unsigned)F && reach < least) least = reach;
+  }
+  least = __reduce_min_sync(kFullMask, least);
+  if (lane == 0) atomicMin(&sh.next, (int)least);
+  __syncthreads();
+  const int next = sh.next, n = next - have;
+  unsigned long long key[ROUNDS];
+#pragma unroll
+  for (int r = 0; r < ROUNDS; ++r) {
+    const int c = tid + r * NT;
+    key[r] = (kept >> r & 1u) && sh.reach[c] == next ? sh.ckey[c] << 32 | (0xFFFFFFFFu - (unsigned)c) : 0ull;
+  }
+  __syncthreads();                                // the keys are free now: the list takes their place
+#pragma unroll
+  for (int r = 0; r < ROUNDS; ++r)
+    if (key[r]) sh.ckey[atomicAdd(&sh.n_equal, 1)] = key[r];
+  if (tid == 0) sh.ckey[n] = 0ull;
+  __syncthreads();
+  unsigned first = 0u;
+#pragma unroll
+  for (int r = 0; r < ROUNDS; ++r) {
+    if (!key[r]) continue;
     int before = 0;
 #pragma unroll 4
-    for (int o = 2 * (tid & 3); o < nc; o += 8) {                                   // (zeros behind the last key)
+    for (int o = 0; o < n; o += 2) {
       const ulonglong2 k = *reinterpret_cast<const ulonglong2 *>(&sh.ckey[o]);
-      before += k.x >= (o < c ? kc : kc1);
-      before += k.y >= (o + 1 < c ? kc : kc1);
+      before += (k.x > key[r]) + (k.y > key[r]);
     }
-    before += __shfl_xor_sync(kFullMask, before, 1);
-    before += __shfl_xor_sync(kFullMask, before, 2);
-    if ((tid & 3) == 0 && c < nc) sh.before[c] = (short)before;
+    first |= (unsigned)(before < F - have) << r;
   }
-  __syncthreads();
+  return first;
 }
 
 // NT: threads of the CTA; b: the sequence; w: the classifier's staged weights.  records == nullptr: the rows come from
@@ -275,6 +298,7 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
     sh.flogP[jf] = flogP;
     sh.fchat[jf] = fchat;
   }
+  if (tid == 0) { sh.next = 0x7FFF; sh.n_equal = 0; }
   __syncthreads();
 
   // ---- features and confidence, a thread per candidate child
@@ -289,7 +313,6 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
     const int c = tid + r * NT;
     keep[r] = false;
     if (r * NT < nc) {                            // (uniform)
-      if (c >= nc && c < nc + 8) sh.ckey[c] = 0ull;
       if (c < nc) {
         const int j = (int)((unsigned)c * per_k >> 16);
         float x;
@@ -320,16 +343,18 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
     sel[r] = keep[r];
   }
 
-  // ---- second pruning: the F survivors that come first under (C desc, index asc).  kParts threads count what comes before a
-  // candidate, first by the upper halves of the keys alone, four to a load: where that leaves F candidates they are the ones.  Else
-  // some are equal in it around the cut, and the whole keys decide (below).
+  // ---- second pruning: the F survivors that come first under (C desc, index asc).  kParts threads count the survivors at or above a
+  // candidate by the upper halves of the keys, four to a load.  Where no more than F of them are, it is selected; those that share the
+  // next larger count have equal upper halves and share what is left: the usual case where K > F, whose cut falls among one row's children (of
+  // ever smaller joint probabilities: their keys share 35 to 60 bits).  Five levels of 9 x 23862 fp32 tokens, K = 10, 12, 14, 16, F = 10: 92, 97,
+  // 106, 106 us; ranked a second time by whole keys where the halves do not decide 92, 102, 120, 121; by whole keys alone 99, 102, 117, 121.
   if (n_keep > F) {
     constexpr int kParts = NT >= 512 ? 4 : 2, kLoads = kCapBlock / kParts / 4;
     const int part = tid % kParts;
     for (int c0 = 0; c0 < nc; c0 += NT / kParts) {
       const int c = c0 + tid / kParts;
       const unsigned kc = c < nc ? sh.chi[c] : 0xFFFFFFFFu;
-      int reach = 0;                                // candidates at or above it, itself among them
+      int n_reach = 0;                              // (itself among them)
 #pragma unroll 1
       for (int o = 0; o < nc; o += kCapBlock) {
 #pragma unroll 1
@@ -345,17 +370,17 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
             more[2] += k[i].z >= kc;
             more[3] += k[i].w >= kc;
           }
-          reach += (more[0] + more[1]) + (more[2] + more[3]);
+          n_reach += (more[0] + more[1]) + (more[2] + more[3]);
         }
       }
 #pragma unroll
-      for (int m = 1; m < kParts; m <<= 1) reach += __shfl_xor_sync(kFullMask, reach, m);
-      if (part == 0 && c < nc) sh.before[c] = (short)reach;
+      for (int m = 1; m < kParts; m <<= 1) n_reach += __shfl_xor_sync(kFullMask, n_reach, m);
+      if (part == 0 && c < nc) sh.reach[c] = (short)n_reach;
     }
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < kRounds; ++r)
-      if (tid + r * NT < nc) sel[r] = keep[r] && sh.before[tid + r * NT] <= F;
+      if (tid + r * NT < nc) sel[r] = keep[r] && sh.reach[tid + r * NT] <= F;
   }
 
   // ---- stable compaction in candidate order; append to the tree, emit the frontier
@@ -373,10 +398,12 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
   };
   int counts = count_up(), total = __reduce_add_sync(kFullMask, counts);
   if (n_keep > F && (total >> 16) != F) {           // (uniform)
-    rank_whole_keys<NT>(sh, nc);
+    unsigned kept = 0u;
 #pragma unroll
-    for (int r = 0; r < kRounds; ++r)
-      if (tid + r * NT < nc) sel[r] = keep[r] && sh.before[tid + r * NT] < F;
+    for (int r = 0; r < kRounds; ++r) kept |= (unsigned)keep[r] << r;
+    const unsigned first = first_of_equals<NT, kRounds>(sh, kept, total >> 16, F);
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) sel[r] = sel[r] || (first >> r & 1u);
     counts = count_up();
     total = __reduce_add_sync(kFullMask, counts);
   }

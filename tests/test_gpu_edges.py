@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+import c2t_inputs
 import oracle
 import paper_2502_13652_b200 as c2t
 from parity_util import gen_inputs, make_configs, run_and_compare
@@ -338,19 +339,61 @@ def test_streamed_rows_around_chunk_edges(dtype, chunk, n, plus):
 
 @pytest.mark.parametrize("B", [2, 60])
 def test_cap_between_confidences_with_equal_upper_halves(B):
-    """Sixteen children one unit in the last place of their fp32 logits apart (1e-6 in their probabilities): the upper 32 bits of
-    neighbouring confidences are equal, so the frontier cap in their middle goes by the whole keys."""
+    """Sixteen children whose fp32 logits of 0.5 to 1 are one unit in the last place apart (6e-8 in their probabilities): the upper 32 bits of
+    neighbouring confidences, 20 of the mantissa, are equal, so the lower ones decide the frontier cap in their middle."""
     V, F, D = 9000, 8, 2
     g = torch.Generator().manual_seed(5)
     draft = []
     for _ in range(D):
-        x = torch.randn(B, F, V, generator=g)
+        x = torch.randn(B, F, V, generator=g) - 6.0
         for b in range(B):
             for j in range(F):
                 at = torch.randperm(V, generator=g)[:16]
-                x[b, j, at] = 10.0 + 0.31 * j + torch.arange(16) * 2.0 ** -20
+                x[b, j, at] = 0.5 + 0.06 * j + torch.arange(16) * 2.0 ** -24
         draft.append(x)
     step(B, V, D, 16, F, 12, 0.0, torch.float32, draft=draft, classifier="identity")
+
+
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+@pytest.mark.parametrize("B,V,K,F", [(2, 23862, 14, 10), (60, 23862, 14, 10), (2, 9000, 32, 32), (30, 9000, 32, 32), (20, 9000, 12, 10),
+                                     (2, 128256, 16, 20)])
+def test_cap_takes_the_first_by_confidence_and_index(B, V, K, F, sign):
+    """Several levels with K above F or near it: joint probabilities shrink from level to level, and a row's children have confidences that
+    share up to all of their upper bits.  What is selected must be the F first under (C desc, index asc), by the confidences that the
+    kernels themselves wrote; with sign -1 the larger ones have the larger index.  The two launches at a level and the one that does both."""
+    D = 4
+    w1, b1, w2, b2 = c2t_inputs.classifier_weights(16, seed=0)
+    _, cfg = make_configs(B, V, D, K, F, 40, 0.0, torch.float32, weights=(w1, b1, sign * w2, b2))
+    draft, _, root, prefix = gen_inputs(B, V, D, F, 8, torch.float32, device="cuda")
+    pad = -(-V // 4) * 4
+    draft = [torch.nn.functional.pad(t.cuda(), (0, pad - V))[:, :, :V] for t in draft]
+    ctx = c2t.Context(cfg)
+    undecided = turned = 0
+    for two in (False, True):
+        ctx.c2t_begin_step(root.cuda(), prefix.cuda())
+        for l in range(D):
+            if two:
+                ctx.c2t_expand_level(l, draft[l]); ctx.c2t_prune(l)
+            else:
+                ctx.c2t_expand_prune_level(l, draft[l])
+            view = ctx.c2t_get_view()
+            n, flags, C = (view[k].cpu().numpy() for k in ("cand_n", "cand_flags", "cand_C"))
+            for b in range(B):
+                m = n[b]
+                keep, c = (flags[b, :m] & 1) != 0, C[b, :m]
+                assert m > 0 and keep.all()
+                order = np.lexsort((np.arange(m), -c))
+                want = np.zeros(m, dtype=bool)
+                want[order[:F]] = True
+                assert np.array_equal(want, (flags[b, :m] & 2) != 0), (l, b)
+                if m > F:
+                    upper = c.view(np.uint64) >> np.uint64(32)
+                    undecided += upper[order[F - 1]] == upper[order[F]]
+                    by_upper = np.lexsort((np.arange(m), -upper.astype(np.int64)))
+                    turned += set(by_upper[:F]) != set(order[:F])
+    ctx.close()
+    if K > F:
+        assert undecided > B and (turned > 0 or sign > 0), (undecided, turned)
 
 
 @pytest.mark.parametrize("B,V,dtype", [(1, 32000, torch.float32), (5, 9001, torch.bfloat16), (40, 20000, torch.bfloat16)])
