@@ -379,7 +379,7 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
   }
   __syncthreads();
   if (warp == 0) {
-    const int n = sh.n, c_n = sh.lost ? kGivenUp : !live || n > kCtaKeys ? kTooMany : n;
+    const int n = sh.n, most = cluster > 1 ? kCtaKeys : kPoolCap, c_n = sh.lost ? kGivenUp : !live || n > most ? kTooMany : n;
     const int handed = c_n < kTooMany ? c_n : 0;
     if (cluster > 1) {
       if (lane < cluster) {
@@ -389,9 +389,8 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
       }
       const uint32_t bar = place_in(&sh.results_in, 0);
       for (int i = lane; i < handed; i += 32) send(place_in(&sh.keys[rank][i], 0), sh.pool[i], bar);
-    } else {
-      for (int i = lane; i < handed; i += 32) sh.keys[0][i] = sh.pool[i];
-      if (lane == 0) sh.counts[0] = c_n;
+    } else if (lane == 0) {
+      sh.counts[0] = c_n;                             // (the keys are where they are ranked)
     }
     __syncwarp();
   }
@@ -455,7 +454,7 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
   const size_t slot = (size_t)b * p.rows_per_seq_max + j;
   if (warp == 0) {
     if (listed) {
-      for (int i = lane; i < total; i += 32) {
+      for (int i = lane; cluster > 1 && i < total; i += 32) {
         int r = 0, before = 0;
 #pragma unroll
         for (int k = 0; k < kRowCluster; ++k)

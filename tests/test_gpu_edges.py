@@ -337,6 +337,19 @@ def test_streamed_rows_around_chunk_edges(dtype, chunk, n, plus):
     step(160, n * chunk + plus, 2, 2, 2, 4, 0.0, dtype, classifier="identity")
 
 
+@pytest.mark.parametrize("dtype,V", [(torch.bfloat16, 4099), (torch.float32, 2050), (torch.bfloat16, 30000)])
+def test_equal_largest_values_around_what_a_block_lists(dtype, V):
+    """40 to 146 equal largest values in a row: a row of one block lists 128 keys, the blocks of a cluster 64 each and 128 together."""
+    B, K = 75, 6
+    g = torch.Generator().manual_seed(7)
+    x = torch.randn(B, 1, V, generator=g)
+    for b in range(B):
+        n = 40 + b + (32 if b >= 40 else 0)
+        at = torch.randperm(V // 4 if b % 3 == 0 else V, generator=g)[:n]
+        x[b, 0, at] = 20.0
+    step(B, V, 1, K, 1, 0, 0.0, dtype, draft=[x.to(dtype)], classifier="identity")
+
+
 @pytest.mark.parametrize("B", [2, 60])
 def test_cap_between_confidences_with_equal_upper_halves(B):
     """Sixteen children whose fp32 logits of 0.5 to 1 are one unit in the last place apart (6e-8 in their probabilities): the upper 32 bits of
