@@ -159,7 +159,7 @@ int rows_bound(const TreeState &t, int level) {
   return bound < t.F ? (int)bound : t.F;
 }
 
-constexpr long long kFusedRowBytes = 32768;            // half of what a block of 512 threads holds
+constexpr long long kFusedRowBytes = 32768;            // (c2t_expand_prune_level)
 
 // the expand pass of a level over rows of `vocab` tokens (the whole vocabulary, or one shard of it)
 PassParams expand_params(const TreeState &t, int level, const void *logits, int64_t seq_stride, int64_t row_stride, int vocab) {
@@ -397,8 +397,10 @@ int c2t_expand_prune_level(c2t_ctx *ctx, int level, const void *logits_dev, int6
                            const c2t_frontier *out, void *stream) {
   if (!ctx || !logits_dev) return C2T_EINVAL;
   const TreeState &t = ctx->t;
-  // One launch where a level is small: few sequences, or long rows in registers (80 rows of 32000 bf16 tokens: 14.3 us a level in two
-  // launches, 12.8 in one).  Short rows, and candidates for which a block's threads do not suffice, leave the pruning too much of the time.
+  // One launch where a level is small: few sequences, or long rows in registers.  On the device one or two launches are alike there, to 0.2 us
+  // of a level of 9 (in a graph; 3 to 12 sequences of 32000 bf16 tokens 8.8, 9.5, 9.8 us in one, 8.7, 9.4, 9.9 in two), and a launch less is 2.5 us
+  // less for the caller.  Below kFusedRowBytes two stay: one is within 0.3 us for 3 and 6 sequences, from 12 on 0.1 to 0.5 us better.  Where
+  // a block's threads do not suffice for the candidates two are better: 3 sequences of 32000, K = 16, F = 24, 12.4 us in one, 11.3 in two.
   const RowPlan rows = row_pass_plan(t.V, (int)ctx->elem_bytes, (long long)t.B * rows_bound(t, level), t.K, ctx->grid_expand);
   const bool small = t.B <= C2T_FUSED_MAX_BATCH ||
                      (rows.cluster > 0 && t.V * (long long)ctx->elem_bytes >= kFusedRowBytes && t.F * t.K <= rows.threads);

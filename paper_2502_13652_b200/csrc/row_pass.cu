@@ -477,9 +477,10 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
 
 // ---------------------------------------------------------------- kernels
 
-// Block x = (row slot, place in the cluster), y = sequence.
+// Block x = (row slot, place in the cluster), y = sequence.  (row_pass_plan leaves an SM 512 threads of them; with the 64 registers that 1024
+// would allow, code spills: 28 sequences of 16000 bf16 tokens 13.3 us a level, so 10.4, 3 of 32000 9.6, so 8.7.)
 template <bool BF16, int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) expand_rows_kernel(const __grid_constant__ PassParams p, int cluster) {
+__global__ void __launch_bounds__(NT, 512 / NT) expand_rows_kernel(const __grid_constant__ PassParams p, int cluster) {
   __shared__ RowShared sh;
   chain_release();
   open_row(sh, cluster);
