@@ -918,6 +918,10 @@ int row_chunks(int vocab, int elem_bytes) {
 #ifdef C2T_DEBUG_BOUNDS
 extern "C" {
 int c2t_debug_task_wait_limit = kTaskWaitLimit;
+// blocks of a row in registers, 0 where the level is streamed: for tests that are about one of the two
+int c2t_debug_row_cluster(int vocab, int elem_bytes, long long rows, int K, int sms) {
+  return c2t::row_pass_plan(vocab, elem_bytes, rows, K, sms).cluster;
+}
 }
 #endif
 

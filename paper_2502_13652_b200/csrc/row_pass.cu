@@ -320,8 +320,8 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
   for (int o = 1; o < width; o <<= 1) g = fmaxf(g, __shfl_xor_sync(kFull, g, o));
   const int to = lane & (width - 1), at = (rank * kW + warp) * (32 / width) + lane / width;
   if (cluster > 1) {
-    if (to < cluster) send(place_in(&sh.group[at], to), __float_as_uint(g), place_in(&sh.maxima_in, to));
-  } else if (to == 0) {
+    if (to < cluster && C2T_IN_BOUNDS(at, groups, p.status)) send(place_in(&sh.group[at], to), __float_as_uint(g), place_in(&sh.maxima_in, to));
+  } else if (to == 0 && C2T_IN_BOUNDS(at, groups, p.status)) {
     sh.group[at] = g;
   }
 
@@ -388,7 +388,8 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
         send(place_in(&sh.counts[rank], lane), (uint32_t)c_n, bar);
       }
       const uint32_t bar = place_in(&sh.results_in, 0);
-      for (int i = lane; i < handed; i += 32) send(place_in(&sh.keys[rank][i], 0), sh.pool[i], bar);
+      for (int i = lane; i < handed; i += 32)
+        if (C2T_IN_BOUNDS(i, kCtaKeys, p.status)) send(place_in(&sh.keys[rank][i], 0), sh.pool[i], bar);
     } else if (lane == 0) {
       sh.counts[0] = c_n;                             // (the keys are where they are ranked)
     }
@@ -411,7 +412,7 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
     sum_lanes(sums);
     sums.equals = __reduce_add_sync(kFull, sums.equals);
   }
-  if (lane == 0) {
+  if (lane == 0 && C2T_IN_BOUNDS(rank * kW + warp, kRowCluster * kMaxRowWarps, p.status)) {
     RowSums *record = &sh.sums[rank * kW + warp];
     if (cluster > 1) {
       const uint32_t bar = place_in(&sh.results_in, 0);
@@ -452,6 +453,7 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
   }
   if (rank != 0) return false;
   const size_t slot = (size_t)b * p.rows_per_seq_max + j;
+  if (!C2T_IN_BOUNDS(slot, (size_t)p.B * p.rows_per_seq_max, p.status)) return true;
   if (warp == 0) {
     if (listed) {
       for (int i = lane; cluster > 1 && i < total; i += 32) {
@@ -459,7 +461,7 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
 #pragma unroll
         for (int k = 0; k < kRowCluster; ++k)
           if (upto[k] <= i) { r = k + 1; before = upto[k]; }
-        sh.pool[i] = sh.keys[r][i - before];
+        if (C2T_IN_BOUNDS(r, cluster, p.status) && C2T_IN_BOUNDS(i - before, kCtaKeys, p.status)) sh.pool[i] = sh.keys[r][i - before];
       }
       __syncwarp();
       n_valid = rank_pool(sh.pool, total, K);
@@ -478,7 +480,7 @@ __device__ __forceinline__ bool expand_row(const PassParams &p, RowShared &sh, i
 // ---------------------------------------------------------------- kernels
 
 // Block x = (row slot, place in the cluster), y = sequence.  (row_pass_plan leaves an SM 512 threads of them; with the 64 registers that 1024
-// would allow, code spills: 28 sequences of 16000 bf16 tokens 13.3 us a level, so 10.4, 3 of 32000 9.6, so 8.7.)
+// would allow, code spills: 28 sequences of 16000 bf16 tokens 13.3 us a level, so 10.8, 3 of 32000 9.6, so 8.7.)
 template <bool BF16, int NT>
 __global__ void __launch_bounds__(NT, 512 / NT) expand_rows_kernel(const __grid_constant__ PassParams p, int cluster) {
   __shared__ RowShared sh;
@@ -512,6 +514,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) expand_rows_prune_kernel(const _
   int n = p.counts[b];
   if (cluster > 1) cluster_wait();
   n = n < p.rows_per_seq_max ? n : p.rows_per_seq_max;
+  if (n > 0 && !C2T_IN_BOUNDS(n - 1, p.rows_bound, p.status)) n = p.rows_bound;      // (or its last row would never be counted)
   if (j >= n && !(n <= 0 && j == 0)) return;
   if (n > 0) {
     if (!expand_row<BF16, NT>(p, sh.row, b, j, cluster, rank)) return;

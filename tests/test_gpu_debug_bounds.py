@@ -23,13 +23,23 @@ cases = [(2, 32000, 5, 10, 10, 40, 0.5, torch.bfloat16, {{}}),
          (3, 5004, 4, 6, 5, 18, 0.5, torch.float32, {{}}),
          (1, 16384, 3, 32, 32, 100, 0.5, torch.bfloat16, dict(hidden=64, wseed=4)),
          (1, 128256, 4, 8, 16, 40, 0.3, torch.bfloat16, {{}}),
-         (2, 4096, 5, 4, 4, 7, 0.0, torch.float32, dict(classifier="identity", tree_add="all"))]
+         (2, 4096, 5, 4, 4, 7, 0.0, torch.float32, dict(classifier="identity", tree_add="all")),
+         # rows in registers: parts of a vector, one vector more than a block, than eight, than blocks of 256 threads hold
+         (2, 1, 2, 1, 1, 3, 0.0, torch.float32, {{}}), (3, 40, 2, 3, 3, 6, 0.0, torch.bfloat16, dict(classifier="identity")),
+         (1, 8193, 3, 5, 6, 12, 0.0, torch.float32, dict(classifier="identity")), (1, 65537, 3, 5, 6, 12, 0.0, torch.float32, dict(classifier="identity")),
+         (90, 16385, 1, 4, 1, 0, 0.0, torch.bfloat16, dict(classifier="identity")),
+         # streamed: in one launch, in two, rows shared by several CTAs and rows inside one, fp32 cells in either place
+         (2, 128256, 3, 20, 20, 40, 0.5, torch.bfloat16, {{}}), (3, 140001, 2, 6, 2, 9, 0.0, torch.float32, dict(classifier="identity")),
+         (160, 2053, 2, 2, 2, 4, 0.0, torch.bfloat16, dict(classifier="identity")), (160, 2053, 2, 2, 2, 4, 0.0, torch.float32, dict(classifier="identity"))]
 for B, V, D, K, F, N, beta, dtype, kw in cases:
     ocfg, gcfg = make_configs(B, V, D, K, F, N, beta, dtype, **kw)
     Nw = c2t.c2t_final_width(gcfg)
     draft, target, root, prefix = gen_inputs(B, V, D, F, Nw, dtype)
-    rep = run_and_compare(ocfg, gcfg, draft, target, root, prefix)
-    assert rep.status_bits == 0, rep.status_bits
+    pad = -(-V // 8) * 8
+    rows = lambda t: torch.nn.functional.pad(t.cuda(), (0, pad - V))[:, :, :V]
+    for fused in (False, True):
+        rep = run_and_compare(ocfg, gcfg, draft, target, root, prefix, draft_dev=[rows(t) for t in draft], target_dev=rows(target), fused=fused)
+        assert rep.status_bits == 0, rep.status_bits
 for kind in ("rising", "uniform", "neg_inf"):
     B, V, D, K, F, N = 2, 20000, 3, 5, 4, 12
     ocfg, gcfg = make_configs(B, V, D, K, F, N, 0.0, torch.bfloat16, classifier="identity")
