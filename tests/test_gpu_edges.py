@@ -1,4 +1,4 @@
-"""GPU parity at the edges of the kernels' tiles and dispatch rules: chunks of the expand pass, the K for which it takes its
+"""GPU parity at the edges of the kernels' tiles and dispatch rules: chunks of the expand pass, rows in registers and rows that are streamed, the K for which it takes its
 bound from half columns, its selection in order, the sizes of the lazy walk's clusters, the rerank of large trees, the short
 and long rows of the arg-max pass, the mask's 16-byte vectors, the host step."""
 import numpy as np
@@ -8,7 +8,7 @@ import torch
 import c2t_inputs
 import oracle
 import paper_2502_13652_b200 as c2t
-from parity_util import gen_inputs, make_configs, run_and_compare
+from parity_util import gen_inputs, make_configs, run_and_compare, special_rows
 
 pytestmark = pytest.mark.gpu
 
@@ -472,3 +472,77 @@ def test_equal_values_in_the_lane_of_the_maximum(dtype):
     assert abs(S[1] / np.exp(-1.3125) - 1) < 5e-7
     for n in S:
         assert abs(S[n] / (n * S[1]) - 1) < 1e-13, (n, S[n] / (n * S[1]) - 1)
+
+
+def blocks_of_a_row(V, dtype, rows, K):
+    """How the level's rows are cut: blocks per row in registers, or 0 where they are streamed."""
+    import ctypes
+    from paper_2502_13652_b200 import build
+    plan = ctypes.CDLL(build.build(debug_bounds=True)).c2t_debug_row_cluster
+    plan.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
+    return plan(V, 2 if dtype == torch.bfloat16 else 4, rows, K, torch.cuda.get_device_properties(0).multi_processor_count)
+
+
+def streamed_row(kind, V, b, dtype):
+    g = torch.Generator().manual_seed(b)
+    if isinstance(kind, float):                        # one value but for a few, just above it too
+        x = torch.full((V,), kind)
+        at = torch.randperm(V, generator=g)[:b % 6 + 3]
+        x[at] = 20.0 + torch.arange(b % 6 + 3)
+        if kind > -1e30 and dtype == torch.float32:
+            up = torch.nextafter(torch.tensor(kind), torch.tensor(100.0))
+            x[V - 1 - 70 * (b % 6)] = up + abs(kind) * 1e-6
+            x[2 * (b % 6)] = up
+    elif kind == "equal":                              # more equal largest values than the pool of a row holds
+        x = torch.randn(V, generator=g)
+        x[::max(1, V // (150 + 9 * (b % 6)))] = 20.0
+    else:
+        x = special_rows(kind, 1, 1, V, torch.float32)[0, 0] + 0.25 * (b % 6)
+    return x.to(dtype)
+
+
+# many short rows in two launches (fp32: cells in shared memory), few long ones (cells in the workspace), two sequences in one launch
+@pytest.mark.parametrize("dtype,B,V", [(torch.bfloat16, 320, 4096), (torch.bfloat16, 300, 20003), (torch.bfloat16, 3, 270000), (torch.bfloat16, 2, 270000),
+                                       (torch.float32, 320, 4096), (torch.float32, 320, 9003), (torch.float32, 3, 140000), (torch.float32, 2, 140000)])
+@pytest.mark.parametrize("kind,K", [(float("-inf"), 10), (-1e9, 10), (0.0, 17), (7.0, 32), ("equal", 6), ("two_valued", 32), ("heavy_ties", 10),
+                                    ("rising", 17), ("late_jump", 16), ("neg_inf", 32)])
+def test_streamed_rows_of_every_kind(dtype, B, V, kind, K):
+    assert blocks_of_a_row(V, dtype, B, K) == 0
+    ocfg, gcfg = make_configs(B, V, 1, K, 1, 0, 0.0, dtype, classifier="identity")
+    pad = -(-V // 8) * 8
+    some = torch.zeros(6, 1, pad, dtype=dtype)
+    for b in range(6):
+        some[b, 0, :V] = streamed_row(kind, V, b, dtype)
+    draft = some[torch.arange(B) % 6].cuda()[:, :, :V]
+    target = torch.zeros(B, c2t.c2t_final_width(gcfg), 8, dtype=dtype, device="cuda").repeat(1, 1, pad // 8)[:, :, :V]
+    ints = torch.zeros(B, dtype=torch.int32)
+    seqs = sorted({0, 1, 2, B // 2, B - 3, B - 2, B - 1} & set(range(B)))
+    rep = run_and_compare(ocfg, gcfg, None, None, ints, ints, seqs=seqs, draft_dev=[draft], target_dev=target, fused=B <= 2)
+    assert rep.status_bits == 0
+
+
+@pytest.mark.parametrize("dtype,B,V", [(torch.bfloat16, 320, 4096), (torch.float32, 320, 4096), (torch.float32, 4, 140000)])
+def test_faults_in_streamed_rows(dtype, B, V):
+    assert blocks_of_a_row(V, dtype, B, 4) == 0
+    _, cfg = make_configs(B, V, 1, 4, 1, 0, 0.0, dtype, classifier="identity")
+    x = torch.randn(B, 1, V, device="cuda").to(dtype)
+    x[1, 0, V - 5] = float("nan"); x[2, 0, 17] = float("inf"); x[3, 0] = float("-inf")
+    ctx = c2t.Context(cfg)
+    ints = torch.zeros(B, dtype=torch.int32, device="cuda")
+    ctx.c2t_begin_step(ints, ints)
+    ctx.c2t_expand_level(0, x); ctx.c2t_prune(0)
+    status = ctx.c2t_status()[1]
+    assert status[:4] == [0, c2t.ST_NAN_LOGIT, c2t.ST_POSINF_LOGIT, c2t.ST_ALL_NEGINF] and not any(status[4:])
+    assert ctx.frontier["count"].tolist() == [1, 0, 0, 0] + [1] * (B - 4)
+    ctx.close()
+
+
+@pytest.mark.parametrize("K,F", [(10, 20), (20, 20), (32, 24)])
+def test_two_sequences_with_streamed_levels_in_one_launch(K, F):
+    """The first level in registers, then more long rows than fit there."""
+    V, dtype = 128256, torch.bfloat16
+    assert blocks_of_a_row(V, dtype, 2, K) > 0 and blocks_of_a_row(V, dtype, 2 * F, K) == 0
+    ocfg, gcfg = make_configs(2, V, 4, K, F, 40, 0.5, dtype)
+    draft, target, root, prefix = gen_inputs(2, V, 4, F, c2t.c2t_final_width(gcfg), dtype)
+    rep = run_and_compare(ocfg, gcfg, draft, target, root, prefix, fused=True)
+    assert rep.status_bits == 0
