@@ -213,6 +213,50 @@ def test_workspace_has_no_pool_where_nothing_is_set_aside(lib):
     ctx.close()
 
 
+def device_step(L, ctx, **change):
+    """Issues a c2t_decode_step; returns its code.  change: fields of the step; levels: {level: (pointer, seq_stride, row_stride)}."""
+    D, V, B = ctx.cfg.max_depth, ctx.cfg.vocab, ctx.cfg.batch
+    rows = [(0x20000000 + l * 0x100000, 4 * V, V) for l in range(D)]
+    for l, r in change.pop("levels", {}).items():
+        rows[l] = r
+    pointers = (C.c_void_p * D)(*[r[0] for r in rows])
+    strides = (C.c_int64 * (2 * D))(*[x for r in rows for x in r[1:]])
+    step = binding.c2t_step(0x1000, 0x2000, pointers, strides, 0x30000000, 16 * V, V, None, None, None)
+    for name, value in change.items():
+        setattr(step, name, value)
+    return L.c2t_decode_step(ctx.h, C.byref(step), C.c_void_p(STREAM))
+
+
+LEVELS = ["expand", "prune"] * 4
+
+
+@pytest.mark.parametrize("change,code,before", [
+    (dict(draft_logits_dev=C.POINTER(C.c_void_p)()), c2t.EINVAL, []), (dict(draft_strides=C.POINTER(C.c_int64)()), c2t.EINVAL, []),
+    (dict(root_tok_dev=None), c2t.EINVAL, []), (dict(prefix_len_dev=None), c2t.EINVAL, []),
+    (dict(levels={0: (None, 16384, 4096)}), c2t.EINVAL, ["begin"]), (dict(levels={2: (None, 16384, 4096)}), c2t.EINVAL, ["begin"] + LEVELS[:4]),
+    (dict(levels={2: (0x20000004, 16384, 4096)}), c2t.EALIGN, ["begin"] + LEVELS[:4]), (dict(levels={1: (0x20000000, 16386, 4096)}), c2t.EALIGN, ["begin"] + LEVELS[:2]),
+    (dict(levels={1: (0x20000000, 16384, 4098)}), c2t.EALIGN, ["begin"] + LEVELS[:2]), (dict(levels={3: (0x20000000, 16384, 4092)}), c2t.EINVAL, ["begin"] + LEVELS[:6]),
+    (dict(levels={3: (0x20000000, -16384, 4096)}), c2t.EINVAL, ["begin"] + LEVELS[:6]),
+    (dict(target_logits_dev=None), c2t.EINVAL, ["begin"] + LEVELS + ["final_prune", "build_verify"]),
+    (dict(target_logits_dev=0x30000008), c2t.EALIGN, ["begin"] + LEVELS + ["final_prune", "build_verify"]),
+    (dict(target_row_stride=4092), c2t.EINVAL, ["begin"] + LEVELS + ["final_prune", "build_verify"]),
+    (dict(), c2t.OK, ["begin"] + LEVELS + ["final_prune", "build_verify", "argmax", "accept_walk"])])
+def test_device_step_stops_at_the_first_call_that_refuses(lib, change, code, before):
+    """With the code of that call, after the launches of those before it; the next step is a whole one."""
+    ctx = Ctx(lib)
+    for what, want, names in ((dict(change), code, before), (dict(), c2t.OK, ["begin"] + LEVELS + ["final_prune", "build_verify", "argmax", "accept_walk"])):
+        lib.fake_reset()
+        assert device_step(lib, ctx, **what) == want
+        assert [c[0] for c in calls(lib)] == names
+    ctx.close()
+
+
+def test_device_step_without_a_step_or_a_context(lib):
+    ctx = Ctx(lib)
+    assert lib.c2t_decode_step(ctx.h, None, None) == c2t.EINVAL and lib.c2t_decode_step(None, None, None) == c2t.EINVAL
+    ctx.close()
+
+
 class Rows:
     """As much of a CUDA tensor as a call's checks look at."""
     is_cuda, dtype = True, c2t.Config(1, 8).torch_dtype
