@@ -240,9 +240,13 @@ struct CtaRange {
   }
 };
 
-// NEAR: the cells of a row inside the CTA's range are in shared memory, those of a row that it shares in the workspace.  For fp32 rows where a
-// CTA has two rows or more: eight levels of 320 rows of 128256 tokens (with the acceptance) 403 -> 396 us; 90 rows of 23862, all of them
-// shared, 111 -> 120.  The bf16 stream, which has no time to spare, loses by the other kind of store (640 rows 465 -> 468).
+// NEAR: the cells of a row inside the CTA's range are in shared memory, those of a row that it shares in the workspace.  For fp32 rows of
+// kNearChunks chunks or more, where a CTA has two rows or more.  Shorter rows lose by it (steps of five levels and the acceptance, cells in
+// shared memory against the workspace: 400 rows of 32000 tokens 145.4 : 143.4 us, of 48000 180.4 : 178.4, of 64000 211.9 : 210.0, of 96000
+// 282.2 : 281.9), long ones gain where a CTA has few (eight levels of 320 rows of 128256 391 : 395, five 295.8 : 296.5, of 480 rows 401.0 : 400.7).
+// With less than two rows a CTA nearly all rows are shared (90 rows of 23862 92.9 : 92.0, 200 of 128256 224 : 221).  The bf16 stream, which has
+// no time to spare, loses by the other kind of store (640 rows 465 -> 468).
+constexpr int kNearChunks = 96;
 template <bool BF16, bool TOPM>
 __device__ __forceinline__ uint32_t *cells_of_row(const PassParams &p, uint32_t *near, const CtaRange<TOPM> &cr, const RowShape<BF16> &rs, int a) {
   return a >= cr.in0 && a < cr.in1 ? near + (size_t)(a - cr.in0) * rs.words * 32 : p.cells + (size_t)a * rs.words * 32;
@@ -933,7 +937,7 @@ static size_t plan_shared(PassParams &p, int elem_bytes, int grid, bool near) {
   const size_t fixed = sizeof(CtaShared) + (size_t)p.cta_tasks * sizeof(unsigned long long) + ((size_t)p.B + 1) * sizeof(int);
   const long long nc = row_chunks(p.V, elem_bytes), per_cta = ((long long)p.B * p.rows_per_seq_max * nc + grid - 1) / grid;
   const size_t at = (fixed + 127) & ~(size_t)127, cells = (size_t)(per_cta / nc + 1) * ((nc + 1) / 2) * 128;
-  p.near_cells = near && elem_bytes == 4 && per_cta >= 2 * nc && at + cells <= kPassSharedBytes ? (int)at : 0;
+  p.near_cells = near && elem_bytes == 4 && nc >= kNearChunks && per_cta >= 2 * nc && at + cells <= kPassSharedBytes ? (int)at : 0;
   return p.near_cells ? at + cells : fixed;
 }
 

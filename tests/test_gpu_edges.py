@@ -501,9 +501,10 @@ def streamed_row(kind, V, b, dtype):
     return x.to(dtype)
 
 
-# many short rows in two launches (fp32: cells in shared memory), few long ones (cells in the workspace), two sequences in one launch
+# many rows in two launches (fp32: the long ones' cells in shared memory, at 96 chunks of 1024 tokens and below), few long ones, two sequences
+# in one launch
 @pytest.mark.parametrize("dtype,B,V", [(torch.bfloat16, 320, 4096), (torch.bfloat16, 300, 20003), (torch.bfloat16, 3, 270000), (torch.bfloat16, 2, 270000),
-                                       (torch.float32, 320, 4096), (torch.float32, 320, 9003), (torch.float32, 3, 140000), (torch.float32, 2, 140000)])
+                                       (torch.float32, 320, 4096), (torch.float32, 300, 97280), (torch.float32, 300, 97281), (torch.float32, 3, 140000), (torch.float32, 2, 140000)])
 @pytest.mark.parametrize("kind,K", [(float("-inf"), 10), (-1e9, 10), (0.0, 17), (7.0, 32), ("equal", 6), ("two_valued", 32), ("heavy_ties", 10),
                                     ("rising", 17), ("late_jump", 16), ("neg_inf", 32)])
 def test_streamed_rows_of_every_kind(dtype, B, V, kind, K):
