@@ -69,7 +69,7 @@ typedef enum { C2T_ADD_FRONTIER = 0, C2T_ADD_ALL_SURVIVORS = 1 } c2t_tree_add;
 #define C2T_MAX_BUDGET    1024
 #define C2T_MAX_TREE      8192   /* nodes per sequence before the Top-N rerank */
 #define C2T_MAX_SHARDS    32     /* vocabulary shards merged by c2t_prune_gathered */
-#define C2T_FUSED_MAX_BATCH 2    /* largest batch for which c2t_expand_prune_level always uses a single launch */
+#define C2T_FUSED_MAX_BATCH 2    /* largest batch for which c2t_expand_prune_level uses a single launch for every level (without entropy_top_m) */
 
 /* per-sequence status bits */
 #define C2T_ST_NAN_LOGIT     1u

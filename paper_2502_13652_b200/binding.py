@@ -340,7 +340,7 @@ class Context:
                                       _stream(stream)), "c2t_expand_level")
 
     def c2t_expand_prune_level(self, level: int, logits: torch.Tensor, stream=None, emit: bool = True) -> None:
-        """c2t_expand_level and c2t_prune of a level as one call (one launch for batches of at most 2 sequences)."""
+        """c2t_expand_level and c2t_prune of a level as one call (one launch for small levels)."""
         assert logits.is_cuda and logits.dtype == self.cfg.torch_dtype and logits.dim() == 3
         assert logits.shape[0] == self.B and logits.shape[2] == self.V and logits.stride(2) == 1
         out = C.byref(self._frontier_c) if emit else None

@@ -199,7 +199,7 @@ extern "C" int c2t_debug_task_wait_limit;       // tests let the wait run out: t
 
 // How a level is cut, if its rows leave an SM no more than 512 threads of them: the smaller blocks where a row fits eight of them, and while
 // half the chip would be idle more of them to a row.  Where the line lies: 64 rows of 128256 bf16 tokens (a step's level 0) in 512 blocks of
-// 256 threads take 8 us more than streamed, 32 of fp32 in 256 blocks of 512 6 us more; 80 rows of 32000 in 160 blocks 4 us less per level.
+// 256 threads take 7 us more than streamed, 32 of fp32 in 256 blocks of 512 6 us more; 80 rows of 32000 in 160 blocks 4 us less per level.
 // Blocks of 512 threads in clusters of eight where those of 256 would do: 16 rows of 128256 19 us per level instead of 14 (a GPC
 // holds two such clusters only while all its SMs are free).
 // And only rows that give data to 1.5 K of the groups whose maxima make the floor, so that few elements reach the K-th of those;
@@ -239,7 +239,7 @@ cudaError_t prepare_accept_lazy();   // once per device
 // the acceptance walk reading only the rows it visits; grid: CTAs of kPassThreads threads that the chip holds
 cudaError_t launch_accept_lazy(const TreeState &t, const void *logits, int64_t seq_stride, int64_t row_stride, const c2t_accept_out *out,
                                int dtype, int grid, cudaStream_t s);
-// expand and prune of a level in one launch (batches of at most C2T_FUSED_MAX_BATCH sequences)
+// expand and prune of a level in one launch (which levels: c2t_expand_prune_level)
 cudaError_t launch_expand_prune(PassParams p, const TreeState &t, int level, const c2t_frontier *out, int dtype,
                                 int grid, cudaStream_t s);
 // ---------------------------------------------------------------- tree state -

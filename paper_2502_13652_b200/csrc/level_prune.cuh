@@ -1,6 +1,6 @@
 // The per-sequence work of a level (Eq. 1, Eq. 4, Alg. 1, Sec. 4.2.2): features, classifier, the two prunings,
 // compaction, tree append, from the results that the expand pass (or the merge of gathered records) has per row.  A device function, so that the pruning kernel
-// (one CTA per sequence) and the expand kernel's last CTA (small batches: expand and prune in one launch) share it.
+// (one CTA per sequence) and the expand kernels that prune in the same launch (by their last CTA, or a sequence's last) share it.
 #pragma once
 
 #include "c2t_internal.h"

@@ -11,10 +11,11 @@
 // elements dealt out to the warp.  So the sums keep fp32 relative accuracy with respect to "everything but the maximum" however peaked the
 // row is.  The threads whose maximum reaches the floor hand their elements over, the leading block ranks the keys and
 // merges the warps' sums in double precision, in a fixed order.
-//   What bounds it: latencies.  Of 9.9 us of a level of 10 rows of 32000 fp32 tokens (clock reads in the kernel, taken once and not kept)
-// the wait for the predecessor takes 0.9, the count 0.35, the loads 0.6, maxima 0.4, sums 0.35, the floor 0.6, what goes between the
-// blocks 0.7, the result 1.4, the count of finished rows 0.7, the pruning 2.6.  Against the streaming pass with the pruning of its time, a step:
-// 1 x 32000 fp32 93 -> 70 us, 1 x 128256 bf16 157 -> 127, 8 x 32000 bf16 143 -> 109, 5 x 32003 fp32 107 -> 84.
+//   What bounds it: latencies.  Of a level of 10 rows of 32000 fp32 tokens (clock reads in the kernel, taken once and not kept, when it took 9.9 us)
+// the wait for the predecessor takes 0.9 us, the count 0.35, the loads 0.6, maxima 0.4, sums 0.35, the floor 0.6, what goes between the
+// blocks 0.7, the result 1.4, the count of finished rows 0.7, the pruning 2.6; the other 1.3 lie outside the block that was read.  Against
+// the streaming pass with the pruning of its time, a step: 1 x 32000 fp32 93 -> 67 us, 1 x 128256 bf16 158 -> 125, 8 x 32000 bf16 142 -> 107,
+// 5 x 32003 fp32 107 -> 81.
 #include "row_sums.cuh"
 
 namespace c2t {
