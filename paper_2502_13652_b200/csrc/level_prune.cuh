@@ -150,7 +150,7 @@ __device__ RowMerge merge_row_records(const TreeState &t, const c2t_row_record *
 }
 
 constexpr int kCapBlock = 128;                 // keys that the frontier cap compares with at a time
-static_assert(kMaxCand % kCapBlock == 0, "");
+static_assert(kMaxCand % kCapBlock == 0 && 256 % kCapBlock == 0, "the last block ends within the threads' last round");
 // The shared memory of prune_level_body.
 struct PruneShared {
   double rowM[C2T_MAX_FRONTIER], rowL[C2T_MAX_FRONTIER], rowH[C2T_MAX_FRONTIER];
@@ -303,7 +303,6 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
 
   // ---- features and confidence, a thread per candidate child
   const int nc = n * K, nc_blocks = (nc + kCapBlock - 1) & ~(kCapBlock - 1);
-  for (int c = nc + tid; c < nc_blocks; c += NT) sh.chi[c] = 0u;
   double C[kRounds], logP[kRounds];
   int tok[kRounds];
   bool keep[kRounds], sel[kRounds];
@@ -313,6 +312,7 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
     const int c = tid + r * NT;
     keep[r] = false;
     if (r * NT < nc) {                            // (uniform)
+      if (c >= nc && c < nc_blocks) sh.chi[c] = 0u;
       if (c < nc) {
         const int j = (int)((unsigned)c * per_k >> 16);
         float x;
