@@ -535,6 +535,7 @@ class Context:
         L, h, s = lib(), self._h, _stream(stream)
         B, V, dtype = self.B, self.V, self.cfg.torch_dtype
         self.c2t_begin_step(root_tok, prefix_len, s)
+        # (a step of nearly empty levels is bound by these calls: nothing is looked up twice)
         expand_prune, out = L.c2t_expand_prune_level, C.byref(self._frontier_c)
         for level in range(self.D):
             t = draft_levels[level]
@@ -542,7 +543,13 @@ class Context:
             n, _, v = t.shape
             seq, row, one = t.stride()
             assert n == B and v == V and one == 1
-            _check(expand_prune(h, level, t.data_ptr(), seq, row, out, s), "c2t_expand_prune_level")
-        self.c2t_prune(FINAL, s)
-        self.c2t_build_verify(s)
+            rc = expand_prune(h, level, t.data_ptr(), seq, row, out, s)
+            if rc:
+                _check(rc, "c2t_expand_prune_level")
+        rc = L.c2t_prune(h, FINAL, None, s)
+        if rc:
+            _check(rc, "c2t_prune")
+        rc = L.c2t_build_verify(h, C.byref(self._verify_c), s)
+        if rc:
+            _check(rc, "c2t_build_verify")
         self.c2t_accept(target, s)
