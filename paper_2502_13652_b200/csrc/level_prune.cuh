@@ -158,7 +158,7 @@ struct PruneShared {
   double fchat[C2T_MAX_FRONTIER];              // its smallest confidence on the path from the root
   int fnode[C2T_MAX_FRONTIER];                 // tree id of every frontier node
   int rowfault[C2T_MAX_FRONTIER];
-  alignas(16) unsigned long long ckey[kMaxCand + 2];   // confidence of every candidate as an orderable integer, 0 for a dropped one
+  alignas(16) unsigned long long ckey[kMaxCand + 2];   // confidence of every candidate as an orderable integer, 0 for a dropped one and behind the last
   alignas(16) unsigned chi[kMaxCand];           // its upper half, zeros behind the last one up to a whole block of kCapBlock
   int count[32];                               // candidates added and selected, per 32
   int next, n_equal;                           // first_of_equals: the smallest reach above the cap, candidates that have it
@@ -312,7 +312,7 @@ __device__ __forceinline__ void prune_level_body(const TreeState &t, int level, 
     const int c = tid + r * NT;
     keep[r] = false;
     if (r * NT < nc) {                            // (uniform)
-      if (c >= nc && c < nc_blocks) sh.chi[c] = 0u;
+      if (c >= nc && c < nc_blocks) { sh.chi[c] = 0u; sh.ckey[c] = 0ull; }
       if (c < nc) {
         const int j = (int)((unsigned)c * per_k >> 16);
         float x;
